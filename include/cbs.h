@@ -174,13 +174,16 @@ cbs_status cbs_hamiltonian_norms(const cbs_hamiltonian *h, double E, double *n_p
 cbs_status cbs_apply(const cbs_hamiltonian *h, int n_sys, const double *z, const double *E,
                      int L, const void *X, void *Y, int dtype, void *stream);
 
-/* Bytes of device workspace cbs_apply_ws needs for n_sys systems of L columns. */
+/* Bytes of device workspace for cbs_apply_ws with n_sys systems of L columns. */
 size_t cbs_apply_workspace_size(const cbs_hamiltonian *h, int n_sys, int L, int dtype);
 
 /* As cbs_apply, with all pointers on the device and caller-provided workspace, so that
  * the call allocates nothing, does not synchronise and can be captured in a CUDA graph:
  * z: DEVICE complex128 [n_sys]; E: DEVICE double [n_sys]; workspace: DEVICE buffer of at
- * least cbs_apply_workspace_size bytes (16-byte aligned), overwritten by the call. */
+ * least cbs_apply_workspace_size bytes (16-byte aligned), overwritten by the call.  In
+ * complex128 a smaller one, down to the projector coefficients alone (n_sys * n_atoms * L *
+ * 4 elements, n_atoms at least 1; 8 instead of 4 with more than 4 projectors per atom), is
+ * accepted and served by the slower FP64 kernels. */
 cbs_status cbs_apply_ws(const cbs_hamiltonian *h, int n_sys, const double *z, const double *E,
                         int L, const void *X, void *Y, int dtype, void *workspace,
                         size_t workspace_bytes, void *stream);
@@ -196,7 +199,8 @@ cbs_status cbs_apply_ws(const cbs_hamiltonian *h, int n_sys, const double *z, co
  * z, E: HOST arrays [n_sys]; X, Y: DEVICE [n_sys][N][L] of type dtype; runs on `stream`
  * and does not synchronise.  L as for cbs_apply, checked before anything is queued.  Sizes
  * whose scratch (about n_sys*L*n_atoms*4*16 bytes in complex128, half that in complex64)
- * exceed the 32 MiB return CBS_EINVAL.  The first call on a device looks up the array's
+ * exceed the 32 MiB return CBS_EINVAL (complex128 sizes above about a quarter of it run on
+ * the slower FP64 kernels).  The first call on a device looks up the array's
  * device address (with that device current); under CUDA's lazy module loading (the
  * default) that first call is also when the 32 MiB are reserved on the device, so make it
  * before a memory pool takes the device's free memory, and before any stream capture.  The

@@ -78,8 +78,7 @@ extern "C" cbs_status cbs_apply(const cbs_hamiltonian *h, int n_sys, const doubl
   if (!apply_supported(h->v, L, dtype, "cbs_apply")) return CBS_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   const HamView &H = h->v;
-  const size_t csz = dtype == CBS_C128 ? sizeof(double2) : sizeof(float2);
-  const size_t dbytes = (size_t)n_sys * (H.n_atoms ? H.n_atoms : 1) * H.np4 * L * csz;
+  const size_t dbytes = apply_ws_bytes(H, n_sys, L, dtype);
   void *scratch = nullptr;
   const size_t sys_bytes = (size_t)n_sys * (sizeof(double2) + sizeof(double));
   CBS_CUDA(cudaMalloc(&scratch, dbytes + sys_bytes + 256));
@@ -92,11 +91,11 @@ extern "C" cbs_status cbs_apply(const cbs_hamiltonian *h, int n_sys, const doubl
   if (e != cudaSuccess) s = cuda_fail(e, "cbs_apply upload");
   if (s == CBS_OK) {
     if (dtype == CBS_C128)
-      s = apply_P<double>(H, n_sys, L, (const double2 *)X, (double2 *)Y, tw, false, Ed, (double2 *)D,
-                          nullptr, st);
+      s = apply_P<double>(H, n_sys, L, (const double2 *)X, (double2 *)Y, tw, false, Ed, D,
+                          dbytes, nullptr, st);
     else
-      s = apply_P<float>(H, n_sys, L, (const float2 *)X, (float2 *)Y, tw, false, Ed, (float2 *)D,
-                         nullptr, st);
+      s = apply_P<float>(H, n_sys, L, (const float2 *)X, (float2 *)Y, tw, false, Ed, D,
+                         dbytes, nullptr, st);
   }
   // the scratch must outlive the kernels: synchronise the stream before freeing it
   cudaError_t e2 = cudaStreamSynchronize(st);
@@ -107,9 +106,7 @@ extern "C" cbs_status cbs_apply(const cbs_hamiltonian *h, int n_sys, const doubl
 
 extern "C" size_t cbs_apply_workspace_size(const cbs_hamiltonian *h, int n_sys, int L, int dtype) {
   if (!h || n_sys < 1 || L < 1) return 0;
-  const HamView &H = h->v;
-  const size_t csz = dtype == CBS_C128 ? sizeof(double2) : sizeof(float2);
-  return (size_t)n_sys * (H.n_atoms ? H.n_atoms : 1) * H.np4 * L * csz;
+  return apply_ws_bytes(h->v, n_sys, L, dtype);
 }
 
 extern "C" cbs_status cbs_apply_ws(const cbs_hamiltonian *h, int n_sys, const double *z, const double *E,
@@ -121,7 +118,7 @@ extern "C" cbs_status cbs_apply_ws(const cbs_hamiltonian *h, int n_sys, const do
   }
   if (dtype != CBS_C128 && dtype != CBS_C64) { set_error("cbs_apply_ws: dtype"); return CBS_EINVAL; }
   if (!apply_supported(h->v, L, dtype, "cbs_apply_ws")) return CBS_EINVAL;
-  if (workspace_bytes < cbs_apply_workspace_size(h, n_sys, L, dtype)) {
+  if (workspace_bytes < apply_coef_bytes(h->v, n_sys, L, dtype)) {
     set_error("cbs_apply_ws: workspace smaller than cbs_apply_workspace_size");
     return CBS_EINVAL;
   }
@@ -129,9 +126,9 @@ extern "C" cbs_status cbs_apply_ws(const cbs_hamiltonian *h, int n_sys, const do
   const HamView &H = h->v;
   if (dtype == CBS_C128)
     return apply_P<double>(H, n_sys, L, (const double2 *)X, (double2 *)Y, (const double2 *)z, false, E,
-                           (double2 *)workspace, nullptr, st);
+                           workspace, workspace_bytes, nullptr, st);
   return apply_P<float>(H, n_sys, L, (const float2 *)X, (float2 *)Y, (const double2 *)z, false, E,
-                        (float2 *)workspace, nullptr, st);
+                        workspace, workspace_bytes, nullptr, st);
 }
 
 // Launch-shape search for the stencil kernel: every admissible (kernel, x-lines per block)
@@ -172,9 +169,9 @@ extern "C" cbs_status cbs_autotune_apply(cbs_hamiltonian *h, int n_sys, int L, i
   float bms = 0.f;
   auto run = [&]() -> cbs_status {
     if (dtype == CBS_C128)
-      return apply_P<double>(H, n_sys, L, (const double2 *)X, (double2 *)Y, tw, false, Ed, (double2 *)D,
+      return apply_P<double>(H, n_sys, L, (const double2 *)X, (double2 *)Y, tw, false, Ed, D, ws,
                              nullptr, st);
-    return apply_P<float>(H, n_sys, L, (const float2 *)X, (float2 *)Y, tw, false, Ed, (float2 *)D,
+    return apply_P<float>(H, n_sys, L, (const float2 *)X, (float2 *)Y, tw, false, Ed, D, ws,
                           nullptr, st);
   };
   do {

@@ -612,17 +612,22 @@ bool apply_supported(const HamView &H, int L, int dtype, const char *who) {
 template <typename R>
 cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *X,
                    typename CT<R>::T *Y, const double2 *twist, bool per_col, const double *E,
-                   typename CT<R>::T *D, const int *sys_active, cudaStream_t st) {
+                   void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st) {
+  typename CT<R>::T *D = (typename CT<R>::T *)ws;
+  if constexpr (sizeof(R) == sizeof(double)) {
+    if (fixed_serves(H, n_sys, L, ws_bytes))
+      return apply_fixed(H, n_sys, L, X, Y, twist, per_col, E, ws, sys_active, st);
+  }
   cbs_status s = launch_proj_gather<R>(H, n_sys, L, X, twist, per_col, D, sys_active, st);
   if (s != CBS_OK) return s;
   return launch_apply<R>(H, n_sys, L, X, Y, twist, per_col, E, D, sys_active, st);
 }
 
 template cbs_status apply_P<double>(const HamView &, int, int, const double2 *, double2 *,
-                                    const double2 *, bool, const double *, double2 *,
+                                    const double2 *, bool, const double *, void *, size_t,
                                     const int *, cudaStream_t);
 template cbs_status apply_P<float>(const HamView &, int, int, const float2 *, float2 *,
-                                   const double2 *, bool, const double *, float2 *,
+                                   const double2 *, bool, const double *, void *, size_t,
                                    const int *, cudaStream_t);
 template cbs_status launch_proj_gather<double>(const HamView &, int, int, const double2 *,
                                                const double2 *, bool, double2 *, const int *,

@@ -1,0 +1,673 @@
+// The complex128 operator apply Y = E X - H(w) X in fixed point (see fixed.cuh for the
+// arithmetic and apply.cu for the operator).  Four kernels:
+//   k_column_max     the largest |component| of every (system, column) over chunks of points,
+//   k_fix_scales     from it the column's scale, with its twist and energy,
+//   k_gather_fixed   D_a = h_a F_a(1/w)^T X per atom, as FP64 and as fixed-point images
+//                    D, w D, w^{-1} D,
+//   k_stencil_fixed  the stencil and the projector scatter.
+// Scratch: D [n_sys][n_atoms][L][4] FP64, then the images [n_sys][3][n_atoms][4][L] as
+// (high, low) word pairs of both components (images of wrap -1, 0, +1), then the scales
+// [n_sys][L], then the chunk maxima [n_sys][chunks][L].
+#include <algorithm>
+#include <type_traits>
+
+#include "fixed.cuh"
+
+namespace cbs {
+
+// What one (system, column) needs besides its vector.
+struct ColumnScale {
+  FixScale f;
+  int base;        // exponent offset of to_fixed
+  long long ef;    // E - diag_kin in the unit of the weights
+  long long pad;
+  double2 w, wi;   // the twist and its inverse
+};
+static_assert(sizeof(ColumnScale) % 16 == 0, "ColumnScale is read in 16-byte pieces");
+
+__device__ __forceinline__ void twist_and_inverse(const double2 *twist, int64_t k, double2 &w, double2 &wi) {
+  w = twist[k];
+  wi = cdiv(make_double2(1.0, 0.0), w);
+}
+
+// Bound by memory: 44 us for 268 MB (32 systems of the 32x32x16 cell, L = 32), 6.1 TB/s.
+// maxhi[s][chunk][c] = max over the chunk's points of the high word of |re|, |im| (the order of
+// non-negative doubles)
+__global__ void k_column_max(int64_t N, int L, int chunk_pts, const double2 *__restrict__ X,
+                             unsigned *__restrict__ maxhi, const int *__restrict__ sys_active) {
+  extern __shared__ unsigned smax[];   // [py][L]
+  const int s = blockIdx.y, c = threadIdx.x, ly = threadIdx.y, py = blockDim.y;
+  if (sys_active && !sys_active[s]) return;
+  const int64_t i0 = (int64_t)blockIdx.x * chunk_pts, i1 = min(N, i0 + chunk_pts);
+  const double2 *Xs = X + (int64_t)s * N * L;
+  unsigned m = 0;
+#pragma unroll 4
+  for (int64_t i = i0 + ly; i < i1; i += py) {
+    const double2 v = Xs[i * L + c];
+    m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+  }
+  smax[ly * L + c] = m;
+  __syncthreads();
+  if (ly == 0) {
+    for (int y = 1; y < py; ++y) m = max(m, smax[y * L + c]);
+    maxhi[((int64_t)s * gridDim.x + blockIdx.x) * L + c] = m;
+  }
+}
+
+// One block per system, one thread per column: the FP64 work of the scales (a division, the
+// conversions) is done here once instead of by every thread of the kernels that use them.
+__global__ void k_fix_scales(const __grid_constant__ HamView H, int L, int chunks, const unsigned *__restrict__ maxhi,
+                             const double2 *__restrict__ twist, int per_col, const double *__restrict__ E,
+                             ColumnScale *__restrict__ scales, const int *__restrict__ sys_active) {
+  const int s = blockIdx.x, c = threadIdx.x;
+  if (sys_active && !sys_active[s]) return;
+  unsigned m = 0;
+#pragma unroll 4
+  for (int k = 0; k < chunks; ++k) m = max(m, maxhi[((int64_t)s * chunks + k) * L + c]);
+  double2 w, wi;
+  twist_and_inverse(twist, per_col ? (int64_t)s * L + c : s, w, wi);
+  ColumnScale o;
+  o.f = fix_scale(H, w, wi, E[s], m);
+  o.base = 1086 + o.f.ex - o.f.Q;
+  o.w = w;
+  o.wi = wi;
+  o.ef = o.f.ok ? round_fixed(E[s] - H.diag_kin, 58 - H.fx_ew) : 0;
+  o.pad = 0;
+  scales[(int64_t)s * L + c] = o;
+}
+
+// FP64 sum of one image of one atom over the entries t0, t0 + step, ...: the columns that
+// fixed point does not serve.
+__device__ __noinline__ void gather_entries_fp64(const HamView *H, int64_t t0, int64_t t1, int step, int L,
+                                                 const double2 *Xc, int image, double2 *out) {
+  double2 acc[4];
+  for (int mu = 0; mu < 4; ++mu) acc[mu] = make_double2(0, 0);
+  for (int64_t t = t0; t < t1; t += step) {
+    if (H->sup_wrap[t] != image) continue;
+    const double2 f = Xc[(int64_t)H->sup_idx[t] * L];
+    for (int mu = 0; mu < H->n_proj; ++mu) {
+      const double p = H->sup_val[t * H->n_proj + mu];
+      acc[mu].x = fma(p, f.x, acc[mu].x);
+      acc[mu].y = fma(p, f.y, acc[mu].y);
+    }
+  }
+  for (int mu = 0; mu < 4; ++mu) out[mu] = acc[mu];
+}
+
+// Bound by integer issue and the latency of the gathered rows: 32 systems of the 32x32x16 cell
+// (40 atoms, L = 32) take 180 us; the FP64 gather, at FP64 issue, 550 us.  84 instructions per
+// entry and column, 24 of them products.
+// One block per (atom, system, group of columns); threadIdx.x a column, threadIdx.y a lane over
+// the atom's support entries.  Per entry: one 16-byte load, two conversions and 3 word
+// products per projector and component.  The projector words are balanced (the low word is
+// signed), so the product of the two low words, left out, has zero mean: it is below 2^-57 of
+// the largest product per entry.
+constexpr int kGatherU = 8;      // entries in flight per thread
+constexpr int kGatherCarry = 2;  // steps of kGatherU entries between carries: |B| grows by less
+                                 // than 2^58.4 per entry
+__global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__ HamView H, int L,
+                                                      const double2 *__restrict__ X,
+                                                      const ColumnScale *__restrict__ scales,
+                                                      double2 *__restrict__ D, int4 *__restrict__ Df,
+                                                      const int *__restrict__ sys_active) {
+  extern __shared__ long long gsm[];
+  const int a = blockIdx.x, s = blockIdx.y;
+  if (sys_active && !sys_active[s]) return;
+  const int cg = blockDim.x, ly = threadIdx.y, py = blockDim.y;
+  const int cx = threadIdx.x;
+  const int c = min((int)(blockIdx.z * cg) + cx, L - 1);
+  const bool own = (int)(blockIdx.z * cg) + cx < L;
+  long long *redA = gsm;                                   // [py][8][cg]
+  long long *redB = redA + (size_t)py * 8 * cg;            // [py][8][cg]
+  double2 *sums = (double2 *)(redB + (size_t)py * 8 * cg); // [4][cg] F_a(1/w)^T X
+  int *seen = (int *)(sums + 4 * cg);                      // [cg] high words met, or-ed
+  const ColumnScale *sc = scales + (int64_t)s * L + c;
+  const FixScale f = sc->f;
+  const int base = sc->base;
+  const double2 *Xc = X + (int64_t)s * H.n * L + c;
+  const char *Xb = (const char *)(X + (int64_t)s * H.n * L);
+  const unsigned row = (unsigned)L * (unsigned)sizeof(double2), col = (unsigned)c * (unsigned)sizeof(double2);
+  const int *gp = H.fx_gptr + 4 * a;
+  if (ly == 0) {
+    seen[cx] = 0;
+    for (int mu = 0; mu < 4; ++mu) sums[mu * cg + cx] = make_double2(0, 0);
+  }
+  __syncthreads();
+  int word = 0;
+  for (int img = 0; img < 3; ++img) {
+    const int t0 = gp[img], t1 = gp[img + 1];
+    if (t0 == t1) continue;
+    long long A[8], B[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) A[k] = B[k] = 0;
+    const int *gi = H.fx_gi + t0 + ly;
+    const int4 *pw = H.fx_gp + 2 * (t0 + ly);
+    int left = (t1 - t0 - ly + py - 1) / py;     // this thread's entries
+    auto fetch = [&](int u) -> double2 { return *(const double2 *)(Xb + ((unsigned)gi[u * py] * row + col)); };
+    auto take = [&](double2 x, const int4 *p) {
+      const int4 p01 = p[0], p23 = p[1];
+      const long long xr = to_fixed(x.x, base, word), xi = to_fixed(x.y, base, word);
+      const int r1 = opaque((int)(xr >> 29)), r0 = opaque((int)xr & 0x1fffffff);
+      const int i1 = opaque((int)(xi >> 29)), i0 = opaque((int)xi & 0x1fffffff);
+      const int p1[4] = {p01.x, p01.z, p23.x, p23.z}, p0[4] = {p01.y, p01.w, p23.y, p23.w};
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu) {
+        madw(A[2 * mu], r1, p1[mu]);
+        madw(B[2 * mu], r1, p0[mu]);
+        madw(B[2 * mu], r0, p1[mu]);
+        madw(A[2 * mu + 1], i1, p1[mu]);
+        madw(B[2 * mu + 1], i1, p0[mu]);
+        madw(B[2 * mu + 1], i0, p1[mu]);
+      }
+    };
+    auto carry = [&]() {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        A[k] += B[k] >> 29;
+        B[k] &= 0x1fffffff;
+      }
+    };
+    int step = 0;
+    for (; left >= kGatherU; left -= kGatherU) {
+      double2 xv[kGatherU];
+#pragma unroll
+      for (int u = 0; u < kGatherU; ++u) xv[u] = fetch(u);
+#pragma unroll
+      for (int u = 0; u < kGatherU; ++u) take(xv[u], pw + 2 * u * py);
+      gi += kGatherU * py;
+      pw += 2 * kGatherU * py;
+      if (++step % kGatherCarry == 0) carry();
+    }
+    carry();
+    for (; left > 0; --left) {
+      take(fetch(0), pw);
+      gi += py;
+      pw += 2 * py;
+    }
+    carry();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      redA[((size_t)ly * 8 + k) * cg + cx] = A[k];
+      redB[((size_t)ly * 8 + k) * cg + cx] = B[k];
+    }
+    __syncthreads();
+    // projector mu of column cx: the image's sum, times w^{-m}
+    for (int mu = ly; mu < 4; mu += py) {
+      long long ar = 0, br = 0, ai = 0, bi = 0;
+      for (int y = 0; y < py; ++y) {
+        ar += redA[((size_t)y * 8 + 2 * mu) * cg + cx];
+        br += redB[((size_t)y * 8 + 2 * mu) * cg + cx];
+        ai += redA[((size_t)y * 8 + 2 * mu + 1) * cg + cx];
+        bi += redB[((size_t)y * 8 + 2 * mu + 1) * cg + cx];
+      }
+      // (A 2^58 + B 2^29) 2^(ex - Q - fp)
+      const double unit = __hiloint2double((1023 + f.ex - f.Q - H.fx_fp + 29) << 20, 0);
+      double2 v = make_double2(fma((double)ar, 536870912.0, (double)br) * unit,
+                               fma((double)ai, 536870912.0, (double)bi) * unit);
+      if (img != 1) v = cmul(img == 2 ? sc->wi : sc->w, v);
+      sums[mu * cg + cx] = cadd(sums[mu * cg + cx], v);
+    }
+    __syncthreads();
+  }
+  if (word) atomicOr(&seen[cx], word);
+  __syncthreads();
+  // columns out of range, or with nothing but small values over this atom: FP64 sums
+  const bool redo = !f.ok || seen[cx] < kFixSmallWord;
+  if (__syncthreads_or(redo)) {
+    double2 *red = (double2 *)gsm;                         // [py][4][cg], the space of redA
+    if (redo && ly == 0)
+      for (int mu = 0; mu < 4; ++mu) sums[mu * cg + cx] = make_double2(0, 0);
+    for (int img = 0; img < 3; ++img) {
+      double2 part[4];
+      if (redo) {
+        gather_entries_fp64(&H, H.sup_ptr[a] + ly, H.sup_ptr[a + 1], py, L, Xc, img - 1, part);
+        for (int mu = 0; mu < 4; ++mu) red[((size_t)ly * 4 + mu) * cg + cx] = part[mu];
+      }
+      __syncthreads();
+      if (redo && ly == 0)
+        for (int mu = 0; mu < 4; ++mu) {
+          double2 v = make_double2(0, 0);
+          for (int y = 0; y < py; ++y) v = cadd(v, red[((size_t)y * 4 + mu) * cg + cx]);
+          if (img != 1) v = cmul(img == 2 ? sc->wi : sc->w, v);
+          sums[mu * cg + cx] = cadd(sums[mu * cg + cx], v);
+        }
+      __syncthreads();
+    }
+  }
+  const double *ha = H.h + (int64_t)a * H.n_proj * H.n_proj;
+  if (!own) return;
+  for (int mu = ly; mu < 4; mu += py) {
+    double2 d = make_double2(0, 0);
+    if (mu < H.n_proj)
+      for (int nu = 0; nu < H.n_proj; ++nu) {
+        const double hv = ha[mu * H.n_proj + nu];
+        const double2 v = sums[nu * cg + cx];
+        d.x = fma(hv, v.x, d.x);
+        d.y = fma(hv, v.y, d.y);
+      }
+    D[(((int64_t)s * H.n_atoms + a) * L + c) * 4 + mu] = d;
+    if (!f.ok) continue;
+    const double2 im[3] = {cmul(sc->wi, d), d, cmul(sc->w, d)};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const long long vr = round_fixed(im[k].x, f.fd), vi = round_fixed(im[k].y, f.fd);
+      Df[((((int64_t)s * 3 + k) * H.n_atoms + a) * 4 + mu) * L + c] =
+          make_int4(balanced_hi(vr), balanced_lo(vr), balanced_hi(vi), balanced_lo(vi));
+    }
+  }
+}
+
+// One output of the FP64 formula (the arithmetic of k_apply_zm<double>).
+__device__ __noinline__ double2 output_fp64(const HamView *H, const double2 *Xc, int L, int ix, int iy, int iz,
+                                            double2 w, double2 wi, double E, const double2 *Dc) {
+  const int nx = H->nx, ny = H->ny, nz = H->nz, nxy = nx * ny;
+  const int pt = (iz * ny + iy) * nx + ix;
+  const double2 x0 = Xc[(int64_t)pt * L];
+  const double dd = (E - H->diag_kin) - H->vloc[pt];
+  double2 acc = make_double2(dd * x0.x, dd * x0.y);
+  for (int k = 1; k <= H->m; ++k) {
+    const int xp = (ix + k) % nx, xm = (ix - k % nx + nx) % nx, yp = (iy + k) % ny, ym = (iy - k % ny + ny) % ny;
+    const double2 a1 = Xc[(int64_t)(pt - ix + xp) * L], a2 = Xc[(int64_t)(pt - ix + xm) * L];
+    const double2 b1 = Xc[(int64_t)(pt + (yp - iy) * nx) * L], b2 = Xc[(int64_t)(pt + (ym - iy) * nx) * L];
+    const int up = iz + k, dn = iz - k;
+    double2 z1 = Xc[(int64_t)(pt + (k - (up >= nz ? nz : 0)) * nxy) * L];
+    double2 z2 = Xc[(int64_t)(pt + ((dn < 0 ? nz : 0) - k) * nxy) * L];
+    if (up >= nz) z1 = cmul(w, z1);
+    if (dn < 0) z2 = cmul(wi, z2);
+    acc.x = fma(-H->wx[k], a1.x + a2.x, acc.x);
+    acc.y = fma(-H->wx[k], a1.y + a2.y, acc.y);
+    acc.x = fma(-H->wy[k], b1.x + b2.x, acc.x);
+    acc.y = fma(-H->wy[k], b1.y + b2.y, acc.y);
+    acc.x = fma(-H->wz[k], z1.x + z2.x, acc.x);
+    acc.y = fma(-H->wz[k], z1.y + z2.y, acc.y);
+  }
+  if (Dc)
+    for (int64_t q = H->pt_ptr[pt]; q < H->pt_ptr[pt + 1]; ++q) {
+      const int2 aw = H->pt_aw[q];
+      const int64_t t = H->pt_ent[q];
+      const double2 *Da = Dc + (int64_t)aw.x * L * 4;
+      double2 v = make_double2(0, 0);
+      for (int mu = 0; mu < H->n_proj; ++mu) {
+        const double p = H->sup_val[t * H->n_proj + mu];
+        v.x = fma(p, Da[mu].x, v.x);
+        v.y = fma(p, Da[mu].y, v.y);
+      }
+      if (aw.y) v = cmul(aw.y > 0 ? w : wi, v);
+      acc = csub(acc, v);
+    }
+  return acc;
+}
+
+struct Fixed2 { long long re, im; };
+
+// sum_k +-n_k s_k as two words: even k enter negative (the signs of c_k alternate)
+struct WeightedSum {
+  long long hi = 0;
+  unsigned long long plus = 0, minus = 0;
+  __device__ __forceinline__ void add(int k, int nk, long long s) {
+    const int s1 = opaque((int)(s >> 32));
+    const unsigned s0 = (unsigned)opaque((int)s);
+    if (k & 1) {
+      madw(hi, s1, nk);
+      madwu(plus, s0, nk);
+    } else {
+      madw(hi, s1, -nk);
+      madwu(minus, s0, nk);
+    }
+  }
+  __device__ __forceinline__ long long shifted(int st) const {   // the sum >> st
+    const long long lo = (long long)(plus - minus);
+    const long long h = hi + (lo >> 32);
+    return (h << (32 - st)) | (long long)((unsigned)lo >> st);
+  }
+};
+
+// The products x * g in words of 31 bits: A 2^62 + B 2^31 + C
+struct Product {
+  long long A = 0, B = 0;
+  unsigned long long C = 0;
+  __device__ __forceinline__ void add(long long x, int g1, int g0) {
+    const int x1 = hi31(x), x0 = lo31(x);
+    madw(A, x1, g1);
+    madw(B, x1, g0);
+    madw(B, x0, g1);
+    madwu(C, x0, g0);
+  }
+  __device__ __forceinline__ long long shifted(int sa) const {   // >> (62 - sa)
+    return (A << sa) + ((B + (long long)(C >> 31)) >> (31 - sa));
+  }
+};
+
+// Projector products in balanced words of 29 bits: A 2^58 + B 2^29 (the product of the low
+// words, of zero mean and below 2^-57 of the largest, is left out).  One entry (4 projectors)
+// adds less than 2^58.6 to |B|: 16 entries between carries.
+struct Scatter {
+  long long A = 0, B = 0;
+  __device__ __forceinline__ void add(int d1, int d0, int p1, int p0) {
+    madw(A, d1, p1);
+    madw(B, d1, p0);
+    madw(B, d0, p1);
+  }
+  __device__ __forceinline__ void carry() {
+    A += B >> 29;
+    B &= 0x1fffffff;
+  }
+  __device__ __forceinline__ long long shifted(int sp) const {   // >> (58 - sp)
+    return (A << sp) + (B >> (29 - sp));
+  }
+};
+
+// Stencil and projector scatter: 664 us on 32 systems of the 32x32x16 cell (L = 32, 16.8 M
+// outputs), of which the stencil is 360; k_apply_zm<double>, at FP64 issue, 2400 us.  About 470
+// instructions per output for the stencil and 110 per covering entry; bound by their issue and,
+// in the scatter, by the latency of its loads (16 warps per SM at 128 registers, of which the
+// z queue takes 36).  8 x 8 x 4 tiles of 256 threads beat 16 x 8 x 4 of 512 (two blocks per SM
+// cover each other's barriers) and 8 x 4 x 8; the columns are cut in fours because the halo,
+// converted once per tile, shrinks with the tile's x-y extent.  A block covers TX x TY lines of CG columns and walks the
+// planes z0 .. z1-1; the plane it is on lies in shared memory with its x-y halo, as
+// fixed-point pairs (two buffers, one barrier per plane), and each thread keeps the 2 MH + 1
+// z neighbours of its point in registers.  The next plane's halo and the plane MH ahead are
+// loaded while the current one is computed.  Offsets inside a plane are 32-bit byte offsets
+// from a base that all threads share.
+template <int MH, int CG, int TX, int TY, bool ISO>
+__global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
+    k_stencil_fixed(const __grid_constant__ HamView H, int L, int groups, int tiles_x, int z_chunk,
+                    const double2 *__restrict__ X, double2 *__restrict__ Y, const double *__restrict__ E,
+                    const ColumnScale *__restrict__ scales,
+                    const double2 *__restrict__ D, const int4 *__restrict__ Df,
+                    const int *__restrict__ sys_active) {
+  constexpr int WX = TX + 2 * MH, WY = TY + 2 * MH, THREADS = CG * TX * TY;
+  constexpr int HALO = 2 * MH * (TX + TY) * CG;
+  constexpr int SLOTS = (HALO + THREADS - 1) / THREADS;
+  constexpr int PLANE = WX * WY * CG;
+  extern __shared__ Fixed2 tile[];   // [2][WY][WX][CG]
+  const int s = blockIdx.z;
+  if (sys_active && !sys_active[s]) return;
+  const int nx = H.nx, ny = H.ny, nz = H.nz;
+  const int g = blockIdx.x % groups, tb = blockIdx.x / groups;
+  const int bx = (tb % tiles_x) * TX, by = (tb / tiles_x) * TY;
+  const int z0 = blockIdx.y * z_chunk, z1 = min(nz, z0 + z_chunk);
+  const int tid = threadIdx.x;
+  const int cl = tid % CG, lx = (tid / CG) % TX, ly = tid / (CG * TX);
+  const int c = min(g * CG + cl, L - 1);
+  const bool own = g * CG + cl < L && bx + lx < nx && by + ly < ny;
+  const int ix = (bx + lx) % nx, iy = (by + ly) % ny;
+  const int line = iy * nx + ix;
+  const int64_t plane_bytes = (int64_t)nx * ny * L * sizeof(double2);
+  const char *Xs = (const char *)(X + (int64_t)s * H.n * L);
+  char *Ys = (char *)(Y + (int64_t)s * H.n * L);
+  const unsigned mine = (unsigned)(line * L + c) * (unsigned)sizeof(double2);
+  auto load = [&](int p, unsigned off) -> double2 { return *(const double2 *)(Xs + p * plane_bytes + off); };
+
+  const ColumnScale *sc = scales + (int64_t)s * L + c;
+  const FixScale f = sc->f;
+  const int base = sc->base;
+  const double2 w = sc->w, wi = sc->wi;
+  const long long ef = sc->ef;
+  auto conv = [&](double2 v) -> Fixed2 { return Fixed2{to_fixed(v.x, base), to_fixed(v.y, base)}; };
+  // this thread's value in plane p of the Bloch-extended field, -nz <= p < 2 nz
+  auto raw = [&](int p) -> double2 { return load(p >= nz ? p - nz : (p < 0 ? p + nz : p), mine); };
+  // halo elements tid, tid + THREADS, ...: 2 MH rows of TX, then 2 MH columns of TY (THREADS is
+  // a multiple of CG, so an element's column is its thread's own)
+  unsigned hoff[SLOTS];
+  int hat[SLOTS];
+#pragma unroll
+  for (int k = 0; k < SLOTS; ++k) {
+    const int h = tid + k * THREADS;
+    const int hp = min(h, HALO - CG + cl) / CG;
+    int px, py;
+    if (hp < 2 * MH * TX) {
+      const int r = hp / TX;
+      px = hp % TX + MH;
+      py = r < MH ? r : r + TY;
+    } else {
+      const int r = (hp - 2 * MH * TX) / TY;
+      py = (hp - 2 * MH * TX) % TY + MH;
+      px = r < MH ? r : r + TX;
+    }
+    int gx = (bx + px - MH) % nx, gy = (by + py - MH) % ny;
+    if (gx < 0) gx += nx;
+    if (gy < 0) gy += ny;
+    hoff[k] = (unsigned)((gy * nx + gx) * L + c) * (unsigned)sizeof(double2);
+    hat[k] = (py * WX + px) * CG + cl;
+  }
+  const int self = ((ly + MH) * WX + lx + MH) * CG + cl;
+
+  Fixed2 q[2 * MH + 1];
+#pragma unroll
+  for (int d = 0; d < 2 * MH; ++d) {
+    double2 v = raw(z0 + d - MH);
+    if (d < MH && z0 < MH) {
+      const double2 t = cmul(wi, v);
+      if (z0 + d - MH < 0) v = t;
+    }
+    if (d > MH && z0 + MH > nz) {
+      const double2 t = cmul(w, v);
+      if (z0 + d - MH >= nz) v = t;
+    }
+    q[d] = conv(v);
+  }
+  double2 head = raw(z0 + MH);
+  tile[self] = q[MH];
+#pragma unroll
+  for (int k = 0; k < SLOTS; ++k) tile[hat[k]] = conv(load(z0, hoff[k]));
+  const bool proj = H.n_atoms > 0;
+  const char *Ds = (const char *)(Df + (int64_t)s * 3 * H.n_atoms * L * 4);
+  const unsigned d_mu = (unsigned)L * (unsigned)sizeof(int4), d_mine = (unsigned)c * (unsigned)sizeof(int4);
+  // the line's tables: entry ranges and V_loc of its planes, one after the other
+  const int *ptr = H.fx_ptr + (int64_t)line * (nz + 1) + z0;
+  const long long *vl = H.fx_v + (int64_t)line * nz + z0;
+  int e0 = 0, e1 = proj ? ptr[0] : 0, e2 = proj ? ptr[1] : 0;
+  // the first entry not yet used (the tables have one spare entry at the end)
+  int img = 0;
+  int4 np01 = make_int4(0, 0, 0, 0), np23 = np01;
+  if (proj) {
+    img = H.fx_img[e1];
+    np01 = H.fx_p[2 * e1];
+    np23 = H.fx_p[2 * e1 + 1];
+  }
+  long long vnext = vl[0];
+  unsigned long long redo = 0;   // planes whose output is left to the FP64 formula
+  // one plane; `twisted`: the plane MH ahead lies in the next cell
+  auto plane = [&](int iz, auto twisted) {
+    const Fixed2 *mid = tile + ((iz - z0) & 1) * PLANE + self;
+    Fixed2 *next = tile + ((iz - z0 + 1) & 1) * PLANE;
+    const bool more = iz + 1 < z1;
+    e0 = e1;
+    e1 = e2;
+    const long long dd = ef - vnext;
+    q[2 * MH] = conv(twisted ? cmul(w, head) : head);
+    double2 hv[SLOTS];
+    if (more) {
+      head = raw(iz + 1 + MH);
+#pragma unroll
+      for (int k = 0; k < SLOTS; ++k) hv[k] = load(iz + 1, hoff[k]);
+      if (proj) e2 = ptr[iz - z0 + 2];
+      vnext = vl[iz - z0 + 1];
+    }
+    __syncthreads();
+    const Fixed2 x0 = q[MH];
+    if (absword(x0.re, x0.im) < kFixSmallWord) {
+      // a small value at the point: its nearest neighbours decide
+      const Fixed2 n1 = mid[CG], n2 = mid[-CG], n3 = mid[WX * CG], n4 = mid[-WX * CG];
+      const int m = max(max(absword(n1.re, n1.im), absword(n2.re, n2.im)),
+                        max(max(absword(n3.re, n3.im), absword(n4.re, n4.im)),
+                            max(absword(q[MH + 1].re, q[MH + 1].im), absword(q[MH - 1].re, q[MH - 1].im))));
+      if (m < kFixSmallWord) redo |= 1ull << (iz - z0);
+    }
+    Product yr, yi;
+    {
+      const int d1 = hi31(dd), d0 = lo31(dd);
+      yr.add(x0.re, d1, d0);
+      yi.add(x0.im, d1, d0);
+    }
+    if (ISO) {
+      WeightedSum tr, ti;
+#pragma unroll
+      for (int k = 1; k <= MH; ++k) {
+        const Fixed2 a1 = mid[k * CG], a2 = mid[-k * CG], b1 = mid[k * WX * CG], b2 = mid[-k * WX * CG];
+        tr.add(k, H.fx_nk[k], (a1.re + a2.re + b1.re) + (b2.re + q[MH + k].re + q[MH - k].re));
+        ti.add(k, H.fx_nk[k], (a1.im + a2.im + b1.im) + (b2.im + q[MH + k].im + q[MH - k].im));
+      }
+      yr.add(tr.shifted(H.fx_st), H.fx_c1[0], H.fx_c0[0]);
+      yi.add(ti.shifted(H.fx_st), H.fx_c1[0], H.fx_c0[0]);
+    } else {
+#pragma unroll
+      for (int dir = 0; dir < 3; ++dir) {
+        WeightedSum tr, ti;
+#pragma unroll
+        for (int k = 1; k <= MH; ++k) {
+          const Fixed2 a = dir == 0 ? mid[k * CG] : dir == 1 ? mid[k * WX * CG] : q[MH + k];
+          const Fixed2 b = dir == 0 ? mid[-k * CG] : dir == 1 ? mid[-k * WX * CG] : q[MH - k];
+          tr.add(k, H.fx_nk[k], a.re + b.re);
+          ti.add(k, H.fx_nk[k], a.im + b.im);
+        }
+        yr.add(tr.shifted(H.fx_st), H.fx_c1[dir], H.fx_c0[dir]);
+        yi.add(ti.shifted(H.fx_st), H.fx_c1[dir], H.fx_c0[dir]);
+      }
+    }
+    long long vr = yr.shifted(f.sa), vi = yi.shifted(f.sa);
+    if (e0 < e1) {
+      Scatter pr, pi;
+      int e = e0;
+      while (true) {
+        const int stop = min(e1, e + 16);
+#pragma unroll 1
+        for (; e < stop; ++e) {
+          const char *Da = Ds + ((unsigned)img * 4 * d_mu + d_mine);
+          const int4 da = *(const int4 *)Da, db = *(const int4 *)(Da + d_mu), dc = *(const int4 *)(Da + 2 * d_mu),
+                     de = *(const int4 *)(Da + 3 * d_mu);
+          const int4 p01 = np01, p23 = np23;
+          // the next entry (of this plane or of the next one with entries)
+          np01 = H.fx_p[2 * (e + 1)];
+          np23 = H.fx_p[2 * (e + 1) + 1];
+          img = H.fx_img[e + 1];
+          pr.add(da.x, da.y, p01.x, p01.y);
+          pi.add(da.z, da.w, p01.x, p01.y);
+          pr.add(db.x, db.y, p01.z, p01.w);
+          pi.add(db.z, db.w, p01.z, p01.w);
+          pr.add(dc.x, dc.y, p23.x, p23.y);
+          pi.add(dc.z, dc.w, p23.x, p23.y);
+          pr.add(de.x, de.y, p23.z, p23.w);
+          pi.add(de.z, de.w, p23.z, p23.w);
+        }
+        if (e == e1) break;
+        pr.carry();
+        pi.carry();
+      }
+      vr -= pr.shifted(f.sp);
+      vi -= pi.shifted(f.sp);
+    }
+    if (own)
+      *(double2 *)(Ys + iz * plane_bytes + mine) = make_double2(from_fixed(vr, f.uy), from_fixed(vi, f.uy));
+#pragma unroll
+    for (int d = 0; d < 2 * MH; ++d) q[d] = q[d + 1];
+    if (more) {
+      next[self] = q[MH];
+#pragma unroll
+      for (int k = 0; k < SLOTS; ++k) next[hat[k]] = conv(hv[k]);
+    }
+  };
+  int iz = z0;
+  for (; iz < min(z1, nz - MH); ++iz) plane(iz, std::false_type());
+  for (; iz < z1; ++iz) plane(iz, std::true_type());
+  if (!f.ok) redo = ~0ull;
+  if (own && redo)
+    for (iz = z0; iz < z1; ++iz)
+      if ((redo >> (iz - z0)) & 1)
+        *(double2 *)(Ys + iz * plane_bytes + mine) =
+            output_fp64(&H, (const double2 *)Xs + c, L, ix, iy, iz, w, wi, E[s],
+                        proj ? D + ((int64_t)s * H.n_atoms * L + c) * 4 : nullptr);
+}
+
+size_t apply_coef_bytes(const HamView &H, int n_sys, int L, int dtype) {
+  const size_t csz = dtype == CBS_C128 ? sizeof(double2) : sizeof(float2);
+  return (size_t)n_sys * (H.n_atoms ? H.n_atoms : 1) * H.np4 * L * csz;
+}
+
+// points per chunk of k_column_max: enough chunks to fill the GPU, at most 64 per system
+static int max_chunks(const HamView &H, int n_sys, int L, int64_t *pts) {
+  const int py = (int)col_block(L).y;
+  int64_t p = std::max<int64_t>((int64_t)py * 16, ceil_div(H.n, 64));
+  while (ceil_div(H.n, p) * (int64_t)n_sys > 152 * 16 && p < (int64_t)py * 256) p *= 2;
+  *pts = p;
+  return ceil_div(H.n, p);
+}
+
+size_t apply_ws_bytes(const HamView &H, int n_sys, int L, int dtype) {
+  const size_t d = apply_coef_bytes(H, n_sys, L, dtype);
+  if (dtype != CBS_C128 || !H.fx_ok || L < 1) return d;
+  int64_t pts;
+  const size_t cols = (size_t)n_sys * L;
+  return (H.n_atoms ? 4 * d : 0) + cols * sizeof(ColumnScale) +
+         cols * max_chunks(H, n_sys, L, &pts) * sizeof(unsigned) + 256;
+}
+
+bool fixed_serves(const HamView &H, int n_sys, int L, size_t ws_bytes) {
+  // offsets inside a system's block and inside its coefficients are 32-bit byte offsets
+  return H.fx_ok && L <= 256 && H.n * L < ((int64_t)1 << 28) &&
+         (int64_t)3 * H.n_atoms * L < ((int64_t)1 << 26) && ws_bytes >= apply_ws_bytes(H, n_sys, L, CBS_C128);
+}
+
+cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y,
+                       const double2 *twist, bool per_col, const double *E, void *ws,
+                       const int *sys_active, cudaStream_t st) {
+  const size_t d = apply_coef_bytes(H, n_sys, L, CBS_C128);
+  double2 *D = (double2 *)ws;
+  int4 *Df = (int4 *)((char *)ws + (H.n_atoms ? d : 0));
+  ColumnScale *scales = (ColumnScale *)((char *)ws + (H.n_atoms ? 4 * d : 0));
+  unsigned *maxhi = (unsigned *)(scales + (size_t)n_sys * L);
+  int64_t pts;
+  const int chunks = max_chunks(H, n_sys, L, &pts);
+  {
+    const dim3 blk = col_block(L);
+    k_column_max<<<dim3((unsigned)chunks, (unsigned)n_sys, 1), blk, (size_t)blk.x * blk.y * sizeof(unsigned), st>>>(
+        H.n, L, (int)pts, X, maxhi, sys_active);
+    k_fix_scales<<<n_sys, L, 0, st>>>(H, L, chunks, maxhi, twist, per_col ? 1 : 0, E, scales, sys_active);
+    count_launches(2);
+    CBS_CUDA(cudaGetLastError());
+  }
+  if (H.n_atoms) {
+    const int groups = ceil_div(L, 32), cg = ceil_div(L, groups);
+    const int py = 256 / cg > 32 ? 32 : 256 / cg;
+    const dim3 blk((unsigned)cg, (unsigned)py, 1), grd((unsigned)H.n_atoms, (unsigned)n_sys, (unsigned)groups);
+    const size_t sm = (size_t)py * 16 * cg * sizeof(long long) + 4 * cg * sizeof(double2) + cg * sizeof(int);
+    k_gather_fixed<<<grd, blk, sm, st>>>(H, L, X, scales, D, Df, sys_active);
+    count_launches(1);
+    CBS_CUDA(cudaGetLastError());
+  }
+  // 8 x 8 lines of 4 columns (64-byte pieces of a point's row)
+  constexpr int CG = 4, TX = 8, TY = 8;
+  const int groups = ceil_div(L, CG), tiles_x = ceil_div(H.nx, TX);
+  const int blocks = groups * tiles_x * ceil_div(H.ny, TY);
+  // planes per block: all of them unless that leaves SMs idle
+  int zc = 1;
+  while (zc < 8 && (int64_t)blocks * n_sys * zc < 152 * 2 && H.nz / (zc * 2) >= 2) zc *= 2;
+  const int z_chunk = std::min(64, ceil_div(H.nz, zc));   // a block marks its planes in 64 bits
+  const dim3 grd((unsigned)blocks, (unsigned)ceil_div(H.nz, z_chunk), (unsigned)n_sys);
+  const size_t sm = (size_t)2 * (TX + 2 * H.m) * (TY + 2 * H.m) * CG * sizeof(Fixed2);
+#define FK(MH, ISO)                                                                                       \
+  do {                                                                                                    \
+    if (sm > 48 * 1024)                                                                                   \
+      CBS_CUDA(cudaFuncSetAttribute(k_stencil_fixed<MH, CG, TX, TY, ISO>,                                 \
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));               \
+    k_stencil_fixed<MH, CG, TX, TY, ISO><<<grd, CG * TX * TY, sm, st>>>(                                  \
+        H, L, groups, tiles_x, z_chunk, X, Y, E, scales, D, Df, sys_active);                              \
+  } while (0)
+#define FM(MH)                     \
+  case MH:                         \
+    if (H.fx_iso) FK(MH, true);    \
+    else FK(MH, false);            \
+    break
+  switch (H.m) {
+    FM(1); FM(2); FM(3); FM(4); FM(5); FM(6);
+    default: set_error("apply: FD half-width must be 1..6"); return CBS_EINVAL;
+  }
+#undef FM
+#undef FK
+  count_launches(1);
+  CBS_CUDA(cudaGetLastError());
+  return CBS_OK;
+}
+
+}  // namespace cbs

@@ -395,7 +395,7 @@ size_t Bicg<R>::bytes_needed(const HamView &H, int n, int L) {
   chunking(H.n, L, &cp, &nc);
   const int64_t vec = (int64_t)2 * n * H.n * L * sizeof(C);
   int64_t b = 4 * align256(vec);
-  b += align256((int64_t)2 * n * (H.n_atoms ? H.n_atoms : 1) * H.np4 * L * sizeof(C));
+  b += align256((int64_t)apply_ws_bytes(H, 2 * n, L, sizeof(R) == 8 ? CBS_C128 : CBS_C64));
   b += align256((int64_t)2 * n * sizeof(double2)) + align256((int64_t)2 * n * sizeof(double));
   b += 4 * align256((int64_t)n * L * sizeof(double2)) + 6 * align256((int64_t)n * L * sizeof(double));
   b += 3 * align256((int64_t)n * L * sizeof(int)) + align256((int64_t)2 * n * sizeof(int)) + 256;
@@ -418,7 +418,8 @@ cbs_status Bicg<R>::alloc(const HamView &H_, int n_, int L_) {
   auto take = [&](int64_t sz) { char *r = b; b += align256(sz); return (void *)r; };
   const int64_t vec = (int64_t)2 * n * N * L * sizeof(C);
   x = (C *)take(vec); r = (C *)take(vec); p = (C *)take(vec); q = (C *)take(vec);
-  D = (C *)take((int64_t)2 * n * (H.n_atoms ? H.n_atoms : 1) * H.np4 * L * sizeof(C));
+  d_bytes = apply_ws_bytes(H, 2 * n, L, sizeof(R) == 8 ? CBS_C128 : CBS_C64);
+  D = take((int64_t)d_bytes);
   tw = (double2 *)take((int64_t)2 * n * sizeof(double2));
   E = (double *)take((int64_t)2 * n * sizeof(double));
   rho = (double2 *)take((int64_t)n * L * sizeof(double2));
@@ -501,7 +502,7 @@ cbs_status Bicg<R>::step(double tol, int max_iter, cudaStream_t st, int kk) {
   const bool prof = profile && kk >= 0 && 2 * kk + 1 < n_prof_ev;
   // recorded as real event nodes of the graph (not capture-dependency markers)
   if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk], st, cudaEventRecordExternal));
-  cbs_status s = apply_P<R>(H, 2 * n, L, p, q, tw, false, E, D, sys_active, st);
+  cbs_status s = apply_P<R>(H, 2 * n, L, p, q, tw, false, E, D, d_bytes, sys_active, st);
   if (s != CBS_OK) return s;
   if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
   k_dot_pq<R><<<grd, blk, red_smem(L), st>>>(n, N, L, chunk_pts, n_chunks, p, q, part, sys_active); cbs::count_launches(1);
@@ -856,7 +857,7 @@ cbs_status MultiShift<R>::step(int max_iter, cudaStream_t st, int kk) {
   CBS_CUDA(cudaGetLastError());
   const bool prof = b.profile && kk >= 0 && 2 * kk + 1 < b.n_prof_ev;
   if (prof) CBS_CUDA(cudaEventRecordWithFlags(b.prof_ev[2 * kk], st, cudaEventRecordExternal));
-  cbs_status s = apply_P<R>(b.H, 2 * n_pt, L, b.p, b.q, b.tw, false, b.E, b.D, b.sys_active, st);
+  cbs_status s = apply_P<R>(b.H, 2 * n_pt, L, b.p, b.q, b.tw, false, b.E, b.D, b.d_bytes, b.sys_active, st);
   if (s != CBS_OK) return s;
   if (prof) CBS_CUDA(cudaEventRecordWithFlags(b.prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
   k_dot_pq<R><<<grd, blk, red_smem(L), st>>>(n_pt, N, L, b.chunk_pts, b.n_chunks, b.p, b.q, b.part, b.sys_active); cbs::count_launches(1);

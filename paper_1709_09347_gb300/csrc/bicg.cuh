@@ -14,7 +14,8 @@ struct Bicg {
   int64_t N = 0;
   int chunk_pts = 0, n_chunks = 0;
   C *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr;   // [2n][N][L]
-  C *D = nullptr;                                             // [2n][n_atoms][n_proj][L]
+  void *D = nullptr;                                          // scratch of the operator apply
+  size_t d_bytes = 0;
   double2 *tw = nullptr;                                      // [2n]
   double *E = nullptr;                                        // [2n]
   double2 *rho = nullptr, *alpha = nullptr, *beta = nullptr;  // [n][L]

@@ -106,6 +106,24 @@ struct HamView {
   // two-columns-per-thread kernel is used (1 = yes, 0 = default, -1 = no)
   int tune_py[2], tune_pz[2];
   int tune_x2;
+  // fixed-point tables of the complex128 apply (fixed.cuh); fx_ok = 0: FP64 kernels only
+  int fx_ok, fx_iso;        // fx_iso: hx = hy = hz
+  int fx_ew;                // weights (diagonal, kinetic factors) are stored as g * 2^(58 - fx_ew)
+  int fx_fp;                // projector values as p * 2^fx_fp
+  int fx_st;                // sum_k n_k < 2^fx_st
+  int fx_nk[kMaxHalf + 1];  // n_k: |c_k| = n_k / den
+  int fx_c1[3], fx_c0[3];   // 2^fx_st / (2 h^2 den) per direction, high and low 31-bit words
+  float fx_wxy, fx_wz;      // sums of |weights| of the x and y arms and of the z arms
+  float fx_db, fx_pb;       // bounds: largest |D| per unit component, largest projector term
+  double fx_vmax;           // max |V_loc|
+  // tables in line order (x-y line by line, along z inside a line)
+  const long long *fx_v;    // [n] V_loc * 2^(58 - fx_ew)
+  const int *fx_ptr;        // [nx ny][nz + 1] entries of each point of a line
+  const int4 *fx_p;         // [nnz+1][2] projector values of the entries: high and low 29-bit words of 4
+  const int *fx_img;        // [nnz+1] (wrap + 1) * n_atoms + atom of the entries
+  const int4 *fx_gp;        // projector values in gather order: per atom, by image -1, 0, +1
+  const int *fx_gi;         // [nnz] grid point, gather order
+  const int *fx_gptr;       // [n_atoms][4] first entry of each image, gather order
 };
 
 }  // namespace cbs
@@ -118,8 +136,9 @@ struct cbs_hamiltonian {
   double fd_c[cbs::kMaxHalf + 1];
   // Frobenius pieces: ||H+||^2, ||H-||^2, off-diagonal part of ||H0||^2, sum d_i, sum d_i^2
   double fro_p2, fro_m2, fro_off0, diag_sum, diag_sum2;
+  int fx_proj_ok;   // the projector values fit the fixed-point tables
   // device allocations owned by the handle
-  void *allocs[24];
+  void *allocs[32];
   int n_allocs;
 };
 
@@ -167,10 +186,19 @@ cbs_status launch_apply(const HamView &H, int n_sys, int L, const typename CT<R>
 // complex128 up to 256 columns; complex64 up to 256, or up to 512 with an even L and at
 // most 4 projectors (two columns per thread).  Sets the error message when it does not.
 bool apply_supported(const HamView &H, int L, int dtype, const char *who);
-// Y = P(w) X for n_sys systems; D is scratch of n_sys*n_atoms*np4*L elements
+// Bytes of scratch of apply_P.  The first apply_coef_bytes of it hold the projector
+// coefficients D; complex128 scratch of only that size is served by the FP64 kernels.
+size_t apply_coef_bytes(const HamView &H, int n_sys, int L, int dtype);
+size_t apply_ws_bytes(const HamView &H, int n_sys, int L, int dtype);
+// Y = P(w) X for n_sys systems; ws: scratch of ws_bytes
 template <typename R>
 cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *X,
                    typename CT<R>::T *Y, const double2 *twist, bool per_col, const double *E,
-                   typename CT<R>::T *D, const int *sys_active, cudaStream_t st);
+                   void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st);
+// apply_fixed.cu: complex128 through fixed point
+bool fixed_serves(const HamView &H, int n_sys, int L, size_t ws_bytes);
+cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y,
+                       const double2 *twist, bool per_col, const double *E, void *ws,
+                       const int *sys_active, cudaStream_t st);
 
 }  // namespace cbs

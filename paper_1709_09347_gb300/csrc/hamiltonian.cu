@@ -12,7 +12,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "common.cuh"
+#include "fixed.cuh"
 
 namespace cbs {
 
@@ -151,6 +151,66 @@ __global__ void k_sum_parts(const double *part, int nparts, double *out) {
   }
 }
 
+// V_loc in the fixed-point unit 2^(ew - 58), line by line
+__global__ void k_fixed_vloc(int64_t n, int nz, int ew, const double *v, long long *fv) {
+  const double up = ldexp(1.0, 58 - ew);
+  const int64_t nxy = n / nz;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    fv[(i % nxy) * nz + i / nxy] = __double2ll_rn(v[i] * up);
+}
+
+// Integer form of the FD coefficients, |c_k| = n_k / den.
+static int64_t fd_integers(int m, int *nk) {
+  static const int den[kMaxHalf + 1] = {0, 1, 12, 180, 5040, 25200, 831600};
+  static const int num[kMaxHalf + 1][kMaxHalf] = {
+      {0}, {1}, {16, 1}, {270, 27, 2}, {8064, 1008, 128, 9}, {42000, 6000, 1000, 125, 8},
+      {1425600, 222750, 44000, 7425, 864, 50}};
+  for (int k = 0; k <= kMaxHalf; ++k) nk[k] = (k >= 1 && k <= m) ? num[m][k - 1] : 0;
+  return den[m];
+}
+
+// The parts of the fixed-point tables that follow the range of V_loc: the common exponent of
+// the weights, the kinetic factors and V_loc in that unit.  fx_ok stays 0 where a range does
+// not fit (the FP64 kernels then serve the cell).
+static cbs_status fixed_weights(cbs_hamiltonian *h, double vmax) {
+  HamView &v = h->v;
+  v.fx_ok = 0;
+  if (v.n_atoms && v.np4 != 4) return CBS_OK;
+  const int64_t den = fd_integers(v.m, v.fx_nk);
+  int64_t sum = 0;
+  for (int k = 1; k <= v.m; ++k) sum += v.fx_nk[k];
+  v.fx_st = 1;
+  while (((int64_t)1 << (v.fx_st - 1)) <= sum) ++v.fx_st;
+  const double hh[3] = {h->hx, h->hy, h->hz};
+  double top = 2.0 * (fabs(v.diag_kin) + vmax), c[3];
+  for (int d = 0; d < 3; ++d) {
+    c[d] = ldexp(1.0, v.fx_st) / (2.0 * hh[d] * hh[d] * (double)den);
+    top = std::max(top, c[d]);
+  }
+  if (!(top < 1e50) || !(top > 1e-50)) return CBS_OK;
+  v.fx_ew = ilogb(top) + 1;
+  for (int d = 0; d < 3; ++d) {
+    const long long f = llrint(ldexp(c[d], 58 - v.fx_ew));
+    v.fx_c1[d] = (int)(f >> 31);
+    v.fx_c0[d] = (int)(f & 0x7fffffff);
+  }
+  v.fx_iso = h->hx == h->hy && h->hy == h->hz;
+  double sxy = 0, sz = 0;
+  for (int k = 1; k <= v.m; ++k) {
+    sxy += 2 * (fabs(v.wx[k]) + fabs(v.wy[k]));
+    sz += 2 * fabs(v.wz[k]);
+  }
+  v.fx_wxy = (float)(sxy * 1.001);
+  v.fx_wz = (float)(sz * 1.001);
+  v.fx_vmax = vmax;
+  k_fixed_vloc<<<(unsigned)std::min<int64_t>(1024, (v.n + 255) / 256), 256>>>(v.n, v.nz, v.fx_ew, v.vloc,
+                                                                              const_cast<long long *>(v.fx_v));
+  count_launches(1);
+  CBS_CUDA(cudaGetLastError());
+  v.fx_ok = h->fx_proj_ok;
+  return CBS_OK;
+}
+
 static cbs_status dalloc(cbs_hamiltonian *h, void **p, size_t bytes) {
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMalloc(p, bytes);
@@ -224,6 +284,90 @@ static cbs_status compute_norms(cbs_hamiltonian *h) {
   return CBS_OK;
 }
 
+// Fixed-point projector tables: values in line order and in gather order (per atom, entries of
+// image -1, then 0, then +1), and the bounds that size the fixed-point sums.
+static cbs_status fixed_projectors(cbs_hamiltonian *h, const cbs_projectors *P, const std::vector<int64_t> &pt_ptr,
+                                   const std::vector<int32_t> &pt_ent, const std::vector<int32_t> &pt_atom) {
+  HamView &v = h->v;
+  const int na = P->n_atoms, np = P->n_proj;
+  const int64_t nnz = P->sup_ptr[na];
+  double pmax = 0, l1max = 0, dmax = 0;
+  for (int a = 0; a < na; ++a) {
+    double l1[4] = {0, 0, 0, 0};
+    for (int64_t t = P->sup_ptr[a]; t < P->sup_ptr[a + 1]; ++t)
+      for (int mu = 0; mu < np; ++mu) {
+        const double p = fabs(P->sup_val[t * np + mu]);
+        pmax = std::max(pmax, p);
+        l1[mu] += p;
+      }
+    for (int mu = 0; mu < np; ++mu) {
+      double d = 0;
+      for (int nu = 0; nu < np; ++nu) d += fabs(P->h[((int64_t)a * np + mu) * np + nu]) * l1[nu];
+      dmax = std::max(dmax, d);
+      l1max = std::max(l1max, l1[mu]);
+    }
+  }
+  double cover = 0;
+  for (int64_t i = 0; i < v.n; ++i) {
+    double c = 0;
+    for (int64_t q = pt_ptr[i]; q < pt_ptr[i + 1]; ++q)
+      for (int mu = 0; mu < np; ++mu) c += fabs(P->sup_val[(int64_t)pt_ent[q] * np + mu]);
+    cover = std::max(cover, c);
+  }
+  if (pmax == 0) pmax = l1max = 1;
+  h->fx_proj_ok = pmax > 1e-50 && l1max < 1e50 && dmax < 1e30 && cover * dmax < 1e30;
+  if (!h->fx_proj_ok) return CBS_OK;
+  // |p| 2^fp < 2^56, and a thread's sum of high words times 2^30 below 2^62
+  v.fx_fp = std::min(56 - (ilogb(pmax) + 1), 61 - (ilogb(l1max) + 1));
+  v.fx_db = (float)(dmax * 1.001);
+  v.fx_pb = (float)(cover * dmax * 1.001);
+  auto words = [&](int64_t t, int4 *out) {
+    int w[8];
+    for (int mu = 0; mu < 4; ++mu) {
+      const long long f = mu < np ? llrint(ldexp(P->sup_val[t * np + mu], v.fx_fp)) : 0;
+      w[2 * mu] = balanced_hi(f);
+      w[2 * mu + 1] = balanced_lo(f);
+    }
+    out[0] = make_int4(w[0], w[1], w[2], w[3]);
+    out[1] = make_int4(w[4], w[5], w[6], w[7]);
+  };
+  std::vector<int4> pp((size_t)nnz * 2 + 2, make_int4(0, 0, 0, 0)), gp((size_t)nnz * 2);   // one spare entry
+  std::vector<int> gi(nnz), gptr((size_t)na * 4), img((size_t)nnz + 1, 0);
+  const int64_t nxy = (int64_t)v.nx * v.ny;
+  std::vector<int> ptr((size_t)nxy * (v.nz + 1));
+  int64_t o = 0;
+  for (int64_t line = 0; line < nxy; ++line) {
+    for (int iz = 0; iz < v.nz; ++iz) {
+      const int64_t i = (int64_t)iz * nxy + line;
+      ptr[(size_t)line * (v.nz + 1) + iz] = (int)o;
+      for (int64_t q = pt_ptr[i]; q < pt_ptr[i + 1]; ++q, ++o) {
+        words(pt_ent[q], &pp[2 * o]);
+        img[o] = ((int)P->sup_wrap[pt_ent[q]] + 1) * na + pt_atom[q];
+      }
+    }
+    ptr[(size_t)line * (v.nz + 1) + v.nz] = (int)o;
+  }
+  o = 0;
+  for (int a = 0; a < na; ++a)
+    for (int m = -1; m <= 2; ++m) {
+      gptr[(size_t)a * 4 + m + 1] = (int)o;
+      if (m == 2) break;
+      for (int64_t t = P->sup_ptr[a]; t < P->sup_ptr[a + 1]; ++t)
+        if (P->sup_wrap[t] == m) {
+          gi[o] = P->sup_idx[t];
+          words(t, &gp[2 * o]);
+          ++o;
+        }
+    }
+  cbs_status s;
+  if ((s = upload(h, pp.data(), pp.size(), &v.fx_p)) != CBS_OK) return s;
+  if ((s = upload(h, img.data(), img.size(), &v.fx_img)) != CBS_OK) return s;
+  if ((s = upload(h, ptr.data(), ptr.size(), &v.fx_ptr)) != CBS_OK) return s;
+  if ((s = upload(h, gp.data(), gp.size(), &v.fx_gp)) != CBS_OK) return s;
+  if ((s = upload(h, gi.data(), gi.size(), &v.fx_gi)) != CBS_OK) return s;
+  return upload(h, gptr.data(), gptr.size(), &v.fx_gptr);
+}
+
 static cbs_status create_impl(const cbs_grid *g, const double *v_loc, const cbs_projectors *P,
                               cbs_hamiltonian *h) {
   HamView &v = h->v;
@@ -266,8 +410,16 @@ static cbs_status create_impl(const cbs_grid *g, const double *v_loc, const cbs_
   s = upload(h, v32.data(), N, &v.vloc32);
   if (s != CBS_OK) return s;
 
+  double vmax = 0;
+  for (size_t i = 0; i < N; ++i) vmax = std::max(vmax, fabs(v_loc[i]));
+  {
+    void *fv = nullptr;
+    if ((s = dalloc(h, &fv, N * sizeof(long long))) != CBS_OK) return s;
+    v.fx_v = (const long long *)fv;
+  }
   // projectors
   v.n_atoms = 0; v.n_proj = 0; h->nnz = 0; v.np4 = 4;
+  h->fx_proj_ok = 1;
   std::vector<int64_t> pt_ptr(N + 1, 0);
   if (P && P->n_atoms > 0) {
     if (P->n_proj < 1 || P->n_proj > kMaxProj) { set_error("n_proj must be 1..8"); return CBS_EINVAL; }
@@ -346,10 +498,11 @@ static cbs_status create_impl(const cbs_grid *g, const double *v_loc, const cbs_
     }
     if ((s = upload(h, aw.data(), (size_t)nnz, &v.pt_aw)) != CBS_OK) return s;
     if (np <= 4 && (s = upload(h, p4.data(), (size_t)nnz, &v.pt_p32)) != CBS_OK) return s;
+    if (np <= 4 && (s = fixed_projectors(h, P, pt_ptr, pt_ent, pt_atom)) != CBS_OK) return s;
   } else {
     if ((s = upload(h, pt_ptr.data(), N + 1, &v.pt_ptr)) != CBS_OK) return s;
   }
-
+  if ((s = fixed_weights(h, vmax)) != CBS_OK) return s;
   return compute_norms(h);
 }
 
@@ -366,14 +519,19 @@ extern "C" cbs_status cbs_create_hamiltonian(const cbs_grid *grid, const double 
 }
 
 namespace cbs {
-// V_loc in single precision from the FP64 copy, and a flag if any value is not finite.
-__global__ void k_vloc32(int64_t n, const double *v, float *v32, int *bad) {
+// V_loc in single precision from the FP64 copy, a flag if any value is not finite, and
+// max |V_loc| (as bits: the order of non-negative doubles).
+__global__ void k_vloc32(int64_t n, const double *v, float *v32, int *bad, unsigned long long *vmax) {
   int b = 0;
+  unsigned long long m = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double x = v[i];
     v32[i] = (float)x;
     b |= !isfinite(x);
+    m = max(m, (unsigned long long)__double_as_longlong(fabs(x)));
   }
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(vmax, m);
   if (__syncthreads_or(b) && threadIdx.x == 0) atomicOr(bad, 1);
 }
 }  // namespace cbs
@@ -386,23 +544,26 @@ extern "C" cbs_status cbs_hamiltonian_set_vloc(cbs_hamiltonian *h, const double 
   double *tmp = nullptr;
   CBS_CUDA(cudaMalloc(&tmp, N * sizeof(double) + 256));
   bad = (int *)((char *)tmp + ((N * sizeof(double) + 127) & ~(size_t)127));
+  unsigned long long *dmax = (unsigned long long *)(bad + 2);
   cbs_status s = CBS_OK;
   cudaError_t e = cudaMemcpy(tmp, v_loc, N * sizeof(double), cudaMemcpyDefault);
-  if (e == cudaSuccess) e = cudaMemset(bad, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(bad, 0, 2 * sizeof(int) + sizeof(unsigned long long));
   if (e == cudaSuccess) {
     // check into a scratch copy first, so a rejected V_loc leaves the handle unchanged
     k_vloc32<<<std::min<int64_t>(1024, ((int64_t)N + 255) / 256), 256>>>((int64_t)N, tmp,
-                                                                         const_cast<float *>(v.vloc32), bad);
+                                                                         const_cast<float *>(v.vloc32), bad, dmax);
     cbs::count_launches(1);
     e = cudaGetLastError();
   }
   int hb = 0;
+  double hmax = 0;
   if (e == cudaSuccess) e = cudaMemcpy(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(&hmax, dmax, sizeof(double), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) s = cuda_fail(e, "cbs_hamiltonian_set_vloc");
   else if (hb) {
     // restore the single-precision copy from the unchanged FP64 one
     k_vloc32<<<std::min<int64_t>(1024, ((int64_t)N + 255) / 256), 256>>>((int64_t)N, v.vloc,
-                                                                         const_cast<float *>(v.vloc32), bad);
+                                                                         const_cast<float *>(v.vloc32), bad, dmax);
     cbs::count_launches(1);
     cudaDeviceSynchronize();
     set_error("v_loc contains a non-finite value");
@@ -413,5 +574,6 @@ extern "C" cbs_status cbs_hamiltonian_set_vloc(cbs_hamiltonian *h, const double 
   }
   cudaFree(tmp);
   if (s != CBS_OK) return s;
+  if ((s = fixed_weights(h, hmax)) != CBS_OK) return s;
   return compute_norms(h);
 }

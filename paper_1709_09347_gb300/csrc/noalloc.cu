@@ -60,8 +60,7 @@ extern "C" cbs_status cbs_apply_noalloc(const cbs_hamiltonian *h, int n_sys, con
   if (!apply_supported(h->v, L, dtype, "cbs_apply_noalloc")) return CBS_EINVAL;
   const size_t tw_bytes = round256((size_t)n_sys * sizeof(double2));
   const size_t e_bytes = round256((size_t)n_sys * sizeof(double));
-  const size_t d_bytes = cbs_apply_workspace_size(h, n_sys, L, dtype);
-  if (tw_bytes + e_bytes + d_bytes > kNoAllocScratchBytes) {
+  if (tw_bytes + e_bytes + apply_coef_bytes(h->v, n_sys, L, dtype) > kNoAllocScratchBytes) {
     set_error("cbs_apply_noalloc: this n_sys x L needs more than the fixed 32 MiB of scratch; "
               "split the batch, or use cbs_apply / cbs_apply_ws");
     return CBS_EINVAL;
@@ -72,15 +71,18 @@ extern "C" cbs_status cbs_apply_noalloc(const cbs_hamiltonian *h, int n_sys, con
   cudaStream_t st = (cudaStream_t)stream;
   double2 *tw = (double2 *)base;
   double *Ed = (double *)((char *)base + tw_bytes);
+  // all that is left of the array: complex128 applies too large for the fixed-point scratch in
+  // it run on the FP64 kernels, which need the coefficients D alone
   void *D = (char *)base + tw_bytes + e_bytes;
+  const size_t d_bytes = kNoAllocScratchBytes - tw_bytes - e_bytes;
   // the twists and energies come from host memory; D is fully written by the projector
   // gather before the stencil reads it, so nothing in the array has to start at zero
   CBS_CUDA(cudaMemcpyAsync(tw, z, (size_t)n_sys * sizeof(double2), cudaMemcpyHostToDevice, st));
   CBS_CUDA(cudaMemcpyAsync(Ed, E, (size_t)n_sys * sizeof(double), cudaMemcpyHostToDevice, st));
   const HamView &H = h->v;
   if (dtype == CBS_C128)
-    return apply_P<double>(H, n_sys, L, (const double2 *)X, (double2 *)Y, tw, false, Ed, (double2 *)D,
-                           nullptr, st);
-  return apply_P<float>(H, n_sys, L, (const float2 *)X, (float2 *)Y, tw, false, Ed, (float2 *)D,
-                        nullptr, st);
+    return apply_P<double>(H, n_sys, L, (const double2 *)X, (double2 *)Y, tw, false, Ed, D,
+                           d_bytes, nullptr, st);
+  return apply_P<float>(H, n_sys, L, (const float2 *)X, (float2 *)Y, tw, false, Ed, D,
+                        d_bytes, nullptr, st);
 }

@@ -180,7 +180,7 @@ cbs_status cbs_internal_rr(const cbs_hamiltonian *h, double E, const double2 *S,
                osig = add(m0 * 8), oinfo = add(64), oCT = add(3 * mm * 16), oLU = add(3 * mm * 16),
                oC = add(4 * mm * 16), oZe = add(4 * mm * 16), otau = add(2 * m0 * 16),
                oYc = add(4 * mm * 16), oring = add(2 * m0 * 4), osm = add(64), oP1 = add(4 * mm * 16),
-               oPsi = add((size_t)N * 2 * m0 * 16), oD = add((size_t)3 * (H.n_atoms ? H.n_atoms : 1) * H.np4 * m0 * 16),
+               oPsi = add((size_t)N * 2 * m0 * 16), oD = add(apply_ws_bytes(H, 3, m0, CBS_C128)),
                otw = add(256), olam = add(2 * m0 * 16);
   char *base = nullptr;
   if (cudaMalloc(&base, bytes) != cudaSuccess) { set_error("cudaMalloc failed (Rayleigh-Ritz workspace)"); return CBS_ENOMEM; }
@@ -190,7 +190,7 @@ cbs_status cbs_internal_rr(const cbs_hamiltonian *h, double E, const double2 *S,
           *Gu = (double2 *)(base + oGu), *Gws = (double2 *)(base + oGws), *CT = (double2 *)(base + oCT),
           *LU = (double2 *)(base + oLU), *C = (double2 *)(base + oC), *Ze = (double2 *)(base + oZe),
           *tau = (double2 *)(base + otau), *Yc = (double2 *)(base + oYc), *P1 = (double2 *)(base + oP1),
-          *Psi = (double2 *)(base + oPsi), *D = (double2 *)(base + oD), *tw = (double2 *)(base + otw),
+          *Psi = (double2 *)(base + oPsi), *tw = (double2 *)(base + otw),
           *lam = (double2 *)(base + olam);
   double *sig = (double *)(base + osig);
   int *info = (int *)(base + oinfo), *ring = (int *)(base + oring), *sm = (int *)(base + osm);
@@ -229,7 +229,8 @@ cbs_status cbs_internal_rr(const cbs_hamiltonian *h, double E, const double2 *S,
   const double hE[3] = {0, 0, 0};
   CBS_CUDA(cudaMemcpyAsync(tw, hw, sizeof(hw), cudaMemcpyHostToDevice, st));
   CBS_CUDA(cudaMemcpyAsync((double *)(tw + 3), hE, sizeof(hE), cudaMemcpyHostToDevice, st));
-  CBS_TRY_RR(apply_P<double>(H, 3, r, X3, R3, tw, false, (const double *)(tw + 3), D, nullptr, st));
+  CBS_TRY_RR(apply_P<double>(H, 3, r, X3, R3, tw, false, (const double *)(tw + 3), base + oD,
+                             apply_ws_bytes(H, 3, m0, CBS_C128), nullptr, st));
   k_rr_blocks<<<152 * 4, 256, 0, st>>>(cntQ, R3, X3);   // X3 <- H0Q, H+Q, H-Q
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());

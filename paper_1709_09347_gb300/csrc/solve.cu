@@ -150,7 +150,8 @@ __global__ void k_scale_rows(int rows, int cols, int64_t ld, const double *sig, 
 struct ResidualCheck {
   DevBuf buf;
   double2 *R = nullptr;
-  double2 *D = nullptr;
+  void *D = nullptr;
+  size_t d_bytes = 0;
   double *cn = nullptr, *bn = nullptr, *bn2 = nullptr, *maxrel = nullptr;
   int *colmask = nullptr, *nunc = nullptr;
   int n = 0, L = 0;
@@ -158,14 +159,14 @@ struct ResidualCheck {
   cbs_status alloc(const HamView &H, int n_, int L_) {
     n = n_; L = L_; N = H.n;
     const size_t vec = (size_t)2 * n * N * L * sizeof(double2);
-    const size_t dsz = (size_t)2 * n * (H.n_atoms ? H.n_atoms : 1) * H.np4 * L * sizeof(double2);
+    const size_t dsz = d_bytes = apply_ws_bytes(H, 2 * n, L, CBS_C128);
     const size_t small = (size_t)2 * n * 64 * L * sizeof(double) + 3 * (size_t)2 * n * L * sizeof(double) +
                          (size_t)n * L * sizeof(int) + 4096;
     CBS_TRY(buf.alloc(vec + dsz + small + 1024));
     char *b = buf.as<char>();
     auto take = [&](size_t sz) { char *r = b; b += (sz + 255) & ~(size_t)255; return (void *)r; };
     R = (double2 *)take(vec);
-    D = (double2 *)take(dsz);
+    D = take(dsz);
     cn = (double *)take((size_t)2 * n * 64 * L * sizeof(double));
     bn = (double *)take((size_t)L * sizeof(double));
     bn2 = (double *)take((size_t)2 * n * L * sizeof(double));
@@ -186,7 +187,7 @@ struct ResidualCheck {
       CBS_CUDA(cudaEventCreate(&e1));
       CBS_CUDA(cudaEventRecord(e0, st));
     }
-    CBS_TRY(apply_P<double>(H, 2 * n, L, Y, R, tw, false, E, D, nullptr, st));
+    CBS_TRY(apply_P<double>(H, 2 * n, L, Y, R, tw, false, E, D, d_bytes, nullptr, st));
     if (profile) {
       CBS_CUDA(cudaEventRecord(e1, st));
       CBS_CUDA(cudaEventSynchronize(e1));
@@ -500,7 +501,7 @@ struct ShiftedSolver {
     size_t free_b = 0, total_b = 0;
     CBS_CUDA(cudaMemGetInfo(&free_b, &total_b));
     const size_t per_e = (size_t)n_pt * (bytes_per_system(H, L, o.precision) + (size_t)2 * H.n * L * 16) +
-                         (size_t)2 * n_pt * (H.n_atoms ? H.n_atoms : 1) * H.np4 * L * 16 * 2;
+                         apply_ws_bytes(H, 2 * n_pt, L, CBS_C128) * 2;
     const int grp = std::max(1, std::min(n_e, (int)((free_b * 8 / 10) / std::max<size_t>(per_e, 1))));
     const size_t blk = (size_t)H.n * L;
     for (int g0 = 0; g0 < n_e; g0 += grp) {
@@ -650,7 +651,7 @@ static cbs_status solve_impl(const cbs_hamiltonian *h, const double *energies, i
   // one wave and as many energies as fit; when not even one energy's points fit at once,
   // all energies (or as many as fit) with as many points per wave as fit.
   const size_t v16 = (size_t)N * L * 16;
-  const size_t dsz = (size_t)2 * (H.n_atoms ? H.n_atoms : 1) * H.np4 * L * 16 * 2;
+  const size_t dsz = apply_ws_bytes(H, 2, L, CBS_C128) * 2;
   const size_t per_sys = ShiftedSolver::bytes_per_system(H, L, o.precision) + dsz;
   const size_t extract_e = (size_t)N * nLM * 16 + (size_t)4 * nLM * nLM * 16 * 6;
   auto peak = [&](size_t ne_, size_t nw_) -> size_t {
@@ -827,12 +828,12 @@ static cbs_status solve_impl(const cbs_hamiltonian *h, const double *energies, i
       auto finish = [&](int cnt, double2 *Psi, const double2 *twr_src, const int *ring_host) -> cbs_status {
         DevBuf vb;
         const size_t psi_bytes = (size_t)N * cnt * sizeof(double2);
-        const size_t dsz = (size_t)(H.n_atoms ? H.n_atoms : 1) * H.np4 * cnt * sizeof(double2);
+        const size_t dsz = apply_ws_bytes(H, 1, cnt, CBS_C128);
         CBS_TRY(vb.alloc(psi_bytes + dsz + (size_t)cnt * 256 + 8192));
         char *p = vb.as<char>();
         auto take = [&](size_t sz) { char *r = p; p += (sz + 255) & ~(size_t)255; return (void *)r; };
         double2 *Res = (double2 *)take(psi_bytes);
-        double2 *Dd = (double2 *)take(dsz);
+        void *Dd = take(dsz);
         double2 *twr = (double2 *)take((size_t)cnt * sizeof(double2));
         double *stats = (double *)take((size_t)cnt * 4 * sizeof(double));
         double *rho_all = (double *)take((size_t)cnt * sizeof(double));
@@ -845,7 +846,7 @@ static cbs_status solve_impl(const cbs_hamiltonian *h, const double *energies, i
         double *Ed = (double *)take(256);
         CBS_CUDA(cudaMemcpyAsync(Ed, &Ee, sizeof(double), cudaMemcpyHostToDevice, st));
         CBS_CUDA(cudaMemcpyAsync(twr, twr_src, (size_t)cnt * sizeof(double2), cudaMemcpyDeviceToDevice, st));
-        CBS_TRY(apply_P<double>(H, 1, cnt, Psi, Res, twr, true, Ed, Dd, nullptr, st));
+        CBS_TRY(apply_P<double>(H, 1, cnt, Psi, Res, twr, true, Ed, Dd, dsz, nullptr, st));
         double nHp, nA, nHm;
         cbs_hamiltonian_norms(h, Ee, &nHp, &nA, &nHm);
         const double a_cell = h->hz * H.nz;
