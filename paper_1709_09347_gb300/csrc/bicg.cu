@@ -45,6 +45,37 @@ __device__ __forceinline__ void block_partials(double (&acc)[4], double *part, i
   }
 }
 
+// Sums over the chunks of one system's partials, NV of the 4 values per column.  Blocks are
+// (L, ry): lane ly adds chunks ly, ly + ry, ... and lane 0 the lanes' sums in order (one thread
+// per column adding 128 chunks is a chain of 128 dependent FP64 additions per value, 40-60 us;
+// with 16 lanes 3-4 us).  The result is returned in lane 0; every thread of the block takes part.
+template <int NV>
+__device__ __forceinline__ void sum_chunks(const double *part, int64_t s, int L, int n_chunks, double (&a)[NV]) {
+  extern __shared__ double csm[];   // [ry][L][NV]
+  const int c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) a[q] = 0;
+#pragma unroll 4
+  for (int ch = ly; ch < n_chunks; ch += ry)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) a[q] += part[((s * n_chunks + ch) * L + c) * 4 + q];
+  if (ry == 1) return;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) csm[((size_t)ly * L + c) * NV + q] = a[q];
+  __syncthreads();
+  if (ly == 0)
+    for (int y = 1; y < ry; ++y)
+#pragma unroll
+      for (int q = 0; q < NV; ++q) a[q] += csm[((size_t)y * L + c) * NV + q];
+}
+
+// Blocks of the kernels that use it: up to 16 lanes, 1024 threads and one lane per chunk.
+static dim3 reduce_block(int L, int n_chunks) {
+  int ry = std::min(16, std::min(1024 / L, n_chunks));
+  return dim3((unsigned)L, (unsigned)std::max(ry, 1), 1);
+}
+static size_t reduce_smem(dim3 blk) { return (size_t)blk.x * blk.y * 4 * sizeof(double); }
+
 template <typename R>
 __global__ void k_init(int n, int64_t N, int L, int chunk_pts, int n_chunks, const double2 *B,
                        int64_t bstride, const double2 *Bd, int64_t bdstride,
@@ -78,26 +109,29 @@ __global__ void k_reduce_init(int n, int L, int n_chunks, const double *part, do
                               const int *colmask, int *sys_active, int *n_active) {
   const int s = blockIdx.x, c = threadIdx.x;
   const int64_t k = (int64_t)s * L + c;
-  double a[4] = {0, 0, 0, 0};
-  for (int ch = 0; ch < n_chunks; ++ch)
-    for (int q = 0; q < 4; ++q) a[q] += part[(((int64_t)s * n_chunks + ch) * L + c) * 4 + q];
-  rho[k] = make_double2(a[0], a[1]);
-  rho_prev[k] = make_double2(0, 0);
-  beta[k] = make_double2(0, 0);
-  nb[k] = sqrt(a[2]);
-  nbd[k] = sqrt(a[3]);
-  // absolute targets: relative to this right-hand side, or to reference norms
-  // ref_norm[2n][L] (primal then dual) when the system solves for a correction
-  tgt[k] = tfloor * (ref_norm ? ref_norm[k] : nb[k]);
-  tgtd[k] = tfloor * (ref_norm ? ref_norm[(int64_t)n * L + k] : nbd[k]);
-  rmax[k] = nb[k];
-  rmaxd[k] = nbd[k];
-  int act = (colmask ? colmask[k] : 1) && a[2] > 0 && a[3] > 0;
-  active[k] = act;
-  iters[k] = 0;
-  flags[k] = 0;
+  double a[4];
+  sum_chunks<4>(part, s, L, n_chunks, a);
+  int act = 0;
+  if (threadIdx.y == 0) {
+    rho[k] = make_double2(a[0], a[1]);
+    rho_prev[k] = make_double2(0, 0);
+    beta[k] = make_double2(0, 0);
+    const double na = sqrt(a[2]), nad = sqrt(a[3]);
+    nb[k] = na;
+    nbd[k] = nad;
+    // absolute targets: relative to this right-hand side, or to reference norms
+    // ref_norm[2n][L] (primal then dual) when the system solves for a correction
+    tgt[k] = tfloor * (ref_norm ? ref_norm[k] : na);
+    tgtd[k] = tfloor * (ref_norm ? ref_norm[(int64_t)n * L + k] : nad);
+    rmax[k] = na;
+    rmaxd[k] = nad;
+    act = (colmask ? colmask[k] : 1) && a[2] > 0 && a[3] > 0;
+    active[k] = act;
+    iters[k] = 0;
+    flags[k] = 0;
+  }
   int any = __syncthreads_or(act);
-  if (c == 0) {
+  if (c == 0 && threadIdx.y == 0) {
     sys_active[s] = any;
     sys_active[n + s] = any;
     if (any) atomicAdd(n_active, 1);
@@ -152,15 +186,13 @@ __global__ void k_reduce_alpha(int n, int L, int n_chunks, const double *part, c
                                unsigned long long *sys_apply) {
   const int s = blockIdx.x, c = threadIdx.x;
   if (!sys_active[s]) return;
+  double a[2];
+  sum_chunks<2>(part, s, L, n_chunks, a);
+  if (threadIdx.y != 0) return;
   if (c == 0 && sys_apply) atomicAdd(sys_apply, 1ull);   // system s went through this apply
   const int64_t k = (int64_t)s * L + c;
   if (!active[k]) { alpha[k] = make_double2(0, 0); return; }
-  double gx = 0, gy = 0;
-  for (int ch = 0; ch < n_chunks; ++ch) {
-    gx += part[(((int64_t)s * n_chunks + ch) * L + c) * 4 + 0];
-    gy += part[(((int64_t)s * n_chunks + ch) * L + c) * 4 + 1];
-  }
-  double2 g = make_double2(gx, gy);
+  double2 g = make_double2(a[0], a[1]);
   double g2 = cabs2(g);
   if (!(g2 > 0) || !isfinite(g2)) {
     flags[k] |= 2;
@@ -217,11 +249,11 @@ __global__ void k_reduce_beta(int n, int L, int n_chunks, const double *part, do
   const int s = blockIdx.x, c = threadIdx.x;
   if (!sys_active[s]) return;   // uniform per block
   const int64_t k = (int64_t)s * L + c;
-  int act = active[k];
+  double a[4];
+  sum_chunks<4>(part, s, L, n_chunks, a);
+  const bool lead = threadIdx.y == 0;
+  int act = lead ? active[k] : 0;
   if (act) {
-    double a[4] = {0, 0, 0, 0};
-    for (int ch = 0; ch < n_chunks; ++ch)
-      for (int q = 0; q < 4; ++q) a[q] += part[(((int64_t)s * n_chunks + ch) * L + c) * 4 + q];
     const int it = iters[k] + 1;
     iters[k] = it;
     const double nr = sqrt(a[2]), nrd = sqrt(a[3]);
@@ -247,9 +279,9 @@ __global__ void k_reduce_beta(int n, int L, int n_chunks, const double *part, do
     }
     active[k] = act;
   }
-  if (!act) beta[k] = make_double2(0, 0);
+  if (lead && !act) beta[k] = make_double2(0, 0);
   int any = __syncthreads_or(act);
-  if (c == 0) {
+  if (lead && c == 0) {
     sys_active[s] = any;
     sys_active[n + s] = any;
     if (any) atomicAdd(n_active, 1);
@@ -334,11 +366,11 @@ __global__ void k_reduce_replace(int n, int L, int n_chunks, const double *part,
                                  int *active, const int *colmask, int *sys_active, int *n_active) {
   const int s = blockIdx.x, c = threadIdx.x;
   const int64_t k = (int64_t)s * L + c;
-  int act = colmask[k];
+  double a[4];
+  sum_chunks<4>(part, s, L, n_chunks, a);
+  const bool lead = threadIdx.y == 0;
+  int act = lead ? colmask[k] : 0;
   if (act) {
-    double a[4] = {0, 0, 0, 0};
-    for (int ch = 0; ch < n_chunks; ++ch)
-      for (int q = 0; q < 4; ++q) a[q] += part[(((int64_t)s * n_chunks + ch) * L + c) * 4 + q];
     const double2 rn = make_double2(a[0], a[1]);
     const double2 rp = rho_prev[k];
     beta[k] = (cabs2(rp) > 0) ? cdiv(rn, rp) : make_double2(0, 0);
@@ -346,12 +378,12 @@ __global__ void k_reduce_replace(int n, int L, int n_chunks, const double *part,
     rmax[k] = sqrt(a[2]);
     rmaxd[k] = sqrt(a[3]);
     if (!(cabs2(rn) > 0) || !isfinite(a[2]) || !isfinite(a[3])) { act = 0; beta[k] = make_double2(0, 0); }
-  } else {
+  } else if (lead) {
     beta[k] = make_double2(0, 0);
   }
-  active[k] = act;
+  if (lead) active[k] = act;
   int any = __syncthreads_or(act);
-  if (c == 0) {
+  if (lead && c == 0) {
     sys_active[s] = any;
     sys_active[n + s] = any;
     if (any) atomicAdd(n_active, 1);
@@ -379,10 +411,15 @@ cbs_status launch_twists(int n, const double2 *z, const double *E, double2 *tw, 
 // ---------------------------------------------------------------- Bicg<R> members
 static int64_t align256(int64_t b) { return (b + 255) & ~(int64_t)255; }
 
-static void chunking(int64_t N, int L, int *chunk_pts, int *n_chunks) {
+// Points per block of the vector kernels.  At most 128 chunks per system and 8 points per
+// thread, fewer points where that would leave SMs without a block: the vector kernels are bound
+// by FP64 issue also on the smallest cells.
+static void chunking(int64_t N, int L, int n, int *chunk_pts, int *n_chunks) {
   dim3 blk = col_block(L);
-  int64_t cp = (N + 127) / 128;                       // at most 128 chunks per system
-  int64_t minp = (int64_t)blk.y * 8;
+  int64_t cp = (N + 127) / 128;
+  int64_t per = 8;
+  while (per > 1 && (int64_t)n * ceil_div(N, blk.y * per) < 152 * 4) per /= 2;
+  const int64_t minp = (int64_t)blk.y * per;
   if (cp < minp) cp = minp;
   cp = ((cp + blk.y - 1) / blk.y) * blk.y;
   *chunk_pts = (int)cp;
@@ -392,7 +429,7 @@ static void chunking(int64_t N, int L, int *chunk_pts, int *n_chunks) {
 template <typename R>
 size_t Bicg<R>::bytes_needed(const HamView &H, int n, int L) {
   int cp, nc;
-  chunking(H.n, L, &cp, &nc);
+  chunking(H.n, L, n, &cp, &nc);
   const int64_t vec = (int64_t)2 * n * H.n * L * sizeof(C);
   int64_t b = 4 * align256(vec);
   b += align256((int64_t)apply_ws_bytes(H, 2 * n, L, sizeof(R) == 8 ? CBS_C128 : CBS_C64));
@@ -406,7 +443,7 @@ size_t Bicg<R>::bytes_needed(const HamView &H, int n, int L) {
 template <typename R>
 cbs_status Bicg<R>::alloc(const HamView &H_, int n_, int L_) {
   H = H_; n = n_; L = L_; N = H.n;
-  chunking(N, L, &chunk_pts, &n_chunks);
+  chunking(N, L, n, &chunk_pts, &n_chunks);
   bytes = bytes_needed(H, n, L);
   cudaError_t e = cudaMalloc(&block, bytes);
   if (e != cudaSuccess) {
@@ -486,7 +523,7 @@ cbs_status Bicg<R>::init(const double2 *B, int64_t bstride, const double2 *Bd, i
                                           x, r, p, part); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   CBS_CUDA(cudaMemsetAsync(n_active, 0, sizeof(int), st));
-  k_reduce_init<<<n, L, 0, st>>>(n, L, n_chunks, part, rho, rho_prev, beta, nb, nbd, tgt, tgtd, rmax,
+  k_reduce_init<<<n, reduce_block(L, n_chunks), reduce_smem(reduce_block(L, n_chunks)), st>>>(n, L, n_chunks, part, rho, rho_prev, beta, nb, nbd, tgt, tgtd, rmax,
                                  rmaxd, tfloor, ref_norm, active, iters, flags, colmask, sys_active,
                                  n_active); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
@@ -507,14 +544,15 @@ cbs_status Bicg<R>::step(double tol, int max_iter, cudaStream_t st, int kk) {
   if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
   k_dot_pq<R><<<grd, blk, red_smem(L), st>>>(n, N, L, chunk_pts, n_chunks, p, q, part, sys_active); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
-  k_reduce_alpha<<<n, L, 0, st>>>(n, L, n_chunks, part, rho, alpha, active, flags, sys_active,
+  const dim3 rblk = reduce_block(L, n_chunks);
+  k_reduce_alpha<<<n, rblk, reduce_smem(rblk), st>>>(n, L, n_chunks, part, rho, alpha, active, flags, sys_active,
                                   sys_apply); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   k_pass_b<R><<<grd, blk, red_smem(L), st>>>(n, N, L, chunk_pts, n_chunks, x, r, p, q, alpha,
                                              active, part, sys_active); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   CBS_CUDA(cudaMemsetAsync(n_active, 0, sizeof(int), st));
-  k_reduce_beta<<<n, L, 0, st>>>(n, L, n_chunks, part, rho, rho_prev, beta, tgt, tgtd, rmax, rmaxd,
+  k_reduce_beta<<<n, rblk, reduce_smem(rblk), st>>>(n, L, n_chunks, part, rho, rho_prev, beta, tgt, tgtd, rmax, rmaxd,
                                  tfac, active, iters, flags, max_iter, sys_active, n_active); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   if (group > 0 && group_need < group) {
@@ -591,7 +629,7 @@ cbs_status Bicg<R>::replace(const double2 *R64, const int *colmask, cudaStream_t
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   CBS_CUDA(cudaMemsetAsync(n_active, 0, sizeof(int), st));
-  k_reduce_replace<<<n, L, 0, st>>>(n, L, n_chunks, part, rho, rho_prev, beta, rmax, rmaxd, active,
+  k_reduce_replace<<<n, reduce_block(L, n_chunks), reduce_smem(reduce_block(L, n_chunks)), st>>>(n, L, n_chunks, part, rho, rho_prev, beta, rmax, rmaxd, active,
                                     colmask, sys_active, n_active);
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
@@ -618,19 +656,20 @@ __global__ void k_ms_init(int n_pt, int n_sh, int L, const int *seed_active, dou
   }
 }
 
-// after alpha_k: pi^{k+1} and the coefficients of this iteration for every energy
+// after alpha_k: pi^{k+1} and the coefficients of this iteration for every energy; blocks are
+// (L, lanes over the energies)
 __global__ void k_ms_coef(int n_pt, int n_sh, int L, const double *sigma, const double2 *alpha,
                           const double2 *beta, double2 *alpha_prev, double2 *pi, double2 *pi_prev,
                           double2 *cb, double2 *ca, int *sactive, int *sflags,
                           const int *seed_sys_active, unsigned long long *upd_cols) {
   const int j = blockIdx.x, c = threadIdx.x;
-  if (!seed_sys_active[j]) return;
-  int live = 0;
+  if (!seed_sys_active[j]) return;   // uniform per block
   const int64_t k = (int64_t)j * L + c;
   const double2 a = alpha[k], b = beta[k], ap = alpha_prev[k];
   const bool first = !(cabs2(b) > 0);
   const double2 g = first ? make_double2(0, 0) : cdiv(cmul(a, b), ap);
-  for (int e = 0; e < n_sh; ++e) {
+  int live = 0;
+  for (int e = threadIdx.y; e < n_sh; e += blockDim.y) {
     const int64_t kk = ((int64_t)e * n_pt + j) * L + c;
     if (!sactive[kk]) {
       cb[kk] = ca[kk] = make_double2(0, 0);
@@ -654,11 +693,9 @@ __global__ void k_ms_coef(int n_pt, int n_sh, int L, const double *sigma, const 
     pi[kk] = pn;
     ++live;
   }
-  alpha_prev[k] = a;
-  if (upd_cols) {
-    for (int o = 16; o > 0; o >>= 1) live += __shfl_xor_sync(0xffffffffu, live, o);
-    if ((c & 31) == 0 && live) atomicAdd(upd_cols, (unsigned long long)live);
-  }
+  __syncthreads();                   // every energy has read alpha_prev
+  if (threadIdx.y == 0) alpha_prev[k] = a;
+  if (upd_cols && live) atomicAdd(upd_cols, (unsigned long long)live);
 }
 
 // p^_e = r + cb p^_e, x_e += ca p^_e (primal; p^_e = pi_e^k p_e, the scaled search
@@ -703,23 +740,27 @@ __global__ void k_ms_reduce_beta(int n_pt, int n_sh, int L, int n_chunks, const 
                                  const double *tgtd, int *active, int *iters, int *flags,
                                  int max_iter, int *sys_active, int *n_active, const double2 *pi,
                                  int *sactive, int *siters, int *sflags) {
-  const int j = blockIdx.x, c = threadIdx.x;
+  const int j = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
   if (!sys_active[j]) return;   // uniform per block
   const int64_t k = (int64_t)j * L + c;
-  int act = active[k];
-  if (act) {
-    double a[4] = {0, 0, 0, 0};
-    for (int ch = 0; ch < n_chunks; ++ch)
-      for (int q = 0; q < 4; ++q) a[q] += part[(((int64_t)j * n_chunks + ch) * L + c) * 4 + q];
-    const int it = iters[k] + 1;
-    iters[k] = it;
-    const double nr = sqrt(a[2]), nrd = sqrt(a[3]);
-    const double2 rn = make_double2(a[0], a[1]);
-    const double2 rold = rho[k];
-    rho_prev[k] = rold;
-    rho[k] = rn;
+  double a[4];
+  sum_chunks<4>(part, j, L, n_chunks, a);
+  // lane 0 hands the column's squared norms to the lanes, which share the energies
+  extern __shared__ double nsm[];   // [L][2] after the sums are read
+  __shared__ int live_any[1024];
+  __syncthreads();
+  if (ly == 0) {
+    nsm[2 * c] = a[2];
+    nsm[2 * c + 1] = a[3];
+    live_any[c] = 0;
+  }
+  __syncthreads();
+  const double nr = sqrt(nsm[2 * c]), nrd = sqrt(nsm[2 * c + 1]);
+  const int was = active[k];
+  const int it = iters[k] + 1;
+  if (was) {
     int live = 0;
-    for (int e = 0; e < n_sh; ++e) {
+    for (int e = ly; e < n_sh; e += ry) {
       const int64_t kk = ((int64_t)e * n_pt + j) * L + c;
       if (!sactive[kk]) continue;
       const double m = sqrt(cabs2(pi[kk]));
@@ -730,8 +771,19 @@ __global__ void k_ms_reduce_beta(int n_pt, int n_sh, int L, int n_chunks, const 
         live = 1;
       }
     }
+    if (live) live_any[c] = 1;
+  }
+  __syncthreads();                 // every lane has read active and iters
+  int act = 0;
+  if (was && ly == 0) {
+    act = 1;
+    iters[k] = it;
+    const double2 rn = make_double2(a[0], a[1]);
+    const double2 rold = rho[k];
+    rho_prev[k] = rold;
+    rho[k] = rn;
     int stop_flag = 0;
-    if (!live) act = 0;
+    if (!live_any[c]) act = 0;
     else if (!isfinite(nr) || !isfinite(nrd) || !(cabs2(rn) > 0)) stop_flag = 2;
     else if (it >= max_iter) stop_flag = 1;
     else beta[k] = cdiv(rn, rold);
@@ -748,9 +800,9 @@ __global__ void k_ms_reduce_beta(int n_pt, int n_sh, int L, int n_chunks, const 
     }
     active[k] = act;
   }
-  if (!act) beta[k] = make_double2(0, 0);
+  if (ly == 0 && !act) beta[k] = make_double2(0, 0);
   int any = __syncthreads_or(act);
-  if (c == 0) {
+  if (c == 0 && ly == 0) {
     sys_active[j] = any;
     sys_active[n_pt + j] = any;
     if (any) atomicAdd(n_active, 1);
@@ -862,10 +914,12 @@ cbs_status MultiShift<R>::step(int max_iter, cudaStream_t st, int kk) {
   if (prof) CBS_CUDA(cudaEventRecordWithFlags(b.prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
   k_dot_pq<R><<<grd, blk, red_smem(L), st>>>(n_pt, N, L, b.chunk_pts, b.n_chunks, b.p, b.q, b.part, b.sys_active); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
-  k_reduce_alpha<<<n_pt, L, 0, st>>>(n_pt, L, b.n_chunks, b.part, b.rho, b.alpha, b.active, b.flags, b.sys_active,
+  const dim3 rblk = reduce_block(L, b.n_chunks);
+  k_reduce_alpha<<<n_pt, rblk, reduce_smem(rblk), st>>>(n_pt, L, b.n_chunks, b.part, b.rho, b.alpha, b.active, b.flags, b.sys_active,
                                      b.sys_apply); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
-  k_ms_coef<<<n_pt, L, 0, st>>>(n_pt, n_sh, L, sigma, b.alpha, b.beta, alpha_prev, pi, pi_prev, cb, ca,
+  const dim3 eblk((unsigned)L, (unsigned)std::max(1, std::min(n_sh, 512 / L)), 1);
+  k_ms_coef<<<n_pt, eblk, 0, st>>>(n_pt, n_sh, L, sigma, b.alpha, b.beta, alpha_prev, pi, pi_prev, cb, ca,
                                 sactive, sflags, b.sys_active, b.profile ? upd_cols : nullptr); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   const bool uprof = b.profile && kk >= 0 && 2 * kk + 1 < n_upd_ev;
@@ -877,7 +931,7 @@ cbs_status MultiShift<R>::step(int max_iter, cudaStream_t st, int kk) {
                                                   b.alpha, b.active, b.part, b.sys_active); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   CBS_CUDA(cudaMemsetAsync(b.n_active, 0, sizeof(int), st));
-  k_ms_reduce_beta<<<n_pt, L, 0, st>>>(n_pt, n_sh, L, b.n_chunks, b.part, b.rho, b.rho_prev, b.beta, b.tgt, b.tgtd,
+  k_ms_reduce_beta<<<n_pt, rblk, reduce_smem(rblk), st>>>(n_pt, n_sh, L, b.n_chunks, b.part, b.rho, b.rho_prev, b.beta, b.tgt, b.tgtd,
                                        b.active, b.iters, b.flags, max_iter, b.sys_active, b.n_active, pi,
                                        sactive, siters, sflags); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
@@ -1032,11 +1086,21 @@ namespace cbs {
 // bnorm: [2n][L] right-hand-side norms.  colmask[s][c] = 1 if the column still needs work.
 __global__ void k_refine_check(int n, int L, int nchunks, const double *colnorm2, const double *bnorm,
                                double tol, int *colmask, int *n_unconv, double *maxrel) {
-  const int s = blockIdx.x, c = threadIdx.x;
+  extern __shared__ double rsm[];   // [ry][L][2]
+  const int s = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
   double a = 0, b = 0;
-  for (int ch = 0; ch < nchunks; ++ch) {
+#pragma unroll 4
+  for (int ch = ly; ch < nchunks; ch += ry) {
     a += colnorm2[((int64_t)s * nchunks + ch) * L + c];
     b += colnorm2[((int64_t)(n + s) * nchunks + ch) * L + c];
+  }
+  rsm[((size_t)ly * L + c) * 2] = a;
+  rsm[((size_t)ly * L + c) * 2 + 1] = b;
+  __syncthreads();
+  if (ly) return;
+  for (int y = 1; y < ry; ++y) {
+    a += rsm[((size_t)y * L + c) * 2];
+    b += rsm[((size_t)y * L + c) * 2 + 1];
   }
   const double nb = bnorm[(int64_t)s * L + c], nbd = bnorm[(int64_t)(n + s) * L + c];
   const double rel = nb > 0 ? sqrt(a) / nb : 0.0, reld = nbd > 0 ? sqrt(b) / nbd : 0.0;
@@ -1049,7 +1113,8 @@ __global__ void k_refine_check(int n, int L, int nchunks, const double *colnorm2
 cbs_status launch_refine_check(int n, int L, int nchunks, const double *colnorm2, const double *bnorm,
                                double tol, int *colmask, int *n_unconv, double *maxrel,
                                cudaStream_t st) {
-  k_refine_check<<<n, L, 0, st>>>(n, L, nchunks, colnorm2, bnorm, tol, colmask, n_unconv, maxrel); cbs::count_launches(1);
+  const dim3 blk((unsigned)L, (unsigned)std::max(1, std::min(16, 1024 / L)), 1);
+  k_refine_check<<<n, blk, (size_t)blk.x * blk.y * 2 * sizeof(double), st>>>(n, L, nchunks, colnorm2, bnorm, tol, colmask, n_unconv, maxrel); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   return CBS_OK;
 }

@@ -12,6 +12,7 @@
 // back-transform and S C) use a tiled complex FP64 GEMM.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "kernels.cuh"
@@ -391,37 +392,48 @@ __device__ __forceinline__ double2 opload(const double2 *A, int64_t ld, int r, i
   return OP == 2 ? cconj(v) : v;
 }
 
-template <int OPA, int OPB>
-__global__ void k_zgemm(int M, int N, int K, double2 alpha, const double2 *A, int64_t lda,
+// Tiles of TM x TN, 256 threads with 2 x 2 results each.  TM = 8 for products of few rows (the
+// bases and eigenvectors of a small rank: 32 rows would be mostly padding, and a warp's FP64
+// instruction costs the same whatever its active lanes).  k_chunk < K: blockIdx.z is a piece
+// of the K range of the one product of the call, whose sum goes to part[z][N][M] instead of C.
+template <int OPA, int OPB, int TM>
+__global__ void __launch_bounds__(256) k_zgemm(int M, int N, int K, double2 alpha, const double2 *A, int64_t lda,
                         int64_t sA, const double2 *B, int64_t ldb, int64_t sB, double2 beta,
-                        double2 *C, int64_t ldc, int64_t sC) {
-  __shared__ double2 As[16][33];
-  __shared__ double2 Bs[16][33];
-  const int bz = blockIdx.z;
+                        double2 *C, int64_t ldc, int64_t sC, int k_chunk, double2 *part) {
+  constexpr int TN = 1024 / TM, RX = TM / 2;
+  __shared__ double2 As[16][TM + 1];
+  __shared__ double2 Bs[16][TN + 1];
+  const int bz = part ? 0 : blockIdx.z;
+  const int kb0 = part ? (int)blockIdx.z * k_chunk : 0, ke = part ? min(K, kb0 + k_chunk) : K;
   A += bz * sA; B += bz * sB; C += bz * sC;
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 16 + tx;
-  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+  const int tid = threadIdx.x, tx = tid % RX, ty = tid / RX;
+  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
+  const bool busy = m0 + tx * 2 < M && n0 + ty * 2 < N;
   double2 acc[2][2];
   for (int a = 0; a < 2; ++a)
     for (int b = 0; b < 2; ++b) acc[a][b] = make_double2(0, 0);
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int t = tid; t < 512; t += 256) {
+  for (int k0 = kb0; k0 < ke; k0 += 16) {
+    for (int t = tid; t < 16 * TM; t += 256) {
       int mm, kk;
-      if (OPA == 0) { mm = t % 32; kk = t / 32; } else { kk = t % 16; mm = t / 16; }
-      As[kk][mm] = opload<OPA>(A, lda, m0 + mm, k0 + kk, M, K);
+      if (OPA == 0) { mm = t % TM; kk = t / TM; } else { kk = t % 16; mm = t / 16; }
+      As[kk][mm] = opload<OPA>(A, lda, m0 + mm, k0 + kk, M, ke);
+    }
+    for (int t = tid; t < 16 * TN; t += 256) {
       int nn2, kb;
-      if (OPB == 0) { kb = t % 16; nn2 = t / 16; } else { nn2 = t % 32; kb = t / 32; }
-      Bs[kb][nn2] = opload<OPB>(B, ldb, k0 + kb, n0 + nn2, K, N);
+      if (OPB == 0) { kb = t % 16; nn2 = t / 16; } else { nn2 = t % TN; kb = t / TN; }
+      Bs[kb][nn2] = opload<OPB>(B, ldb, k0 + kb, n0 + nn2, ke, N);
     }
     __syncthreads();
+    if (busy) {
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      double2 a0 = As[kk][tx * 2], a1 = As[kk][tx * 2 + 1];
-      double2 b0 = Bs[kk][ty * 2], b1 = Bs[kk][ty * 2 + 1];
-      acc[0][0] = cfma(a0, b0, acc[0][0]);
-      acc[0][1] = cfma(a0, b1, acc[0][1]);
-      acc[1][0] = cfma(a1, b0, acc[1][0]);
-      acc[1][1] = cfma(a1, b1, acc[1][1]);
+      for (int kk = 0; kk < 16; ++kk) {
+        double2 a0 = As[kk][tx * 2], a1 = As[kk][tx * 2 + 1];
+        double2 b0 = Bs[kk][ty * 2], b1 = Bs[kk][ty * 2 + 1];
+        acc[0][0] = cfma(a0, b0, acc[0][0]);
+        acc[0][1] = cfma(a0, b1, acc[0][1]);
+        acc[1][0] = cfma(a1, b0, acc[1][0]);
+        acc[1][1] = cfma(a1, b1, acc[1][1]);
+      }
     }
     __syncthreads();
   }
@@ -429,6 +441,10 @@ __global__ void k_zgemm(int M, int N, int K, double2 alpha, const double2 *A, in
     for (int b = 0; b < 2; ++b) {
       const int r = m0 + tx * 2 + a, c = n0 + ty * 2 + b;
       if (r < M && c < N) {
+        if (part) {
+          part[((int64_t)blockIdx.z * N + c) * M + r] = acc[a][b];
+          continue;
+        }
         double2 *cp = C + r + (int64_t)c * ldc;
         double2 v = cmul(alpha, acc[a][b]);
         if (beta.x != 0.0 || beta.y != 0.0) v = cfma(beta, *cp, v);
@@ -437,13 +453,48 @@ __global__ void k_zgemm(int M, int N, int K, double2 alpha, const double2 *A, in
     }
 }
 
+// C = alpha (sum of the pieces, in order) + beta C
+__global__ void k_zgemm_sum(int M, int N, int pieces, const double2 *part, double2 alpha, double2 beta, double2 *C,
+                            int64_t ldc) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= M * N) return;
+  double2 t = make_double2(0, 0);
+#pragma unroll 8
+  for (int z = 0; z < pieces; ++z) t = cadd(t, part[(int64_t)z * M * N + idx]);
+  double2 *cp = C + idx % M + (int64_t)(idx / M) * ldc;
+  double2 v = cmul(alpha, t);
+  if (beta.x != 0.0 || beta.y != 0.0) v = cfma(beta, *cp, v);
+  *cp = v;
+}
+
+// scratch (scratch_elems complex numbers, or NULL): where a single product with a long K and few
+// tiles is cut into pieces of K, so that more than a few SMs work on it.
 cbs_status zgemm(int opa, int opb, int M, int N, int K, double2 alpha, const double2 *A,
                  int64_t lda, int64_t sA, const double2 *B, int64_t ldb, int64_t sB,
-                 double2 beta, double2 *C, int64_t ldc, int64_t sC, int batch, cudaStream_t st) {
+                 double2 beta, double2 *C, int64_t ldc, int64_t sC, int batch, cudaStream_t st,
+                 double2 *scratch, size_t scratch_elems) {
   if (M <= 0 || N <= 0 || batch <= 0) return CBS_OK;
-  dim3 blk(16, 16, 1);
-  dim3 grd((unsigned)ceil_div(M, 32), (unsigned)ceil_div(N, 32), (unsigned)batch);
-#define ZG(a, b) k_zgemm<a, b><<<grd, blk, 0, st>>>(M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC)
+  const int tm = M <= 8 ? 8 : 32, tn = 1024 / tm;
+  dim3 grd((unsigned)ceil_div(M, tm), (unsigned)ceil_div(N, tn), (unsigned)batch);
+  int k_chunk = K;
+  double2 *part = nullptr;
+  if (batch == 1 && scratch && (int64_t)M * N < (1 << 30)) {
+    // two blocks per SM, pieces of at least 128
+    int pieces = std::min(ceil_div(K, 128), ceil_div(304, (int64_t)grd.x * grd.y));
+    pieces = (int)std::min<size_t>(pieces, scratch_elems / ((size_t)M * N));
+    if (pieces > 1) {
+      k_chunk = ceil_div(ceil_div(K, pieces), 16) * 16;
+      part = scratch;
+      grd.z = (unsigned)ceil_div(K, k_chunk);
+    }
+  }
+#define ZG(a, b)                                                                                                  \
+  do {                                                                                                            \
+    if (tm == 8)                                                                                                  \
+      k_zgemm<a, b, 8><<<grd, 256, 0, st>>>(M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, k_chunk, part);  \
+    else                                                                                                          \
+      k_zgemm<a, b, 32><<<grd, 256, 0, st>>>(M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, k_chunk, part); \
+  } while (0)
   if (opa == 0 && opb == 0) ZG(0, 0);
   else if (opa == 0 && opb == 1) ZG(0, 1);
   else if (opa == 0 && opb == 2) ZG(0, 2);
@@ -454,6 +505,11 @@ cbs_status zgemm(int opa, int opb, int M, int N, int K, double2 alpha, const dou
 #undef ZG
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
+  if (part) {
+    k_zgemm_sum<<<ceil_div((int64_t)M * N, 128), 128, 0, st>>>(M, N, (int)grd.z, part, alpha, beta, C, ldc);
+    cbs::count_launches(1);
+    CBS_CUDA(cudaGetLastError());
+  }
   return CBS_OK;
 }
 

@@ -26,7 +26,8 @@ cbs_status launch_svd(int n_e, int n, double2 *A, double2 *W, double2 *U, double
 cbs_status launch_rank(int n_e, int n, const double *sig, double delta, int *mhat, cudaStream_t st);
 cbs_status zgemm(int opa, int opb, int M, int N, int K, double2 alpha, const double2 *A,
                  int64_t lda, int64_t sA, const double2 *B, int64_t ldb, int64_t sB,
-                 double2 beta, double2 *C, int64_t ldc, int64_t sC, int batch, cudaStream_t st);
+                 double2 beta, double2 *C, int64_t ldc, int64_t sC, int batch, cudaStream_t st,
+                 double2 *scratch = nullptr, size_t scratch_elems = 0);
 cbs_status launch_scale(int n_e, int rows, int ld, const int *mhat, const double *sig, double2 *B,
                         int rows_scale, cudaStream_t st);
 cbs_status launch_eig(int n_e, int ld, const int *mhat, double2 *B, double2 *Z, double2 *tau,

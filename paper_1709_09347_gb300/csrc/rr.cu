@@ -181,7 +181,8 @@ cbs_status cbs_internal_rr(const cbs_hamiltonian *h, double E, const double2 *S,
                oC = add(4 * mm * 16), oZe = add(4 * mm * 16), otau = add(2 * m0 * 16),
                oYc = add(4 * mm * 16), oring = add(2 * m0 * 4), osm = add(64), oP1 = add(4 * mm * 16),
                oPsi = add((size_t)N * 2 * m0 * 16), oD = add(apply_ws_bytes(H, 3, m0, CBS_C128)),
-               otw = add(256), olam = add(2 * m0 * 16);
+               otw = add(256), olam = add(2 * m0 * 16),
+               opart = add((320 * 1024 + mm) * 16);   // pieces of the products over the grid
   char *base = nullptr;
   if (cudaMalloc(&base, bytes) != cudaSuccess) { set_error("cudaMalloc failed (Rayleigh-Ritz workspace)"); return CBS_ENOMEM; }
   *ws_out = base;
@@ -192,6 +193,7 @@ cbs_status cbs_internal_rr(const cbs_hamiltonian *h, double E, const double2 *S,
           *tau = (double2 *)(base + otau), *Yc = (double2 *)(base + oYc), *P1 = (double2 *)(base + oP1),
           *Psi = (double2 *)(base + oPsi), *tw = (double2 *)(base + otw),
           *lam = (double2 *)(base + olam);
+  double2 *part = (double2 *)(base + opart);
   double *sig = (double *)(base + osig);
   int *info = (int *)(base + oinfo), *ring = (int *)(base + oring), *sm = (int *)(base + osm);
   // Z^T (m x N, ld m) = W1^T S^T
@@ -201,7 +203,7 @@ cbs_status cbs_internal_rr(const cbs_hamiltonian *h, double E, const double2 *S,
   const double2 *src = Z;
   std::vector<double> hs(m0);
   for (int pass = 0; pass < 2; ++pass) {
-    CBS_TRY_RR(zgemm(0, 2, r, r, (int)N, one, src, r, 0, src, r, 0, zero, G, r, 0, 1, st));
+    CBS_TRY_RR(zgemm(0, 2, r, r, (int)N, one, src, r, 0, src, r, 0, zero, G, r, 0, 1, st, part, 320 * 1024 + mm));
     CBS_TRY_RR(launch_svd(1, r, G, Gw, Gu, Gws, sig, info, st));
     CBS_CUDA(cudaMemcpyAsync(hs.data(), sig, (size_t)r * sizeof(double), cudaMemcpyDeviceToHost, st));
     CBS_CUDA(cudaStreamSynchronize(st));
@@ -236,9 +238,9 @@ cbs_status cbs_internal_rr(const cbs_hamiltonian *h, double E, const double2 *S,
   CBS_CUDA(cudaGetLastError());
   // CT_l = (Q^dagger X_l)^T = X_l^T conj(Q): zgemm(N, C) on the column-major transposes
   const size_t rr2 = (size_t)r * r;
-  CBS_TRY_RR(zgemm(0, 2, r, r, (int)N, one, X3 + cntQ, r, 0, Q, r, 0, zero, CT, r, 0, 1, st));          // A2
-  CBS_TRY_RR(zgemm(0, 2, r, r, (int)N, one, X3, r, 0, Q, r, 0, zero, CT + rr2, r, 0, 1, st));          // Q^dagger H0 Q
-  CBS_TRY_RR(zgemm(0, 2, r, r, (int)N, one, X3 + 2 * cntQ, r, 0, Q, r, 0, zero, CT + 2 * rr2, r, 0, 1, st));  // A0
+  CBS_TRY_RR(zgemm(0, 2, r, r, (int)N, one, X3 + cntQ, r, 0, Q, r, 0, zero, CT, r, 0, 1, st, part, 320 * 1024 + mm));          // A2
+  CBS_TRY_RR(zgemm(0, 2, r, r, (int)N, one, X3, r, 0, Q, r, 0, zero, CT + rr2, r, 0, 1, st, part, 320 * 1024 + mm));          // Q^dagger H0 Q
+  CBS_TRY_RR(zgemm(0, 2, r, r, (int)N, one, X3 + 2 * cntQ, r, 0, Q, r, 0, zero, CT + 2 * rr2, r, 0, 1, st, part, 320 * 1024 + mm));  // A0
   // shift inside the ring, off the unit circle (propagating eigenvalues sit on it)
   const double2 shift = make_double2(0.7 * cos(2.399963), 0.7 * sin(2.399963));
   k_rr_companion<<<1, kLuThreads, 0, st>>>(r, CT, CT + rr2, CT + 2 * rr2, E, shift, LU, C, info);

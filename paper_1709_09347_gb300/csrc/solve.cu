@@ -119,10 +119,17 @@ static cbs_status check_finite_block(int64_t count, const double2 *A, const char
   return CBS_OK;
 }
 
+// One block of (L, lanes over the points).
 __global__ void k_col_norms(int64_t N, int L, const double2 *B, double *out) {
-  const int c = threadIdx.x;
+  extern __shared__ double sm[];   // [lanes][L]
+  const int c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
   double a = 0;
-  for (int64_t i = 0; i < N; ++i) a += cabs2(B[i * L + c]);
+#pragma unroll 4
+  for (int64_t i = ly; i < N; i += ry) a += cabs2(B[i * L + c]);
+  sm[ly * L + c] = a;
+  __syncthreads();
+  if (ly) return;
+  for (int y = 1; y < ry; ++y) a += sm[y * L + c];
   out[c] = sqrt(a);
 }
 
@@ -201,7 +208,7 @@ struct ResidualCheck {
     }
     CBS_TRY(launch_residual(2 * n, N, L, B, 0, B, 0, n, R, cn, st));
     if (!have_bn) {   // the right-hand sides do not change between calls
-      k_col_norms<<<1, L, 0, st>>>(N, L, B, bn); cbs::count_launches(1);
+      k_col_norms<<<1, dim3((unsigned)L, (unsigned)(1024 / L), 1), (size_t)L * (1024 / L) * sizeof(double), st>>>(N, L, B, bn); cbs::count_launches(1);
       k_bnorm_expand<<<2 * n, L, 0, st>>>(2 * n, L, bn, bn2); cbs::count_launches(1);
       CBS_CUDA(cudaGetLastError());
       have_bn = true;
