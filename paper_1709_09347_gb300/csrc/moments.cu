@@ -43,17 +43,18 @@ cbs_status launch_contour(int n_int, int M, double lambda_min, double2 *coef, do
 // solutions stored in Y[2n][N][L], n = n_e * n_w, of quadrature points j = j0 + jj; with
 // `accumulate` the wave's sum is added to S (points streamed in waves), else it replaces S.
 // mirror > 0: the solutions at the conjugate point j' = mirror - 1 - j (z_j' = conj(z_j),
-// same for the dual twists) are conj(Y_j), which holds for real blocks and a real V, and
-// enter with their own coefficients.
+// same for the dual twists) are conj(Y_j), which holds for real blocks and a real V; S is then
+// real, and its imaginary parts, which would hold nothing but the rounding of terms that
+// cancel, are set to zero (the Hankel matrices and all that follows stay real with them).
 template <int MM, bool MIR>
 __global__ void k_moments(int n, int n_w, int j0, int M, int64_t N, int L, const double2 *__restrict__ Y,
                           const double2 *__restrict__ coef, double2 *__restrict__ S, int accumulate,
                           int mirror) {
   // MIR: a point and its conjugate enter together through
-  //   a y + a' conj(y) = (a + a') Re y + i (a - a') Im y,
-  // two complex-by-real products instead of two complex ones; the four combined
-  // coefficients of each (point, k) are formed once per block in shared memory.
-  extern __shared__ double2 mc[];   // [n_w][4][M]: a+a', i(a-a'), -(b+b'), -i(b-b')
+  //   Re(a y + a' conj(y)) = Re(a + a') Re y - Im(a - a') Im y,
+  // two real products; the four combined coefficients of each (point, k) are formed once per
+  // block in shared memory.
+  extern __shared__ double mc[];   // [n_w][4][M]: Re(a+a'), -Im(a-a'), -Re(b+b'), Im(b-b')
   const int e = blockIdx.y, c = threadIdx.x, ly = threadIdx.y, py = blockDim.y;
   const int M2 = 2 * M;
   if (MIR) {
@@ -64,11 +65,11 @@ __global__ void k_moments(int n, int n_w, int j0, int M, int64_t N, int L, const
       const double2 b = coef[((int64_t)(j0 + jj) * 2 + 1) * M2 + k];
       const double2 am = coef[((int64_t)jm * 2 + 0) * M2 + k];
       const double2 bm = coef[((int64_t)jm * 2 + 1) * M2 + k];
-      double2 *q = mc + (int64_t)jj * 4 * M;
-      q[k] = make_double2(a.x + am.x, a.y + am.y);
-      q[M + k] = make_double2(-(a.y - am.y), a.x - am.x);
-      q[2 * M + k] = make_double2(-(b.x + bm.x), -(b.y + bm.y));
-      q[3 * M + k] = make_double2(b.y - bm.y, -(b.x - bm.x));
+      double *q = mc + (int64_t)jj * 4 * M;
+      q[k] = a.x + am.x;
+      q[M + k] = -(a.y - am.y);
+      q[2 * M + k] = -(b.x + bm.x);
+      q[3 * M + k] = b.y - bm.y;
     }
     __syncthreads();
   }
@@ -85,14 +86,11 @@ __global__ void k_moments(int n, int n_w, int j0, int M, int64_t N, int L, const
       const double2 y1 = Y[(s * N + i) * L + c];
       const double2 y2 = Y[((n + s) * N + i) * L + c];
       if (MIR) {
-        const double2 *q = mc + (int64_t)jj * 4 * M;
+        const double *q = mc + (int64_t)jj * 4 * M;
 #pragma unroll
         for (int k = 0; k < MM; ++k)
-          if (k < M) {
-            const double2 p0 = q[k], p1 = q[M + k], p2 = q[2 * M + k], p3 = q[3 * M + k];
-            acc[k].x = fma(p3.x, y2.y, fma(p2.x, y2.x, fma(p1.x, y1.y, fma(p0.x, y1.x, acc[k].x))));
-            acc[k].y = fma(p3.y, y2.y, fma(p2.y, y2.x, fma(p1.y, y1.y, fma(p0.y, y1.x, acc[k].y))));
-          }
+          if (k < M)
+            acc[k].x = fma(q[3 * M + k], y2.y, fma(q[2 * M + k], y2.x, fma(q[M + k], y1.y, fma(q[k], y1.x, acc[k].x))));
       } else {
         const double2 *a = coef + (int64_t)(j0 + jj) * 2 * M2;
         const double2 *b = a + M2;
@@ -117,7 +115,7 @@ __global__ void k_moments(int n, int n_w, int j0, int M, int64_t N, int L, const
     }
 #pragma unroll
     for (int k = 0; k < MM; ++k)
-      if (k < M) Se[(int64_t)k * L + c] = acc[k];
+      if (k < M) Se[(int64_t)k * L + c] = mirror > 0 ? make_double2(acc[k].x, 0) : acc[k];
   }
 }
 
@@ -125,7 +123,7 @@ cbs_status launch_moments(int n, int n_e, int n_w, int j0, int M, int64_t N, int
                           const double2 *coef, double2 *S, bool accumulate, int mirror, cudaStream_t st) {
   dim3 blk = col_block(L);
   dim3 grd((unsigned)ceil_div(N, (int64_t)blk.y * 4), (unsigned)n_e, 1);
-  const size_t msm = (size_t)n_w * 4 * M * sizeof(double2);
+  const size_t msm = (size_t)n_w * 4 * M * sizeof(double);
   const bool mir = mirror > 0 && msm <= 48 * 1024;
   const int acc = accumulate ? 1 : 0;
   if (M <= 8) {
@@ -196,7 +194,7 @@ __global__ void k_vhy(int64_t N, int L, int n_chunks, const double2 *__restrict_
 
 // mu[e][k][c1][c2] (+)= sum_jj sum_chunks a_{j0+jj,k} G_jj - b_{j0+jj,k} G~_jj over the wave's
 // points; mirror > 0: plus the conjugate points' terms, whose G = V^dagger conj(Y_j) is
-// conj(G_j) for a real V
+// conj(G_j) for a real V; mu is then real, as S is
 __global__ void k_mu(int n, int n_w, int j0, int M2, int L, int n_chunks, const double2 *part,
                      const double2 *coef, double2 *mu, int accumulate, int mirror) {
   const int e = blockIdx.y, k = blockIdx.x;
@@ -223,6 +221,7 @@ __global__ void k_mu(int n, int n_w, int j0, int M2, int L, int n_chunks, const 
         acc = cfma(make_double2(-bm.x, -bm.y), cconj(gd), acc);
       }
     }
+    if (mirror > 0) acc.y = 0;
     *out = acc;
   }
 }
