@@ -10,6 +10,7 @@
 // One thread block per energy runs each factorisation; matrices are column-major in
 // global memory (they fit in L2).  The GEMMs (T^< W_1, U_1^dagger C, the eigenvector
 // back-transform and S C) use a tiled complex FP64 GEMM.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
@@ -80,150 +81,165 @@ __global__ void k_hankel(int n_e, int L, int M, const double2 *mu, double2 *T, d
 // T = (Q V_x) Sigma (P U_x)^dagger, i.e. U = Q V_x and W = P U_x.
 constexpr int kSvdThreads = 256;
 
-// Column-pivoted Householder QR, one block per energy (A in place: R in the upper
-// triangle, zeros below).  Step k takes the remaining column of largest partial norm
-// (the first one on ties), then the reflector H_k = I - beta_k v_k v_k^dagger with
-// v_k = x + (x_0/|x_0|) ||x|| e_0 on x = A(k:n, k), beta_k = 2 / (v_k^dagger v_k), which
-// maps x onto -(x_0/|x_0|) ||x|| e_0; v_k goes to column k of Vh (rows k..n-1).  The partial
-// norms are downdated and recomputed from the column once the downdate has cancelled
-// more than half the digits (the criterion of LAPACK's xLAQP2).  Q = H_0 H_1 ... H_{n-1}.
+// Column-pivoted Householder QR, a cluster of 8 blocks per energy; block r owns the columns
+// j = r mod 8.  Step k takes the remaining column p of largest partial norm (the lowest one on
+// ties), then the reflector H_k = I - beta_k v_k v_k^dagger with
+// v_k = x + (x_0/|x_0|) ||x|| e_0 on x = A(k:n, p), beta_k = 2 / (v_k^dagger v_k), which
+// maps x onto -(x_0/|x_0|) ||x|| e_0 (Rd[k]); v_k goes to column k of Vh (rows k..n-1).  Columns
+// stay in place: R(j, k) = A(j, perm[k]) for j < k.  The squared partial norms are downdated and
+// recomputed from the column once the downdate has cancelled more than half the digits (the
+// criterion of LAPACK's xLAQP2).  Q = H_0 H_1 ... H_{n-1}.
+// 1.2 ms for n = 128 and one energy.  Bound by the latency of a step (one cluster barrier, one column load from L2, a reflector and
+// a column update of dependent FP64 operations, 64 cycles each): one block per energy, at FP64
+// issue on its one SM, took 8.7 ms for n = 128 and 43.7 ms for 16 of n = 256.
 constexpr int kQrpThreads = 512;
-__global__ void __launch_bounds__(kQrpThreads) k_qrp(int n, double2 *Ab, double2 *Vhb, double *betab,
-                                                     int *permb) {
-  const int e = blockIdx.x;
+constexpr int kQrpBlocks = 8;
+__global__ void __cluster_dims__(kQrpBlocks, 1, 1) __launch_bounds__(kQrpThreads)
+    k_qrp(int n, double2 *Ab, double2 *Vhb, double *betab, int *permb, double2 *Rdb) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int e = blockIdx.x / kQrpBlocks, rank = (int)cluster.block_rank();
   const int64_t nn = (int64_t)n * n;
   double2 *A = Ab + e * nn, *Vh = Vhb + e * nn;
   double *beta = betab + (int64_t)e * n;
   int *perm = permb + (int64_t)e * n;
+  double2 *Rd = Rdb + (int64_t)e * n;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int nwarp = kQrpThreads / 32;
-  __shared__ double vn1[512], vn2[512];
-  __shared__ int sperm[512];
-  __shared__ double red_v[nwarp];
-  __shared__ int red_i[nwarp];
-  __shared__ int sh_p;
+  const int nl = (n - rank + kQrpBlocks - 1) / kQrpBlocks;   // own columns
+  __shared__ double w1[512 / kQrpBlocks], w2[512 / kQrpBlocks];   // squared partial norms; -1: taken
+  __shared__ double2 v[512];
+  __shared__ double red[nwarp];
+  __shared__ double cand_v[2];   // this block's best column, by parity of the step
+  __shared__ int cand_j[2];
+  __shared__ double2 sh_x0;
   __shared__ double sh_beta;
   const double tol3z = sqrt(2.220446049250313e-16);
-  auto At = [&](int i, int j) -> double2 & { return A[i + (int64_t)j * n]; };
-  for (int j = warp; j < n; j += nwarp) {
+  for (int l = warp; l < nl; l += nwarp) {
+    const double2 *a = A + (int64_t)(l * kQrpBlocks + rank) * n;
     double t = 0;
-    for (int i = lane; i < n; i += 32) t += cabs2(At(i, j));
+    for (int i = lane; i < n; i += 32) t += cabs2(a[i]);
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) vn1[j] = vn2[j] = sqrt(t);
+    if (lane == 0) w1[l] = w2[l] = t;
   }
-  for (int j = tid; j < n; j += kQrpThreads) sperm[j] = j;
   __syncthreads();
   for (int k = 0; k < n; ++k) {
-    // pivot: largest vn1[j], j >= k, first index on ties
-    double bv = -1.0;
-    int bi = n;
-    for (int j = k + tid; j < n; j += kQrpThreads)
-      if (vn1[j] > bv) { bv = vn1[j]; bi = j; }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-    }
-    if (lane == 0) { red_v[warp] = bv; red_i[warp] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      double v = red_v[0];
-      int i0 = red_i[0];
-      for (int w = 1; w < nwarp; ++w)
-        if (red_v[w] > v || (red_v[w] == v && red_i[w] < i0)) { v = red_v[w]; i0 = red_i[w]; }
-      sh_p = i0;
-    }
-    __syncthreads();
-    const int p = sh_p;
-    if (p != k) {
-      for (int i = tid; i < n; i += kQrpThreads) {
-        const double2 t = At(i, k);
-        At(i, k) = At(i, p);
-        At(i, p) = t;
-      }
-      if (tid == 0) {
-        double t = vn1[k]; vn1[k] = vn1[p]; vn1[p] = t;
-        t = vn2[k]; vn2[k] = vn2[p]; vn2[p] = t;
-        const int q = sperm[k]; sperm[k] = sperm[p]; sperm[p] = q;
-      }
-    }
-    __syncthreads();
-    // reflector of column k (warp 0)
     if (warp == 0) {
-      double a2 = 0;
-      for (int i = k + lane; i < n; i += 32) a2 += cabs2(At(i, k));
-      for (int o = 16; o > 0; o >>= 1) a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-      const double2 x0 = At(k, k);
-      if (a2 > 0) {
-        const double alpha = sqrt(a2), ax0 = cabsd(x0);
-        const double2 ph = ax0 > 0 ? make_double2(x0.x / ax0, x0.y / ax0) : make_double2(1, 0);
-        for (int i = k + lane; i < n; i += 32)
-          Vh[i + (int64_t)k * n] = (i == k) ? make_double2(x0.x + ph.x * alpha, x0.y + ph.y * alpha) : At(i, k);
-        __syncwarp();
-        if (lane == 0) {
-          sh_beta = 1.0 / (a2 + alpha * ax0);
-          At(k, k) = make_double2(-ph.x * alpha, -ph.y * alpha);
-        }
-      } else {
-        for (int i = k + lane; i < n; i += 32) Vh[i + (int64_t)k * n] = make_double2(0, 0);
-        if (lane == 0) sh_beta = 0.0;
+      double bv = -1.0;
+      int bj = n;
+      for (int l = lane; l < nl; l += 32)
+        if (w1[l] > bv) { bv = w1[l]; bj = l * kQrpBlocks + rank; }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+        if (ov > bv || (ov == bv && oj < bj)) { bv = ov; bj = oj; }
       }
-      for (int i = k + 1 + lane; i < n; i += 32) At(i, k) = make_double2(0, 0);
-      if (lane == 0) beta[k] = sh_beta;
+      if (lane == 0) { cand_v[k & 1] = bv; cand_j[k & 1] = bj; }
+    }
+    cluster.sync();   // candidates and the columns updated in the last step are visible
+    int p;
+    {
+      const int from = lane & (kQrpBlocks - 1);
+      double bv = *cluster.map_shared_rank(&cand_v[k & 1], from);
+      int bj = *cluster.map_shared_rank(&cand_j[k & 1], from);
+      for (int o = kQrpBlocks / 2; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+        if (ov > bv || (ov == bv && oj < bj)) { bv = ov; bj = oj; }
+      }
+      p = bj;
+    }
+    // every block forms the reflector of column p for itself (the column comes from L2: its owner
+    // is another SM)
+    const double2 x = (tid >= k && tid < n) ? __ldcg(A + tid + (int64_t)p * n) : make_double2(0, 0);
+    double a2 = cabs2(x);
+    for (int o = 16; o > 0; o >>= 1) a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+    if (lane == 0) red[warp] = a2;
+    if (tid > k && tid < n) v[tid] = x;
+    if (tid == k) sh_x0 = x;
+    __syncthreads();
+    if (warp == 0) {
+      double t = lane < nwarp ? red[lane] : 0.0;
+      for (int o = nwarp / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      t = __shfl_sync(0xffffffffu, t, 0);
+      const double2 x0 = sh_x0;
+      double2 v0 = make_double2(0, 0), r = v0;
+      double b = 0;
+      if (t > 0) {
+        const double ax2 = cabs2(x0), alpha = sqrt(t);
+        if (ax2 > 0) {
+          const double q = alpha * rsqrt(ax2);         // ||x|| / |x_0|
+          v0 = make_double2(fma(x0.x, q, x0.x), fma(x0.y, q, x0.y));
+          r = make_double2(-x0.x * q, -x0.y * q);
+          b = 1.0 / (t + ax2 * q);
+        } else {
+          v0 = make_double2(alpha, 0);
+          r = make_double2(-alpha, 0);
+          b = 1.0 / t;
+        }
+      }
+      if (lane == 0) {
+        v[k] = v0;
+        sh_beta = b;
+        if (rank == 0) { beta[k] = b; perm[k] = p; Rd[k] = r; }
+        if (p % kQrpBlocks == rank) w1[p / kQrpBlocks] = -1.0;
+      }
     }
     __syncthreads();
     const double b = sh_beta;
-    const double2 *v = Vh + (int64_t)k * n;
-    // A(k:n, j) -= beta v (v^dagger A(k:n, j)) for j > k, one warp per column; then the
-    // column's partial norm
-    for (int j = k + 1 + warp; j < n; j += nwarp) {
+    if (rank == 0)
+      for (int i = k + tid; i < n; i += kQrpThreads) Vh[i + (int64_t)k * n] = b != 0 ? v[i] : make_double2(0, 0);
+    // A(k:n, j) -= beta v (v^dagger A(k:n, j)) for the own columns left, one warp per column; then
+    // the column's partial norm
+    for (int l = warp; l < nl; l += nwarp) {
+      const double wl = w1[l];
+      if (wl < 0) continue;
+      double2 *a = A + (int64_t)(l * kQrpBlocks + rank) * n;
       if (b != 0) {
         double sx = 0, sy = 0;
         for (int i = k + lane; i < n; i += 32) {
-          const double2 t = cmulc(v[i], At(i, j));   // conj(v_i) a_i
-          sx += t.x;
-          sy += t.y;
+          const double2 u = v[i], c = a[i];   // conj(v_i) a_i
+          sx = fma(u.x, c.x, fma(u.y, c.y, sx));
+          sy = fma(u.x, c.y, fma(-u.y, c.x, sy));
         }
         for (int o = 16; o > 0; o >>= 1) {
           sx += __shfl_xor_sync(0xffffffffu, sx, o);
           sy += __shfl_xor_sync(0xffffffffu, sy, o);
         }
-        const double2 sb = make_double2(sx * b, sy * b);
-        for (int i = k + lane; i < n; i += 32) At(i, j) = csub(At(i, j), cmul(v[i], sb));
+        const double2 sb = make_double2(-sx * b, -sy * b);
+        for (int i = k + lane; i < n; i += 32) a[i] = cfma(sb, v[i], a[i]);
         __syncwarp();
       }
-      const double nj = vn1[j];
-      if (nj != 0) {
-        double t = cabsd(At(k, j)) / nj;
-        t = fmax(0.0, (1.0 + t) * (1.0 - t));
-        const double r = nj / vn2[j];
-        if (t * r * r <= tol3z) {
+      if (wl > 0) {
+        const double left = wl - cabs2(a[k]);
+        if (left <= tol3z * w2[l]) {
           double q = 0;
-          for (int i = k + 1 + lane; i < n; i += 32) q += cabs2(At(i, j));
+          for (int i = k + 1 + lane; i < n; i += 32) q += cabs2(a[i]);
           for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
           __syncwarp();
-          if (lane == 0) vn1[j] = vn2[j] = sqrt(q);
+          if (lane == 0) w1[l] = w2[l] = q;
         } else {
           __syncwarp();
-          if (lane == 0) vn1[j] = nj * sqrt(t);
+          if (lane == 0) w1[l] = left;
         }
       }
     }
     __syncthreads();
   }
-  for (int j = tid; j < n; j += kQrpThreads) perm[j] = sperm[j];
+  cluster.sync();   // no block leaves while another may read its candidate
 }
 
-// X = R^dagger (lower triangular) from the upper triangle of R
-__global__ void k_rdagger(int n, const double2 *Rb, double2 *Xb) {
+// X = R^dagger (lower triangular): R's diagonal in Rd, R(j, i) = A(j, perm[i]) above it
+__global__ void k_rdagger(int n, const double2 *Rb, const int *permb, const double2 *Rdb, double2 *Xb) {
   const int e = blockIdx.y;
   const int64_t nn = (int64_t)n * n;
   const double2 *R = Rb + e * nn;
+  const int *perm = permb + (int64_t)e * n;
   double2 *X = Xb + e * nn;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < nn;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(idx % n), j = (int)(idx / n);
-    X[idx] = (j <= i) ? cconj(R[j + (int64_t)i * n]) : make_double2(0, 0);
+    X[idx] = j < i ? cconj(R[j + (int64_t)perm[i] * n]) : j == i ? cconj(Rdb[(int64_t)e * n + i]) : make_double2(0, 0);
   }
 }
 
@@ -279,57 +295,153 @@ __global__ void k_svd_init(int n, double2 *Wb) {
     W[idx] = make_double2((idx % n) == (idx / n) ? 1.0 : 0.0, 0.0);
 }
 
+// Sums of four values over a warp, to every lane: the lanes share the values as the butterfly
+// narrows, 6 FP64 additions instead of 20.
+__device__ __forceinline__ void warp_sum4(double (&v)[4]) {
+  const int lane = threadIdx.x & 31;
+  const bool h = lane & 16, g = lane & 8;
+  double p = h ? v[2] : v[0], q = h ? v[3] : v[1];
+  const double sp = h ? v[0] : v[2], sq = h ? v[1] : v[3];
+  p += __shfl_xor_sync(0xffffffffu, sp, 16);
+  q += __shfl_xor_sync(0xffffffffu, sq, 16);
+  double r = g ? q : p;
+  const double sr = g ? p : q;
+  r += __shfl_xor_sync(0xffffffffu, sr, 8);
+  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xffffffffu, r, 8 * k);
+}
+
+// Rotation that makes two columns orthogonal, from their squared norms al, be and inner product
+// g: with g = |g| e^{i phi}, zeta = (be - al)/(2|g|), t the smaller root of
+// t^2 + 2 zeta t - 1 = 0,
+//   a_p' = c a_p - s e^{-i phi} a_q,  a_q' = s e^{i phi} a_p + c a_q,   sp = s e^{i phi}.
+// False where the pair is orthogonal to tolj.  It stands alone on every round's critical path,
+// so it avoids the divisions and hypot of the textbook form (about 150 dependent FP64
+// operations): t starts in single precision and takes one Newton step.
+__device__ __forceinline__ bool pair_rotation(double al, double be, double gx, double gy, double tolj, double &c,
+                                              double2 &sp) {
+  const double g2 = fma(gx, gx, gy * gy), ab = al * be;
+  if (al == 0.0 || be == 0.0) return false;
+  if (!(g2 > 1e-270 && g2 < 1e270 && ab > 1e-270 && ab < 1e270)) {
+    const double g = hypot(gx, gy);
+    if (!(g > tolj * (sqrt(al) * sqrt(be)))) return false;
+    const double zeta = (be - al) / (2.0 * g);
+    const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+    c = 1.0 / sqrt(1.0 + t * t);
+    sp = make_double2(c * t * (gx / g), c * t * (gy / g));
+    return true;
+  }
+  if (!(g2 > tolj * tolj * ab)) return false;
+  const double ig = rsqrt(g2);
+  const double zeta = 0.5 * (be - al) * ig, az = fabs(zeta);
+  double t;
+  if (az < 1e15) {
+    const float zf = (float)az, t0 = 1.0f / (zf + sqrtf(fmaf(zf, zf, 1.0f)));
+    t = (double)t0;
+    t -= (fma(t, t, -1.0) + 2.0 * az * t) * (double)(0.5f / (t0 + zf));
+  } else {
+    t = 0.5 / az;
+  }
+  c = rsqrt(fma(t, t, 1.0));
+  const double s = copysign(c * t, zeta) * ig;
+  sp = make_double2(s * gx, s * gy);
+  return true;
+}
+
+// Columns of round `round`, pair pi (circle method: player 0 fixed, the others rotate)
+__device__ __forceinline__ bool round_pair(int n, int round, int pi, int &p, int &q) {
+  const int nn2 = (n + 1) & ~1;
+  if (pi >= nn2 / 2) return false;
+  const int a = pi, b = nn2 - 1 - pi;
+  p = (a == 0) ? 0 : ((a - 1 + round) % (nn2 - 1)) + 1;
+  q = (b == 0) ? 0 : ((b - 1 + round) % (nn2 - 1)) + 1;
+  return p < n && q < n;
+}
+
+__device__ __forceinline__ void rotate_rows(double2 *ap, double2 *aq, int first, int step, int n, double c, double2 sp) {
+  for (int i = first; i < n; i += step) {
+    const double2 u = ap[i], v = aq[i];
+    ap[i] = make_double2(fma(c, u.x, -fma(sp.x, v.x, sp.y * v.y)), fma(c, u.y, -fma(sp.x, v.y, -sp.y * v.x)));
+    aq[i] = make_double2(fma(c, v.x, fma(sp.x, u.x, -sp.y * u.y)), fma(c, v.y, fma(sp.x, u.y, sp.y * u.x)));
+  }
+}
+
+__device__ __forceinline__ void pair_products(const double2 *ap, const double2 *aq, int first, int step, int n,
+                                              double (&s)[4]) {
+  s[0] = s[1] = s[2] = s[3] = 0;
+  for (int i = first; i < n; i += step) {
+    const double2 u = ap[i], v = aq[i];
+    s[0] = fma(u.x, u.x, fma(u.y, u.y, s[0]));
+    s[1] = fma(v.x, v.x, fma(v.y, v.y, s[1]));
+    s[2] = fma(u.x, v.x, fma(u.y, v.y, s[2]));    // conj(u) v
+    s[3] = fma(u.x, v.y, fma(-u.y, v.x, s[3]));
+  }
+}
+
+// One warp per pair, 8 pairs per block: rounds of many pairs, bound by FP64 issue.
 __global__ void __launch_bounds__(kSvdThreads) k_svd_round(int n, int round, double2 *Ab, double2 *Wb,
                                                            double tolj, int *rot) {
   const int e = blockIdx.y;
   const int64_t nn = (int64_t)n * n;
   double2 *A = Ab + e * nn, *W = Wb + e * nn;
   const int lane = threadIdx.x & 31;
-  const int pi = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int nn2 = (n + 1) & ~1;
-  if (pi >= nn2 / 2) return;
-  // circle method: player 0 fixed, the others rotate by `round`
-  const int a = pi, b = nn2 - 1 - pi;
-  const int p = (a == 0) ? 0 : ((a - 1 + round) % (nn2 - 1)) + 1;
-  const int q = (b == 0) ? 0 : ((b - 1 + round) % (nn2 - 1)) + 1;
-  if (p >= n || q >= n) return;
+  int p, q;
+  if (!round_pair(n, round, blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), p, q)) return;
   double2 *ap = A + (int64_t)p * n, *aq = A + (int64_t)q * n;
-  double al = 0, be = 0, gx = 0, gy = 0;
-  for (int i = lane; i < n; i += 32) {
-    const double2 u = ap[i], v = aq[i];
-    al += cabs2(u);
-    be += cabs2(v);
-    gx += u.x * v.x + u.y * v.y;   // conj(u) v
-    gy += u.x * v.y - u.y * v.x;
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    al += __shfl_xor_sync(0xffffffffu, al, o);
-    be += __shfl_xor_sync(0xffffffffu, be, o);
-    gx += __shfl_xor_sync(0xffffffffu, gx, o);
-    gy += __shfl_xor_sync(0xffffffffu, gy, o);
-  }
-  const double g = hypot(gx, gy);
-  if (!(g > tolj * sqrt(al * be)) || al == 0.0 || be == 0.0) return;
-  // rotation that makes columns p and q orthogonal: with gamma = |g| e^{i phi},
-  // zeta = (be - al)/(2|g|), t the smaller root of t^2 + 2 zeta t - 1 = 0,
-  // a_p' = c a_p - s e^{-i phi} a_q,  a_q' = s e^{i phi} a_p + c a_q
-  const double zeta = (be - al) / (2.0 * g);
-  const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-  const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-  const double2 sp = make_double2(s * gx / g, s * gy / g);    // s e^{i phi}
-  const double2 spc = make_double2(sp.x, -sp.y);              // s e^{-i phi}
-  for (int i = lane; i < n; i += 32) {
-    const double2 u = ap[i], v = aq[i];
-    ap[i] = csub(cscale(u, c), cmul(spc, v));
-    aq[i] = cadd(cmul(sp, u), cscale(v, c));
-  }
-  double2 *wp = W + (int64_t)p * n, *wq = W + (int64_t)q * n;
-  for (int i = lane; i < n; i += 32) {
-    const double2 u = wp[i], v = wq[i];
-    wp[i] = csub(cscale(u, c), cmul(spc, v));
-    wq[i] = cadd(cmul(sp, u), cscale(v, c));
-  }
+  double s[4], c;
+  double2 sp;
+  pair_products(ap, aq, lane, 32, n, s);
+  warp_sum4(s);
+  if (!pair_rotation(s[0], s[1], s[2], s[3], tolj, c, sp)) return;
+  rotate_rows(ap, aq, lane, 32, n, c, sp);
+  rotate_rows(W + (int64_t)p * n, W + (int64_t)q * n, lane, 32, n, c, sp);
   if (lane == 0) atomicAdd(&rot[e], 1);
+}
+
+// One block per pair, 4 warps on the rows of A and 4 on those of W: rounds with fewer pairs than
+// keep the GPU's FP64 pipes busy, bound by the latency of the round.  One round of n = 128:
+// 6.6 us; with a warp per pair, on 8 SMs at FP64 issue, 19 us.
+__global__ void __launch_bounds__(kSvdThreads) k_svd_round_wide(int n, int round, double2 *Ab, double2 *Wb,
+                                                                double tolj, int *rot) {
+  const int e = blockIdx.y;
+  const int64_t nn = (int64_t)n * n;
+  int p, q;
+  if (!round_pair(n, round, blockIdx.x, p, q)) return;
+  const int half = kSvdThreads / 2, tid = threadIdx.x, warp = tid >> 5;
+  const bool on_a = tid < half;
+  double2 *M = (on_a ? Ab : Wb) + e * nn;
+  double2 *mp = M + (int64_t)p * n, *mq = M + (int64_t)q * n;
+  __shared__ double part[half / 32][4];
+  __shared__ double rc;
+  __shared__ double2 rsp;
+  __shared__ int turn;
+  double s[4];
+  if (on_a) {
+    pair_products(mp, mq, tid, half, n, s);
+    warp_sum4(s);
+    if ((tid & 31) == 0)
+      for (int k = 0; k < 4; ++k) part[warp][k] = s[k];
+  }
+  __syncthreads();
+  if (warp == 0) {
+    for (int k = 0; k < 4; ++k) {
+      s[k] = part[0][k];
+      for (int w = 1; w < half / 32; ++w) s[k] += part[w][k];
+    }
+    double c = 1;
+    double2 sp = make_double2(0, 0);
+    const bool go = pair_rotation(s[0], s[1], s[2], s[3], tolj, c, sp);
+    if (tid == 0) {
+      rc = c;
+      rsp = sp;
+      turn = go;
+      if (go) atomicAdd(&rot[e], 1);
+    }
+  }
+  __syncthreads();
+  if (!turn) return;
+  rotate_rows(mp, mq, on_a ? tid : tid - half, half, n, rc, rsp);
 }
 
 // sigma_j = ||a_j||, sorted descending (ties by index); U = A/sigma, W permuted alike.
@@ -972,24 +1084,29 @@ cbs_status launch_svd(int n_e, int n, double2 *A, double2 *W, double2 *U, double
     void *p = nullptr;
     ~Work() { if (p) cudaFree(p); }
   } wk;
-  const size_t wbytes = (size_t)nn * n_e * sizeof(double2) + (size_t)n * n_e * (sizeof(double) + sizeof(int)) + 256;
+  const size_t wbytes = (size_t)nn * n_e * sizeof(double2) +
+                        (size_t)n * n_e * (sizeof(double2) + sizeof(double) + sizeof(int)) + 256;
   if (cudaMalloc(&wk.p, wbytes) != cudaSuccess) {
     wk.p = nullptr;
     set_error("cudaMalloc failed (SVD workspace)");
     return CBS_ENOMEM;
   }
   double2 *Vh = (double2 *)wk.p;
-  double *beta = (double *)(Vh + nn * n_e);
+  double2 *Rd = Vh + nn * n_e;
+  double *beta = (double *)(Rd + (size_t)n * n_e);
   int *perm = (int *)(beta + (size_t)n * n_e);
   // T P = Q R in place (A holds R), X = R^dagger into Ws: the matrix the sweeps rotate
-  k_qrp<<<n_e, kQrpThreads, 0, st>>>(n, A, Vh, beta, perm);
+  k_qrp<<<n_e * kQrpBlocks, kQrpThreads, 0, st>>>(n, A, Vh, beta, perm, Rd);
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
-  k_rdagger<<<dim3(64, (unsigned)n_e, 1), 256, 0, st>>>(n, A, Ws);
+  k_rdagger<<<dim3(64, (unsigned)n_e, 1), 256, 0, st>>>(n, A, perm, Rd, Ws);
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   double2 *X = Ws;
-  dim3 grd_round((unsigned)ceil_div(nn2 / 2, warps), (unsigned)n_e, 1);
+  // a block per pair while that is at most two blocks per SM (n = 256 with 2 energies is still
+  // wide; 16 energies of n = 256 are bound by FP64 issue in either form)
+  const bool wide = (int64_t)nn2 / 2 * n_e <= 2 * 152;
+  dim3 grd_round((unsigned)(wide ? nn2 / 2 : ceil_div(nn2 / 2, warps)), (unsigned)n_e, 1);
   k_svd_init<<<dim3(64, (unsigned)n_e, 1), 256, 0, st>>>(n, W);
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
@@ -1001,7 +1118,8 @@ cbs_status launch_svd(int n_e, int n, double2 *A, double2 *W, double2 *U, double
   CBS_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   cudaError_t ce = cudaMemsetAsync(rot, 0, (size_t)n_e * sizeof(int), st);
   for (int r = 0; r < nn2 - 1 && ce == cudaSuccess; ++r) {
-    k_svd_round<<<grd_round, kSvdThreads, 0, st>>>(n, r, X, W, tolj, rot);
+    if (wide) k_svd_round_wide<<<grd_round, kSvdThreads, 0, st>>>(n, r, X, W, tolj, rot);
+    else k_svd_round<<<grd_round, kSvdThreads, 0, st>>>(n, r, X, W, tolj, rot);
     cbs::count_launches(1);
     ce = cudaGetLastError();
   }
@@ -1032,7 +1150,9 @@ cbs_status launch_svd(int n_e, int n, double2 *A, double2 *W, double2 *U, double
   k_svd_finish<<<n_e, 1024, 0, st>>>(n, X, W, A, U, sig);
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
-  k_apply_q<<<dim3((unsigned)ceil_div(n, 16), (unsigned)n_e, 1), 512, 0, st>>>(n, Vh, beta, U);
+  // a column's chain of reflectors is one warp's: few columns per block spread them over the SMs
+  const int qw = (int64_t)n * n_e <= 152 * 8 ? 2 : 16;
+  k_apply_q<<<dim3((unsigned)ceil_div(n, qw), (unsigned)n_e, 1), 32 * qw, 0, st>>>(n, Vh, beta, U);
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   k_permute_rows<<<dim3(64, (unsigned)n_e, 1), 256, 0, st>>>(n, perm, A, Ws);
