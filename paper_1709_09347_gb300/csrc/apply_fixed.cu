@@ -15,21 +15,6 @@
 
 namespace cbs {
 
-// What one (system, column) needs besides its vector.
-struct ColumnScale {
-  FixScale f;
-  int base;        // exponent offset of to_fixed
-  long long ef;    // E - diag_kin in the unit of the weights
-  long long pad;
-  double2 w, wi;   // the twist and its inverse
-};
-static_assert(sizeof(ColumnScale) % 16 == 0, "ColumnScale is read in 16-byte pieces");
-
-__device__ __forceinline__ void twist_and_inverse(const double2 *twist, int64_t k, double2 &w, double2 &wi) {
-  w = twist[k];
-  wi = cdiv(make_double2(1.0, 0.0), w);
-}
-
 // Bound by memory: 44 us for 268 MB (32 systems of the 32x32x16 cell, L = 32), 6.1 TB/s.
 // maxhi[s][chunk][c] = max over the chunk's points of the high word of |re|, |im| (the order of
 // non-negative doubles)
@@ -54,26 +39,21 @@ __global__ void k_column_max(int64_t N, int L, int chunk_pts, const double2 *__r
   }
 }
 
-// One block per system, one thread per column: the FP64 work of the scales (a division, the
+// One block of (L, lanes over the chunks) per system: the FP64 work of the scales (a division, the
 // conversions) is done here once instead of by every thread of the kernels that use them.
 __global__ void k_fix_scales(const __grid_constant__ HamView H, int L, int chunks, const unsigned *__restrict__ maxhi,
                              const double2 *__restrict__ twist, int per_col, const double *__restrict__ E,
                              ColumnScale *__restrict__ scales, const int *__restrict__ sys_active) {
-  const int s = blockIdx.x, c = threadIdx.x;
+  extern __shared__ unsigned smax[];   // [lanes][L]
+  const int s = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
   if (sys_active && !sys_active[s]) return;
   unsigned m = 0;
-#pragma unroll 4
-  for (int k = 0; k < chunks; ++k) m = max(m, maxhi[((int64_t)s * chunks + k) * L + c]);
-  double2 w, wi;
-  twist_and_inverse(twist, per_col ? (int64_t)s * L + c : s, w, wi);
-  ColumnScale o;
-  o.f = fix_scale(H, w, wi, E[s], m);
-  o.base = 1086 + o.f.ex - o.f.Q;
-  o.w = w;
-  o.wi = wi;
-  o.ef = o.f.ok ? round_fixed(E[s] - H.diag_kin, 58 - H.fx_ew) : 0;
-  o.pad = 0;
-  scales[(int64_t)s * L + c] = o;
+  for (int k = ly; k < chunks; k += ry) m = max(m, maxhi[((int64_t)s * chunks + k) * L + c]);
+  smax[ly * L + c] = m;
+  __syncthreads();
+  if (ly) return;
+  for (int y = 1; y < ry; ++y) m = max(m, smax[y * L + c]);
+  scales[(int64_t)s * L + c] = column_scale(H, twist[per_col ? (int64_t)s * L + c : s], E[s], m, false);
 }
 
 // FP64 sum of one image of one atom over the entries t0, t0 + step, ...: the columns that
@@ -212,7 +192,7 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
   if (word) atomicOr(&seen[cx], word);
   __syncthreads();
   // columns out of range, or with nothing but small values over this atom: FP64 sums
-  const bool redo = !f.ok || seen[cx] < kFixSmallWord;
+  const bool redo = !sc->skip && (!f.ok || seen[cx] < kFixSmallWord);
   if (__syncthreads_or(redo)) {
     double2 *red = (double2 *)gsm;                         // [py][4][cg], the space of redA
     if (redo && ly == 0)
@@ -369,13 +349,13 @@ struct Scatter {
 // z neighbours of its point in registers.  The next plane's halo and the plane MH ahead are
 // loaded while the current one is computed.  Offsets inside a plane are 32-bit byte offsets
 // from a base that all threads share.
-template <int MH, int CG, int TX, int TY, bool ISO>
+template <int MH, int CG, int TX, int TY, bool ISO, bool DOT>
 __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
     k_stencil_fixed(const __grid_constant__ HamView H, int L, int groups, int tiles_x, int z_chunk,
                     const double2 *__restrict__ X, double2 *__restrict__ Y, const double *__restrict__ E,
                     const ColumnScale *__restrict__ scales,
                     const double2 *__restrict__ D, const int4 *__restrict__ Df,
-                    const int *__restrict__ sys_active) {
+                    const int *__restrict__ sys_active, const FixedDot dot) {
   constexpr int WX = TX + 2 * MH, WY = TY + 2 * MH, THREADS = CG * TX * TY;
   constexpr int HALO = 2 * MH * (TX + TY) * CG;
   constexpr int SLOTS = (HALO + THREADS - 1) / THREADS;
@@ -390,7 +370,6 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
   const int tid = threadIdx.x;
   const int cl = tid % CG, lx = (tid / CG) % TX, ly = tid / (CG * TX);
   const int c = min(g * CG + cl, L - 1);
-  const bool own = g * CG + cl < L && bx + lx < nx && by + ly < ny;
   const int ix = (bx + lx) % nx, iy = (by + ly) % ny;
   const int line = iy * nx + ix;
   const int64_t plane_bytes = (int64_t)nx * ny * L * sizeof(double2);
@@ -402,6 +381,15 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
   const ColumnScale *sc = scales + (int64_t)s * L + c;
   const FixScale f = sc->f;
   const int base = sc->base;
+  const bool own = g * CG + cl < L && bx + lx < nx && by + ly < ny && !sc->skip;
+  // (p~, q): this thread's share, for primal systems
+  const bool dotted = DOT && s < dot.n;
+  const char *Xd = Xs + (DOT ? (int64_t)dot.n * H.n * L * (int64_t)sizeof(double2) : 0);
+  double dx = 0, dy = 0;
+  auto add_dot = [&](double2 pd, double2 q) {
+    dx = fma(pd.x, q.x, fma(pd.y, q.y, dx));
+    dy = fma(pd.x, q.y, fma(-pd.y, q.x, dy));
+  };
   const double2 w = sc->w, wi = sc->wi;
   const long long ef = sc->ef;
   auto conv = [&](double2 v) -> Fixed2 { return Fixed2{to_fixed(v.x, base), to_fixed(v.y, base)}; };
@@ -558,8 +546,11 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
       vr -= pr.shifted(f.sp);
       vi -= pi.shifted(f.sp);
     }
-    if (own)
-      *(double2 *)(Ys + iz * plane_bytes + mine) = make_double2(from_fixed(vr, f.uy), from_fixed(vi, f.uy));
+    if (own) {
+      const double2 out = make_double2(from_fixed(vr, f.uy), from_fixed(vi, f.uy));
+      *(double2 *)(Ys + iz * plane_bytes + mine) = out;
+      if (dotted && f.ok && !((redo >> (iz - z0)) & 1)) add_dot(*(const double2 *)(Xd + iz * plane_bytes + mine), out);
+    }
 #pragma unroll
     for (int d = 0; d < 2 * MH; ++d) q[d] = q[d + 1];
     if (more) {
@@ -574,10 +565,38 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
   if (!f.ok) redo = ~0ull;
   if (own && redo)
     for (iz = z0; iz < z1; ++iz)
-      if ((redo >> (iz - z0)) & 1)
-        *(double2 *)(Ys + iz * plane_bytes + mine) =
-            output_fp64(&H, (const double2 *)Xs + c, L, ix, iy, iz, w, wi, E[s],
-                        proj ? D + ((int64_t)s * H.n_atoms * L + c) * 4 : nullptr);
+      if ((redo >> (iz - z0)) & 1) {
+        const double2 out = output_fp64(&H, (const double2 *)Xs + c, L, ix, iy, iz, w, wi, E[s],
+                                        proj ? D + ((int64_t)s * H.n_atoms * L + c) * 4 : nullptr);
+        *(double2 *)(Ys + iz * plane_bytes + mine) = out;
+        if (dotted) add_dot(*(const double2 *)(Xd + iz * plane_bytes + mine), out);
+      }
+  if (dotted) {
+    // the block's sum per column, lines in order of the shuffles: fixed for a given grid
+    double *red = (double *)tile;   // [warps][CG][2]
+    for (int o = CG; o < 32; o <<= 1) {
+      dx += __shfl_xor_sync(0xffffffffu, dx, o);
+      dy += __shfl_xor_sync(0xffffffffu, dy, o);
+    }
+    __syncthreads();
+    if (tid % 32 < CG) {
+      red[(tid / 32 * CG + cl) * 2] = dx;
+      red[(tid / 32 * CG + cl) * 2 + 1] = dy;
+    }
+    __syncthreads();
+    const int tiles = gridDim.x / groups, parts = tiles * gridDim.y;
+    if (tid < CG && g * CG + tid < L) {
+      for (int k = 1; k < THREADS / 32; ++k) {
+        dx += red[(k * CG + tid) * 2];
+        dy += red[(k * CG + tid) * 2 + 1];
+      }
+      double *o = dot.part + (((int64_t)s * parts + blockIdx.y * tiles + tb) * L + g * CG + tid) * 2;
+      o[0] = dx;
+      o[1] = dy;
+    }
+    if (last_block(dot.tail.count + s, gridDim.x * gridDim.y))
+      alpha_tail<2>(dot.tail, dot.part, s, L, parts, tid, THREADS, (double *)tile);
+  }
 }
 
 size_t apply_coef_bytes(const HamView &H, int n_sys, int L, int dtype) {
@@ -609,24 +628,36 @@ bool fixed_serves(const HamView &H, int n_sys, int L, size_t ws_bytes) {
          (int64_t)3 * H.n_atoms * L < ((int64_t)1 << 26) && ws_bytes >= apply_ws_bytes(H, n_sys, L, CBS_C128);
 }
 
-cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y,
-                       const double2 *twist, bool per_col, const double *E, void *ws,
-                       const int *sys_active, cudaStream_t st) {
-  const size_t d = apply_coef_bytes(H, n_sys, L, CBS_C128);
+ColumnScale *fixed_scales(const HamView &H, int n_sys, int L, void *ws) {
+  return (ColumnScale *)((char *)ws + (H.n_atoms ? 4 * apply_coef_bytes(H, n_sys, L, CBS_C128) : 0));
+}
+
+// 8 x 8 lines of 4 columns (64-byte pieces of a point's row)
+constexpr int kFixCG = 4, kFixTX = 8, kFixTY = 8;
+struct FixGrid { int groups, tiles_x, tiles, z_chunk, z_blocks; };
+static FixGrid fix_grid(const HamView &H, int n_sys, int L) {
+  FixGrid g;
+  g.groups = ceil_div(L, kFixCG);
+  g.tiles_x = ceil_div(H.nx, kFixTX);
+  g.tiles = g.tiles_x * ceil_div(H.ny, kFixTY);
+  // planes per block: all of them unless that leaves SMs idle
+  int zc = 1;
+  while (zc < 8 && (int64_t)g.groups * g.tiles * n_sys * zc < 152 * 2 && H.nz / (zc * 2) >= 2) zc *= 2;
+  g.z_chunk = std::min(64, ceil_div(H.nz, zc));   // a block marks its planes in 64 bits
+  g.z_blocks = ceil_div(H.nz, g.z_chunk);
+  return g;
+}
+
+int fixed_dot_parts(const HamView &H, int n_sys, int L) {
+  const FixGrid g = fix_grid(H, n_sys, L);
+  return g.tiles * g.z_blocks;
+}
+
+cbs_status apply_fixed_scaled(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y, const double *E,
+                              void *ws, const int *sys_active, cudaStream_t st, const FixedDot *dot) {
   double2 *D = (double2 *)ws;
-  int4 *Df = (int4 *)((char *)ws + (H.n_atoms ? d : 0));
-  ColumnScale *scales = (ColumnScale *)((char *)ws + (H.n_atoms ? 4 * d : 0));
-  unsigned *maxhi = (unsigned *)(scales + (size_t)n_sys * L);
-  int64_t pts;
-  const int chunks = max_chunks(H, n_sys, L, &pts);
-  {
-    const dim3 blk = col_block(L);
-    k_column_max<<<dim3((unsigned)chunks, (unsigned)n_sys, 1), blk, (size_t)blk.x * blk.y * sizeof(unsigned), st>>>(
-        H.n, L, (int)pts, X, maxhi, sys_active);
-    k_fix_scales<<<n_sys, L, 0, st>>>(H, L, chunks, maxhi, twist, per_col ? 1 : 0, E, scales, sys_active);
-    count_launches(2);
-    CBS_CUDA(cudaGetLastError());
-  }
+  int4 *Df = (int4 *)((char *)ws + (H.n_atoms ? apply_coef_bytes(H, n_sys, L, CBS_C128) : 0));
+  const ColumnScale *scales = fixed_scales(H, n_sys, L, ws);
   if (H.n_atoms) {
     const int groups = ceil_div(L, 32), cg = ceil_div(L, groups);
     const int py = 256 / cg > 32 ? 32 : 256 / cg;
@@ -636,28 +667,27 @@ cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, dou
     count_launches(1);
     CBS_CUDA(cudaGetLastError());
   }
-  // 8 x 8 lines of 4 columns (64-byte pieces of a point's row)
-  constexpr int CG = 4, TX = 8, TY = 8;
-  const int groups = ceil_div(L, CG), tiles_x = ceil_div(H.nx, TX);
-  const int blocks = groups * tiles_x * ceil_div(H.ny, TY);
-  // planes per block: all of them unless that leaves SMs idle
-  int zc = 1;
-  while (zc < 8 && (int64_t)blocks * n_sys * zc < 152 * 2 && H.nz / (zc * 2) >= 2) zc *= 2;
-  const int z_chunk = std::min(64, ceil_div(H.nz, zc));   // a block marks its planes in 64 bits
-  const dim3 grd((unsigned)blocks, (unsigned)ceil_div(H.nz, z_chunk), (unsigned)n_sys);
-  const size_t sm = (size_t)2 * (TX + 2 * H.m) * (TY + 2 * H.m) * CG * sizeof(Fixed2);
-#define FK(MH, ISO)                                                                                       \
-  do {                                                                                                    \
-    if (sm > 48 * 1024)                                                                                   \
-      CBS_CUDA(cudaFuncSetAttribute(k_stencil_fixed<MH, CG, TX, TY, ISO>,                                 \
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));               \
-    k_stencil_fixed<MH, CG, TX, TY, ISO><<<grd, CG * TX * TY, sm, st>>>(                                  \
-        H, L, groups, tiles_x, z_chunk, X, Y, E, scales, D, Df, sys_active);                              \
+  const FixGrid g = fix_grid(H, n_sys, L);
+  const dim3 grd((unsigned)(g.groups * g.tiles), (unsigned)g.z_blocks, (unsigned)n_sys);
+  const size_t sm = (size_t)2 * (kFixTX + 2 * H.m) * (kFixTY + 2 * H.m) * kFixCG * sizeof(Fixed2);
+  const FixedDot d = dot ? *dot : FixedDot();
+#define FK(MH, ISO, DOT)                                                                                   \
+  do {                                                                                                     \
+    if (sm > 48 * 1024)                                                                                    \
+      CBS_CUDA(cudaFuncSetAttribute(k_stencil_fixed<MH, kFixCG, kFixTX, kFixTY, ISO, DOT>,                 \
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));                \
+    k_stencil_fixed<MH, kFixCG, kFixTX, kFixTY, ISO, DOT><<<grd, kFixCG * kFixTX * kFixTY, sm, st>>>(      \
+        H, L, g.groups, g.tiles_x, g.z_chunk, X, Y, E, scales, D, Df, sys_active, d);                      \
   } while (0)
-#define FM(MH)                     \
-  case MH:                         \
-    if (H.fx_iso) FK(MH, true);    \
-    else FK(MH, false);            \
+#define FM(MH)                        \
+  case MH:                            \
+    if (H.fx_iso) {                   \
+      if (d.n) FK(MH, true, true);    \
+      else FK(MH, true, false);       \
+    } else {                          \
+      if (d.n) FK(MH, false, true);   \
+      else FK(MH, false, false);      \
+    }                                 \
     break
   switch (H.m) {
     FM(1); FM(2); FM(3); FM(4); FM(5); FM(6);
@@ -668,6 +698,24 @@ cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, dou
   count_launches(1);
   CBS_CUDA(cudaGetLastError());
   return CBS_OK;
+}
+
+cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y,
+                       const double2 *twist, bool per_col, const double *E, void *ws,
+                       const int *sys_active, cudaStream_t st) {
+  ColumnScale *scales = fixed_scales(H, n_sys, L, ws);
+  unsigned *maxhi = (unsigned *)(scales + (size_t)n_sys * L);
+  int64_t pts;
+  const int chunks = max_chunks(H, n_sys, L, &pts);
+  const dim3 blk = col_block(L);
+  k_column_max<<<dim3((unsigned)chunks, (unsigned)n_sys, 1), blk, (size_t)blk.x * blk.y * sizeof(unsigned), st>>>(
+      H.n, L, (int)pts, X, maxhi, sys_active);
+  const dim3 sblk((unsigned)L, (unsigned)std::max(1, std::min(chunks, 512 / L)), 1);
+  k_fix_scales<<<n_sys, sblk, (size_t)sblk.x * sblk.y * sizeof(unsigned), st>>>(H, L, chunks, maxhi, twist, per_col ? 1 : 0,
+                                                                               E, scales, sys_active);
+  count_launches(2);
+  CBS_CUDA(cudaGetLastError());
+  return apply_fixed_scaled(H, n_sys, L, X, Y, E, ws, sys_active, st, nullptr);
 }
 
 }  // namespace cbs

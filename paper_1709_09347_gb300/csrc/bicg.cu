@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "bicg.cuh"
+#include "fixed.cuh"
 
 #define CBS_TRY_B(x)               \
   do {                             \
@@ -58,8 +59,9 @@ __device__ __forceinline__ void sum_chunks(const double *part, int64_t s, int L,
 #pragma unroll 4
   for (int ch = ly; ch < n_chunks; ch += ry)
 #pragma unroll
-    for (int q = 0; q < NV; ++q) a[q] += part[((s * n_chunks + ch) * L + c) * 4 + q];
+    for (int q = 0; q < NV; ++q) a[q] += __ldcg(&part[((s * n_chunks + ch) * L + c) * 4 + q]);
   if (ry == 1) return;
+  __syncthreads();   // the shared memory may hold a block sum that is still read
 #pragma unroll
   for (int q = 0; q < NV; ++q) csm[((size_t)ly * L + c) * NV + q] = a[q];
   __syncthreads();
@@ -138,30 +140,81 @@ __global__ void k_reduce_init(int n, int L, int n_chunks, const double *part, do
   }
 }
 
-template <typename R>
-__global__ void k_update_p(int n, int64_t N, int L, int chunk_pts, const typename CT<R>::T *r,
-                           typename CT<R>::T *p, const double2 *beta, const int *active,
-                           const int *sys_active) {
+// The scales of the fixed-point apply of p, from the maxima that k_update_p meets.
+struct ScaleTail {
+  const double2 *tw = nullptr;     // [2n] twists
+  const double *E = nullptr;       // [2n]
+  unsigned *maxhi = nullptr;       // [2n][n_chunks][L]
+  unsigned *count = nullptr;       // [n] blocks done
+  ColumnScale *scales = nullptr;   // [2n][L]
+};
+
+// p = r + beta p and its dual.  FIXED (complex128 applies in fixed point): also the largest
+// component of every column of p, and by the last block of a system the columns' scales.  The
+// count of active systems is cleared here for the end of the iteration.
+template <typename R, bool FIXED>
+__global__ void k_update_p(const __grid_constant__ HamView H, int n, int64_t N, int L, int chunk_pts,
+                           const typename CT<R>::T *r, typename CT<R>::T *p, const double2 *beta, const int *active,
+                           const int *sys_active, int *n_active, const ScaleTail tail) {
   typedef typename CT<R>::T C;
+  extern __shared__ unsigned umax[];   // [2][py][L]
   const int s = blockIdx.y, chunk = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, py = blockDim.y;
+  if (s == 0 && chunk == 0 && c == 0 && ly == 0) *n_active = 0;
   if (!sys_active[s]) return;
   const int64_t k = (int64_t)s * L + c;
-  if (!active[k]) return;
-  const C b = from_d<R>(beta[k]), bc = cconj(b);
-  const int64_t i0 = (int64_t)chunk * chunk_pts;
-  const int64_t i1 = min(N, i0 + chunk_pts);
-  for (int64_t i = i0 + ly; i < i1; i += py) {
-    const int64_t e = ((int64_t)s * N + i) * L + c, ed = ((int64_t)(n + s) * N + i) * L + c;
-    p[e] = cfma(b, p[e], r[e]);
-    p[ed] = cfma(bc, p[ed], r[ed]);
+  const bool act = active[k];
+  if (!FIXED && !act) return;
+  unsigned m = 0, md = 0;
+  if (act) {
+    const C b = from_d<R>(beta[k]), bc = cconj(b);
+    const int64_t i0 = (int64_t)chunk * chunk_pts;
+    const int64_t i1 = min(N, i0 + chunk_pts);
+#pragma unroll 2
+    for (int64_t i = i0 + ly; i < i1; i += py) {
+      const int64_t e = ((int64_t)s * N + i) * L + c, ed = ((int64_t)(n + s) * N + i) * L + c;
+      const C v = cfma(b, p[e], r[e]), vd = cfma(bc, p[ed], r[ed]);
+      p[e] = v;
+      p[ed] = vd;
+      if constexpr (FIXED) {
+        m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+        md = max(md, max((unsigned)__double2hiint(vd.x) & 0x7fffffffu, (unsigned)__double2hiint(vd.y) & 0x7fffffffu));
+      }
+    }
+  }
+  if constexpr (FIXED) {
+    umax[ly * L + c] = m;
+    umax[(py + ly) * L + c] = md;
+    __syncthreads();
+    for (int d = ly; d < 2; d += py) {
+      unsigned t = 0;
+      for (int y = 0; y < py; ++y) t = max(t, umax[(d * py + y) * L + c]);
+      tail.maxhi[((int64_t)(d * n + s) * gridDim.x + chunk) * L + c] = t;
+    }
+    if (!last_block(tail.count + s, gridDim.x)) return;
+    for (int d = 0; d < 2; ++d) {
+      unsigned t = 0;
+      for (int ch = ly; ch < (int)gridDim.x; ch += py)
+        t = max(t, __ldcg(&tail.maxhi[((int64_t)(d * n + s) * gridDim.x + ch) * L + c]));
+      umax[(d * py + ly) * L + c] = t;
+    }
+    __syncthreads();
+    for (int d = ly; d < 2; d += py) {
+      unsigned t = 0;
+      for (int y = 0; y < py; ++y) t = max(t, umax[(d * py + y) * L + c]);
+      const int64_t q = (int64_t)d * n + s;
+      tail.scales[q * L + c] = column_scale(H, tail.tw[q], tail.E[q], t, !act);
+    }
   }
 }
 
+// (p~, q), and alpha by the last block of each system (complex64, and complex128 cells that fixed
+// point does not serve; else k_stencil_fixed sums it).
 template <typename R>
 __global__ void k_dot_pq(int n, int64_t N, int L, int chunk_pts, int n_chunks,
                          const typename CT<R>::T *p, const typename CT<R>::T *q, double *part,
-                         const int *sys_active) {
+                         const int *sys_active, const AlphaTail tail) {
   typedef typename CT<R>::T C;
+  extern __shared__ double red[];
   const int s = blockIdx.y, chunk = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, py = blockDim.y;
   if (!sys_active[s]) return;
   double acc[4] = {0, 0, 0, 0};
@@ -174,40 +227,76 @@ __global__ void k_dot_pq(int n, int64_t N, int L, int chunk_pts, int n_chunks,
   for (int64_t i = i0 + ly; i < i1; i += py) {
     const double2 pd = to_d(p[((int64_t)(n + s) * N + i) * L + c]);
     const double2 qq = to_d(q[((int64_t)s * N + i) * L + c]);
-    ax += pd.x * qq.x + pd.y * qq.y;
-    ay += pd.x * qq.y - pd.y * qq.x;
+    ax = fma(pd.x, qq.x, fma(pd.y, qq.y, ax));
+    ay = fma(pd.x, qq.y, fma(-pd.y, qq.x, ay));
   }
   acc[0] = ax; acc[1] = ay;
   block_partials<R>(acc, part, (int64_t)s * n_chunks + chunk);
+  if (last_block(tail.count + s, gridDim.x)) alpha_tail<4>(tail, part, s, L, n_chunks, ly * L + c, py * L, red);
 }
 
-__global__ void k_reduce_alpha(int n, int L, int n_chunks, const double *part, const double2 *rho,
-                               double2 *alpha, int *active, int *flags, const int *sys_active,
-                               unsigned long long *sys_apply) {
-  const int s = blockIdx.x, c = threadIdx.x;
-  if (!sys_active[s]) return;
-  double a[2];
-  sum_chunks<2>(part, s, L, n_chunks, a);
-  if (threadIdx.y != 0) return;
-  if (c == 0 && sys_apply) atomicAdd(sys_apply, 1ull);   // system s went through this apply
+// What follows the residual update of one BiCG iteration.
+struct BetaTail {
+  unsigned *count = nullptr;   // [n] blocks done
+  double2 *rho = nullptr, *rho_prev = nullptr, *beta = nullptr;
+  const double *tgt = nullptr, *tgtd = nullptr;
+  double *rmax = nullptr, *rmaxd = nullptr;
+  double tfac = 0;
+  int *active = nullptr, *iters = nullptr, *flags = nullptr;
+  int max_iter = 0;
+  int *sys_active = nullptr, *n_active = nullptr;
+};
+
+// rho, the norms, the stop tests and beta of system s; blocks are (L, lanes)
+__device__ __forceinline__ void beta_tail(const BetaTail &b, const double *part, int n, int s, int L, int n_chunks) {
+  const int c = threadIdx.x;
   const int64_t k = (int64_t)s * L + c;
-  if (!active[k]) { alpha[k] = make_double2(0, 0); return; }
-  double2 g = make_double2(a[0], a[1]);
-  double g2 = cabs2(g);
-  if (!(g2 > 0) || !isfinite(g2)) {
-    flags[k] |= 2;
-    active[k] = 0;
-    alpha[k] = make_double2(0, 0);
-    return;
+  double a[4];
+  sum_chunks<4>(part, s, L, n_chunks, a);
+  const bool lead = threadIdx.y == 0;
+  int act = lead ? b.active[k] : 0;
+  if (act) {
+    const int it = b.iters[k] + 1;
+    b.iters[k] = it;
+    const double nr = sqrt(a[2]), nrd = sqrt(a[3]);
+    const double2 rn = make_double2(a[0], a[1]);
+    const double2 rold = b.rho[k];
+    b.rho_prev[k] = rold;                  // kept for a later residual replacement
+    b.rho[k] = rn;
+    // stop (or pause until the next residual replacement) below max(tfac * the largest
+    // residual norm since the last replacement, the absolute target)
+    const double mx = fmax(b.rmax[k], nr), mxd = fmax(b.rmaxd[k], nrd);
+    b.rmax[k] = mx;
+    b.rmaxd[k] = mxd;
+    if (nr <= fmax(b.tfac * mx, b.tgt[k]) && nrd <= fmax(b.tfac * mxd, b.tgtd[k])) {
+      act = 0;
+    } else if (!isfinite(nr) || !isfinite(nrd) || !(cabs2(rn) > 0)) {
+      b.flags[k] |= 2;
+      act = 0;
+    } else if (it >= b.max_iter) {
+      b.flags[k] |= 1;
+      act = 0;
+    } else {
+      b.beta[k] = cdiv(rn, rold);
+    }
+    b.active[k] = act;
   }
-  alpha[k] = cdiv(rho[k], g);
+  if (lead && !act) b.beta[k] = make_double2(0, 0);
+  int any = __syncthreads_or(act);
+  if (lead && c == 0) {
+    b.sys_active[s] = any;
+    b.sys_active[n + s] = any;
+    if (any) atomicAdd(b.n_active, 1);
+  }
 }
 
-template <typename R>
+// x += alpha p, r -= alpha q and their duals, (r~, r) and the norms; then, by the last block of
+// each system, beta and the stop tests (TAIL; the shifted family's are a kernel of their own).
+template <typename R, bool TAIL>
 __global__ void k_pass_b(int n, int64_t N, int L, int chunk_pts, int n_chunks,
                          typename CT<R>::T *x, typename CT<R>::T *r, const typename CT<R>::T *p,
                          const typename CT<R>::T *q, const double2 *alpha, const int *active,
-                         double *part, const int *sys_active) {
+                         double *part, const int *sys_active, const BetaTail tail) {
   typedef typename CT<R>::T C;
   const int s = blockIdx.y, chunk = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, py = blockDim.y;
   if (!sys_active[s]) return;
@@ -231,61 +320,15 @@ __global__ void k_pass_b(int n, int64_t N, int L, int chunk_pts, int n_chunks,
       C rd = cfma(nac, q[ed], r[ed]);
       r[ed] = rd;
       const double2 r1 = to_d(rr), r2 = to_d(rd);
-      s0 += r2.x * r1.x + r2.y * r1.y;
-      s1 += r2.x * r1.y - r2.y * r1.x;
-      s2 += rr.x * rr.x + rr.y * rr.y;
-      s3 += rd.x * rd.x + rd.y * rd.y;
+      s0 = fma(r2.x, r1.x, fma(r2.y, r1.y, s0));
+      s1 = fma(r2.x, r1.y, fma(-r2.y, r1.x, s1));
+      s2 = fma(rr.x, rr.x, fma(rr.y, rr.y, s2));
+      s3 = fma(rd.x, rd.x, fma(rd.y, rd.y, s3));
     }
   }
   double acc[4] = {s0, s1, (double)s2, (double)s3};
   block_partials<R>(acc, part, (int64_t)s * n_chunks + chunk);
-}
-
-__global__ void k_reduce_beta(int n, int L, int n_chunks, const double *part, double2 *rho,
-                              double2 *rho_prev, double2 *beta, const double *tgt,
-                              const double *tgtd, double *rmax, double *rmaxd, double tfac,
-                              int *active, int *iters, int *flags, int max_iter, int *sys_active,
-                              int *n_active) {
-  const int s = blockIdx.x, c = threadIdx.x;
-  if (!sys_active[s]) return;   // uniform per block
-  const int64_t k = (int64_t)s * L + c;
-  double a[4];
-  sum_chunks<4>(part, s, L, n_chunks, a);
-  const bool lead = threadIdx.y == 0;
-  int act = lead ? active[k] : 0;
-  if (act) {
-    const int it = iters[k] + 1;
-    iters[k] = it;
-    const double nr = sqrt(a[2]), nrd = sqrt(a[3]);
-    const double2 rn = make_double2(a[0], a[1]);
-    const double2 rold = rho[k];
-    rho_prev[k] = rold;                  // kept for a later residual replacement
-    rho[k] = rn;
-    // stop (or pause until the next residual replacement) below max(tfac * the largest
-    // residual norm since the last replacement, the absolute target)
-    const double mx = fmax(rmax[k], nr), mxd = fmax(rmaxd[k], nrd);
-    rmax[k] = mx;
-    rmaxd[k] = mxd;
-    if (nr <= fmax(tfac * mx, tgt[k]) && nrd <= fmax(tfac * mxd, tgtd[k])) {
-      act = 0;
-    } else if (!isfinite(nr) || !isfinite(nrd) || !(cabs2(rn) > 0)) {
-      flags[k] |= 2;
-      act = 0;
-    } else if (it >= max_iter) {
-      flags[k] |= 1;
-      act = 0;
-    } else {
-      beta[k] = cdiv(rn, rold);
-    }
-    active[k] = act;
-  }
-  if (lead && !act) beta[k] = make_double2(0, 0);
-  int any = __syncthreads_or(act);
-  if (lead && c == 0) {
-    sys_active[s] = any;
-    sys_active[n + s] = any;
-    if (any) atomicAdd(n_active, 1);
-  }
+  if (TAIL && last_block(tail.count + s, gridDim.x)) beta_tail(tail, part, n, s, L, n_chunks);
 }
 
 // Load-balance rule of §3.3 (second stopping rule): the systems of one energy are its
@@ -437,6 +480,10 @@ size_t Bicg<R>::bytes_needed(const HamView &H, int n, int L) {
   b += 4 * align256((int64_t)n * L * sizeof(double2)) + 6 * align256((int64_t)n * L * sizeof(double));
   b += 3 * align256((int64_t)n * L * sizeof(int)) + align256((int64_t)2 * n * sizeof(int)) + 256;
   b += align256((int64_t)n * nc * L * 4 * sizeof(double)) + 256;
+  b += align256((int64_t)3 * n * sizeof(unsigned));
+  if (sizeof(R) == sizeof(double) && fixed_serves(H, 2 * n, L, ~(size_t)0))
+    b += align256((int64_t)2 * n * nc * L * sizeof(unsigned)) +
+         align256((int64_t)n * fixed_dot_parts(H, 2 * n, L) * L * 2 * sizeof(double));
   return (size_t)b;
 }
 
@@ -477,6 +524,13 @@ cbs_status Bicg<R>::alloc(const HamView &H_, int n_, int L_) {
   part = (double *)take((int64_t)n * n_chunks * L * 4 * sizeof(double));
   sys_apply = (unsigned long long *)take(256);
   CBS_CUDA(cudaMemset(sys_apply, 0, sizeof(unsigned long long)));
+  done = (unsigned *)take((int64_t)3 * n * sizeof(unsigned));
+  CBS_CUDA(cudaMemset(done, 0, (size_t)3 * n * sizeof(unsigned)));
+  fixed = sizeof(R) == sizeof(double) && fixed_serves(H, 2 * n, L, d_bytes);
+  if (fixed) {
+    maxhi = (unsigned *)take((int64_t)2 * n * n_chunks * L * sizeof(unsigned));
+    dot_part = (double *)take((int64_t)n * fixed_dot_parts(H, 2 * n, L) * L * 2 * sizeof(double));
+  }
   return CBS_OK;
 }
 
@@ -530,30 +584,77 @@ cbs_status Bicg<R>::init(const double2 *B, int64_t bstride, const double2 *Bd, i
   return CBS_OK;
 }
 
+// The first half of an iteration: p, q = P p and alpha.  Three launches with fixed-point applies
+// (two without projectors), else four.
+template <typename R>
+cbs_status Bicg<R>::advance(cudaStream_t st, int kk) {
+  dim3 blk = col_block(L);
+  dim3 grd((unsigned)n_chunks, (unsigned)n, 1);
+  const size_t msm = (size_t)2 * blk.x * blk.y * sizeof(unsigned);
+  AlphaTail at;
+  at.count = done + n;
+  at.rho = rho;
+  at.alpha = alpha;
+  at.active = active;
+  at.flags = flags;
+  at.sys_apply = sys_apply;
+  const bool prof = profile && kk >= 0 && 2 * kk + 1 < n_prof_ev;
+  // (events are recorded as real event nodes of the graph, not capture-dependency markers)
+  if constexpr (sizeof(R) == sizeof(double)) {
+    if (fixed) {
+      ScaleTail sc;
+      sc.tw = tw;
+      sc.E = E;
+      sc.maxhi = maxhi;
+      sc.count = done;
+      sc.scales = fixed_scales(H, 2 * n, L, D);
+      k_update_p<R, true><<<grd, blk, msm, st>>>(H, n, N, L, chunk_pts, r, p, beta, active, sys_active, n_active, sc);
+      cbs::count_launches(1);
+      CBS_CUDA(cudaGetLastError());
+      FixedDot dot;
+      dot.n = n;
+      dot.part = dot_part;
+      dot.tail = at;
+      if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk], st, cudaEventRecordExternal));
+      CBS_TRY_B(apply_fixed_scaled(H, 2 * n, L, p, q, E, D, sys_active, st, &dot));
+      if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
+      return CBS_OK;
+    }
+  }
+  k_update_p<R, false><<<grd, blk, 0, st>>>(H, n, N, L, chunk_pts, r, p, beta, active, sys_active, n_active, ScaleTail());
+  cbs::count_launches(1);
+  CBS_CUDA(cudaGetLastError());
+  if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk], st, cudaEventRecordExternal));
+  CBS_TRY_B(apply_P<R>(H, 2 * n, L, p, q, tw, false, E, D, d_bytes, sys_active, st));
+  if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
+  k_dot_pq<R><<<grd, blk, red_smem(L), st>>>(n, N, L, chunk_pts, n_chunks, p, q, part, sys_active, at); cbs::count_launches(1);
+  CBS_CUDA(cudaGetLastError());
+  return CBS_OK;
+}
+
 template <typename R>
 cbs_status Bicg<R>::step(double tol, int max_iter, cudaStream_t st, int kk) {
   dim3 blk = col_block(L);
   dim3 grd((unsigned)n_chunks, (unsigned)n, 1);
-  k_update_p<R><<<grd, blk, 0, st>>>(n, N, L, chunk_pts, r, p, beta, active, sys_active); cbs::count_launches(1);
-  CBS_CUDA(cudaGetLastError());
-  const bool prof = profile && kk >= 0 && 2 * kk + 1 < n_prof_ev;
-  // recorded as real event nodes of the graph (not capture-dependency markers)
-  if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk], st, cudaEventRecordExternal));
-  cbs_status s = apply_P<R>(H, 2 * n, L, p, q, tw, false, E, D, d_bytes, sys_active, st);
-  if (s != CBS_OK) return s;
-  if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
-  k_dot_pq<R><<<grd, blk, red_smem(L), st>>>(n, N, L, chunk_pts, n_chunks, p, q, part, sys_active); cbs::count_launches(1);
-  CBS_CUDA(cudaGetLastError());
-  const dim3 rblk = reduce_block(L, n_chunks);
-  k_reduce_alpha<<<n, rblk, reduce_smem(rblk), st>>>(n, L, n_chunks, part, rho, alpha, active, flags, sys_active,
-                                  sys_apply); cbs::count_launches(1);
-  CBS_CUDA(cudaGetLastError());
-  k_pass_b<R><<<grd, blk, red_smem(L), st>>>(n, N, L, chunk_pts, n_chunks, x, r, p, q, alpha,
-                                             active, part, sys_active); cbs::count_launches(1);
-  CBS_CUDA(cudaGetLastError());
-  CBS_CUDA(cudaMemsetAsync(n_active, 0, sizeof(int), st));
-  k_reduce_beta<<<n, rblk, reduce_smem(rblk), st>>>(n, L, n_chunks, part, rho, rho_prev, beta, tgt, tgtd, rmax, rmaxd,
-                                 tfac, active, iters, flags, max_iter, sys_active, n_active); cbs::count_launches(1);
+  CBS_TRY_B(advance(st, kk));
+  BetaTail bt;
+  bt.count = done + 2 * n;
+  bt.rho = rho;
+  bt.rho_prev = rho_prev;
+  bt.beta = beta;
+  bt.tgt = tgt;
+  bt.tgtd = tgtd;
+  bt.rmax = rmax;
+  bt.rmaxd = rmaxd;
+  bt.tfac = tfac;
+  bt.active = active;
+  bt.iters = iters;
+  bt.flags = flags;
+  bt.max_iter = max_iter;
+  bt.sys_active = sys_active;
+  bt.n_active = n_active;
+  k_pass_b<R, true><<<grd, blk, red_smem(L), st>>>(n, N, L, chunk_pts, n_chunks, x, r, p, q, alpha,
+                                                   active, part, sys_active, bt); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   if (group > 0 && group_need < group) {
     k_group_stop<<<n / group, ((group + 31) / 32) * 32, 0, st>>>(n, group, L, group_need, active, flags, sys_active);
@@ -905,19 +1006,7 @@ cbs_status MultiShift<R>::step(int max_iter, cudaStream_t st, int kk) {
   Bicg<R> &b = seed;
   dim3 blk = col_block(L);
   dim3 grd((unsigned)b.n_chunks, (unsigned)n_pt, 1);
-  k_update_p<R><<<grd, blk, 0, st>>>(n_pt, N, L, b.chunk_pts, b.r, b.p, b.beta, b.active, b.sys_active); cbs::count_launches(1);
-  CBS_CUDA(cudaGetLastError());
-  const bool prof = b.profile && kk >= 0 && 2 * kk + 1 < b.n_prof_ev;
-  if (prof) CBS_CUDA(cudaEventRecordWithFlags(b.prof_ev[2 * kk], st, cudaEventRecordExternal));
-  cbs_status s = apply_P<R>(b.H, 2 * n_pt, L, b.p, b.q, b.tw, false, b.E, b.D, b.d_bytes, b.sys_active, st);
-  if (s != CBS_OK) return s;
-  if (prof) CBS_CUDA(cudaEventRecordWithFlags(b.prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
-  k_dot_pq<R><<<grd, blk, red_smem(L), st>>>(n_pt, N, L, b.chunk_pts, b.n_chunks, b.p, b.q, b.part, b.sys_active); cbs::count_launches(1);
-  CBS_CUDA(cudaGetLastError());
-  const dim3 rblk = reduce_block(L, b.n_chunks);
-  k_reduce_alpha<<<n_pt, rblk, reduce_smem(rblk), st>>>(n_pt, L, b.n_chunks, b.part, b.rho, b.alpha, b.active, b.flags, b.sys_active,
-                                     b.sys_apply); cbs::count_launches(1);
-  CBS_CUDA(cudaGetLastError());
+  CBS_TRY_B(b.advance(st, kk));
   const dim3 eblk((unsigned)L, (unsigned)std::max(1, std::min(n_sh, 512 / L)), 1);
   k_ms_coef<<<n_pt, eblk, 0, st>>>(n_pt, n_sh, L, sigma, b.alpha, b.beta, alpha_prev, pi, pi_prev, cb, ca,
                                 sactive, sflags, b.sys_active, b.profile ? upd_cols : nullptr); cbs::count_launches(1);
@@ -927,10 +1016,10 @@ cbs_status MultiShift<R>::step(int max_iter, cudaStream_t st, int kk) {
   k_ms_update<R><<<grd, blk, 0, st>>>(n_pt, n_sh, N, L, b.chunk_pts, b.r, P, X, cb, ca, sactive, b.sys_active); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   if (uprof) CBS_CUDA(cudaEventRecordWithFlags(upd_ev[2 * kk + 1], st, cudaEventRecordExternal));
-  k_pass_b<R><<<grd, blk, red_smem(L), st>>>(n_pt, N, L, b.chunk_pts, b.n_chunks, nullptr, b.r, b.p, b.q,
-                                                  b.alpha, b.active, b.part, b.sys_active); cbs::count_launches(1);
+  k_pass_b<R, false><<<grd, blk, red_smem(L), st>>>(n_pt, N, L, b.chunk_pts, b.n_chunks, nullptr, b.r, b.p, b.q,
+                                                    b.alpha, b.active, b.part, b.sys_active, BetaTail()); cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
-  CBS_CUDA(cudaMemsetAsync(b.n_active, 0, sizeof(int), st));
+  const dim3 rblk = reduce_block(L, b.n_chunks);
   k_ms_reduce_beta<<<n_pt, rblk, reduce_smem(rblk), st>>>(n_pt, n_sh, L, b.n_chunks, b.part, b.rho, b.rho_prev, b.beta, b.tgt, b.tgtd,
                                        b.active, b.iters, b.flags, max_iter, b.sys_active, b.n_active, pi,
                                        sactive, siters, sflags); cbs::count_launches(1);
@@ -1027,7 +1116,7 @@ __global__ void k_residual(int n, int64_t N, int L, const double2 *B, int64_t bs
     const int64_t e = ((int64_t)s2 * N + i) * L + c;
     double2 v = csub(b[i * L + c], AY[e]);
     AY[e] = v;
-    acc += cabs2(v);
+    acc = fma(v.x, v.x, fma(v.y, v.y, acc));
   }
   extern __shared__ double red1[];
   red1[ly * L + c] = acc;

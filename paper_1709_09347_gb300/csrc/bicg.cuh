@@ -28,6 +28,10 @@ struct Bicg {
   int *sys_active = nullptr;                                  // [2n]
   int *n_active = nullptr;                                    // [1]
   double *part = nullptr;                                     // [n][n_chunks][L][4]
+  unsigned *done = nullptr;                                   // [3][n] blocks done: p, (p~, q), x/r
+  bool fixed = false;                                         // applies in fixed point, scales by k_update_p
+  unsigned *maxhi = nullptr;                                  // [2n][n_chunks][L] largest components of p
+  double *dot_part = nullptr;                                 // partial (p~, q) of the fixed-point stencil
   void *block = nullptr;
   size_t bytes = 0;
   // profiling of the operator-apply launches (events around each apply inside the graph)
@@ -65,6 +69,8 @@ struct Bicg {
   // Residual replacement from FP64 true residuals R64 [2n][N][L]; columns with
   // colmask != 0 resume from them.
   cbs_status replace(const double2 *R64, const int *colmask, cudaStream_t st);
+  // p, q = P p and alpha of one iteration
+  cbs_status advance(cudaStream_t st, int k);
   // one iteration (captured into graphs); k indexes the iteration inside the graph
   cbs_status step(double tol, int max_iter, cudaStream_t st, int k);
   // outputs written by the apply launches so far (2 * active systems * N * L)

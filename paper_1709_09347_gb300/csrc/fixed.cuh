@@ -15,7 +15,7 @@
 // whose twist or energy is out of range take the FP64 formula instead, point by point.
 #pragma once
 
-#include "common.cuh"
+#include "tails.cuh"
 
 namespace cbs {
 
@@ -126,5 +126,40 @@ __device__ __forceinline__ int absword(long long a, long long b) {
   const int h0 = (int)(a >> 32), h1 = (int)(b >> 32);
   return max(h0 ^ (h0 >> 31), h1 ^ (h1 >> 31));
 }
+
+// What one (system, column) needs besides its vector.
+struct ColumnScale {
+  FixScale f;
+  int base;        // exponent offset of to_fixed
+  long long ef;    // E - diag_kin in the unit of the weights
+  long long skip;  // 1: the column takes no part (its output is not written)
+  double2 w, wi;   // the twist and its inverse
+};
+static_assert(sizeof(ColumnScale) % 16 == 0, "ColumnScale is read in 16-byte pieces");
+
+__device__ __forceinline__ ColumnScale column_scale(const HamView &H, double2 w, double E, unsigned maxhi, bool skip) {
+  ColumnScale o;
+  o.w = w;
+  o.wi = cdiv(make_double2(1.0, 0.0), w);
+  o.f = fix_scale(H, w, o.wi, E, maxhi);
+  o.base = 1086 + o.f.ex - o.f.Q;
+  o.ef = o.f.ok ? round_fixed(E - H.diag_kin, 58 - H.fx_ew) : 0;
+  o.skip = skip;
+  return o;
+}
+
+// The same apply with the columns' scales already in place (fixed_scales of the scratch), for
+// callers that know the maxima; with `dot`, the stencil also sums (p~, q) over the columns of
+// the first dot->n systems, p~ the input of system n + s, and its last block per system forms
+// alpha.
+struct FixedDot {
+  int n = 0;
+  double *part = nullptr;   // [n][fixed_dot_parts][L][2]
+  AlphaTail tail;
+};
+ColumnScale *fixed_scales(const HamView &H, int n_sys, int L, void *ws);
+int fixed_dot_parts(const HamView &H, int n_sys, int L);
+cbs_status apply_fixed_scaled(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y, const double *E,
+                              void *ws, const int *sys_active, cudaStream_t st, const FixedDot *dot);
 
 }  // namespace cbs
