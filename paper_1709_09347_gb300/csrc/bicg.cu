@@ -32,27 +32,57 @@
 
 namespace cbs {
 
-template <typename R>
+// Sums over the lanes of a (L, lanes) block, per column: on return every thread of lane 0 holds
+// its column's NV sums (the order is fixed by the block's shape).  The values are shared out
+// over the lanes, in two stages: FP64 issue is what these sums cost, and one warp instruction
+// of a narrow block then serves several values.  sm: threads x NV doubles.
+template <int NV>
+__device__ __forceinline__ void lane_sums(double (&a)[NV], double *sm) {
+  const int c = threadIdx.x, ly = threadIdx.y, L = blockDim.x, py = blockDim.y;
+  if (py == 1) return;
+  __syncthreads();   // the shared memory may still be read
+#pragma unroll
+  for (int q = 0; q < NV; ++q) sm[((size_t)ly * L + c) * NV + q] = a[q];
+  __syncthreads();
+  if (py < 2 * NV) {
+    if (ly == 0)
+      for (int y = 1; y < py; ++y)
+#pragma unroll
+        for (int q = 0; q < NV; ++q) a[q] += sm[((size_t)y * L + c) * NV + q];
+    return;
+  }
+  const int v = ly % NV, seg = ly / NV, nseg = py / NV;
+  double t = 0;
+  if (seg < nseg)
+    for (int y = seg; y < py; y += nseg) t += sm[((size_t)y * L + c) * NV + v];
+  __syncthreads();
+  if (seg < nseg) sm[((size_t)seg * L + c) * NV + v] = t;
+  __syncthreads();
+  if (seg == 0) {
+    for (int y = 1; y < nseg; ++y) t += sm[((size_t)y * L + c) * NV + v];
+    sm[(size_t)c * NV + v] = t;      // row 0: read by its own thread only
+  }
+  __syncthreads();
+  if (ly == 0)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) a[q] = sm[(size_t)c * NV + q];
+}
+
 __device__ __forceinline__ void block_partials(double (&acc)[4], double *part, int64_t slot) {
   extern __shared__ double red[];  // [py][L][4]
-  const int c = threadIdx.x, ly = threadIdx.y, L = blockDim.x, py = blockDim.y;
-  for (int k = 0; k < 4; ++k) red[((int64_t)ly * L + c) * 4 + k] = acc[k];
-  __syncthreads();
-  if (ly == 0) {
-    double s[4] = {0, 0, 0, 0};
-    for (int y = 0; y < py; ++y)
-      for (int k = 0; k < 4; ++k) s[k] += red[((int64_t)y * L + c) * 4 + k];
-    for (int k = 0; k < 4; ++k) part[(slot * L + c) * 4 + k] = s[k];
-  }
+  const int c = threadIdx.x, L = blockDim.x;
+  lane_sums<4>(acc, red);
+  if (threadIdx.y == 0)
+    for (int k = 0; k < 4; ++k) part[(slot * L + c) * 4 + k] = acc[k];
 }
 
 // Sums over the chunks of one system's partials, NV of the 4 values per column.  Blocks are
-// (L, ry): lane ly adds chunks ly, ly + ry, ... and lane 0 the lanes' sums in order (one thread
-// per column adding 128 chunks is a chain of 128 dependent FP64 additions per value, 40-60 us;
-// with 16 lanes 3-4 us).  The result is returned in lane 0; every thread of the block takes part.
+// (L, lanes): a lane adds every lanes-th chunk, then the lanes' sums are added (one thread per
+// column adding 128 chunks is a chain of 128 dependent FP64 additions per value, 40-60 us;
+// with 16 lanes 3-4 us).  The result is in lane 0; every thread of the block takes part.
 template <int NV>
 __device__ __forceinline__ void sum_chunks(const double *part, int64_t s, int L, int n_chunks, double (&a)[NV]) {
-  extern __shared__ double csm[];   // [ry][L][NV]
+  extern __shared__ double csm[];   // [lanes][L][NV]
   const int c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
 #pragma unroll
   for (int q = 0; q < NV; ++q) a[q] = 0;
@@ -60,15 +90,7 @@ __device__ __forceinline__ void sum_chunks(const double *part, int64_t s, int L,
   for (int ch = ly; ch < n_chunks; ch += ry)
 #pragma unroll
     for (int q = 0; q < NV; ++q) a[q] += __ldcg(&part[((s * n_chunks + ch) * L + c) * 4 + q]);
-  if (ry == 1) return;
-  __syncthreads();   // the shared memory may hold a block sum that is still read
-#pragma unroll
-  for (int q = 0; q < NV; ++q) csm[((size_t)ly * L + c) * NV + q] = a[q];
-  __syncthreads();
-  if (ly == 0)
-    for (int y = 1; y < ry; ++y)
-#pragma unroll
-      for (int q = 0; q < NV; ++q) a[q] += csm[((size_t)y * L + c) * NV + q];
+  lane_sums<NV>(a, csm);
 }
 
 // Blocks of the kernels that use it: up to 16 lanes, 1024 threads and one lane per chunk.
@@ -101,7 +123,7 @@ __global__ void k_init(int n, int64_t N, int L, int chunk_pts, int n_chunks, con
     acc[2] += cabs2(bb);
     acc[3] += cabs2(bdd);
   }
-  block_partials<R>(acc, part, (int64_t)s * n_chunks + chunk);
+  block_partials(acc, part, (int64_t)s * n_chunks + chunk);
 }
 
 __global__ void k_reduce_init(int n, int L, int n_chunks, const double *part, double2 *rho,
@@ -231,7 +253,7 @@ __global__ void k_dot_pq(int n, int64_t N, int L, int chunk_pts, int n_chunks,
     ay = fma(pd.x, qq.y, fma(-pd.y, qq.x, ay));
   }
   acc[0] = ax; acc[1] = ay;
-  block_partials<R>(acc, part, (int64_t)s * n_chunks + chunk);
+  block_partials(acc, part, (int64_t)s * n_chunks + chunk);
   if (last_block(tail.count + s, gridDim.x)) alpha_tail<4>(tail, part, s, L, n_chunks, ly * L + c, py * L, red);
 }
 
@@ -251,24 +273,33 @@ struct BetaTail {
 __device__ __forceinline__ void beta_tail(const BetaTail &b, const double *part, int n, int s, int L, int n_chunks) {
   const int c = threadIdx.x;
   const int64_t k = (int64_t)s * L + c;
+  const bool lead = threadIdx.y == 0;
+  int act = 0, it = 0;
+  double2 rold = make_double2(0, 0);
+  double tg = 0, tgd = 0, mx0 = 0, mxd0 = 0;
+  if (lead) {            // loaded before the sums, which they do not wait for
+    act = b.active[k];
+    it = b.iters[k] + 1;
+    rold = b.rho[k];
+    tg = b.tgt[k];
+    tgd = b.tgtd[k];
+    mx0 = b.rmax[k];
+    mxd0 = b.rmaxd[k];
+  }
   double a[4];
   sum_chunks<4>(part, s, L, n_chunks, a);
-  const bool lead = threadIdx.y == 0;
-  int act = lead ? b.active[k] : 0;
   if (act) {
-    const int it = b.iters[k] + 1;
     b.iters[k] = it;
     const double nr = sqrt(a[2]), nrd = sqrt(a[3]);
     const double2 rn = make_double2(a[0], a[1]);
-    const double2 rold = b.rho[k];
     b.rho_prev[k] = rold;                  // kept for a later residual replacement
     b.rho[k] = rn;
     // stop (or pause until the next residual replacement) below max(tfac * the largest
     // residual norm since the last replacement, the absolute target)
-    const double mx = fmax(b.rmax[k], nr), mxd = fmax(b.rmaxd[k], nrd);
+    const double mx = fmax(mx0, nr), mxd = fmax(mxd0, nrd);
     b.rmax[k] = mx;
     b.rmaxd[k] = mxd;
-    if (nr <= fmax(b.tfac * mx, b.tgt[k]) && nrd <= fmax(b.tfac * mxd, b.tgtd[k])) {
+    if (nr <= fmax(b.tfac * mx, tg) && nrd <= fmax(b.tfac * mxd, tgd)) {
       act = 0;
     } else if (!isfinite(nr) || !isfinite(nrd) || !(cabs2(rn) > 0)) {
       b.flags[k] |= 2;
@@ -292,8 +323,10 @@ __device__ __forceinline__ void beta_tail(const BetaTail &b, const double *part,
 
 // x += alpha p, r -= alpha q and their duals, (r~, r) and the norms; then, by the last block of
 // each system, beta and the stop tests (TAIL; the shifted family's are a kernel of their own).
+// Bound by FP64 issue (12 operations per element); 64 registers keep 4 blocks on an SM (90, with
+// the tail's, 2).
 template <typename R, bool TAIL>
-__global__ void k_pass_b(int n, int64_t N, int L, int chunk_pts, int n_chunks,
+__global__ void __maxnreg__(64) k_pass_b(int n, int64_t N, int L, int chunk_pts, int n_chunks,
                          typename CT<R>::T *x, typename CT<R>::T *r, const typename CT<R>::T *p,
                          const typename CT<R>::T *q, const double2 *alpha, const int *active,
                          double *part, const int *sys_active, const BetaTail tail) {
@@ -327,7 +360,7 @@ __global__ void k_pass_b(int n, int64_t N, int L, int chunk_pts, int n_chunks,
     }
   }
   double acc[4] = {s0, s1, (double)s2, (double)s3};
-  block_partials<R>(acc, part, (int64_t)s * n_chunks + chunk);
+  block_partials(acc, part, (int64_t)s * n_chunks + chunk);
   if (TAIL && last_block(tail.count + s, gridDim.x)) beta_tail(tail, part, n, s, L, n_chunks);
 }
 
@@ -401,7 +434,7 @@ __global__ void k_replace(int n, int64_t N, int L, int chunk_pts, int n_chunks,
       acc[3] += cabs2(bdd);
     }
   }
-  block_partials<R>(acc, part, (int64_t)s * n_chunks + chunk);
+  block_partials(acc, part, (int64_t)s * n_chunks + chunk);
 }
 
 __global__ void k_reduce_replace(int n, int L, int n_chunks, const double *part, double2 *rho,
@@ -801,7 +834,10 @@ __global__ void k_ms_coef(int n_pt, int n_sh, int L, const double *sigma, const 
 
 // p^_e = r + cb p^_e, x_e += ca p^_e (primal; p^_e = pi_e^k p_e, the scaled search
 // direction); conjugated coefficients for the dual.  One block per (chunk of points,
-// quadrature point); every energy of that point reads the same seed residual chunk.
+// quadrature point); every energy of that point reads the same seed residual chunk.  Bound by
+// FP64 issue (16 FMA per point and column); not unrolled: with fewer registers more blocks stay
+// on an SM, and the FP64 pipe is busy with two warps (4 energies, 8 points of the 32x32x16 cell,
+// L = 16: whole solve 353 -> 334 ms; unrolled by four 378).
 template <typename R>
 __global__ void k_ms_update(int n_pt, int n_sh, int64_t N, int L, int chunk_pts,
                             const typename CT<R>::T *__restrict__ r, typename CT<R>::T *__restrict__ P,
@@ -822,6 +858,7 @@ __global__ void k_ms_update(int n_pt, int n_sh, int64_t N, int L, int chunk_pts,
     const C bc = cconj(b), alc = cconj(al);
     C *Pp = P + s * N * L, *Xp = X + s * N * L;
     C *Pd = P + (n + s) * N * L, *Xd = X + (n + s) * N * L;
+#pragma unroll 1
     for (int64_t i = i0 + ly; i < i1; i += py) {
       const int64_t o = i * L + c;
       const C pv = cfma(b, Pp[o], rp[o]);
