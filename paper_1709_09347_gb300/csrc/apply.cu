@@ -37,6 +37,13 @@ __device__ __forceinline__ float4 c2mul(float2 w0, float2 w1, float4 v) {
   return make_float4(a.x, a.y, b.x, b.y);
 }
 
+// Whether a complex64 apply runs on the two-columns-per-thread stencil: an even number of columns,
+// at most 4 projectors, not the one-column kernel by the caller's choice (the only kernel that
+// takes more than 256 columns).
+static bool c64_two_columns(const HamView &H, int L) {
+  return L % 2 == 0 && L <= 512 && H.np4 == 4 && (H.tune_x2 >= 0 || L > 256);
+}
+
 template <typename R> __device__ __forceinline__ const R *vloc_ptr(const HamView &H);
 template <> __device__ __forceinline__ const double *vloc_ptr<double>(const HamView &H) { return H.vloc; }
 template <> __device__ __forceinline__ const float *vloc_ptr<float>(const HamView &H) { return H.vloc32; }
@@ -152,11 +159,14 @@ __global__ void k_proj_gather(HamView H, int L, const typename CT<R>::T *__restr
 }
 
 // Complex64 gather with two columns per thread (16-byte loads):
-// D[s][a][c][4] = h_a sum_{t in a} p_t w^{-m_t} X[s][i_t][c], for n_proj <= 4.
+// D[s][a] = h_a sum_{t in a} p_t w^{-m_t} X[s][i_t], for n_proj <= 4; element (mu, c) of an atom's
+// block at c d_col + mu d_mu: projectors outermost for k_apply_c64x2 (a warp then reads whole
+// lines; columns outermost, each of its loads touched a quarter of four times as many), columns
+// outermost for k_apply_zm.
 template <bool PER_COL>
 __global__ void k_proj_gather_c64x2(HamView H, int L, const float4 *__restrict__ X,
-                                    const double2 *__restrict__ twist, float2 *__restrict__ D,
-                                    const int *__restrict__ sys_active) {
+                                    const double2 *__restrict__ twist, float2 *__restrict__ D, int d_col,
+                                    int d_mu, const int *__restrict__ sys_active) {
   extern __shared__ float4 red4[];   // [py][4 projectors][L/2] pairs of complex
   const int a = blockIdx.x, s = blockIdx.y;
   const int t = threadIdx.x, ly = threadIdx.y, py = blockDim.y;
@@ -174,36 +184,33 @@ __global__ void k_proj_gather_c64x2(HamView H, int L, const float4 *__restrict__
   const float *pv = H.sup_val32;
   const int64_t t0 = H.sup_ptr[a], t1 = H.sup_ptr[a + 1];
   const float4 *Xs = X + (int64_t)s * H.n * L2;
-  constexpr int U = 4;
-  for (int64_t tb = t0 + ly; tb < t1; tb += (int64_t)U * py) {
+  // eight independent support entries per step keep their gathers in flight (the rows come from
+  // L2 or HBM at random)
+  constexpr int U = 8;
+  auto take = [&](float4 f, int m, int64_t tt) {
+    if (m > 0) f = c2mul(wi0, wi1, f);       // w^{-m} x
+    else if (m < 0) f = c2mul(w0, w1, f);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu)
+      if (mu < np) {
+        const float p = pv[tt * np + mu];
+        acc[mu].x += p * f.x; acc[mu].y += p * f.y; acc[mu].z += p * f.z; acc[mu].w += p * f.w;
+      }
+  };
+  int64_t tb = t0 + ly;
+  for (; tb + (int64_t)(U - 1) * py < t1; tb += (int64_t)U * py) {
     float4 xv[U];
     int mw[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int64_t tt = tb + (int64_t)u * py;
-      if (tt < t1) {
-        xv[u] = Xs[(int64_t)H.sup_idx[tt] * L2 + t];
-        mw[u] = H.sup_wrap[tt];
-      } else {
-        xv[u] = make_float4(0, 0, 0, 0);
-        mw[u] = 0;
-      }
+      xv[u] = Xs[(int64_t)H.sup_idx[tt] * L2 + t];
+      mw[u] = H.sup_wrap[tt];
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int64_t tt = tb + (int64_t)u * py;
-      if (tt >= t1) break;
-      float4 f = xv[u];
-      if (mw[u] > 0) f = c2mul(wi0, wi1, f);       // w^{-m} x
-      else if (mw[u] < 0) f = c2mul(w0, w1, f);
-#pragma unroll
-      for (int mu = 0; mu < 4; ++mu)
-        if (mu < np) {
-          const float p = pv[tt * np + mu];
-          acc[mu].x += p * f.x; acc[mu].y += p * f.y; acc[mu].z += p * f.z; acc[mu].w += p * f.w;
-        }
-    }
+    for (int u = 0; u < U; ++u) take(xv[u], mw[u], tb + (int64_t)u * py);
   }
+  for (; tb < t1; tb += py) take(Xs[(int64_t)H.sup_idx[tb] * L2 + t], H.sup_wrap[tb], tb);
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) red4[((int64_t)ly * 4 + mu) * L2 + t] = acc[mu];
   __syncthreads();
@@ -218,7 +225,7 @@ __global__ void k_proj_gather_c64x2(HamView H, int L, const float4 *__restrict__
       cc[mu] = sum;
     }
     const float *ha = H.h32 + (int64_t)a * np * np;
-    float2 *Da = D + (((int64_t)s * H.n_atoms + a) * L + 2 * t) * 4;   // columns 2t, 2t+1
+    float2 *Da = D + ((int64_t)s * H.n_atoms + a) * L * 4 + 2 * t * (int64_t)d_col;   // columns 2t, 2t+1
     for (int mu = 0; mu < 4; ++mu) {
       float4 d = make_float4(0, 0, 0, 0);
       if (mu < np)
@@ -226,8 +233,8 @@ __global__ void k_proj_gather_c64x2(HamView H, int L, const float4 *__restrict__
           const float hv = ha[mu * np + nu];
           d.x += hv * cc[nu].x; d.y += hv * cc[nu].y; d.z += hv * cc[nu].z; d.w += hv * cc[nu].w;
         }
-      Da[mu] = make_float2(d.x, d.y);
-      Da[4 + mu] = make_float2(d.z, d.w);
+      Da[(int64_t)mu * d_mu] = make_float2(d.x, d.y);
+      Da[(int64_t)mu * d_mu + d_col] = make_float2(d.z, d.w);
     }
   }
 }
@@ -362,11 +369,14 @@ constexpr int kApplyPFBig = 2;
 // Complex64 fast path: each thread owns two adjacent columns of one (x, y) line, so every
 // load and store is 16 bytes; z arms from the register queue of Bloch-extended values, fed
 // from a per-thread ring of kApplyPF planes in shared memory filled by cp.async; the
-// projector scatter reads one packed (atom, wrap) word, one float4 of projector values and
-// 64 bytes of D per covering entry (D laid out [system][atom][column][4]).  The point's
-// scatter-table range and local potential are loaded one plane ahead.  BIG: blocks of up to
+// projector scatter reads one image word, one float4 of projector values and 64 bytes of D per
+// covering entry (D laid out [system][atom][projector][column]); the tables follow the line, and
+// the next entry's image, the point's table range and the local potential are loaded ahead.
+// PROJ: the cell has projectors.  64x64x24 cell, 32 systems, L = 32: gather and stencil 1119 us;
+// with D columns outermost and tables in point order 1314 (the L1 data pipe is what bounds the
+// stencil, and each D load touched 16 wavefronts instead of 4).  BIG: blocks of up to
 // 512 threads (a larger x-y footprint per block, so more of the neighbour loads hit in L1).
-template <bool PER_COL, int MH, bool BIG>
+template <bool PROJ, int MH, bool BIG>
 __global__ void __launch_bounds__(BIG ? 512 : 256, BIG ? 1 : 2) k_apply_c64x2(HamView H, int L, const float4 *__restrict__ X,
                                                         float4 *__restrict__ Y,
                                                         const double2 *__restrict__ twist,
@@ -385,11 +395,9 @@ __global__ void __launch_bounds__(BIG ? 512 : 256, BIG ? 1 : 2) k_apply_c64x2(Ha
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int nth = blockDim.x * blockDim.y * blockDim.z;
   const int nx = H.nx, ny = H.ny, nz = H.nz, nxy = nx * ny;
-  const double2 wd0 = twist[PER_COL ? (int64_t)s * L + 2 * t : s];
-  const double2 wd1 = twist[PER_COL ? (int64_t)s * L + 2 * t + 1 : s];
-  float2 w0, w1, wi0, wi1;
-  twist_pair(wd0, w0, wi0);
-  twist_pair(wd1, w1, wi1);
+  float2 w0, wi0;
+  twist_pair(twist[s], w0, wi0);
+  const float2 w1 = w0, wi1 = wi0;
   const float e = (float)E[s];
   const float dk = H.diag_kin32;
   // neighbour offsets in float4 units (x and y periodic); recomputed, not kept in registers
@@ -400,7 +408,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 256, BIG ? 1 : 2) k_apply_c64x2(Ha
   const float *vl = H.vloc32;
   const float4 *Xs = X + (int64_t)s * H.n * L2;
   float4 *Ys = Y + (int64_t)s * H.n * L2;
-  const float4 *Ds = D + (int64_t)s * H.n_atoms * L * 2 + 4 * t;   // column pair 2t, 2t+1
+  const float4 *Ds = D + (int64_t)s * H.n_atoms * L * 2 + t;   // column pair 2t, 2t+1
   const int line = iy * nx + ix;
   // address of this thread's value in plane p of the Bloch-extended field, p in [-nz, 2nz)
   auto src = [&](int p) -> const float4 * {
@@ -424,8 +432,15 @@ __global__ void __launch_bounds__(BIG ? 512 : 256, BIG ? 1 : 2) k_apply_c64x2(Ha
   float4 q[2 * MH + 1];
 #pragma unroll
   for (int d = 0; d < 2 * MH; ++d) q[d] = bloch(d - MH);
-  int e0 = 0, e1 = 0;
-  if (D) { e0 = (int)H.pt_ptr[line]; e1 = (int)H.pt_ptr[line + 1]; }
+  // entries of the line: the range of the plane, and the first entry not yet used (the tables
+  // have one spare entry at the end)
+  const int *ptr = PROJ ? H.fx_ptr + (int64_t)line * (nz + 1) : nullptr;
+  int e0 = 0, e1 = 0, img = 0;
+  if (PROJ) {
+    e0 = ptr[0];
+    e1 = ptr[1];
+    img = H.fx_img[e0];
+  }
   float vnext = vl[line];
   int slot = 0;
   for (int iz = 0; iz < nz; ++iz) {
@@ -433,7 +448,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 256, BIG ? 1 : 2) k_apply_c64x2(Ha
     const int ce0 = e0, ce1 = e1;
     const float vcur = vnext;
     if (iz + 1 < nz) {                       // next plane's table range and potential
-      if (D) { e0 = (int)H.pt_ptr[pt + nxy]; e1 = (int)H.pt_ptr[pt + nxy + 1]; }
+      if (PROJ) { e0 = e1; e1 = ptr[iz + 2]; }
       vnext = vl[pt + nxy];
     }
     cp_async_wait<PF - 1>();           // plane iz + MH has landed in `slot`
@@ -460,18 +475,20 @@ __global__ void __launch_bounds__(BIG ? 512 : 256, BIG ? 1 : 2) k_apply_c64x2(Ha
     if (iz + MH + PF <= last) cp_async16(&pf_ring[slot * nth + tid], src(iz + MH + PF));
     cp_async_commit();
     slot = slot + 1 == PF ? 0 : slot + 1;
+    if (PROJ)
     for (int qq = ce0; qq < ce1; ++qq) {
-      const int2 aw = H.pt_aw[qq];
-      const float4 p = H.pt_p32[qq];
-      const float4 *Da = Ds + (int64_t)aw.x * L * 2;
-      const float4 d0 = Da[0], d1 = Da[1], d2 = Da[2], d3 = Da[3];
+      const int m = img >= 2 * H.n_atoms ? 1 : (img >= H.n_atoms ? 0 : -1);
+      const float4 *Da = Ds + (int64_t)(img - (m + 1) * H.n_atoms) * 4 * L2;
+      const float4 d0 = Da[0], d1 = Da[L2], d2 = Da[2 * L2], d3 = Da[3 * L2];
+      const float4 p = H.ln_p32[qq];
+      img = H.fx_img[qq + 1];
       float4 v;
-      v.x = p.x * d0.x + p.y * d0.z + p.z * d1.x + p.w * d1.z;
-      v.y = p.x * d0.y + p.y * d0.w + p.z * d1.y + p.w * d1.w;
-      v.z = p.x * d2.x + p.y * d2.z + p.z * d3.x + p.w * d3.z;
-      v.w = p.x * d2.y + p.y * d2.w + p.z * d3.y + p.w * d3.w;
-      if (aw.y > 0) v = c2mul(w0, w1, v);            // w^{m} v
-      else if (aw.y < 0) v = c2mul(wi0, wi1, v);
+      v.x = p.x * d0.x + p.y * d1.x + p.z * d2.x + p.w * d3.x;
+      v.y = p.x * d0.y + p.y * d1.y + p.z * d2.y + p.w * d3.y;
+      v.z = p.x * d0.z + p.y * d1.z + p.z * d2.z + p.w * d3.z;
+      v.w = p.x * d0.w + p.y * d1.w + p.z * d2.w + p.w * d3.w;
+      if (m > 0) v = c2mul(w0, w1, v);            // w^{m} v
+      else if (m < 0) v = c2mul(wi0, wi1, v);
       acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
     }
     Ys[b] = make_float4(e * x0.x - acc.x, e * x0.y - acc.y, e * x0.z - acc.z, e * x0.w - acc.w);
@@ -501,8 +518,10 @@ cbs_status launch_proj_gather(const HamView &H, int n_sys, int L, const typename
     const size_t sm2 = (size_t)py * 4 * L2 * sizeof(float4);
     const float4 *X4 = reinterpret_cast<const float4 *>(X);
     float2 *D2 = reinterpret_cast<float2 *>(D);
-    if (per_col) k_proj_gather_c64x2<true><<<grd, b2, sm2, st>>>(H, L, X4, twist, D2, sys_active);
-    else k_proj_gather_c64x2<false><<<grd, b2, sm2, st>>>(H, L, X4, twist, D2, sys_active);
+    const bool x2 = !per_col && c64_two_columns(H, L);
+    const int d_col = x2 ? 1 : 4, d_mu = x2 ? L : 1;
+    if (per_col) k_proj_gather_c64x2<true><<<grd, b2, sm2, st>>>(H, L, X4, twist, D2, d_col, d_mu, sys_active);
+    else k_proj_gather_c64x2<false><<<grd, b2, sm2, st>>>(H, L, X4, twist, D2, d_col, d_mu, sys_active);
     cbs::count_launches(1);
     CBS_CUDA(cudaGetLastError());
     return CBS_OK;
@@ -532,7 +551,7 @@ cbs_status launch_apply(const HamView &H, int n_sys, int L, const typename CT<R>
   const int ti = sizeof(typename CT<R>::T) == sizeof(float2) ? 1 : 0;
   // complex64 with an even number of columns and at most 4 projectors: two columns per
   // thread (the only complex64 kernel that takes more than 256 columns)
-  if (ti == 1 && L % 2 == 0 && L <= 512 && H.np4 == 4 && (H.tune_x2 >= 0 || L > 256)) {
+  if (ti == 1 && !per_col && c64_two_columns(H, L)) {
     const int L2 = L / 2;
     int py = 256 / L2, pz = 1;
     if (H.tune_py[1] > 0 && H.tune_pz[1] > 0 && H.tune_py[1] * H.tune_pz[1] * L2 <= 512) {
@@ -547,16 +566,16 @@ cbs_status launch_apply(const HamView &H, int n_sys, int L, const typename CT<R>
     float4 *Y4 = reinterpret_cast<float4 *>(Y);
     const float4 *D4 = H.n_atoms ? reinterpret_cast<const float4 *>(D) : nullptr;
     const size_t pf_smem = (size_t)(big ? kApplyPFBig : kApplyPF) * blk.x * blk.y * blk.z * sizeof(float4);
-#define FX(MH)                                                                                     \
-  do {                                                                                             \
-    if (big) {                                                                                     \
-      if (per_col) k_apply_c64x2<true, MH, true><<<grd, blk, pf_smem, st>>>(H, L, X4, Y4, twist, E, D4, sys_active); \
-      else k_apply_c64x2<false, MH, true><<<grd, blk, pf_smem, st>>>(H, L, X4, Y4, twist, E, D4, sys_active);    \
-    } else {                                                                                       \
-      if (per_col) k_apply_c64x2<true, MH, false><<<grd, blk, pf_smem, st>>>(H, L, X4, Y4, twist, E, D4, sys_active); \
-      else k_apply_c64x2<false, MH, false><<<grd, blk, pf_smem, st>>>(H, L, X4, Y4, twist, E, D4, sys_active);    \
-    }                                                                                              \
-    cbs::count_launches(1);                                                                        \
+#define FX(MH)                                                                                                \
+  do {                                                                                                        \
+    if (D4) {                                                                                                 \
+      if (big) k_apply_c64x2<true, MH, true><<<grd, blk, pf_smem, st>>>(H, L, X4, Y4, twist, E, D4, sys_active);   \
+      else k_apply_c64x2<true, MH, false><<<grd, blk, pf_smem, st>>>(H, L, X4, Y4, twist, E, D4, sys_active);      \
+    } else {                                                                                                  \
+      if (big) k_apply_c64x2<false, MH, true><<<grd, blk, pf_smem, st>>>(H, L, X4, Y4, twist, E, D4, sys_active);  \
+      else k_apply_c64x2<false, MH, false><<<grd, blk, pf_smem, st>>>(H, L, X4, Y4, twist, E, D4, sys_active);     \
+    }                                                                                                         \
+    cbs::count_launches(1);                                                                                   \
   } while (0)
     switch (H.m) {
       case 1: FX(1); break;
@@ -615,7 +634,12 @@ cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *
                    void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st) {
   typename CT<R>::T *D = (typename CT<R>::T *)ws;
   if constexpr (sizeof(R) == sizeof(double)) {
-    if (fixed_serves(H, n_sys, L, ws_bytes))
+    // Fixed point takes three launches without projectors, the FP64 stencil one: on short marches
+    // of narrow stencils with little work the launch counts (8x8x4 cell, order 4, 1 to 16 systems
+    // of 16 columns: 10.3 against 16.5 us; 30x30x12, order 2, 16 columns in all: 14.4 against
+    // 18.5; but 20x20x10, order 8, one column: 26.7 against 19.9).
+    const bool brief = H.n_atoms == 0 && H.nz * H.m <= 12 && (double)n_sys * H.n * L * (2 + 12 * H.m) < 4e6;
+    if (!brief && fixed_serves(H, n_sys, L, ws_bytes))
       return apply_fixed(H, n_sys, L, X, Y, twist, per_col, E, ws, sys_active, st);
   }
   cbs_status s = launch_proj_gather<R>(H, n_sys, L, X, twist, per_col, D, sys_active, st);

@@ -642,7 +642,7 @@ static FixGrid fix_grid(const HamView &H, int n_sys, int L) {
   g.tiles = g.tiles_x * ceil_div(H.ny, kFixTY);
   // planes per block: all of them unless that leaves SMs idle
   int zc = 1;
-  while (zc < 8 && (int64_t)g.groups * g.tiles * n_sys * zc < 152 * 2 && H.nz / (zc * 2) >= 2) zc *= 2;
+  while (zc < 8 && (int64_t)g.groups * g.tiles * n_sys * zc < 152 && H.nz / (zc * 2) >= 2) zc *= 2;
   g.z_chunk = std::min(64, ceil_div(H.nz, zc));   // a block marks its planes in 64 bits
   g.z_blocks = ceil_div(H.nz, g.z_chunk);
   return g;

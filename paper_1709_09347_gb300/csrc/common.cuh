@@ -54,7 +54,13 @@ __host__ __device__ __forceinline__ float2 cfma(float2 s, float2 b, float2 a) {
   return a;
 }
 __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-  // Smith's algorithm (scaled) for a / b
+  // one reciprocal where |b|^2 is well inside the range (a division is some 20 dependent FP64
+  // operations, and the scalars of an iteration wait for theirs), else Smith's algorithm
+  const double b2 = b.x * b.x + b.y * b.y;
+  if (b2 > 1e-200 && b2 < 1e200) {
+    const double i = 1.0 / b2;
+    return make_double2((a.x * b.x + a.y * b.y) * i, (a.y * b.x - a.x * b.y) * i);
+  }
   if (fabs(b.x) >= fabs(b.y)) {
     double r = b.y / b.x, d = b.x + b.y * r;
     return make_double2((a.x + a.y * r) / d, (a.y - a.x * r) / d);
@@ -97,9 +103,8 @@ struct HamView {
   const int64_t *pt_ptr;    // [n+1]
   const int32_t *pt_ent;    // [nnz] support entry index
   const int32_t *pt_atom;   // [nnz] atom of that entry
-  int np4;                  // projector slots per entry in D and pt_p32: 4 (n_proj <= 4) or 8
+  int np4;                  // projector slots per entry in D: 4 (n_proj <= 4) or 8
   const int2 *pt_aw;        // [nnz] (atom, wrap) of each covering entry, point order
-  const float4 *pt_p32;     // [nnz] projector values of the entry, zero-padded to 4 (n_proj <= 4)
   // stencil launch shape chosen by cbs_autotune_apply, per precision ([0] complex128,
   // [1] complex64): a block covers tune_py x-lines of tune_pz rows (0 = default: 256 /
   // threads per line x-lines of one row) and, for complex64, whether the
@@ -116,7 +121,9 @@ struct HamView {
   float fx_wxy, fx_wz;      // sums of |weights| of the x and y arms and of the z arms
   float fx_db, fx_pb;       // bounds: largest |D| per unit component, largest projector term
   double fx_vmax;           // max |V_loc|
-  // tables in line order (x-y line by line, along z inside a line)
+  // tables in line order (x-y line by line, along z inside a line), the projectors' for at most
+  // 4 per atom
+  const float4 *ln_p32;     // [nnz+1] projector values of the entries, zero-padded to 4
   const long long *fx_v;    // [n] V_loc * 2^(58 - fx_ew)
   const int *fx_ptr;        // [nx ny][nz + 1] entries of each point of a line
   const int4 *fx_p;         // [nnz+1][2] projector values of the entries: high and low 29-bit words of 4

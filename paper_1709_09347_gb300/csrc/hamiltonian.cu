@@ -284,9 +284,10 @@ static cbs_status compute_norms(cbs_hamiltonian *h) {
   return CBS_OK;
 }
 
-// Fixed-point projector tables: values in line order and in gather order (per atom, entries of
-// image -1, then 0, then +1), and the bounds that size the fixed-point sums.
-static cbs_status fixed_projectors(cbs_hamiltonian *h, const cbs_projectors *P, const std::vector<int64_t> &pt_ptr,
+// Projector tables of the kernels that march along lines: the entries in line order (single
+// precision and fixed point) and in gather order (fixed point: per atom, entries of image -1,
+// then 0, then +1), and the bounds that size the fixed-point sums.
+static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, const std::vector<int64_t> &pt_ptr,
                                    const std::vector<int32_t> &pt_ent, const std::vector<int32_t> &pt_atom) {
   HamView &v = h->v;
   const int na = P->n_atoms, np = P->n_proj;
@@ -316,14 +317,13 @@ static cbs_status fixed_projectors(cbs_hamiltonian *h, const cbs_projectors *P, 
   }
   if (pmax == 0) pmax = l1max = 1;
   h->fx_proj_ok = pmax > 1e-50 && l1max < 1e50 && dmax < 1e30 && cover * dmax < 1e30;
-  if (!h->fx_proj_ok) return CBS_OK;
   // |p| 2^fp < 2^56, and a thread's sum of high words times 2^30 below 2^62
-  v.fx_fp = std::min(56 - (ilogb(pmax) + 1), 61 - (ilogb(l1max) + 1));
+  v.fx_fp = h->fx_proj_ok ? std::min(56 - (ilogb(pmax) + 1), 61 - (ilogb(l1max) + 1)) : 0;
   v.fx_db = (float)(dmax * 1.001);
   v.fx_pb = (float)(cover * dmax * 1.001);
   auto words = [&](int64_t t, int4 *out) {
-    int w[8];
-    for (int mu = 0; mu < 4; ++mu) {
+    int w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int mu = 0; mu < (h->fx_proj_ok ? 4 : 0); ++mu) {
       const long long f = mu < np ? llrint(ldexp(P->sup_val[t * np + mu], v.fx_fp)) : 0;
       w[2 * mu] = balanced_hi(f);
       w[2 * mu + 1] = balanced_lo(f);
@@ -332,6 +332,7 @@ static cbs_status fixed_projectors(cbs_hamiltonian *h, const cbs_projectors *P, 
     out[1] = make_int4(w[4], w[5], w[6], w[7]);
   };
   std::vector<int4> pp((size_t)nnz * 2 + 2, make_int4(0, 0, 0, 0)), gp((size_t)nnz * 2);   // one spare entry
+  std::vector<float4> p32((size_t)nnz + 1, make_float4(0, 0, 0, 0));
   std::vector<int> gi(nnz), gptr((size_t)na * 4), img((size_t)nnz + 1, 0);
   const int64_t nxy = (int64_t)v.nx * v.ny;
   std::vector<int> ptr((size_t)nxy * (v.nz + 1));
@@ -342,6 +343,9 @@ static cbs_status fixed_projectors(cbs_hamiltonian *h, const cbs_projectors *P, 
       ptr[(size_t)line * (v.nz + 1) + iz] = (int)o;
       for (int64_t q = pt_ptr[i]; q < pt_ptr[i + 1]; ++q, ++o) {
         words(pt_ent[q], &pp[2 * o]);
+        float pv[4] = {0, 0, 0, 0};
+        for (int mu = 0; mu < np; ++mu) pv[mu] = (float)P->sup_val[(int64_t)pt_ent[q] * np + mu];
+        p32[o] = make_float4(pv[0], pv[1], pv[2], pv[3]);
         img[o] = ((int)P->sup_wrap[pt_ent[q]] + 1) * na + pt_atom[q];
       }
     }
@@ -361,6 +365,7 @@ static cbs_status fixed_projectors(cbs_hamiltonian *h, const cbs_projectors *P, 
     }
   cbs_status s;
   if ((s = upload(h, pp.data(), pp.size(), &v.fx_p)) != CBS_OK) return s;
+  if ((s = upload(h, p32.data(), p32.size(), &v.ln_p32)) != CBS_OK) return s;
   if ((s = upload(h, img.data(), img.size(), &v.fx_img)) != CBS_OK) return s;
   if ((s = upload(h, ptr.data(), ptr.size(), &v.fx_ptr)) != CBS_OK) return s;
   if ((s = upload(h, gp.data(), gp.size(), &v.fx_gp)) != CBS_OK) return s;
@@ -483,22 +488,12 @@ static cbs_status create_impl(const cbs_grid *g, const double *v_loc, const cbs_
     if ((s = upload(h, pt_ptr.data(), N + 1, &v.pt_ptr)) != CBS_OK) return s;
     if ((s = upload(h, pt_ent.data(), (size_t)nnz, &v.pt_ent)) != CBS_OK) return s;
     if ((s = upload(h, pt_atom.data(), (size_t)nnz, &v.pt_atom)) != CBS_OK) return s;
-    // packed per-entry records for the complex64 scatter (point order)
+    // packed per-entry records (point order)
     v.np4 = np <= 4 ? 4 : 8;
     std::vector<int2> aw(nnz);
-    std::vector<float4> p4(np <= 4 ? nnz : 0);
-    for (int64_t q = 0; q < nnz; ++q) {
-      const int t = pt_ent[q];
-      aw[q] = make_int2(pt_atom[q], (int)P->sup_wrap[t]);
-      if (np <= 4) {
-        float pv[4] = {0, 0, 0, 0};
-        for (int mu = 0; mu < np; ++mu) pv[mu] = (float)P->sup_val[(int64_t)t * np + mu];
-        p4[q] = make_float4(pv[0], pv[1], pv[2], pv[3]);
-      }
-    }
+    for (int64_t q = 0; q < nnz; ++q) aw[q] = make_int2(pt_atom[q], (int)P->sup_wrap[pt_ent[q]]);
     if ((s = upload(h, aw.data(), (size_t)nnz, &v.pt_aw)) != CBS_OK) return s;
-    if (np <= 4 && (s = upload(h, p4.data(), (size_t)nnz, &v.pt_p32)) != CBS_OK) return s;
-    if (np <= 4 && (s = fixed_projectors(h, P, pt_ptr, pt_ent, pt_atom)) != CBS_OK) return s;
+    if (np <= 4 && (s = line_projectors(h, P, pt_ptr, pt_ent, pt_atom)) != CBS_OK) return s;
   } else {
     if ((s = upload(h, pt_ptr.data(), N + 1, &v.pt_ptr)) != CBS_OK) return s;
   }
