@@ -127,8 +127,11 @@ __global__ void __cluster_dims__(kQrpBlocks, 1, 1) __launch_bounds__(kQrpThreads
     if (warp == 0) {
       double bv = -1.0;
       int bj = n;
-      for (int l = lane; l < nl; l += 32)
-        if (w1[l] > bv) { bv = w1[l]; bj = l * kQrpBlocks + rank; }
+      for (int l = lane; l < nl; l += 32) {
+        // a norm that is not a number (an overflow) counts as the largest: every step has a pivot
+        const double wl = w1[l] == w1[l] ? w1[l] : HUGE_VAL;
+        if (wl > bv) { bv = wl; bj = l * kQrpBlocks + rank; }
+      }
       for (int o = 16; o > 0; o >>= 1) {
         const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
         const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
