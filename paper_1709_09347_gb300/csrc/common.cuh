@@ -121,6 +121,7 @@ struct HamView {
   float fx_wxy, fx_wz;      // sums of |weights| of the x and y arms and of the z arms
   float fx_db, fx_pb;       // bounds: largest |D| per unit component, largest projector term
   double fx_vmax;           // max |V_loc|
+  long long fx_diag;        // kinetic diagonal in the unit of the weights
   // tables in line order (x-y line by line, along z inside a line), the projectors' for at most
   // 4 per atom
   const float4 *ln_p32;     // [nnz+1] projector values of the entries, zero-padded to 4

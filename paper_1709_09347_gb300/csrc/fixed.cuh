@@ -143,7 +143,7 @@ __device__ __forceinline__ ColumnScale column_scale(const HamView &H, double2 w,
   o.wi = cdiv(make_double2(1.0, 0.0), w);
   o.f = fix_scale(H, w, o.wi, E, maxhi);
   o.base = 1086 + o.f.ex - o.f.Q;
-  o.ef = o.f.ok ? round_fixed(E - H.diag_kin, 58 - H.fx_ew) : 0;
+  o.ef = o.f.ok ? round_fixed(E, 58 - H.fx_ew) - H.fx_diag : 0;
   o.skip = skip;
   return o;
 }

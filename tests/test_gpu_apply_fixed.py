@@ -135,3 +135,15 @@ def test_error_not_above_the_fp64_kernels():
     ref = P @ X[0].astype(np.clongdouble)
     err = [float(np.sqrt((np.abs(_apply(H, 3, z, E, X, k)[0] - ref) ** 2).sum())) for k in (False, True)]
     assert err[0] <= err[1]
+
+
+def test_constant_field_keeps_the_weights_of_the_fp64_kernels():
+    """On a constant column the neighbours' coefficients must not add up to another energy than the
+    FP64 weights: mean difference to the FP64 kernels below one rounding of E minus the kinetic
+    diagonal (23.4, half an ulp 1.8e-15) and the mean of the 840 points' own roundings (exact
+    coefficients beside the rounded diagonal: 5.8e-15)."""
+    cell = _cell(12, 10, 7, 4, 0)
+    X = np.ones((1, cell[0].n, 1), complex)
+    H, z = _handle(cell), np.array([1.0])
+    a, b = (_apply(H, 0, z, ES[:1], X, k) for k in (False, True))
+    assert abs((a - b).real.mean()) < 3e-15
