@@ -163,8 +163,13 @@ __global__ void k_proj_gather(HamView H, int L, const typename CT<R>::T *__restr
 // block at c d_col + mu d_mu: projectors outermost for k_apply_c64x2 (a warp then reads whole
 // lines; columns outermost, each of its loads touched a quarter of four times as many), columns
 // outermost for k_apply_zm.
+// Bound by the latency of the gathered rows, so warps in flight count: 64 registers and four blocks
+// per SM, 63x61x24 cell, 32 systems of 20 columns 124 us; eight rows per thread and two or four
+// blocks 190, two rows and eight blocks 191.  The values come as one 16-byte load in gather order,
+// and the entry's position tells its image.  64x64x24 cell, 32 systems, L = 32: gather and stencil
+// 1152 -> 1102 us; 4 systems 184 -> 169.
 template <bool PER_COL>
-__global__ void k_proj_gather_c64x2(HamView H, int L, const float4 *__restrict__ X,
+__global__ void __launch_bounds__(256, 4) k_proj_gather_c64x2(HamView H, int L, const float4 *__restrict__ X,
                                     const double2 *__restrict__ twist, float2 *__restrict__ D, int d_col,
                                     int d_mu, const int *__restrict__ sys_active) {
   extern __shared__ float4 red4[];   // [py][4 projectors][L/2] pairs of complex
@@ -181,36 +186,41 @@ __global__ void k_proj_gather_c64x2(HamView H, int L, const float4 *__restrict__
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) acc[mu] = make_float4(0, 0, 0, 0);
   const int np = H.n_proj;
-  const float *pv = H.sup_val32;
-  const int64_t t0 = H.sup_ptr[a], t1 = H.sup_ptr[a + 1];
-  const float4 *Xs = X + (int64_t)s * H.n * L2;
-  // eight independent support entries per step keep their gathers in flight (the rows come from
-  // L2 or HBM at random)
-  constexpr int U = 8;
-  auto take = [&](float4 f, int m, int64_t tt) {
-    if (m > 0) f = c2mul(wi0, wi1, f);       // w^{-m} x
-    else if (m < 0) f = c2mul(w0, w1, f);
+  // the atom's entries in gather order: image -1, then 0, then +1
+  const int4 gp = *reinterpret_cast<const int4 *>(H.fx_gptr + 4 * a);
+  const float4 *Xs = X + (int64_t)s * H.n * L2 + t;
+  // four support entries per step keep their gathers in flight (the rows come from L2 or HBM at
+  // random); the next step's grid points are loaded meanwhile
+  constexpr int U = 4;
+  int row[U];
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu)
-      if (mu < np) {
-        const float p = pv[tt * np + mu];
-        acc[mu].x += p * f.x; acc[mu].y += p * f.y; acc[mu].z += p * f.z; acc[mu].w += p * f.w;
-      }
-  };
-  int64_t tb = t0 + ly;
-  for (; tb + (int64_t)(U - 1) * py < t1; tb += (int64_t)U * py) {
+  for (int u = 0; u < U; ++u) row[u] = gp.x + ly + u * py < gp.w ? H.fx_gi[gp.x + ly + u * py] : -1;
+  for (int tb = gp.x + ly; tb < gp.w; tb += U * py) {
     float4 xv[U];
-    int mw[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int64_t tt = tb + (int64_t)u * py;
-      xv[u] = Xs[(int64_t)H.sup_idx[tt] * L2 + t];
-      mw[u] = H.sup_wrap[tt];
+      xv[u] = make_float4(0, 0, 0, 0);
+      if (row[u] >= 0) xv[u] = Xs[row[u] * L2];
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) take(xv[u], mw[u], tb + (int64_t)u * py);
+    for (int u = 0; u < U; ++u) {
+      const int tn = tb + (U + u) * py;
+      row[u] = tn < gp.w ? H.fx_gi[tn] : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int tt = tb + u * py;
+      if (tt >= gp.w) break;
+      float4 f = xv[u];
+      if (tt >= gp.z) f = c2mul(wi0, wi1, f);       // w^{-m} x
+      else if (tt < gp.y) f = c2mul(w0, w1, f);
+      const float4 p = H.fx_gp32[tt];
+      acc[0].x += p.x * f.x; acc[0].y += p.x * f.y; acc[0].z += p.x * f.z; acc[0].w += p.x * f.w;
+      acc[1].x += p.y * f.x; acc[1].y += p.y * f.y; acc[1].z += p.y * f.z; acc[1].w += p.y * f.w;
+      acc[2].x += p.z * f.x; acc[2].y += p.z * f.y; acc[2].z += p.z * f.z; acc[2].w += p.z * f.w;
+      acc[3].x += p.w * f.x; acc[3].y += p.w * f.y; acc[3].z += p.w * f.z; acc[3].w += p.w * f.w;
+    }
   }
-  for (; tb < t1; tb += py) take(Xs[(int64_t)H.sup_idx[tb] * L2 + t], H.sup_wrap[tb], tb);
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) red4[((int64_t)ly * 4 + mu) * L2 + t] = acc[mu];
   __syncthreads();
@@ -372,7 +382,7 @@ constexpr int kApplyPFBig = 2;
 // projector scatter reads one image word, one float4 of projector values and 64 bytes of D per
 // covering entry (D laid out [system][atom][projector][column]); the tables follow the line, and
 // the next entry's image, the point's table range and the local potential are loaded ahead.
-// PROJ: the cell has projectors.  64x64x24 cell, 32 systems, L = 32: gather and stencil 1119 us;
+// PROJ: the cell has projectors.  64x64x24 cell, 32 systems, L = 32: 909 us, gather and stencil 1152;
 // with D columns outermost and tables in point order 1314 (the L1 data pipe is what bounds the
 // stencil, and each D load touched 16 wavefronts instead of 4).  BIG: blocks of up to
 // 512 threads (a larger x-y footprint per block, so more of the neighbour loads hit in L1).

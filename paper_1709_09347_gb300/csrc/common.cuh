@@ -130,6 +130,7 @@ struct HamView {
   const int4 *fx_p;         // [nnz+1][2] projector values of the entries: high and low 29-bit words of 4
   const int *fx_img;        // [nnz+1] (wrap + 1) * n_atoms + atom of the entries
   const int4 *fx_gp;        // projector values in gather order: per atom, by image -1, 0, +1
+  const float4 *fx_gp32;    // [nnz] projector values in gather order, zero-padded to 4
   const int *fx_gi;         // [nnz] grid point, gather order
   const int *fx_gptr;       // [n_atoms][4] first entry of each image, gather order
 };

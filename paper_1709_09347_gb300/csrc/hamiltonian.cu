@@ -368,8 +368,13 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
     out[1] = make_int4(w[4], w[5], w[6], w[7]);
   };
   std::vector<int4> pp((size_t)nnz * 2 + 2, make_int4(0, 0, 0, 0)), gp((size_t)nnz * 2);   // one spare entry
-  std::vector<float4> p32((size_t)nnz + 1, make_float4(0, 0, 0, 0));
+  std::vector<float4> p32((size_t)nnz + 1, make_float4(0, 0, 0, 0)), gp32(nnz);
   std::vector<int> gi(nnz), gptr((size_t)na * 4), img((size_t)nnz + 1, 0);
+  auto single = [&](int64_t t) {
+    float pv[4] = {0, 0, 0, 0};
+    for (int mu = 0; mu < np; ++mu) pv[mu] = (float)P->sup_val[t * np + mu];
+    return make_float4(pv[0], pv[1], pv[2], pv[3]);
+  };
   const int64_t nxy = (int64_t)v.nx * v.ny;
   std::vector<int> ptr((size_t)nxy * (v.nz + 1));
   int64_t o = 0;
@@ -379,9 +384,7 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
       ptr[(size_t)line * (v.nz + 1) + iz] = (int)o;
       for (int64_t q = pt_ptr[i]; q < pt_ptr[i + 1]; ++q, ++o) {
         words(pt_ent[q], &pp[2 * o]);
-        float pv[4] = {0, 0, 0, 0};
-        for (int mu = 0; mu < np; ++mu) pv[mu] = (float)P->sup_val[(int64_t)pt_ent[q] * np + mu];
-        p32[o] = make_float4(pv[0], pv[1], pv[2], pv[3]);
+        p32[o] = single(pt_ent[q]);
         img[o] = ((int)P->sup_wrap[pt_ent[q]] + 1) * na + pt_atom[q];
       }
     }
@@ -396,6 +399,7 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
         if (P->sup_wrap[t] == m) {
           gi[o] = P->sup_idx[t];
           words(t, &gp[2 * o]);
+          gp32[o] = single(t);
           ++o;
         }
     }
@@ -405,6 +409,7 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
   if ((s = upload(h, img.data(), img.size(), &v.fx_img)) != CBS_OK) return s;
   if ((s = upload(h, ptr.data(), ptr.size(), &v.fx_ptr)) != CBS_OK) return s;
   if ((s = upload(h, gp.data(), gp.size(), &v.fx_gp)) != CBS_OK) return s;
+  if ((s = upload(h, gp32.data(), gp32.size(), &v.fx_gp32)) != CBS_OK) return s;
   if ((s = upload(h, gi.data(), gi.size(), &v.fx_gi)) != CBS_OK) return s;
   return upload(h, gptr.data(), gptr.size(), &v.fx_gptr);
 }
