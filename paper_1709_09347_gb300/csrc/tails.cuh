@@ -38,7 +38,7 @@ struct AlphaTail {
 template <int ST>
 __device__ __forceinline__ void alpha_tail(const AlphaTail &a, const double *part, int s, int L, int parts, int t, int nt,
                                            double *smem) {
-  const int c = t % L, ly = t / L, ry = nt / L;
+  const int c = t % L, ly = t / L, ry = min(nt / L, parts);   // no lane without a part
   const int64_t k0 = (int64_t)s * L + c;
   const double2 rho = ly == 0 ? a.rho[k0] : make_double2(0, 0);   // before the sums
   double gx = 0, gy = 0;
