@@ -299,8 +299,8 @@ static cbs_status compute_norms(cbs_hamiltonian *h) {
   const int nb = ceil_div(v.n, kFroWarps);
   double *part = nullptr, *out = nullptr;
   int *err = nullptr;
-  CBS_CUDA(cudaMalloc(&part, (size_t)nb * 5 * sizeof(double)));
-  CBS_CUDA(cudaMalloc(&out, 5 * sizeof(double) + sizeof(int)));
+  CBS_CUDA(cudaMalloc(&part, ((size_t)nb * 5 + 6) * sizeof(double)));
+  out = part + (size_t)nb * 5;
   err = (int *)(out + 5);
   CBS_CUDA(cudaMemset(err, 0, sizeof(int)));
   k_frobenius<<<nb, 32 * kFroWarps>>>(v, part, err); cbs::count_launches(1);
@@ -310,7 +310,6 @@ static cbs_status compute_norms(cbs_hamiltonian *h) {
   cudaError_t e1 = cudaMemcpy(res, out, sizeof(res), cudaMemcpyDeviceToHost);
   cudaError_t e2 = cudaMemcpy(&herr, err, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(part);
-  cudaFree(out);
   if (e1 != cudaSuccess) return cuda_fail(e1, "Frobenius norm kernel");
   if (e2 != cudaSuccess) return cuda_fail(e2, "Frobenius norm kernel");
   if (herr == 1) { set_error("more than 64 atoms cover one grid point"); return CBS_EINVAL; }
@@ -450,19 +449,19 @@ static cbs_status create_impl(const cbs_grid *g, const double *v_loc, const cbs_
   const size_t N = (size_t)v.n;
   for (size_t i = 0; i < N; ++i)
     if (!isfinite(v_loc[i])) { set_error("v_loc contains a non-finite value"); return CBS_EINVAL; }
-  cbs_status s = upload(h, v_loc, N, &v.vloc);
+  // V_loc in FP64 and in fixed point: one allocation (on small cells they are what creation costs)
+  void *pv = nullptr;
+  cbs_status s = dalloc(h, &pv, 2 * N * sizeof(double));
   if (s != CBS_OK) return s;
+  CBS_CUDA(cudaMemcpy(pv, v_loc, N * sizeof(double), cudaMemcpyHostToDevice));
+  v.vloc = (const double *)pv;
+  v.fx_v = (const long long *)((double *)pv + N);
   std::vector<float> v32(v_loc, v_loc + N);
   s = upload(h, v32.data(), N, &v.vloc32);
   if (s != CBS_OK) return s;
 
   double vmax = 0;
   for (size_t i = 0; i < N; ++i) vmax = std::max(vmax, fabs(v_loc[i]));
-  {
-    void *fv = nullptr;
-    if ((s = dalloc(h, &fv, N * sizeof(long long))) != CBS_OK) return s;
-    v.fx_v = (const long long *)fv;
-  }
   // projectors
   v.n_atoms = 0; v.n_proj = 0; h->nnz = 0; v.np4 = 4;
   h->fx_proj_ok = 1;
