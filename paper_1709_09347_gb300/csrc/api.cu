@@ -175,7 +175,8 @@ extern "C" cbs_status cbs_autotune_apply(cbs_hamiltonian *h, int n_sys, int L, i
                           nullptr, st);
   };
   do {
-    cudaError_t e = cudaMemsetAsync(X, 0, vec, st);
+    // an ordinary number in either type: a column of zeros takes the fixed-point apply's FP64 formula
+    cudaError_t e = cudaMemsetAsync(X, 0x3f, vec, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(tw, hz.data(), n_sys * sizeof(double2), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(Ed, hE.data(), n_sys * sizeof(double), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
