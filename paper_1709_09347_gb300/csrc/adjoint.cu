@@ -138,7 +138,7 @@ extern "C" cbs_status cbs_objective(const cbs_hamiltonian *h, double E, const cb
     s = CBS_OK;
     const double2 *G = nullptr;
     if (grad_vloc || grad_E) {
-      if ((s = adj.alloc(H, n, L)) != CBS_OK) break;
+      if ((s = adj.alloc(H, n, L, st)) != CBS_OK) break;
       if ((s = adj.set_systems(z1, Es, st)) != CBS_OK) break;
       // primal right-hand sides Y2 (systems n..2n-1 of Y), dual right-hand sides Y1
       if ((s = adj.init(Y + (size_t)n * N * L, N * L, Y, N * L, nullptr, o.tol, 0.0, st)) != CBS_OK) break;

@@ -521,7 +521,7 @@ size_t Bicg<R>::bytes_needed(const HamView &H, int n, int L) {
 }
 
 template <typename R>
-cbs_status Bicg<R>::alloc(const HamView &H_, int n_, int L_) {
+cbs_status Bicg<R>::alloc(const HamView &H_, int n_, int L_, cudaStream_t st) {
   H = H_; n = n_; L = L_; N = H.n;
   chunking(N, L, n, &chunk_pts, &n_chunks);
   bytes = bytes_needed(H, n, L);
@@ -556,9 +556,9 @@ cbs_status Bicg<R>::alloc(const HamView &H_, int n_, int L_) {
   n_active = (int *)take(256);
   part = (double *)take((int64_t)n * n_chunks * L * 4 * sizeof(double));
   sys_apply = (unsigned long long *)take(256);
-  CBS_CUDA(cudaMemset(sys_apply, 0, sizeof(unsigned long long)));
+  CBS_CUDA(cudaMemsetAsync(sys_apply, 0, sizeof(unsigned long long), st));
   done = (unsigned *)take((int64_t)3 * n * sizeof(unsigned));
-  CBS_CUDA(cudaMemset(done, 0, (size_t)3 * n * sizeof(unsigned)));
+  CBS_CUDA(cudaMemsetAsync(done, 0, (size_t)3 * n * sizeof(unsigned), st));
   fixed = sizeof(R) == sizeof(double) && fixed_serves(H, 2 * n, L, d_bytes);
   if (fixed) {
     maxhi = (unsigned *)take((int64_t)2 * n * n_chunks * L * sizeof(unsigned));
@@ -958,9 +958,9 @@ size_t MultiShift<R>::bytes_needed(const HamView &H, int n_pt, int n_sh, int L) 
 }
 
 template <typename R>
-cbs_status MultiShift<R>::alloc(const HamView &H, int n_pt_, int n_sh_, int L_) {
+cbs_status MultiShift<R>::alloc(const HamView &H, int n_pt_, int n_sh_, int L_, cudaStream_t st) {
   n_pt = n_pt_; n_sh = n_sh_; L = L_; N = H.n;
-  CBS_TRY_B(seed.alloc(H, n_pt, L));
+  CBS_TRY_B(seed.alloc(H, n_pt, L, st));
   const int64_t n = (int64_t)n_pt * n_sh;
   const int64_t vec = align256(2 * n * N * L * (int64_t)sizeof(C));
   const int64_t bytes = (int64_t)bytes_needed(H, n_pt, n_sh, L) - (int64_t)Bicg<R>::bytes_needed(H, n_pt, L) - vec;
@@ -988,7 +988,7 @@ cbs_status MultiShift<R>::alloc(const HamView &H, int n_pt_, int n_sh_, int L_) 
   siters = (int *)take(n * L * (int64_t)sizeof(int));
   sflags = (int *)take(n * L * (int64_t)sizeof(int));
   upd_cols = (unsigned long long *)take(256);
-  CBS_CUDA(cudaMemset(upd_cols, 0, sizeof(unsigned long long)));
+  CBS_CUDA(cudaMemsetAsync(upd_cols, 0, sizeof(unsigned long long), st));
   return CBS_OK;
 }
 

@@ -51,7 +51,9 @@ struct Bicg {
   int group = 0, group_need = 0;
 
   static size_t bytes_needed(const HamView &H, int n, int L);
-  cbs_status alloc(const HamView &H, int n, int L);
+  // st: the stream of every later call.  The block counters are cleared on it: the legacy stream is
+  // not ordered against a non-blocking one, and a count begun on other contents is never completed.
+  cbs_status alloc(const HamView &H, int n, int L, cudaStream_t st);
   void release();
   // Set twists/energies: primal twist z[s], dual twist 1/conj(z[s]); z, E on device.
   cbs_status set_systems(const double2 *z, const double *Es, cudaStream_t st);
@@ -125,7 +127,7 @@ struct MultiShift {
   static size_t bytes_needed(const HamView &H, int n_pt, int n_sh, int L);
   cbs_status update_columns(cudaStream_t st, double *out);
   // twists z1 [n_pt] (device), shifts sigma_h [n_sh] (host) relative to E0.
-  cbs_status alloc(const HamView &H, int n_pt, int n_sh, int L);
+  cbs_status alloc(const HamView &H, int n_pt, int n_sh, int L, cudaStream_t st);
   cbs_status init(const double2 *z1, double E0, const double *sigma_h, const double2 *B,
                   double tol, cudaStream_t st);
   cbs_status step(int max_iter, cudaStream_t st, int k);

@@ -328,7 +328,7 @@ struct ShiftedSolver {
     rc.profile = o.profile != 0;
     b64.profile = b32.profile = o.profile != 0;
     if (o.precision == CBS_FP64) {
-      CBS_TRY(b64.alloc(H, n, L));
+      CBS_TRY(b64.alloc(H, n, L, st));
       if (group > 0 && o.stop_fraction < 1.0) {
         b64.group = group;
         b64.group_need = stop_need(o, group);
@@ -377,7 +377,7 @@ struct ShiftedSolver {
       //   R~ = B - P(z)^dagger Y~ are formed in FP64, and the columns above tol continue
       //   from R (rounded) with their search directions kept.  Stop targets are relative
       //   to the original right-hand side.
-      CBS_TRY(b32.alloc(H, n, L));
+      CBS_TRY(b32.alloc(H, n, L, st));
       CBS_TRY(b32.set_systems(zs, Es, st));
       CBS_TRY(b32.init(rc.R, (int64_t)H.n * L, rc.R + (size_t)n * H.n * L, (int64_t)H.n * L,
                        rc.colmask, 0.25 * o.tol, o.inner_tol, st, rc.bn2));
@@ -425,7 +425,7 @@ struct ShiftedSolver {
     if (unconv > 0) {
       // FP64 BiCG for the columns left: P(z) D = R, P(z)^dagger D~ = R~ to tol relative to
       // the original right-hand side, then Y += D
-      CBS_TRY(b64.alloc(H, n, L));
+      CBS_TRY(b64.alloc(H, n, L, st));
       CBS_TRY(b64.set_systems(zs, Es, st));
       CBS_TRY(b64.init(rc.R, (int64_t)H.n * L, rc.R + (size_t)n * H.n * L, (int64_t)H.n * L,
                        rc.colmask, 0.5 * o.tol, 0.0, st, rc.bn2));
@@ -471,7 +471,7 @@ struct ShiftedSolver {
     for (int e = 0; e < n_e; ++e) sig[e] = energies_h[e] - E0;
     const bool mixed = sizeof(R) == sizeof(float);
     const double ftol = mixed ? std::max(o.tol, o.family_tol > 0 ? o.family_tol : 1e-6) : o.tol;
-    CBS_TRY(fam.alloc(H, n_pt, n_e, L));
+    CBS_TRY(fam.alloc(H, n_pt, n_e, L, st));
     fam.group_need = stop_need(o, n_pt);
     CBS_TRY(fam.init(z1, E0, sig.data(), B, ftol, st));
     int done = 0;
