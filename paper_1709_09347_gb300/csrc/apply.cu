@@ -553,10 +553,6 @@ cbs_status launch_apply(const HamView &H, int n_sys, int L, const typename CT<R>
                         typename CT<R>::T *Y, const double2 *twist, bool per_col,
                         const double *E, const typename CT<R>::T *D, const int *sys_active,
                         cudaStream_t st) {
-  if ((int64_t)H.n * L >= ((int64_t)1 << 31)) {
-    set_error("apply: N*L must be below 2^31");
-    return CBS_EINVAL;
-  }
   const typename CT<R>::T *Dp = H.n_atoms ? D : nullptr;
   const int ti = sizeof(typename CT<R>::T) == sizeof(float2) ? 1 : 0;
   // complex64 with an even number of columns and at most 4 projectors: two columns per
@@ -651,6 +647,11 @@ cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *
     const bool brief = H.n_atoms == 0 && H.nz * H.m <= 12 && (double)n_sys * H.n * L * (2 + 12 * H.m) < 4e6;
     if (!brief && fixed_serves(H, n_sys, L, ws_bytes))
       return apply_fixed(H, n_sys, L, X, Y, twist, per_col, E, ws, sys_active, st);
+  }
+  // 32-bit indices inside a system, in the gather too: refused before anything is queued
+  if ((int64_t)H.n * L >= ((int64_t)1 << 31)) {
+    set_error("apply: N*L must be below 2^31");
+    return CBS_EINVAL;
   }
   cbs_status s = launch_proj_gather<R>(H, n_sys, L, X, twist, per_col, D, sys_active, st);
   if (s != CBS_OK) return s;
