@@ -153,7 +153,9 @@ void cbs_hamiltonian_free(cbs_hamiltonian *h);
 /* Replaces the local potential of h (§2: V_loc on the diagonal of H0) in place:
  * v_loc: N doubles, HOST or DEVICE pointer (detected).  The single-precision copy and the
  * Frobenius norms are recomputed on the device; the projector table and launch shapes are
- * kept.  A non-finite value returns CBS_EINVAL and leaves h unchanged.  Synchronises the
+ * kept.  A non-finite value returns CBS_EINVAL and leaves h unchanged.  Applies captured in a
+ * CUDA graph stay valid and see the new potential (complex128 ones captured with a potential
+ * of clearly another range run on the slower FP64 formula: capture again).  Synchronises the
  * device; must not run concurrently with other work that uses h.  Lets a caller that
  * differentiates with respect to V_loc (cbs_objective) keep V_loc on the device. */
 cbs_status cbs_hamiltonian_set_vloc(cbs_hamiltonian *h, const double *v_loc);

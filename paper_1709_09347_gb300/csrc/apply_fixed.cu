@@ -497,8 +497,8 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
         tr.add(k, H.fx_nk[k], (a1.re + a2.re + b1.re) + (b2.re + q[MH + k].re + q[MH - k].re));
         ti.add(k, H.fx_nk[k], (a1.im + a2.im + b1.im) + (b2.im + q[MH + k].im + q[MH - k].im));
       }
-      yr.add(tr.shifted(H.fx_st), __ldg(&H.fx_u->c1[0]), __ldg(&H.fx_u->c0[0]));
-      yi.add(ti.shifted(H.fx_st), __ldg(&H.fx_u->c1[0]), __ldg(&H.fx_u->c0[0]));
+      yr.add(tr.shifted(H.fx_st), H.fx_c1[0], H.fx_c0[0]);
+      yi.add(ti.shifted(H.fx_st), H.fx_c1[0], H.fx_c0[0]);
     } else {
 #pragma unroll
       for (int dir = 0; dir < 3; ++dir) {
@@ -510,8 +510,8 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
           tr.add(k, H.fx_nk[k], a.re + b.re);
           ti.add(k, H.fx_nk[k], a.im + b.im);
         }
-        yr.add(tr.shifted(H.fx_st), __ldg(&H.fx_u->c1[dir]), __ldg(&H.fx_u->c0[dir]));
-        yi.add(ti.shifted(H.fx_st), __ldg(&H.fx_u->c1[dir]), __ldg(&H.fx_u->c0[dir]));
+        yr.add(tr.shifted(H.fx_st), H.fx_c1[dir], H.fx_c0[dir]);
+        yi.add(ti.shifted(H.fx_st), H.fx_c1[dir], H.fx_c0[dir]);
       }
     }
     long long vr = yr.shifted(f.sa), vi = yi.shifted(f.sa);

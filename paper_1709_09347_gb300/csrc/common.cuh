@@ -81,16 +81,14 @@ template <> __host__ __device__ __forceinline__ float2 from_d<float>(double2 a) 
 constexpr int kMaxHalf = 6;   // fd_order <= 12
 constexpr int kMaxProj = 8;
 
-// The unit of the fixed-point weights and what is stored in it (fixed.cuh).  It follows the range
-// of V_loc, which may be replaced in place: it lives in device memory beside the table of V_loc in
-// that unit, so that an apply captured in a graph reads the present one.
-struct FixedUnits {
-  int ok;            // 0: the ranges do not fit, every point takes the FP64 formula
-  int ew;            // weights (diagonal, kinetic factors) are stored as g * 2^(58 - ew)
-  double vmax;       // max |V_loc|
-  long long diag;    // kinetic diagonal
-  int c1[3], c0[3];  // 2^fx_st / (2 h^2 den) per direction, high and low 31-bit words
+// The unit that the device table fx_v holds V_loc in, and the range of V_loc.  V_loc may be replaced in
+// place, so these lie in device memory: an apply captured in a graph with another unit takes the
+// FP64 formula (column_scale), which reads V_loc itself.
+struct VlocUnit {
+  int ew;        // fx_v holds V_loc * 2^(58 - ew); kNoUnit: it does not fit
+  double vmax;   // max |V_loc|
 };
+constexpr int kNoUnit = -(1 << 30);
 
 // Device view, passed by value to kernels.
 struct HamView {
@@ -125,15 +123,18 @@ struct HamView {
   // fixed-point tables of the complex128 apply (fixed.cuh); fx_ok = 0: FP64 kernels only
   int fx_ok, fx_iso;        // fx_iso: hx = hy = hz
   int fx_fp;                // projector values as p * 2^fx_fp
+  int fx_ew;                // weights (diagonal, kinetic factors) are stored as g * 2^(58 - fx_ew)
   int fx_st;                // sum_k n_k < 2^fx_st
   int fx_nk[kMaxHalf + 1];  // n_k: |c_k| = n_k / den
+  int fx_c1[3], fx_c0[3];   // 2^fx_st / (2 h^2 den) per direction, high and low 31-bit words
   float fx_wxy, fx_wz;      // sums of |weights| of the x and y arms and of the z arms
   float fx_db, fx_pb;       // bounds: largest |D| per unit component, largest projector term
-  const FixedUnits *fx_u;
+  long long fx_diag;        // kinetic diagonal in the unit of the weights
+  const VlocUnit *fx_u;
   // tables in line order (x-y line by line, along z inside a line), the projectors' for at most
   // 4 per atom
   const float4 *ln_p32;     // [nnz+1] projector values of the entries, zero-padded to 4
-  const long long *fx_v;    // [n] V_loc * 2^(58 - ew)
+  const long long *fx_v;    // [n] V_loc * 2^(58 - fx_u->ew)
   const int *fx_ptr;        // [nx ny][nz + 1] entries of each point of a line
   const int4 *fx_p;         // [nnz+1][2] projector values of the entries: high and low 29-bit words of 4
   const int *fx_img;        // [nnz+1] (wrap + 1) * n_atoms + atom of the entries

@@ -37,7 +37,7 @@ __device__ __forceinline__ int float_exp_above(float f) {   // 2^r > f for a pos
 }
 
 // maxhi: largest high word of |component| over the column.
-__device__ __forceinline__ FixScale fix_scale(const HamView &H, const FixedUnits &u, double2 w, double2 wi, double E,
+__device__ __forceinline__ FixScale fix_scale(const HamView &H, const VlocUnit &u, double2 w, double2 wi, double E,
                                               unsigned maxhi) {
   FixScale s;
   const float a = fmaxf(fmaxf(fabsf((float)w.x), fabsf((float)w.y)), fmaxf(fabsf((float)wi.x), fabsf((float)wi.y)));
@@ -45,7 +45,7 @@ __device__ __forceinline__ FixScale fix_scale(const HamView &H, const FixedUnits
   s.ex = (int)(maxhi >> 20) - 1022;
   // (a NaN would pass through fmaxf: the products with zero are NaN for it)
   const bool finite = w.x * 0.0 + w.y * 0.0 + wi.x * 0.0 + wi.y * 0.0 == 0.0;
-  s.ok = u.ok && finite && a < 8.0f && s.ex > -700 && s.ex < 700 && __double2hiint(de) < ((1023 + u.ew) << 20) && de >= 0.0;
+  s.ok = u.ew == H.fx_ew && finite && a < 8.0f && s.ex > -700 && s.ex < 700 && __double2hiint(de) < ((1023 + H.fx_ew) << 20) && de >= 0.0;
   if (!s.ok) {
     s.Q = kFixMaxQ; s.ex = 0; s.sa = 0; s.uy = 0; s.sp = 0; s.fd = 0;
     return s;
@@ -56,10 +56,10 @@ __device__ __forceinline__ FixScale fix_scale(const HamView &H, const FixedUnits
                                             (float)wi.x * (float)wi.x + (float)wi.y * (float)wi.y)) * 1.0001f);
   const float tw = 1.4143f * wm;
   s.Q = min(kFixMaxQ, 63 - float_exp_above(4.0f + 2.0f * tw));
-  const float yb = H.fx_wxy + H.fx_wz * tw + exp2f((float)u.ew) * 1.0001f + H.fx_pb * tw * tw;
+  const float yb = H.fx_wxy + H.fx_wz * tw + exp2f((float)H.fx_ew) * 1.0001f + H.fx_pb * tw * tw;
   const int lb = float_exp_above(yb * 1.0001f);
-  s.sa = min(24, 66 + u.ew - s.Q - lb);
-  s.uy = s.ex - s.Q + u.ew + 4 - s.sa;
+  s.sa = min(24, 66 + H.fx_ew - s.Q - lb);
+  s.uy = s.ex - s.Q + H.fx_ew + 4 - s.sa;
   // the coefficients (and their twisted images) in 57 bits
   s.sp = H.fx_db > 0 ? max(0, 1 + float_exp_above(H.fx_db * tw * tw * 1.0001f) + s.ex - H.fx_fp - s.uy) : 0;
   s.fd = 58 - H.fx_fp - s.sp - s.uy;
@@ -141,10 +141,10 @@ __device__ __forceinline__ ColumnScale column_scale(const HamView &H, double2 w,
   ColumnScale o;
   o.w = w;
   o.wi = cdiv(make_double2(1.0, 0.0), w);
-  const FixedUnits u = *H.fx_u;
+  const VlocUnit u = *H.fx_u;
   o.f = fix_scale(H, u, w, o.wi, E, maxhi);
   o.base = 1086 + o.f.ex - o.f.Q;
-  o.ef = o.f.ok ? round_fixed(E, 58 - u.ew) - u.diag : 0;
+  o.ef = o.f.ok ? round_fixed(E, 58 - H.fx_ew) - H.fx_diag : 0;
   o.skip = skip;
   return o;
 }

@@ -172,10 +172,10 @@ __global__ void k_sum_parts(const double *part, int nparts, double *out) {
   }
 }
 
-// The units of the fixed-point weights into device memory, and V_loc in that unit, line by line
-__global__ void k_fixed_vloc(int64_t n, int nz, FixedUnits u, const double *v, FixedUnits *du, long long *fv) {
+// V_loc in the fixed-point unit 2^(ew - 58), line by line, and that unit for the applies
+__global__ void k_fixed_vloc(int64_t n, int nz, VlocUnit u, const double *v, VlocUnit *du, long long *fv) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *du = u;
-  if (!u.ok) return;
+  if (u.ew == kNoUnit) return;
   const double up = ldexp(1.0, 58 - u.ew);
   const int64_t nxy = n / nz;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -193,11 +193,10 @@ static int64_t fd_integers(int m, int *nk) {
 }
 
 // The parts of the fixed-point tables that follow the range of V_loc: the common exponent of
-// the weights, the kinetic factors and V_loc in that unit.  Where a range does not fit, fx_ok (and
-// the units' ok, for captured applies) stays 0 and the FP64 kernels serve the cell.
+// the weights, the kinetic factors and V_loc in that unit.  Where a range does not fit, fx_ok stays 0
+// (the FP64 kernels then serve the cell) and captured applies are told by kNoUnit.
 static cbs_status fixed_weights(cbs_hamiltonian *h, double vmax) {
   HamView &v = h->v;
-  FixedUnits u = {};
   v.fx_ok = 0;
   if (v.n_atoms && v.np4 != 4) return CBS_OK;
   const int64_t den = fd_integers(v.m, v.fx_nk);
@@ -211,14 +210,13 @@ static cbs_status fixed_weights(cbs_hamiltonian *h, double vmax) {
     c[d] = ldexp(1.0, v.fx_st) / (2.0 * hh[d] * hh[d] * (double)den);
     top = std::max(top, c[d]);
   }
-  if (top < 1e50 && top > 1e-50) {
-    u.ok = 1;
-    u.ew = ilogb(top) + 1;
-    u.vmax = vmax;
+  const bool fits = top < 1e50 && top > 1e-50;
+  if (fits) {
+    v.fx_ew = ilogb(top) + 1;
     for (int d = 0; d < 3; ++d) {
-      const long long f = llrint(ldexp(c[d], 58 - u.ew));
-      u.c1[d] = (int)(f >> 31);
-      u.c0[d] = (int)(f & 0x7fffffff);
+      const long long f = llrint(ldexp(c[d], 58 - v.fx_ew));
+      v.fx_c1[d] = (int)(f >> 31);
+      v.fx_c0[d] = (int)(f & 0x7fffffff);
     }
     // The neighbours' coefficients n_k c differ from the FP64 weights by up to half an ulp each.
     // What a constant field sees of the difference goes onto the diagonal: left out, the operator
@@ -227,15 +225,15 @@ static cbs_status fixed_weights(cbs_hamiltonian *h, double vmax) {
     // kernels': 2.1e-14).
     double shift = 0;
     for (int d = 0; d < 3; ++d) {
-      const long long f = ((long long)u.c1[d] << 31) + u.c0[d];
+      const long long f = ((long long)v.fx_c1[d] << 31) + v.fx_c0[d];
       const double fh = (double)f, fl = (double)(f - (long long)fh);   // f = fh + fl
       const double *w = d == 0 ? v.wx : d == 1 ? v.wy : v.wz;
       for (int k = 1; k <= v.m; ++k) {
-        const double n = ldexp(k & 1 ? 1.0 : -1.0, u.ew - 58 - v.fx_st) * v.fx_nk[k];
+        const double n = ldexp(k & 1 ? 1.0 : -1.0, v.fx_ew - 58 - v.fx_st) * v.fx_nk[k];
         shift += 2 * (fma(fh, n, w[k]) + fl * n);   // w_k = -n_k c: what is left of it
       }
     }
-    u.diag = llrint(ldexp(v.diag_kin, 58 - u.ew)) + llrint(ldexp(shift, 58 - u.ew));
+    v.fx_diag = llrint(ldexp(v.diag_kin, 58 - v.fx_ew)) + llrint(ldexp(shift, 58 - v.fx_ew));
   }
   v.fx_iso = h->hx == h->hy && h->hy == h->hz;
   double sxy = 0, sz = 0;
@@ -245,11 +243,12 @@ static cbs_status fixed_weights(cbs_hamiltonian *h, double vmax) {
   }
   v.fx_wxy = (float)(sxy * 1.001);
   v.fx_wz = (float)(sz * 1.001);
+  const VlocUnit unit = {fits ? v.fx_ew : kNoUnit, vmax};
   k_fixed_vloc<<<(unsigned)std::min<int64_t>(1024, (v.n + 255) / 256), 256>>>(
-      v.n, v.nz, u, v.vloc, const_cast<FixedUnits *>(v.fx_u), const_cast<long long *>(v.fx_v));
+      v.n, v.nz, unit, v.vloc, const_cast<VlocUnit *>(v.fx_u), const_cast<long long *>(v.fx_v));
   count_launches(1);
   CBS_CUDA(cudaGetLastError());
-  v.fx_ok = u.ok && h->fx_proj_ok;
+  v.fx_ok = fits && h->fx_proj_ok;
   return CBS_OK;
 }
 
@@ -457,12 +456,12 @@ static cbs_status create_impl(const cbs_grid *g, const double *v_loc, const cbs_
   // V_loc in FP64 and in fixed point with its unit: one allocation (on small cells they are what
   // creation costs)
   void *pv = nullptr;
-  cbs_status s = dalloc(h, &pv, 2 * N * sizeof(double) + sizeof(FixedUnits));
+  cbs_status s = dalloc(h, &pv, 2 * N * sizeof(double) + sizeof(VlocUnit));
   if (s != CBS_OK) return s;
   CBS_CUDA(cudaMemcpy(pv, v_loc, N * sizeof(double), cudaMemcpyHostToDevice));
   v.vloc = (const double *)pv;
   v.fx_v = (const long long *)((double *)pv + N);
-  v.fx_u = (const FixedUnits *)(v.fx_v + N);
+  v.fx_u = (const VlocUnit *)(v.fx_v + N);
   std::vector<float> v32(v_loc, v_loc + N);
   s = upload(h, v32.data(), N, &v.vloc32);
   if (s != CBS_OK) return s;
