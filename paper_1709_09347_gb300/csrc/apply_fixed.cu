@@ -39,38 +39,98 @@ __global__ void k_column_max(int64_t N, int L, int chunk_pts, const double2 *__r
   }
 }
 
-// One block of (L, lanes over the chunks) per system: the FP64 work of the scales (a division, the
-// conversions) is done here once instead of by every thread of the kernels that use them.
-__global__ void k_fix_scales(const __grid_constant__ HamView H, int L, int chunks, const unsigned *__restrict__ maxhi,
-                             const double2 *__restrict__ twist, int per_col, const double *__restrict__ E,
-                             ColumnScale *__restrict__ scales, const int *__restrict__ sys_active) {
-  extern __shared__ unsigned smax[];   // [lanes][L]
+// Sample k of a cell of n points: hashed, since steps that divide the grid's would meet one corner of
+// it only.
+__device__ __forceinline__ int sample_point(int k, int64_t n) {
+  return (int)(((unsigned long long)((k + 1) * 0x9e3779b9u) * (unsigned long long)n) >> 32);
+}
+
+__device__ __forceinline__ unsigned point_word(const double2 *Xc, int L, int i) {
+  const double2 v = Xc[(int64_t)i * L];
+  return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+}
+
+// Whether the nearest neighbours of point i of a column (Xc its first element) are all below lim.
+__device__ __forceinline__ bool small_neighbours(const HamView &H, const double2 *Xc, int L, int i, unsigned lim) {
+  const int nx = H.nx, ny = H.ny, nz = H.nz, sz = nx * ny;
+  const int ix = i % nx, iy = i / nx % ny, iz = i / sz;
+  return max(max(max(point_word(Xc, L, i + (ix + 1 < nx ? 1 : 1 - nx)), point_word(Xc, L, i - (ix > 0 ? 1 : 1 - nx))),
+                 max(point_word(Xc, L, i + (iy + 1 < ny ? nx : nx - sz)), point_word(Xc, L, i - (iy > 0 ? nx : nx - sz)))),
+             max(point_word(Xc, L, i + (iz + 1 < nz ? sz : sz - sz * nz)),
+                 point_word(Xc, L, i - (iz > 0 ? sz : sz - sz * nz)))) < lim;
+}
+
+// One block of (L, lanes) per system: the FP64 work of the scales (a division, the conversions) is
+// done here once instead of by every thread of the kernels that use them.  The lanes share the
+// chunks and the samples of a column; bound by latency, so the samples are loaded beside the maxima.
+__global__ void __launch_bounds__(1024) k_fix_scales(const __grid_constant__ HamView H, int L, int chunks,
+                                                     const unsigned *__restrict__ maxhi, const double2 *__restrict__ X,
+                                                     const double2 *__restrict__ twist, int per_col,
+                                                     const double *__restrict__ E, ColumnScale *__restrict__ scales,
+                                                     const int *__restrict__ sys_active) {
+  extern __shared__ unsigned smax[];   // [lanes][L], lim [L], poor [L]
+  __shared__ int bad[256 / kFixRoute];
   const int s = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
   if (sys_active && !sys_active[s]) return;
+  const double2 *Xc = X + (int64_t)s * H.n * L + c;
+  constexpr int U = kFixSamples / 4;   // at least 4 lanes
+  unsigned word[U];
+#pragma unroll
+  for (int j = 0; j < U; ++j) word[j] = ly + j * ry < kFixSamples ? point_word(Xc, L, sample_point(ly + j * ry, H.n)) : ~0u;
   unsigned m = 0;
   for (int k = ly; k < chunks; k += ry) m = max(m, maxhi[((int64_t)s * chunks + k) * L + c]);
   smax[ly * L + c] = m;
+  unsigned *lim = smax + ry * L, *poor = lim + L;
+  __syncthreads();
+  ColumnScale o;
+  if (ly == 0) {
+    for (int y = 1; y < ry; ++y) m = max(m, smax[y * L + c]);
+    o = column_scale(H, twist[per_col ? (int64_t)s * L + c : s], E[s], m, false);
+    lim[c] = o.f.ok ? (unsigned)(o.f.ex - o.f.Q + 53 + 1023) << 20 : 0u;
+    poor[c] = 0;
+    if (c % kFixRoute == 0) bad[c / kFixRoute] = 0;
+  }
+  __syncthreads();
+  const unsigned lm = lim[c];
+  int p = 0;
+#pragma unroll
+  for (int j = 0; j < U; ++j)
+    if (word[j] < lm) p += small_neighbours(H, Xc, L, sample_point(ly + j * ry, H.n), lm);
+  if (p) atomicAdd(&poor[c], (unsigned)p);
+  __syncthreads();
+  if (ly == 0 && (!o.f.ok || poor[c] >= kFixPoor)) bad[c / kFixRoute] = 1;
   __syncthreads();
   if (ly) return;
-  for (int y = 1; y < ry; ++y) m = max(m, smax[y * L + c]);
-  scales[(int64_t)s * L + c] = column_scale(H, twist[per_col ? (int64_t)s * L + c : s], E[s], m, false);
+  if (bad[c / kFixRoute]) o.skip = 2;
+  scales[(int64_t)s * L + c] = o;
 }
 
-// FP64 sum of one image of one atom over the entries t0, t0 + step, ...: the columns that
-// fixed point does not serve.
-__device__ __noinline__ void gather_entries_fp64(const HamView *H, int64_t t0, int64_t t1, int step, int L,
-                                                 const double2 *Xc, int image, double2 *out) {
+// FP64 sums of one image of one atom over the entries t0, t0 + step, ... in gather order: the columns
+// that fixed point does not serve.  Bound by FP64 issue, as k_proj_gather is.
+__device__ __noinline__ void gather_entries_fp64(const HamView *H, int t0, int t1, int step, int L, const double2 *Xc,
+                                                 double2 *out) {
   double2 acc[4];
+#pragma unroll
   for (int mu = 0; mu < 4; ++mu) acc[mu] = make_double2(0, 0);
-  for (int64_t t = t0; t < t1; t += step) {
-    if (H->sup_wrap[t] != image) continue;
-    const double2 f = Xc[(int64_t)H->sup_idx[t] * L];
-    for (int mu = 0; mu < H->n_proj; ++mu) {
-      const double p = H->sup_val[t * H->n_proj + mu];
-      acc[mu].x = fma(p, f.x, acc[mu].x);
-      acc[mu].y = fma(p, f.y, acc[mu].y);
+  const int np = H->n_proj;
+  constexpr int U = 4;   // rows in flight
+  for (int tb = t0; tb < t1; tb += U * step) {
+    double2 x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u] = tb + u * step < t1 ? Xc[(int64_t)H->fx_gi[tb + u * step] * L] : make_double2(0, 0);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (tb + u * step >= t1) break;
+      const double *p = H->sup_val + (int64_t)H->fx_gt[tb + u * step] * np;
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu)
+        if (mu < np) {
+          acc[mu].x = fma(p[mu], x[u].x, acc[mu].x);
+          acc[mu].y = fma(p[mu], x[u].y, acc[mu].y);
+        }
     }
   }
+#pragma unroll
   for (int mu = 0; mu < 4; ++mu) out[mu] = acc[mu];
 }
 
@@ -112,9 +172,11 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
     seen[cx] = 0;
     for (int mu = 0; mu < 4; ++mu) sums[mu * cg + cx] = make_double2(0, 0);
   }
-  __syncthreads();
+  // a warp pays for its FP64 sums whatever its active lanes: one column without a scale takes the
+  // block's others along
+  const bool all64 = __syncthreads_or(sc->skip != 1 && (!f.ok || sc->skip == 2));
   int word = 0;
-  for (int img = 0; img < 3; ++img) {
+  for (int img = 0; img < 3 && !all64; ++img) {
     const int t0 = gp[img], t1 = gp[img + 1];
     if (t0 == t1) continue;
     long long A[8], B[8];
@@ -192,20 +254,22 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
   if (word) atomicOr(&seen[cx], word);
   __syncthreads();
   // columns out of range, or with nothing but small values over this atom: FP64 sums
-  const bool redo = !sc->skip && (!f.ok || seen[cx] < kFixSmallWord);
+  const bool redo = sc->skip != 1 && (all64 || seen[cx] < kFixSmallWord);
   if (__syncthreads_or(redo)) {
     double2 *red = (double2 *)gsm;                         // [py][4][cg], the space of redA
     if (redo && ly == 0)
       for (int mu = 0; mu < 4; ++mu) sums[mu * cg + cx] = make_double2(0, 0);
     for (int img = 0; img < 3; ++img) {
-      double2 part[4];
+      const int t0 = gp[img], t1 = gp[img + 1];   // empty ones too: w may not be finite
       if (redo) {
-        gather_entries_fp64(&H, H.sup_ptr[a] + ly, H.sup_ptr[a + 1], py, L, Xc, img - 1, part);
+        double2 part[4];
+        gather_entries_fp64(&H, t0 + ly, t1, py, L, Xc, part);
+#pragma unroll
         for (int mu = 0; mu < 4; ++mu) red[((size_t)ly * 4 + mu) * cg + cx] = part[mu];
       }
       __syncthreads();
-      if (redo && ly == 0)
-        for (int mu = 0; mu < 4; ++mu) {
+      if (redo)
+        for (int mu = ly; mu < 4; mu += py) {
           double2 v = make_double2(0, 0);
           for (int y = 0; y < py; ++y) v = cadd(v, red[((size_t)y * 4 + mu) * cg + cx]);
           if (img != 1) v = cmul(img == 2 ? sc->wi : sc->w, v);
@@ -226,7 +290,7 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
         d.y = fma(hv, v.y, d.y);
       }
     D[(((int64_t)s * H.n_atoms + a) * L + c) * 4 + mu] = d;
-    if (!f.ok) continue;
+    if (!f.ok || sc->skip) continue;
     const double2 im[3] = {cmul(sc->wi, d), d, cmul(sc->w, d)};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -276,6 +340,98 @@ __device__ __noinline__ double2 output_fp64(const HamView *H, const double2 *Xc,
       acc = csub(acc, v);
     }
   return acc;
+}
+
+// A block's share of a group of columns that takes the FP64 formula throughout: the blocks of the
+// group's columns split the lines of their tile, columns innermost (the march of
+// k_apply_zm<double>, at FP64 issue: 2.35 ms on 32 systems of the 32x32x16 cell, L = 32).
+template <int MH, int CG, int TX, int TY>
+__device__ __noinline__ void tile_fp64(const HamView &H, int L, int groups, int tiles_x, int z_chunk, const double2 *X,
+                                       double2 *Y, const double *E, const ColumnScale *scales, const double2 *D) {
+  const int nx = H.nx, ny = H.ny, nz = H.nz, nxy = nx * ny;
+  const int s = blockIdx.z, g = blockIdx.x % groups, tb = blockIdx.x / groups;
+  const int bx = (tb % tiles_x) * TX, by = (tb / tiles_x) * TY;
+  const int z0 = blockIdx.y * z_chunk, z1 = min(nz, z0 + z_chunk);
+  const double2 *Xs = X + (int64_t)s * H.n * L;
+  double2 *Ys = Y + (int64_t)s * H.n * L;
+  scales += (int64_t)s * L;
+  D += (int64_t)s * H.n_atoms * L * 4;
+  const int c0 = g * CG / kFixRoute * kFixRoute, cols = min(kFixRoute, L - c0);
+  const int blocks = (cols + CG - 1) / CG, per = CG * TX * TY / cols;
+  const int tid = threadIdx.x, c = c0 + tid % cols;
+  if (tid >= per * cols) return;
+  const double2 w = scales[c].w, wi = scales[c].wi;
+  const double ed = E[s] - H.diag_kin;
+  for (int ln = tid / cols + per * (g - c0 / CG); ln < TX * TY; ln += per * blocks) {
+    const int ix = bx + ln % TX, iy = by + ln / TX;
+    if (ix >= nx || iy >= ny) continue;
+    const int line = iy * nx + ix;
+    auto fold = [](int j, int n) {
+      while (j >= n) j -= n;
+      while (j < 0) j += n;
+      return j;
+    };
+    int ox_p[MH + 1], ox_m[MH + 1], oy_p[MH + 1], oy_m[MH + 1];
+#pragma unroll
+    for (int k = 1; k <= MH; ++k) {
+      ox_p[k] = (fold(ix + k, nx) - ix) * L;
+      ox_m[k] = (fold(ix - k, nx) - ix) * L;
+      oy_p[k] = (fold(iy + k, ny) - iy) * nx * L;
+      oy_m[k] = (fold(iy - k, ny) - iy) * nx * L;
+    }
+    auto bloch = [&](int p) -> double2 {
+      if (p >= nz) return cmul(w, Xs[((p - nz) * nxy + line) * L + c]);
+      if (p < 0) return cmul(wi, Xs[((p + nz) * nxy + line) * L + c]);
+      return Xs[(p * nxy + line) * L + c];
+    };
+    double2 q[2 * MH + 1];
+#pragma unroll
+    for (int d = 0; d < 2 * MH; ++d) q[d] = bloch(z0 + d - MH);
+    for (int iz = z0; iz < z1; ++iz) {
+      const int pt = iz * nxy + line, b = pt * L + c;
+      int e0 = 0, e1 = 0;
+      if (H.n_atoms) { e0 = (int)H.pt_ptr[pt]; e1 = (int)H.pt_ptr[pt + 1]; }
+      q[2 * MH] = bloch(iz + MH);
+      const double2 x0 = q[MH];
+      const double dd = ed - H.vloc[pt];
+      double2 acc = make_double2(dd * x0.x, dd * x0.y);
+#pragma unroll
+      for (int k = 1; k <= MH; ++k) {
+        const double2 a1 = Xs[b + ox_p[k]], a2 = Xs[b + ox_m[k]], b1 = Xs[b + oy_p[k]], b2 = Xs[b + oy_m[k]];
+        const double2 z1 = q[MH + k], z2 = q[MH - k];
+        acc.x = fma(-H.wx[k], a1.x + a2.x, acc.x);
+        acc.y = fma(-H.wx[k], a1.y + a2.y, acc.y);
+        acc.x = fma(-H.wy[k], b1.x + b2.x, acc.x);
+        acc.y = fma(-H.wy[k], b1.y + b2.y, acc.y);
+        acc.x = fma(-H.wz[k], z1.x + z2.x, acc.x);
+        acc.y = fma(-H.wz[k], z1.y + z2.y, acc.y);
+      }
+      for (int e = e0; e < e1; ++e) {
+        const int2 aw = H.pt_aw[e];
+        const double *p = H.sup_val + (int64_t)H.pt_ent[e] * H.n_proj;
+        const double2 *Da = D + ((int64_t)aw.x * L + c) * 4;
+        if (aw.y == 0) {
+          for (int mu = 0; mu < H.n_proj; ++mu) {
+            const double2 d = Da[mu];
+            acc.x = fma(-p[mu], d.x, acc.x);
+            acc.y = fma(-p[mu], d.y, acc.y);
+          }
+        } else {
+          double2 v = make_double2(0, 0);
+          for (int mu = 0; mu < H.n_proj; ++mu) {
+            const double2 d = Da[mu];
+            v.x = fma(p[mu], d.x, v.x);
+            v.y = fma(p[mu], d.y, v.y);
+          }
+          const double2 t = aw.y > 0 ? w : wi;
+          acc = cfma(make_double2(-t.x, -t.y), v, acc);
+        }
+      }
+      Ys[b] = acc;
+#pragma unroll
+      for (int d = 0; d < 2 * MH; ++d) q[d] = q[d + 1];
+    }
+  }
 }
 
 struct Fixed2 { long long re, im; };
@@ -365,6 +521,10 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
   if (sys_active && !sys_active[s]) return;
   const int nx = H.nx, ny = H.ny, nz = H.nz;
   const int g = blockIdx.x % groups, tb = blockIdx.x / groups;
+  if (!DOT && scales[(int64_t)s * L + g * CG].skip) {   // the same for the columns of the block
+    tile_fp64<MH, CG, TX, TY>(H, L, groups, tiles_x, z_chunk, X, Y, E, scales, D);
+    return;
+  }
   const int bx = (tb % tiles_x) * TX, by = (tb / tiles_x) * TY;
   const int z0 = blockIdx.y * z_chunk, z1 = min(nz, z0 + z_chunk);
   const int tid = threadIdx.x;
@@ -710,8 +870,8 @@ cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, dou
   const dim3 blk = col_block(L);
   k_column_max<<<dim3((unsigned)chunks, (unsigned)n_sys, 1), blk, (size_t)blk.x * blk.y * sizeof(unsigned), st>>>(
       H.n, L, (int)pts, X, maxhi, sys_active);
-  const dim3 sblk((unsigned)L, (unsigned)std::max(1, std::min(chunks, 512 / L)), 1);
-  k_fix_scales<<<n_sys, sblk, (size_t)sblk.x * sblk.y * sizeof(unsigned), st>>>(H, L, chunks, maxhi, twist, per_col ? 1 : 0,
+  const dim3 sblk((unsigned)L, (unsigned)std::min(kFixSamples, 1024 / L), 1);
+  k_fix_scales<<<n_sys, sblk, (size_t)(sblk.y + 2) * L * sizeof(unsigned), st>>>(H, L, chunks, maxhi, X, twist, per_col ? 1 : 0,
                                                                                E, scales, sys_active);
   count_launches(2);
   CBS_CUDA(cudaGetLastError());

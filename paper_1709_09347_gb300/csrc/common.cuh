@@ -141,6 +141,7 @@ struct HamView {
   const int4 *fx_gp;        // projector values in gather order: per atom, by image -1, 0, +1
   const float4 *fx_gp32;    // [nnz] projector values in gather order, zero-padded to 4
   const int *fx_gi;         // [nnz] grid point, gather order
+  const int *fx_gt;         // [nnz] support entry, gather order
   const int *fx_gptr;       // [n_atoms][4] first entry of each image, gather order
 };
 

@@ -22,6 +22,14 @@ namespace cbs {
 constexpr int kFixMaxQ = 59;
 constexpr int kFixSmallWord = 1 << (53 - 32);   // high word of the smallest value that counts
 
+// Columns of which too many points would leave fixed point take the FP64 formula as a whole: point
+// by point the fixed-point sums are paid as well, and a warp pays for an FP64 output whatever its
+// active lanes (32x32x16 cell, 32 systems of 32 columns: fixed point 0.9 ms, FP64 3.0, point by
+// point on localised columns 4.5).  At one point in 24, two warps in three hold one and the two
+// cost about the same; 32 points of each column are looked at.  An FP64 warp covers 32 columns, so
+// one such column takes the 32 along.
+constexpr int kFixSamples = 32, kFixPoor = 2, kFixRoute = 32;
+
 // Exponents of one (system, column).
 struct FixScale {
   int ok;     // 0: FP64 formula for every point of the column
@@ -132,7 +140,7 @@ struct ColumnScale {
   FixScale f;
   int base;        // exponent offset of to_fixed
   long long ef;    // E - diag_kin in the unit of the weights
-  long long skip;  // 1: the column takes no part (its output is not written)
+  long long skip;  // 1: the column takes no part (its output is not written); 2: it takes the FP64 formula
   double2 w, wi;   // the twist and its inverse
 };
 static_assert(sizeof(ColumnScale) % 16 == 0, "ColumnScale is read in 16-byte pieces");

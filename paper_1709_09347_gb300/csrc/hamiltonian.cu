@@ -372,7 +372,7 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
   };
   std::vector<int4> pp((size_t)nnz * 2 + 2, make_int4(0, 0, 0, 0)), gp((size_t)nnz * 2);   // one spare entry
   std::vector<float4> p32((size_t)nnz + 1, make_float4(0, 0, 0, 0)), gp32(nnz);
-  std::vector<int> gi(nnz), gptr((size_t)na * 4), img((size_t)nnz + 1, 0);
+  std::vector<int> gi(nnz), gt(nnz), gptr((size_t)na * 4), img((size_t)nnz + 1, 0);
   auto single = [&](int64_t t) {
     float pv[4] = {0, 0, 0, 0};
     for (int mu = 0; mu < np; ++mu) pv[mu] = (float)P->sup_val[t * np + mu];
@@ -401,6 +401,7 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
       for (int64_t t = P->sup_ptr[a]; t < P->sup_ptr[a + 1]; ++t)
         if (P->sup_wrap[t] == m) {
           gi[o] = P->sup_idx[t];
+          gt[o] = (int)t;
           words(t, &gp[2 * o]);
           gp32[o] = single(t);
           ++o;
@@ -414,6 +415,7 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
   if ((s = upload(h, gp.data(), gp.size(), &v.fx_gp)) != CBS_OK) return s;
   if ((s = upload(h, gp32.data(), gp32.size(), &v.fx_gp32)) != CBS_OK) return s;
   if ((s = upload(h, gi.data(), gi.size(), &v.fx_gi)) != CBS_OK) return s;
+  if ((s = upload(h, gt.data(), gt.size(), &v.fx_gt)) != CBS_OK) return s;
   return upload(h, gptr.data(), gptr.size(), &v.fx_gptr);
 }
 
