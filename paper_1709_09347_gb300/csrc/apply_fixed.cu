@@ -45,19 +45,26 @@ __device__ __forceinline__ int sample_point(int k, int64_t n) {
   return (int)(((unsigned long long)((k + 1) * 0x9e3779b9u) * (unsigned long long)n) >> 32);
 }
 
-__device__ __forceinline__ unsigned point_word(const double2 *Xc, int L, int i) {
+// High words of the magnitudes of both components of a point.
+__device__ __forceinline__ uint2 point_words(const double2 *Xc, int L, int i) {
   const double2 v = Xc[(int64_t)i * L];
-  return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+  return make_uint2((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
 }
 
-// Whether the nearest neighbours of point i of a column (Xc its first element) are all below lim.
-__device__ __forceinline__ bool small_neighbours(const HamView &H, const double2 *Xc, int L, int i, unsigned lim) {
+// Whether a component of point i (words `own`) and of its nearest neighbours, in a column whose first
+// element is Xc, is below lim throughout.
+__device__ __forceinline__ bool small_around(const HamView &H, const double2 *Xc, int L, int i, uint2 own, unsigned lim) {
   const int nx = H.nx, ny = H.ny, nz = H.nz, sz = nx * ny;
   const int ix = i % nx, iy = i / nx % ny, iz = i / sz;
-  return max(max(max(point_word(Xc, L, i + (ix + 1 < nx ? 1 : 1 - nx)), point_word(Xc, L, i - (ix > 0 ? 1 : 1 - nx))),
-                 max(point_word(Xc, L, i + (iy + 1 < ny ? nx : nx - sz)), point_word(Xc, L, i - (iy > 0 ? nx : nx - sz)))),
-             max(point_word(Xc, L, i + (iz + 1 < nz ? sz : sz - sz * nz)),
-                 point_word(Xc, L, i - (iz > 0 ? sz : sz - sz * nz)))) < lim;
+  const int step[6] = {ix + 1 < nx ? 1 : 1 - nx,    ix > 0 ? -1 : nx - 1,   iy + 1 < ny ? nx : nx - sz,
+                       iy > 0 ? -nx : sz - nx, iz + 1 < nz ? sz : sz - sz * nz, iz > 0 ? -sz : sz * nz - sz};
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const uint2 v = point_words(Xc, L, i + step[k]);
+    own.x = max(own.x, v.x);
+    own.y = max(own.y, v.y);
+  }
+  return min(own.x, own.y) < lim;
 }
 
 // One block of (L, lanes) per system: the FP64 work of the scales (a division, the conversions) is
@@ -74,9 +81,10 @@ __global__ void __launch_bounds__(1024) k_fix_scales(const __grid_constant__ Ham
   if (sys_active && !sys_active[s]) return;
   const double2 *Xc = X + (int64_t)s * H.n * L + c;
   constexpr int U = kFixSamples / 4;   // at least 4 lanes
-  unsigned word[U];
+  uint2 word[U];
 #pragma unroll
-  for (int j = 0; j < U; ++j) word[j] = ly + j * ry < kFixSamples ? point_word(Xc, L, sample_point(ly + j * ry, H.n)) : ~0u;
+  for (int j = 0; j < U; ++j)
+    word[j] = ly + j * ry < kFixSamples ? point_words(Xc, L, sample_point(ly + j * ry, H.n)) : make_uint2(~0u, ~0u);
   unsigned m = 0;
   for (int k = ly; k < chunks; k += ry) m = max(m, maxhi[((int64_t)s * chunks + k) * L + c]);
   smax[ly * L + c] = m;
@@ -95,7 +103,7 @@ __global__ void __launch_bounds__(1024) k_fix_scales(const __grid_constant__ Ham
   int p = 0;
 #pragma unroll
   for (int j = 0; j < U; ++j)
-    if (word[j] < lm) p += small_neighbours(H, Xc, L, sample_point(ly + j * ry, H.n), lm);
+    if (min(word[j].x, word[j].y) < lm) p += small_around(H, Xc, L, sample_point(ly + j * ry, H.n), word[j], lm);
   if (p) atomicAdd(&poor[c], (unsigned)p);
   __syncthreads();
   if (ly == 0 && (!o.f.ok || poor[c] >= kFixPoor)) bad[c / kFixRoute] = 1;
@@ -140,11 +148,16 @@ __device__ __noinline__ void gather_entries_fp64(const HamView *H, int t0, int t
 // One block per (atom, system, group of columns); threadIdx.x a column, threadIdx.y a lane over
 // the atom's support entries.  Per entry: one 16-byte load, two conversions and 3 word
 // products per projector and component.  The projector words are balanced (the low word is
-// signed), so the product of the two low words, left out, has zero mean: it is below 2^-57 of
-// the largest product per entry.
+// signed), so the product of the two low words, left out but for its mean (which depends on the
+// projector alone), is below 2^-58 of the largest product per entry.
+// A sum is about as accurate as the FP64 one where one of its larger projector values (a quarter of the
+// largest) meets a component of at least 2^54 units.  PARTS: each projector is watched for that, the
+// real and the imaginary parts for themselves, and a column without it over the atom is summed in
+// FP64 (175 -> 194 us).  BiCG, which mixes the parts, has the moduli over the atom looked at.
 constexpr int kGatherU = 8;      // entries in flight per thread
 constexpr int kGatherCarry = 2;  // steps of kGatherU entries between carries: |B| grows by less
                                  // than 2^58.4 per entry
+template <bool PARTS>
 __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__ HamView H, int L,
                                                       const double2 *__restrict__ X,
                                                       const ColumnScale *__restrict__ scales,
@@ -160,7 +173,7 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
   long long *redA = gsm;                                   // [py][8][cg]
   long long *redB = redA + (size_t)py * 8 * cg;            // [py][8][cg]
   double2 *sums = (double2 *)(redB + (size_t)py * 8 * cg); // [4][cg] F_a(1/w)^T X
-  int *seen = (int *)(sums + 4 * cg);                      // [cg] high words met, or-ed
+  int *seen = (int *)(sums + 4 * cg);                      // [2][cg] large components met
   const ColumnScale *sc = scales + (int64_t)s * L + c;
   const FixScale f = sc->f;
   const int base = sc->base;
@@ -169,13 +182,13 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
   const unsigned row = (unsigned)L * (unsigned)sizeof(double2), col = (unsigned)c * (unsigned)sizeof(double2);
   const int *gp = H.fx_gptr + 4 * a;
   if (ly == 0) {
-    seen[cx] = 0;
+    seen[cx] = seen[cg + cx] = 0;
     for (int mu = 0; mu < 4; ++mu) sums[mu * cg + cx] = make_double2(0, 0);
   }
   // a warp pays for its FP64 sums whatever its active lanes: one column without a scale takes the
   // block's others along
   const bool all64 = __syncthreads_or(sc->skip != 1 && (!f.ok || sc->skip == 2));
-  int word = 0;
+  int met01 = 0, met23 = 0;   // PARTS: a byte per projector and part, else high words
   for (int img = 0; img < 3 && !all64; ++img) {
     const int t0 = gp[img], t1 = gp[img + 1];
     if (t0 == t1) continue;
@@ -184,11 +197,21 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
     for (int k = 0; k < 8; ++k) A[k] = B[k] = 0;
     const int *gi = H.fx_gi + t0 + ly;
     const int4 *pw = H.fx_gp + 2 * (t0 + ly);
+    const int2 *pm = H.fx_gm + t0 + ly;
     int left = (t1 - t0 - ly + py - 1) / py;     // this thread's entries
     auto fetch = [&](int u) -> double2 { return *(const double2 *)(Xb + ((unsigned)gi[u * py] * row + col)); };
-    auto take = [&](double2 x, const int4 *p) {
+    auto take = [&](double2 x, const int4 *p, const int2 *large) {
       const int4 p01 = p[0], p23 = p[1];
-      const long long xr = to_fixed(x.x, base, word), xi = to_fixed(x.y, base, word);
+      int wr = 0, wi = 0;
+      const long long xr = to_fixed(x.x, base, wr), xi = to_fixed(x.y, base, wi);
+      if constexpr (PARTS) {
+        const int2 m = *large;
+        const int met = __byte_perm((wr >> 22) | (wi >> 22) << 8, 0, 0x1010);
+        met01 |= met & m.x;
+        met23 |= met & m.y;
+      } else {
+        met01 |= wr | wi;
+      }
       const int r1 = opaque((int)(xr >> 29)), r0 = opaque((int)xr & 0x1fffffff);
       const int i1 = opaque((int)(xi >> 29)), i0 = opaque((int)xi & 0x1fffffff);
       const int p1[4] = {p01.x, p01.z, p23.x, p23.z}, p0[4] = {p01.y, p01.w, p23.y, p23.w};
@@ -215,16 +238,18 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
 #pragma unroll
       for (int u = 0; u < kGatherU; ++u) xv[u] = fetch(u);
 #pragma unroll
-      for (int u = 0; u < kGatherU; ++u) take(xv[u], pw + 2 * u * py);
+      for (int u = 0; u < kGatherU; ++u) take(xv[u], pw + 2 * u * py, pm + u * py);
       gi += kGatherU * py;
       pw += 2 * kGatherU * py;
+      pm += kGatherU * py;
       if (++step % kGatherCarry == 0) carry();
     }
     carry();
     for (; left > 0; --left) {
-      take(fetch(0), pw);
+      take(fetch(0), pw, pm);
       gi += py;
       pw += 2 * py;
+      pm += py;
     }
     carry();
 #pragma unroll
@@ -235,7 +260,9 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
     __syncthreads();
     // projector mu of column cx: the image's sum, times w^{-m}
     for (int mu = ly; mu < 4; mu += py) {
-      long long ar = 0, br = 0, ai = 0, bi = 0;
+      // the mean of the products of the low words, 2^28 times the sum of the projector's
+      const long long low = H.fx_gc[(a * 3 + img) * 4 + mu];
+      long long ar = 0, br = low, ai = 0, bi = low;
       for (int y = 0; y < py; ++y) {
         ar += redA[((size_t)y * 8 + 2 * mu) * cg + cx];
         br += redB[((size_t)y * 8 + 2 * mu) * cg + cx];
@@ -251,10 +278,16 @@ __global__ void __launch_bounds__(256, 2) k_gather_fixed(const __grid_constant__
     }
     __syncthreads();
   }
-  if (word) atomicOr(&seen[cx], word);
+  if (met01) atomicOr(&seen[cx], met01);
+  if (met23) atomicOr(&seen[cg + cx], met23);
   __syncthreads();
-  // columns out of range, or with nothing but small values over this atom: FP64 sums
-  const bool redo = sc->skip != 1 && (all64 || seen[cx] < kFixSmallWord);
+  // columns out of range, or with a sum of nothing but small terms: FP64 sums
+  bool redo = all64;
+  if (PARTS)
+    for (int k = 0; k < 2 * H.n_proj; ++k) redo |= !(seen[k / 4 * cg + cx] >> (k % 4 * 8) & 255);
+  else
+    redo |= seen[cx] < kFixSmallWord;
+  redo &= sc->skip != 1;
   if (__syncthreads_or(redo)) {
     double2 *red = (double2 *)gsm;                         // [py][4][cg], the space of redA
     if (redo && ly == 0)
@@ -550,7 +583,18 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
     dx = fma(pd.x, q.x, fma(pd.y, q.y, dx));
     dy = fma(pd.x, q.y, fma(-pd.y, q.x, dy));
   };
-  const double2 w = sc->w, wi = sc->wi;
+  const double2 w0 = sc->w, wi0 = sc->wi;
+  // In the widest stencils the twist is read again where it is used (the last planes, the FP64
+  // formula): kept, it would hold 8 registers through the march (13x10x6 cell, order 12, with the
+  // neighbours of the test below: 21.4 -> 19.4 us; at order 8 the loads cost more, 677 -> 687).
+  auto twist = [&](bool inverse) -> double2 {
+    if constexpr (MH > 4) {
+      const ColumnScale *t = sc;
+      asm volatile("" : "+l"(t));
+      return inverse ? t->wi : t->w;
+    }
+    return inverse ? wi0 : w0;
+  };
   const long long ef = sc->ef;
   auto conv = [&](double2 v) -> Fixed2 { return Fixed2{to_fixed(v.x, base), to_fixed(v.y, base)}; };
   // this thread's value in plane p of the Bloch-extended field, -nz <= p < 2 nz
@@ -586,11 +630,11 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
   for (int d = 0; d < 2 * MH; ++d) {
     double2 v = raw(z0 + d - MH);
     if (d < MH && z0 < MH) {
-      const double2 t = cmul(wi, v);
+      const double2 t = cmul(wi0, v);
       if (z0 + d - MH < 0) v = t;
     }
     if (d > MH && z0 + MH > nz) {
-      const double2 t = cmul(w, v);
+      const double2 t = cmul(w0, v);
       if (z0 + d - MH >= nz) v = t;
     }
     q[d] = conv(v);
@@ -624,7 +668,7 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
     e0 = e1;
     e1 = e2;
     const long long dd = ef - vnext;
-    q[2 * MH] = conv(twisted ? cmul(w, head) : head);
+    q[2 * MH] = conv(twisted ? cmul(twist(false), head) : head);
     double2 hv[SLOTS];
     if (more) {
       head = raw(iz + 1 + MH);
@@ -635,12 +679,13 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
     }
     __syncthreads();
     const Fixed2 x0 = q[MH];
-    if (absword(x0.re, x0.im) < kFixSmallWord) {
-      // a small value at the point: its nearest neighbours decide
-      const Fixed2 n1 = mid[CG], n2 = mid[-CG], n3 = mid[WX * CG], n4 = mid[-WX * CG];
-      const int m = max(max(absword(n1.re, n1.im), absword(n2.re, n2.im)),
-                        max(max(absword(n3.re, n3.im), absword(n4.re, n4.im)),
-                            max(absword(q[MH + 1].re, q[MH + 1].im), absword(q[MH - 1].re, q[MH - 1].im))));
+    if (DOT && max(absword(x0.re), absword(x0.im)) < kFixSmallWord) {
+      // small at the point: its nearest neighbours decide (the moduli, since BiCG mixes the parts: its
+      // updates round each against the larger one)
+      const Fixed2 n[6] = {mid[CG], mid[-CG], mid[WX * CG], mid[-WX * CG], q[MH + 1], q[MH - 1]};
+      int m = 0;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) m = max(m, max(absword(n[k].re), absword(n[k].im)));
       if (m < kFixSmallWord) redo |= 1ull << (iz - z0);
     }
     Product yr, yi;
@@ -649,13 +694,17 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
       yr.add(x0.re, d1, d0);
       yi.add(x0.im, d1, d0);
     }
+    int near_re = 0, near_im = 0;   // high words of the sums over the nearest neighbours
     if (ISO) {
       WeightedSum tr, ti;
 #pragma unroll
       for (int k = 1; k <= MH; ++k) {
         const Fixed2 a1 = mid[k * CG], a2 = mid[-k * CG], b1 = mid[k * WX * CG], b2 = mid[-k * WX * CG];
-        tr.add(k, H.fx_nk[k], (a1.re + a2.re + b1.re) + (b2.re + q[MH + k].re + q[MH - k].re));
-        ti.add(k, H.fx_nk[k], (a1.im + a2.im + b1.im) + (b2.im + q[MH + k].im + q[MH - k].im));
+        const long long sr = (a1.re + a2.re + b1.re) + (b2.re + q[MH + k].re + q[MH - k].re);
+        const long long si = (a1.im + a2.im + b1.im) + (b2.im + q[MH + k].im + q[MH - k].im);
+        if (k == 1) { near_re = (int)(sr >> 32); near_im = (int)(si >> 32); }
+        tr.add(k, H.fx_nk[k], sr);
+        ti.add(k, H.fx_nk[k], si);
       }
       yr.add(tr.shifted(H.fx_st), H.fx_c1[0], H.fx_c0[0]);
       yi.add(ti.shifted(H.fx_st), H.fx_c1[0], H.fx_c0[0]);
@@ -667,12 +716,28 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
         for (int k = 1; k <= MH; ++k) {
           const Fixed2 a = dir == 0 ? mid[k * CG] : dir == 1 ? mid[k * WX * CG] : q[MH + k];
           const Fixed2 b = dir == 0 ? mid[-k * CG] : dir == 1 ? mid[-k * WX * CG] : q[MH - k];
+          if (k == 1) { near_re += (int)((a.re + b.re) >> 32); near_im += (int)((a.im + b.im) >> 32); }
           tr.add(k, H.fx_nk[k], a.re + b.re);
           ti.add(k, H.fx_nk[k], a.im + b.im);
         }
         yr.add(tr.shifted(H.fx_st), H.fx_c1[dir], H.fx_c0[dir]);
         yi.add(ti.shifted(H.fx_st), H.fx_c1[dir], H.fx_c0[dir]);
       }
+    }
+    if (!DOT && ((within((int)(x0.re >> 32), kFixSmallWord) && within(near_re, 8 * kFixSmallWord)) ||
+                 (within((int)(x0.im >> 32), kFixSmallWord) && within(near_im, 8 * kFixSmallWord)))) {
+      // a part that is small at the point, and may be at its nearest neighbours: their sum, which
+      // is at hand, is then below 6 times the limit (seldom otherwise)
+      const Fixed2 *at = mid;
+      if constexpr (MH > 4) asm volatile("" : "+l"(at));   // read again, as the twist
+      const Fixed2 n[6] = {at[CG], at[-CG], at[WX * CG], at[-WX * CG], q[MH + 1], q[MH - 1]};
+      int mr = absword(x0.re), mi = absword(x0.im);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        mr = max(mr, absword(n[k].re));
+        mi = max(mi, absword(n[k].im));
+      }
+      if (min(mr, mi) < kFixSmallWord) redo |= 1ull << (iz - z0);
     }
     long long vr = yr.shifted(f.sa), vi = yi.shifted(f.sa);
     if (e0 < e1) {
@@ -726,7 +791,7 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
   if (own && redo)
     for (iz = z0; iz < z1; ++iz)
       if ((redo >> (iz - z0)) & 1) {
-        const double2 out = output_fp64(&H, (const double2 *)Xs + c, L, ix, iy, iz, w, wi, E[s],
+        const double2 out = output_fp64(&H, (const double2 *)Xs + c, L, ix, iy, iz, twist(false), twist(true), E[s],
                                         proj ? D + ((int64_t)s * H.n_atoms * L + c) * 4 : nullptr);
         *(double2 *)(Ys + iz * plane_bytes + mine) = out;
         if (dotted) add_dot(*(const double2 *)(Xd + iz * plane_bytes + mine), out);
@@ -822,8 +887,9 @@ cbs_status apply_fixed_scaled(const HamView &H, int n_sys, int L, const double2 
     const int groups = ceil_div(L, 32), cg = ceil_div(L, groups);
     const int py = 256 / cg > 32 ? 32 : 256 / cg;
     const dim3 blk((unsigned)cg, (unsigned)py, 1), grd((unsigned)H.n_atoms, (unsigned)n_sys, (unsigned)groups);
-    const size_t sm = (size_t)py * 16 * cg * sizeof(long long) + 4 * cg * sizeof(double2) + cg * sizeof(int);
-    k_gather_fixed<<<grd, blk, sm, st>>>(H, L, X, scales, D, Df, sys_active);
+    const size_t sm = (size_t)py * 16 * cg * sizeof(long long) + 4 * cg * sizeof(double2) + 2 * cg * sizeof(int);
+    if (dot) k_gather_fixed<false><<<grd, blk, sm, st>>>(H, L, X, scales, D, Df, sys_active);
+    else k_gather_fixed<true><<<grd, blk, sm, st>>>(H, L, X, scales, D, Df, sys_active);
     count_launches(1);
     CBS_CUDA(cudaGetLastError());
   }

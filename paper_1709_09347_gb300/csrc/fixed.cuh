@@ -9,10 +9,13 @@
 // enter as the integers n_k of c_k = +-n_k / den, and every product keeps both words of both
 // factors, so an output is rounded once, when it is converted back to FP64.  The error of an
 // output is about 2^(ex - Q) / 4 times the root of the sum of the squared weights; the FP64
-// kernels' is about 2^-53 of the local partial sums.  The fixed-point one is the smaller
-// wherever the neighbourhood of a point holds a component of at least 2^53 units; a point
-// without one, a column whose largest component is zero, not finite or extreme, and a system
-// whose twist or energy is out of range take the FP64 formula instead, point by point.
+// kernels' is about 2^-53 of the local partial sums, of each part for itself.  The fixed-point one is
+// no larger where the real parts over a point and its nearest neighbours hold one of at least 2^53
+// units, and the imaginary parts too (k_gather_fixed has its own test, on the terms of its sums).
+// A point without them (one of a real field, say), a column whose largest component is zero, not
+// finite or extreme, and a system whose twist or energy is out of range take the FP64 formula
+// instead, point by point.  Inside BiCG the moduli are looked at: its updates with complex scalars
+// round a part against the larger of the two.
 #pragma once
 
 #include "tails.cuh"
@@ -129,11 +132,14 @@ __host__ __device__ __forceinline__ int balanced_lo(long long v) {
   return (int)((v + (1 << 28)) & 0x1fffffff) - (1 << 28);
 }
 
-// largest |high word| of a pair of fixed-point components
-__device__ __forceinline__ int absword(long long a, long long b) {
-  const int h0 = (int)(a >> 32), h1 = (int)(b >> 32);
-  return max(h0 ^ (h0 >> 31), h1 ^ (h1 >> 31));
+// high word of a fixed-point component's magnitude (of |v| - 1 for a negative one)
+__device__ __forceinline__ int absword(long long v) {
+  const int h = (int)(v >> 32);
+  return h ^ (h >> 31);
 }
+
+// -lim <= h < lim
+__device__ __forceinline__ bool within(int h, int lim) { return (unsigned)(h + lim) < 2u * (unsigned)lim; }
 
 // What one (system, column) needs besides its vector.
 struct ColumnScale {

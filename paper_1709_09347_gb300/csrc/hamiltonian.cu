@@ -372,6 +372,8 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
   };
   std::vector<int4> pp((size_t)nnz * 2 + 2, make_int4(0, 0, 0, 0)), gp((size_t)nnz * 2);   // one spare entry
   std::vector<float4> p32((size_t)nnz + 1, make_float4(0, 0, 0, 0)), gp32(nnz);
+  std::vector<int2> gm(nnz, make_int2(0, 0));
+  std::vector<long long> gc((size_t)na * 12, 0);
   std::vector<int> gi(nnz), gt(nnz), gptr((size_t)na * 4), img((size_t)nnz + 1, 0);
   auto single = [&](int64_t t) {
     float pv[4] = {0, 0, 0, 0};
@@ -394,7 +396,10 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
     ptr[(size_t)line * (v.nz + 1) + v.nz] = (int)o;
   }
   o = 0;
-  for (int a = 0; a < na; ++a)
+  for (int a = 0; a < na; ++a) {
+    double top[4] = {0, 0, 0, 0};
+    for (int64_t t = P->sup_ptr[a]; t < P->sup_ptr[a + 1]; ++t)
+      for (int mu = 0; mu < np; ++mu) top[mu] = std::max(top[mu], fabs(P->sup_val[t * np + mu]));
     for (int m = -1; m <= 2; ++m) {
       gptr[(size_t)a * 4 + m + 1] = (int)o;
       if (m == 2) break;
@@ -403,10 +408,17 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
           gi[o] = P->sup_idx[t];
           gt[o] = (int)t;
           words(t, &gp[2 * o]);
+          const int4 w0 = gp[2 * o], w1 = gp[2 * o + 1];
+          const int low[4] = {w0.y, w0.w, w1.y, w1.w};
+          for (int mu = 0; mu < 4; ++mu) gc[((size_t)a * 3 + m + 1) * 4 + mu] += low[mu];
           gp32[o] = single(t);
+          for (int mu = 0; mu < np; ++mu)
+            if (4 * fabs(P->sup_val[t * np + mu]) >= top[mu]) (mu < 2 ? gm[o].x : gm[o].y) |= mu % 2 ? (int)0xffff0000 : 0xffff;
           ++o;
         }
     }
+  }
+  for (long long &c : gc) c /= 2;   // 2^28 of the 2^29 that a low word stands for
   cbs_status s;
   if ((s = upload(h, pp.data(), pp.size(), &v.fx_p)) != CBS_OK) return s;
   if ((s = upload(h, p32.data(), p32.size(), &v.ln_p32)) != CBS_OK) return s;
@@ -415,6 +427,8 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
   if ((s = upload(h, gp.data(), gp.size(), &v.fx_gp)) != CBS_OK) return s;
   if ((s = upload(h, gp32.data(), gp32.size(), &v.fx_gp32)) != CBS_OK) return s;
   if ((s = upload(h, gi.data(), gi.size(), &v.fx_gi)) != CBS_OK) return s;
+  if ((s = upload(h, gc.data(), gc.size(), &v.fx_gc)) != CBS_OK) return s;
+  if ((s = upload(h, gm.data(), gm.size(), &v.fx_gm)) != CBS_OK) return s;
   if ((s = upload(h, gt.data(), gt.size(), &v.fx_gt)) != CBS_OK) return s;
   return upload(h, gptr.data(), gptr.size(), &v.fx_gptr);
 }
