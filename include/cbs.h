@@ -171,8 +171,9 @@ cbs_status cbs_hamiltonian_norms(const cbs_hamiltonian *h, double E, double *n_p
  * z: host array of n_sys complex128 twists; E: host array of n_sys energies.
  * X, Y: DEVICE pointers to [n_sys][N][L] blocks of element type dtype (CBS_C128 or
  * CBS_C64).  1 <= L <= 256 (complex64 with even L: <= 512).  Runs on `stream`
- * (cudaStream_t, NULL = legacy default);
- * scratch is allocated per call and freed after synchronising that stream. */
+ * (cudaStream_t, NULL = legacy default) and synchronises it.  Up to 16 MiB of scratch stay with
+ * h, for one call at a time; larger scratch, and that of calls on h that overlap in several
+ * threads, is allocated per call and freed. */
 cbs_status cbs_apply(const cbs_hamiltonian *h, int n_sys, const double *z, const double *E,
                      int L, const void *X, void *Y, int dtype, void *stream);
 

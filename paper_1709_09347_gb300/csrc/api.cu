@@ -68,6 +68,49 @@ extern "C" cbs_status cbs_options_default(cbs_options *o) {
   return CBS_OK;
 }
 
+namespace cbs {
+
+// Scratch of one cbs_apply.  What an allocation and its release cost depends on the other small
+// allocations of the process (a few microseconds, or 175 where they open and close a page of the
+// device's memory), so up to kKeepScratch of it stays with the handle.  The call synchronises its
+// stream before it gives the scratch back, so the next one may use it on any stream; a call that
+// finds it taken (another thread's) allocates its own.
+constexpr size_t kKeepScratch = (size_t)16 << 20;
+
+struct ApplyScratch {
+  cbs_hamiltonian *h = nullptr;   // whose kept scratch is in use
+  void *p = nullptr;
+  cudaError_t take(const cbs_hamiltonian *from, size_t bytes) {
+    if (bytes <= kKeepScratch) {
+      cbs_hamiltonian *o = const_cast<cbs_hamiltonian *>(from);
+      if (!__atomic_exchange_n(&o->scratch_busy, 1, __ATOMIC_ACQUIRE)) {
+        h = o;
+        if (o->scratch_bytes < bytes) {
+          size_t size = (size_t)64 << 10;
+          while (size < bytes) size *= 2;
+          if (o->scratch) cudaFree(o->scratch);
+          o->scratch_bytes = 0;
+          const cudaError_t e = cudaMalloc(&o->scratch, size);
+          if (e != cudaSuccess) {
+            o->scratch = nullptr;
+            return e;
+          }
+          o->scratch_bytes = size;
+        }
+        p = o->scratch;
+        return cudaSuccess;
+      }
+    }
+    return cudaMalloc(&p, bytes);
+  }
+  ~ApplyScratch() {
+    if (h) __atomic_store_n(&h->scratch_busy, 0, __ATOMIC_RELEASE);
+    else if (p) cudaFree(p);
+  }
+};
+
+}  // namespace cbs
+
 extern "C" cbs_status cbs_apply(const cbs_hamiltonian *h, int n_sys, const double *z, const double *E,
                                 int L, const void *X, void *Y, int dtype, void *stream) {
   if (!h || !z || !E || !X || !Y || n_sys < 1 || L < 1 || L > 512) {
@@ -79,12 +122,12 @@ extern "C" cbs_status cbs_apply(const cbs_hamiltonian *h, int n_sys, const doubl
   cudaStream_t st = (cudaStream_t)stream;
   const HamView &H = h->v;
   const size_t dbytes = apply_ws_bytes(H, n_sys, L, dtype);
-  void *scratch = nullptr;
+  ApplyScratch scratch;
   const size_t sys_bytes = (size_t)n_sys * (sizeof(double2) + sizeof(double));
-  CBS_CUDA(cudaMalloc(&scratch, dbytes + sys_bytes + 256));
-  double2 *tw = (double2 *)scratch;
+  CBS_CUDA(scratch.take(h, dbytes + sys_bytes + 256));
+  double2 *tw = (double2 *)scratch.p;
   double *Ed = (double *)(tw + n_sys);
-  void *D = (char *)scratch + ((sys_bytes + 255) & ~(size_t)255);
+  void *D = (char *)scratch.p + ((sys_bytes + 255) & ~(size_t)255);
   cbs_status s = CBS_OK;
   cudaError_t e = cudaMemcpyAsync(tw, z, (size_t)n_sys * sizeof(double2), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(Ed, E, (size_t)n_sys * sizeof(double), cudaMemcpyHostToDevice, st);
@@ -97,9 +140,8 @@ extern "C" cbs_status cbs_apply(const cbs_hamiltonian *h, int n_sys, const doubl
       s = apply_P<float>(H, n_sys, L, (const float2 *)X, (float2 *)Y, tw, false, Ed, D,
                          dbytes, nullptr, st);
   }
-  // the scratch must outlive the kernels: synchronise the stream before freeing it
+  // the scratch must outlive the kernels: synchronise the stream before it is given back
   cudaError_t e2 = cudaStreamSynchronize(st);
-  cudaFree(scratch);
   if (s == CBS_OK && e2 != cudaSuccess) s = cuda_fail(e2, "cbs_apply");
   return s;
 }

@@ -159,6 +159,10 @@ struct cbs_hamiltonian {
   // Frobenius pieces: ||H+||^2, ||H-||^2, off-diagonal part of ||H0||^2, sum d_i, sum d_i^2
   double fro_p2, fro_m2, fro_off0, diag_sum, diag_sum2;
   int fx_proj_ok;   // the projector values fit the fixed-point tables
+  // scratch of one-call applies, kept between calls: taken by one call at a time (scratch_busy)
+  void *scratch;
+  size_t scratch_bytes;
+  int scratch_busy;
   // device allocations owned by the handle
   void *allocs[32];
   int n_allocs;

@@ -280,6 +280,7 @@ using namespace cbs;
 extern "C" void cbs_hamiltonian_free(cbs_hamiltonian *h) {
   if (!h) return;
   for (int k = 0; k < h->n_allocs; ++k) cudaFree(h->allocs[k]);
+  if (h->scratch) cudaFree(h->scratch);
   free(h);
 }
 
