@@ -54,12 +54,16 @@ __host__ __device__ __forceinline__ float2 cfma(float2 s, float2 b, float2 a) {
   return a;
 }
 __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-  // one reciprocal where |b|^2 is well inside the range (a division is some 20 dependent FP64
-  // operations, and the scalars of an iteration wait for theirs), else Smith's algorithm
-  const double b2 = b.x * b.x + b.y * b.y;
-  if (b2 > 1e-200 && b2 < 1e200) {
+  // One reciprocal and a correction by the residual a - q b where both moduli are well inside the range
+  // (a division is some 20 dependent FP64 operations, and the scalars of an iteration wait for
+  // theirs; the correction is 5, and the error at most 1.9 half ulps of the modulus, Smith's 2.7,
+  // without the correction 4.3), else Smith's algorithm.
+  const double b2 = fma(b.x, b.x, b.y * b.y), a1 = fabs(a.x) + fabs(a.y);
+  if (b2 > 1e-200 && b2 < 1e200 && a1 > 1e-150 && a1 < 1e150) {
     const double i = 1.0 / b2;
-    return make_double2((a.x * b.x + a.y * b.y) * i, (a.y * b.x - a.x * b.y) * i);
+    const double qx = fma(a.x, b.x, a.y * b.y) * i, qy = fma(a.y, b.x, -(a.x * b.y)) * i;
+    const double rx = fma(-qx, b.x, fma(qy, b.y, a.x)), ry = fma(-qx, b.y, fma(-qy, b.x, a.y));
+    return make_double2(fma(fma(rx, b.x, ry * b.y), i, qx), fma(fma(ry, b.x, -(rx * b.y)), i, qy));
   }
   if (fabs(b.x) >= fabs(b.y)) {
     double r = b.y / b.x, d = b.x + b.y * r;
