@@ -221,10 +221,11 @@ cbs_status cbs_apply_noalloc(const cbs_hamiltonian *h, int n_sys, const double *
  * columns per thread), with CUDA events on `stream`, a few applies each, and stores the
  * fastest in h:
  * every later apply of that precision through h (cbs_apply*, cbs_solve*, cbs_objective)
- * uses it.  Allocates and frees its own buffers (about 2 n_sys N L elements) and
+ * uses it.  In complex128 the shapes are those of the FP64 kernels, which are timed for them;
+ * the fixed-point kernels that serve most complex128 applies have one shape.  Allocates and frees its own buffers (about 2 n_sys N L elements) and
  * synchronises `stream`.  Outputs (may be NULL): best_py, best_pz (x-lines and rows per
  * block), best_x2 (1 two columns per thread, -1 one, 0 not applicable), best_ms (one
- * apply, milliseconds).
+ * apply as later calls run it, milliseconds).
  * Must not run concurrently with other work that uses h.  Every shape computes the same
  * arithmetic per output; the one- and two-column complex64 kernels may differ in the last
  * bit. */
