@@ -168,7 +168,6 @@ __global__ void k_proj_gather(HamView H, int L, const typename CT<R>::T *__restr
 // blocks 190, two rows and eight blocks 191.  The values come as one 16-byte load in gather order,
 // and the entry's position tells its image.  64x64x24 cell, 32 systems, L = 32: gather and stencil
 // 1152 -> 1102 us; 4 systems 184 -> 169.
-template <bool PER_COL>
 __global__ void __launch_bounds__(256, 4) k_proj_gather_c64x2(HamView H, int L, const float4 *__restrict__ X,
                                     const double2 *__restrict__ twist, float2 *__restrict__ D, int d_col,
                                     int d_mu, const int *__restrict__ sys_active) {
@@ -177,11 +176,8 @@ __global__ void __launch_bounds__(256, 4) k_proj_gather_c64x2(HamView H, int L, 
   const int t = threadIdx.x, ly = threadIdx.y, py = blockDim.y;
   const int L2 = L >> 1;
   if (sys_active && !sys_active[s]) return;
-  const double2 wd0 = twist[PER_COL ? (int64_t)s * L + 2 * t : s];
-  const double2 wd1 = twist[PER_COL ? (int64_t)s * L + 2 * t + 1 : s];
-  float2 w0, w1, wi0, wi1;
-  twist_pair(wd0, w0, wi0);
-  twist_pair(wd1, w1, wi1);
+  float2 w, wi;
+  twist_pair(twist[s], w, wi);
   float4 acc[4];
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) acc[mu] = make_float4(0, 0, 0, 0);
@@ -212,8 +208,8 @@ __global__ void __launch_bounds__(256, 4) k_proj_gather_c64x2(HamView H, int L, 
       const int tt = tb + u * py;
       if (tt >= gp.w) break;
       float4 f = xv[u];
-      if (tt >= gp.z) f = c2mul(wi0, wi1, f);       // w^{-m} x
-      else if (tt < gp.y) f = c2mul(w0, w1, f);
+      if (tt >= gp.z) f = c2mul(wi, wi, f);       // w^{-m} x
+      else if (tt < gp.y) f = c2mul(w, w, f);
       const float4 p = H.fx_gp32[tt];
       acc[0].x += p.x * f.x; acc[0].y += p.x * f.y; acc[0].z += p.x * f.z; acc[0].w += p.x * f.w;
       acc[1].x += p.y * f.x; acc[1].y += p.y * f.y; acc[1].z += p.y * f.z; acc[1].w += p.y * f.w;
@@ -508,6 +504,9 @@ __global__ void __launch_bounds__(BIG ? 512 : 256, BIG ? 1 : 2) k_apply_c64x2(Ha
   cp_async_wait<0>();
 }
 
+// Twists per column come from the residual check of the eigenpairs, in complex128 only.
+template <typename R> constexpr bool kPerCol = sizeof(R) == sizeof(double);
+
 template <typename R>
 cbs_status launch_proj_gather(const HamView &H, int n_sys, int L, const typename CT<R>::T *X,
                               const double2 *twist, bool per_col, typename CT<R>::T *D,
@@ -528,21 +527,24 @@ cbs_status launch_proj_gather(const HamView &H, int n_sys, int L, const typename
     const size_t sm2 = (size_t)py * 4 * L2 * sizeof(float4);
     const float4 *X4 = reinterpret_cast<const float4 *>(X);
     float2 *D2 = reinterpret_cast<float2 *>(D);
-    const bool x2 = !per_col && c64_two_columns(H, L);
-    const int d_col = x2 ? 1 : 4, d_mu = x2 ? L : 1;
-    if (per_col) k_proj_gather_c64x2<true><<<grd, b2, sm2, st>>>(H, L, X4, twist, D2, d_col, d_mu, sys_active);
-    else k_proj_gather_c64x2<false><<<grd, b2, sm2, st>>>(H, L, X4, twist, D2, d_col, d_mu, sys_active);
+    const bool x2 = c64_two_columns(H, L);
+    k_proj_gather_c64x2<<<grd, b2, sm2, st>>>(H, L, X4, twist, D2, x2 ? 1 : 4, x2 ? L : 1, sys_active);
     cbs::count_launches(1);
     CBS_CUDA(cudaGetLastError());
     return CBS_OK;
   }
-  if (H.n_proj <= 4) {
-    if (per_col) k_proj_gather<R, true, 4><<<grd, blk, sm, st>>>(H, L, X, twist, D, sys_active);
-    else k_proj_gather<R, false, 4><<<grd, blk, sm, st>>>(H, L, X, twist, D, sys_active);
+#define PG(PER_COL)                                                                                               \
+  do {                                                                                                            \
+    if (H.n_proj <= 4) k_proj_gather<R, PER_COL, 4><<<grd, blk, sm, st>>>(H, L, X, twist, D, sys_active);          \
+    else k_proj_gather<R, PER_COL, kMaxProj><<<grd, blk, sm, st>>>(H, L, X, twist, D, sys_active);                 \
+  } while (0)
+  if constexpr (kPerCol<R>) {
+    if (per_col) PG(true);
+    else PG(false);
   } else {
-    if (per_col) k_proj_gather<R, true, kMaxProj><<<grd, blk, sm, st>>>(H, L, X, twist, D, sys_active);
-    else k_proj_gather<R, false, kMaxProj><<<grd, blk, sm, st>>>(H, L, X, twist, D, sys_active);
+    PG(false);
   }
+#undef PG
   cbs::count_launches(1);
   CBS_CUDA(cudaGetLastError());
   return CBS_OK;
@@ -557,7 +559,7 @@ cbs_status launch_apply(const HamView &H, int n_sys, int L, const typename CT<R>
   const int ti = sizeof(typename CT<R>::T) == sizeof(float2) ? 1 : 0;
   // complex64 with an even number of columns and at most 4 projectors: two columns per
   // thread (the only complex64 kernel that takes more than 256 columns)
-  if (ti == 1 && !per_col && c64_two_columns(H, L)) {
+  if (ti == 1 && c64_two_columns(H, L)) {
     const int L2 = L / 2;
     int py = 256 / L2, pz = 1;
     if (H.tune_py[1] > 0 && H.tune_pz[1] > 0 && H.tune_py[1] * H.tune_pz[1] * L2 <= 512) {
@@ -608,8 +610,10 @@ cbs_status launch_apply(const HamView &H, int n_sys, int L, const typename CT<R>
   dim3 grd((unsigned)ceil_div(H.nx, blk.y), (unsigned)ceil_div(H.ny, blk.z), (unsigned)n_sys);
 #define ZM(MH)                                                                                  \
   do {                                                                                          \
-    if (per_col) k_apply_zm<R, true, MH><<<grd, blk, 0, st>>>(H, L, X, Y, twist, E, Dp, sys_active); \
-    else k_apply_zm<R, false, MH><<<grd, blk, 0, st>>>(H, L, X, Y, twist, E, Dp, sys_active);   \
+    if (kPerCol<R> && per_col)                                                                  \
+      k_apply_zm<R, kPerCol<R>, MH><<<grd, blk, 0, st>>>(H, L, X, Y, twist, E, Dp, sys_active); \
+    else                                                                                        \
+      k_apply_zm<R, false, MH><<<grd, blk, 0, st>>>(H, L, X, Y, twist, E, Dp, sys_active);      \
     cbs::count_launches(1);                                                                     \
   } while (0)
   switch (H.m) {
@@ -639,6 +643,10 @@ cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *
                    typename CT<R>::T *Y, const double2 *twist, bool per_col, const double *E,
                    void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st) {
   typename CT<R>::T *D = (typename CT<R>::T *)ws;
+  if (per_col && !kPerCol<R>) {
+    set_error("apply: twists per column need complex128");
+    return CBS_EINVAL;
+  }
   if constexpr (sizeof(R) == sizeof(double)) {
     // Fixed point takes three launches without projectors, the FP64 stencil one: on short marches
     // of narrow stencils with little work the launch counts (8x8x4 cell, order 4, 1 to 16 systems
