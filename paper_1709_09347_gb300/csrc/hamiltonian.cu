@@ -356,7 +356,8 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
     cover = std::max(cover, c);
   }
   if (pmax == 0) pmax = l1max = 1;
-  h->fx_proj_ok = pmax > 1e-50 && l1max < 1e50 && dmax < 1e30 && cover * dmax < 1e30;
+  // (the kernels count the two words of an entry's values in 32 bits)
+  h->fx_proj_ok = nnz < (int64_t)1 << 30 && pmax > 1e-50 && l1max < 1e50 && dmax < 1e30 && cover * dmax < 1e30;
   // |p| 2^fp < 2^56, and a thread's sum of high words times 2^30 below 2^62
   v.fx_fp = h->fx_proj_ok ? std::min(56 - (ilogb(pmax) + 1), 61 - (ilogb(l1max) + 1)) : 0;
   v.fx_db = (float)(dmax * 1.001);
