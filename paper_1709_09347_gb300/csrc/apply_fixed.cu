@@ -143,8 +143,8 @@ __device__ __noinline__ void gather_entries_fp64(const HamView *H, int t0, int t
 }
 
 // Bound by integer issue and the latency of the gathered rows: 32 systems of the 32x32x16 cell
-// (40 atoms, L = 32) take 180 us; the FP64 gather, at FP64 issue, 550 us.  84 instructions per
-// entry and column, 24 of them products.
+// (40 atoms, L = 32) take 194 us (175 without PARTS); the FP64 gather, at FP64 issue, 550 us.  About 90
+// instructions per entry and column, 24 of them products.
 // One block per (atom, system, group of columns); threadIdx.x a column, threadIdx.y a lane over
 // the atom's support entries.  Per entry: one 16-byte load, two conversions and 3 word
 // products per projector and component.  The projector words are balanced (the low word is
@@ -153,7 +153,7 @@ __device__ __noinline__ void gather_entries_fp64(const HamView *H, int t0, int t
 // A sum is about as accurate as the FP64 one where one of its larger projector values (a quarter of the
 // largest) meets a component of at least 2^54 units.  PARTS: each projector is watched for that, the
 // real and the imaginary parts for themselves, and a column without it over the atom is summed in
-// FP64 (175 -> 194 us).  BiCG, which mixes the parts, has the moduli over the atom looked at.
+// FP64.  BiCG, which mixes the parts, has the moduli over the atom looked at.
 constexpr int kGatherU = 8;      // entries in flight per thread
 constexpr int kGatherCarry = 2;  // steps of kGatherU entries between carries: |B| grows by less
                                  // than 2^58.4 per entry
@@ -469,7 +469,9 @@ __device__ __noinline__ void tile_fp64(const HamView &H, int L, int groups, int 
 
 struct Fixed2 { long long re, im; };
 
-// sum_k +-n_k s_k as two words: even k enter negative (the signs of c_k alternate)
+// sum_k +-n_k s_k as two words: even k enter negative (the signs of c_k alternate).  The sums s_k stay
+// below 2^63 by the choice of Q, and sum_k n_k below 2^(fx_st - 1), so shifted(fx_st) stays below 2^62:
+// what Product::add, which cuts its factor at 31 bits, can hold.
 struct WeightedSum {
   long long hi = 0;
   unsigned long long plus = 0, minus = 0;
@@ -526,18 +528,19 @@ struct Scatter {
   }
 };
 
-// Stencil and projector scatter: 664 us on 32 systems of the 32x32x16 cell (L = 32, 16.8 M
-// outputs), of which the stencil is 360; k_apply_zm<double>, at FP64 issue, 2400 us.  About 470
+// Stencil and projector scatter: 677 us on 32 systems of the 32x32x16 cell (L = 32, 16.8 M
+// outputs), of which the stencil is 360; k_apply_zm<double>, at FP64 issue, 2400 us.  About 480
 // instructions per output for the stencil and 110 per covering entry; bound by their issue and,
 // in the scatter, by the latency of its loads (16 warps per SM at 128 registers, of which the
-// z queue takes 36).  8 x 8 x 4 tiles of 256 threads beat 16 x 8 x 4 of 512 (two blocks per SM
+// z queue takes 36; the widest stencils, of half-width 5 and 6, spill 30 to 270 bytes per thread).
+// 8 x 8 x 4 tiles of 256 threads beat 16 x 8 x 4 of 512 (two blocks per SM
 // cover each other's barriers) and 8 x 4 x 8; the columns are cut in fours because the halo,
-// converted once per tile, shrinks with the tile's x-y extent.  A block covers TX x TY lines of CG columns and walks the
-// planes z0 .. z1-1; the plane it is on lies in shared memory with its x-y halo, as
-// fixed-point pairs (two buffers, one barrier per plane), and each thread keeps the 2 MH + 1
-// z neighbours of its point in registers.  The next plane's halo and the plane MH ahead are
-// loaded while the current one is computed.  Offsets inside a plane are 32-bit byte offsets
-// from a base that all threads share.
+// converted once per tile, shrinks with the tile's x-y extent.  A block covers TX x TY lines of CG
+// columns and walks the planes z0 .. z1-1; the plane it is on lies in shared memory with its x-y
+// halo, as fixed-point pairs (two buffers, one barrier per plane), and each thread keeps the
+// 2 MH + 1 z neighbours of its point in registers.  The next plane's halo and the plane MH ahead
+// are loaded while the current one is computed.  Offsets inside a plane are 32-bit byte offsets
+// from a base that all threads share.  DOT: one of BiCG's iterations, with (p~, q).
 template <int MH, int CG, int TX, int TY, bool ISO, bool DOT>
 __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
     k_stencil_fixed(const __grid_constant__ HamView H, int L, int groups, int tiles_x, int z_chunk,

@@ -11,10 +11,12 @@
 //
 // All systems of a batch advance together; every kernel covers [2n][N][L] (primal
 // systems then their duals).  Inner products are reduced in two deterministic levels:
-// per-block partial sums over a chunk of grid points, then one thread per (system,
-// column) adding the chunks in order.  One iteration = 6 launches (update p, apply,
-// (p~, q), alpha, update x/r, beta); `check_every` iterations are captured in a CUDA
-// graph and replayed until the device-side count of active systems reaches zero.
+// per-block partial sums over a chunk of grid points, then the chunks by lanes in a fixed
+// order, in the last block of a system to finish (tails.cuh).  One iteration = 4 launches with
+// fixed-point applies (update p with the columns' scales; projector gather; stencil with
+// (p~, q) and alpha; update x/r with beta and the stop tests), 5 with other applies, one fewer
+// without projectors; `check_every` iterations are captured in a CUDA graph and replayed until the
+// device-side count of active systems reaches zero.
 #include <stdio.h>
 #include <stdlib.h>
 
@@ -324,7 +326,7 @@ __device__ __forceinline__ void beta_tail(const BetaTail &b, const double *part,
 // x += alpha p, r -= alpha q and their duals, (r~, r) and the norms; then, by the last block of
 // each system, beta and the stop tests (TAIL; the shifted family's are a kernel of their own).
 // Bound by FP64 issue (12 operations per element); 64 registers keep 4 blocks on an SM (90, with
-// the tail's, 2).
+// the tail's, 2; the cap spills some 50 to 120 bytes, most of them the tail's).
 template <typename R, bool TAIL>
 __global__ void __maxnreg__(64) k_pass_b(int n, int64_t N, int L, int chunk_pts, int n_chunks,
                          typename CT<R>::T *x, typename CT<R>::T *r, const typename CT<R>::T *p,

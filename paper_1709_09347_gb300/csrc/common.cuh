@@ -128,7 +128,7 @@ struct HamView {
   int fx_ok, fx_iso;        // fx_iso: hx = hy = hz
   int fx_fp;                // projector values as p * 2^fx_fp
   int fx_ew;                // weights (diagonal, kinetic factors) are stored as g * 2^(58 - fx_ew)
-  int fx_st;                // sum_k n_k < 2^fx_st
+  int fx_st;                // sum_k n_k < 2^(fx_st - 1): half the range, see WeightedSum
   int fx_nk[kMaxHalf + 1];  // n_k: |c_k| = n_k / den
   int fx_c1[3], fx_c0[3];   // 2^fx_st / (2 h^2 den) per direction, high and low 31-bit words
   float fx_wxy, fx_wz;      // sums of |weights| of the x and y arms and of the z arms

@@ -7,8 +7,9 @@
 //   lambda = tau,  psi = S W_1 Sigma_1^{-1} phi,  S = [S_0 ... S_{M-1}].
 // followed by the residual check of every in-ring pair and the filter.
 //
-// One thread block per energy runs each factorisation; matrices are column-major in
-// global memory (they fit in L2).  The GEMMs (T^< W_1, U_1^dagger C, the eigenvector
+// The QR runs in a cluster of 8 blocks per energy, a Jacobi round in a launch over all pairs, the
+// eigen-solver in one block per energy; matrices are column-major in global memory (they fit in
+// L2).  The GEMMs (T^< W_1, U_1^dagger C, the eigenvector
 // back-transform and S C) use a tiled complex FP64 GEMM.
 #include <cooperative_groups.h>
 #include <math.h>

@@ -202,7 +202,7 @@ static cbs_status fixed_weights(cbs_hamiltonian *h, double vmax) {
   const int64_t den = fd_integers(v.m, v.fx_nk);
   int64_t sum = 0;
   for (int k = 1; k <= v.m; ++k) sum += v.fx_nk[k];
-  v.fx_st = 1;
+  v.fx_st = 1;   // sum < 2^(fx_st - 1), not just 2^fx_st: Product::add takes the sums' upper words as ints
   while (((int64_t)1 << (v.fx_st - 1)) <= sum) ++v.fx_st;
   const double hh[3] = {h->hx, h->hy, h->hz};
   double top = 2.0 * (fabs(v.diag_kin) + vmax), c[3];
