@@ -51,20 +51,20 @@ __device__ __forceinline__ uint2 point_words(const double2 *Xc, int L, int i) {
   return make_uint2((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
 }
 
-// Whether a component of point i (words `own`) and of its nearest neighbours, in a column whose first
-// element is Xc, is below lim throughout.
-__device__ __forceinline__ bool small_around(const HamView &H, const double2 *Xc, int L, int i, uint2 own, unsigned lim) {
+// The larger of these over point i and its nearest neighbours, in a column whose first element is Xc.
+__device__ __forceinline__ uint2 words_around(const HamView &H, const double2 *Xc, int L, int i) {
   const int nx = H.nx, ny = H.ny, nz = H.nz, sz = nx * ny;
   const int ix = i % nx, iy = i / nx % ny, iz = i / sz;
-  const int step[6] = {ix + 1 < nx ? 1 : 1 - nx,    ix > 0 ? -1 : nx - 1,   iy + 1 < ny ? nx : nx - sz,
-                       iy > 0 ? -nx : sz - nx, iz + 1 < nz ? sz : sz - sz * nz, iz > 0 ? -sz : sz * nz - sz};
+  const int step[6] = {ix + 1 < nx ? 1 : 1 - nx, ix > 0 ? -1 : nx - 1,        iy + 1 < ny ? nx : nx - sz,
+                       iy > 0 ? -nx : sz - nx,   iz + 1 < nz ? sz : sz - sz * nz, iz > 0 ? -sz : sz * nz - sz};
+  uint2 m = point_words(Xc, L, i);
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const uint2 v = point_words(Xc, L, i + step[k]);
-    own.x = max(own.x, v.x);
-    own.y = max(own.y, v.y);
+    m.x = max(m.x, v.x);
+    m.y = max(m.y, v.y);
   }
-  return min(own.x, own.y) < lim;
+  return m;
 }
 
 // One block of (L, lanes) per system: the FP64 work of the scales (a division, the conversions) is
@@ -80,20 +80,31 @@ __global__ void __launch_bounds__(1024) k_fix_scales(const __grid_constant__ Ham
   const int s = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
   if (sys_active && !sys_active[s]) return;
   const double2 *Xc = X + (int64_t)s * H.n * L + c;
-  constexpr int U = kFixSamples / 4;   // at least 4 lanes
-  uint2 word[U];
-#pragma unroll
-  for (int j = 0; j < U; ++j)
-    word[j] = ly + j * ry < kFixSamples ? point_words(Xc, L, sample_point(ly + j * ry, H.n)) : make_uint2(~0u, ~0u);
   unsigned m = 0;
   for (int k = ly; k < chunks; k += ry) m = max(m, maxhi[((int64_t)s * chunks + k) * L + c]);
+  double2 w = make_double2(1, 0);
+  double energy = 0;
+  if (ly == 0) {
+    w = twist[per_col ? (int64_t)s * L + c : s];
+    energy = E[s];
+  }
+  constexpr int U = kFixSamples / 4;   // at least 4 lanes
+  unsigned word[U];                    // the smaller part's
+#pragma unroll
+  for (int j = 0; j < U; ++j) {
+    word[j] = ~0u;
+    if (ly + j * ry < kFixSamples) {
+      const uint2 v = words_around(H, Xc, L, sample_point(ly + j * ry, H.n));
+      word[j] = min(v.x, v.y);
+    }
+  }
   smax[ly * L + c] = m;
   unsigned *lim = smax + ry * L, *poor = lim + L;
   __syncthreads();
   ColumnScale o;
   if (ly == 0) {
-    for (int y = 1; y < ry; ++y) m = max(m, smax[y * L + c]);
-    o = column_scale(H, twist[per_col ? (int64_t)s * L + c : s], E[s], m, false);
+    for (int y = 1; y < min(ry, chunks); ++y) m = max(m, smax[y * L + c]);
+    o = column_scale(H, w, energy, m, false);
     lim[c] = o.f.ok ? (unsigned)(o.f.ex - o.f.Q + 53 + 1023) << 20 : 0u;
     poor[c] = 0;
     if (c % kFixRoute == 0) bad[c / kFixRoute] = 0;
@@ -102,8 +113,7 @@ __global__ void __launch_bounds__(1024) k_fix_scales(const __grid_constant__ Ham
   const unsigned lm = lim[c];
   int p = 0;
 #pragma unroll
-  for (int j = 0; j < U; ++j)
-    if (min(word[j].x, word[j].y) < lm) p += small_around(H, Xc, L, sample_point(ly + j * ry, H.n), word[j], lm);
+  for (int j = 0; j < U; ++j) p += word[j] < lm;
   if (p) atomicAdd(&poor[c], (unsigned)p);
   __syncthreads();
   if (ly == 0 && (!o.f.ok || poor[c] >= kFixPoor)) bad[c / kFixRoute] = 1;
@@ -151,7 +161,7 @@ __device__ __noinline__ void gather_entries_fp64(const HamView *H, int t0, int t
 // signed), so the product of the two low words, left out but for its mean (which depends on the
 // projector alone), is below 2^-58 of the largest product per entry.
 // A sum is about as accurate as the FP64 one where one of its larger projector values (a quarter of the
-// largest) meets a component of at least 2^54 units.  PARTS: each projector is watched for that, the
+// largest, at least six of them) meets a component of at least 2^54 units.  PARTS: each projector is watched for that, the
 // real and the imaginary parts for themselves, and a column without it over the atom is summed in
 // FP64.  BiCG, which mixes the parts, has the moduli over the atom looked at.
 constexpr int kGatherU = 8;      // entries in flight per thread

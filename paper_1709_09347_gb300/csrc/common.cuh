@@ -143,8 +143,8 @@ struct HamView {
   const int4 *fx_p;         // [nnz+1][2] projector values of the entries: high and low 29-bit words of 4
   const int *fx_img;        // [nnz+1] (wrap + 1) * n_atoms + atom of the entries
   const int4 *fx_gp;        // projector values in gather order: per atom, by image -1, 0, +1
-  const int2 *fx_gm;        // [nnz] gather order: ones in the 16 bits of projector mu where |p| is at least a
-                            // quarter of the atom's largest
+  const int2 *fx_gm;        // [nnz] gather order: ones in the 16 bits of projector mu where |p| is one of the
+                            // atom's larger (a quarter of the largest, at least six of them)
   const long long *fx_gc;   // [n_atoms][3][4] half the sum of the low words of the projector values of each image
   const float4 *fx_gp32;    // [nnz] projector values in gather order, zero-padded to 4
   const int *fx_gi;         // [nnz] grid point, gather order

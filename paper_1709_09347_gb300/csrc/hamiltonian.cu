@@ -10,6 +10,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <vector>
 
 #include "fixed.cuh"
@@ -399,9 +400,17 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
   }
   o = 0;
   for (int a = 0; a < na; ++a) {
-    double top[4] = {0, 0, 0, 0};
-    for (int64_t t = P->sup_ptr[a]; t < P->sup_ptr[a + 1]; ++t)
-      for (int mu = 0; mu < np; ++mu) top[mu] = std::max(top[mu], fabs(P->sup_val[t * np + mu]));
+    // the larger values of each projector: a quarter of the largest, at least six of them (a narrow
+    // projector has one or two, and an ordinary column often something small there)
+    double large[4] = {0, 0, 0, 0};
+    const int64_t t0 = P->sup_ptr[a], entries = P->sup_ptr[a + 1] - t0;
+    std::vector<double> size(entries);
+    for (int mu = 0; mu < np && entries > 0; ++mu) {
+      for (int64_t t = 0; t < entries; ++t) size[t] = fabs(P->sup_val[(t0 + t) * np + mu]);
+      const int64_t sixth = std::min<int64_t>(6, entries) - 1;
+      std::nth_element(size.begin(), size.begin() + sixth, size.end(), std::greater<double>());
+      large[mu] = std::min(size[sixth], *std::max_element(size.begin(), size.begin() + sixth + 1) / 4);
+    }
     for (int m = -1; m <= 2; ++m) {
       gptr[(size_t)a * 4 + m + 1] = (int)o;
       if (m == 2) break;
@@ -415,7 +424,7 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
           for (int mu = 0; mu < 4; ++mu) gc[((size_t)a * 3 + m + 1) * 4 + mu] += low[mu];
           gp32[o] = single(t);
           for (int mu = 0; mu < np; ++mu)
-            if (4 * fabs(P->sup_val[t * np + mu]) >= top[mu]) (mu < 2 ? gm[o].x : gm[o].y) |= mu % 2 ? (int)0xffff0000 : 0xffff;
+            if (fabs(P->sup_val[t * np + mu]) >= large[mu]) (mu < 2 ? gm[o].x : gm[o].y) |= mu % 2 ? (int)0xffff0000 : 0xffff;
           ++o;
         }
     }
