@@ -648,12 +648,7 @@ cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *
     return CBS_EINVAL;
   }
   if constexpr (sizeof(R) == sizeof(double)) {
-    // Fixed point takes three launches without projectors, the FP64 stencil one: on short marches
-    // of narrow stencils with little work the launch counts (8x8x4 cell, order 4, 1 to 16 systems
-    // of 16 columns: 10.3 against 16.5 us; 30x30x12, order 2, 16 columns in all: 14.4 against
-    // 18.5; but 20x20x10, order 8, one column: 26.7 against 19.9).
-    const bool brief = H.n_atoms == 0 && H.nz * H.m <= 12 && (double)n_sys * H.n * L * (2 + 12 * H.m) < 4e6;
-    if (!brief && fixed_serves(H, n_sys, L, ws_bytes))
+    if (!fp64_quicker(H, n_sys, L) && fixed_serves(H, n_sys, L, ws_bytes))
       return apply_fixed(H, n_sys, L, X, Y, twist, per_col, E, ws, sys_active, st);
   }
   // 32-bit indices inside a system, in the gather too: refused before anything is queued

@@ -8,6 +8,8 @@
 // Scratch: D [n_sys][n_atoms][L][4] FP64, then the images [n_sys][3][n_atoms][4][L] as
 // (high, low) word pairs of both components (images of wrap -1, 0, +1), then the scales
 // [n_sys][L], then the chunk maxima [n_sys][chunks][L].
+#include <math.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -884,6 +886,35 @@ static FixGrid fix_grid(const HamView &H, int n_sys, int L) {
   g.z_chunk = std::min(64, ceil_div(H.nz, zc));   // a block marks its planes in 64 bits
   g.z_blocks = ceil_div(H.nz, g.z_chunk);
   return g;
+}
+
+// Fixed point takes three launches without projectors, the FP64 stencil one, and its tiles of 8 x 8
+// lines and 4 columns are padded where the cell or the block is narrower.  The times of both in
+// microseconds, fitted to 900 cells without projectors (4..96 x 4..96 x 4..32, orders 2..12, 1..64
+// columns and systems, up to 4 M outputs; 9 and 5 per cent off in the mean).  The FP64 march is
+// bound by the latency of a line, in rounds of the blocks that the SMs hold (by registers), or by the
+// FP64 issue of the fullest SM; fixed point by its rounds of two blocks per SM.  A microsecond on top
+// is the host's for two more launches.  The choice was 0.6 per cent from the better of the two in
+// the mean, one of the 900 more than a twentieth slower than the FP64 stencil (62x9x16, order 2,
+// one column of 14 systems: 16.5 against 34 us; 8x8x4, order 4, 16 columns: 10 against 17; but
+// 47x14x6, order 8, 14 columns: 35 against 23).
+bool fp64_quicker(const HamView &H, int n_sys, int L) {
+  const double outputs = (double)n_sys * H.n * L;
+  if (H.n_atoms || outputs > 4e6) return false;
+  static const int resident[kMaxHalf + 1] = {0, 5, 4, 3, 2, 2, 2};   // blocks of the FP64 stencil per SM
+  const int lines = std::max(1, 256 / L), across = ceil_div(H.nx, lines);
+  const double blocks64 = (double)across * H.ny * n_sys;
+  const int widest = ceil_div((int64_t)std::min(H.nx, lines) * L, 32);   // warps of the fullest block
+  const int last = ceil_div((int64_t)(H.nx - (across - 1) * lines) * L, 32);
+  const double mean = across > 1 ? (double)((across - 1) * widest + last) / across : widest;
+  const double latency = H.nz * (0.033 + 0.542 * H.m) * std::max(1.0, blocks64 / (152 * resident[H.m]));
+  const double warps = std::max(ceil(blocks64 / 152) * mean, blocks64 <= 152 ? (double)widest : 0.0);
+  const double fp64 = 4.85 + std::max(latency, warps * H.nz * (2 + 12 * H.m) * 0.0124);
+  const FixGrid g = fix_grid(H, n_sys, L);
+  const int64_t blocks = (int64_t)g.groups * g.tiles * g.z_blocks * n_sys, rest = blocks % 304;
+  const double rounds = 1.64 * (double)(blocks / 304) + (rest == 0 ? 0.0 : rest <= 152 ? 1.0 : 1.64);
+  const double fixed = 10.8 + (g.z_chunk + 2.5) * (0.21 + 0.2 * H.m) * rounds + 7.3e-6 * outputs;
+  return fp64 < fixed + 1;
 }
 
 int fixed_dot_parts(const HamView &H, int n_sys, int L) {

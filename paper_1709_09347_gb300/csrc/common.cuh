@@ -227,6 +227,8 @@ cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *
                    void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st);
 // apply_fixed.cu: complex128 through fixed point
 bool fixed_serves(const HamView &H, int n_sys, int L, size_t ws_bytes);
+// whether the FP64 stencil takes about as long or less on a cell without projectors
+bool fp64_quicker(const HamView &H, int n_sys, int L);
 cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y,
                        const double2 *twist, bool per_col, const double *E, void *ws,
                        const int *sys_active, cudaStream_t st);

@@ -96,3 +96,35 @@ def test_widest_stencil_on_an_alternating_column(modulus):
     X = np.repeat(np.stack([x, x.conj(), x.real, 1j * x.imag], 1)[None], len(z), 0)
     E = np.zeros(len(z))
     _parts_within(cell, z, E, X, _apply(_handle(cell), 0, z, E, X))
+
+
+@pytest.mark.parametrize("L,systems,nx,ny,nz,fd,launches", [
+    (1, 14, 62, 9, 16, 2, 1), (16, 1, 8, 8, 4, 4, 1), (1, 8, 9, 32, 5, 8, 1),
+    (14, 1, 47, 14, 6, 8, 3), (16, 8, 30, 20, 16, 4, 3),
+])
+def test_short_marches_of_few_columns_stay_on_one_launch(L, systems, nx, ny, nz, fd, launches):
+    """Without projectors the FP64 stencil is a single launch, and quicker where there is little to do
+    or where tiles of 8 x 8 lines and 4 columns would be mostly padding; both against the oracle."""
+    need_gpu()
+    from paper_1709_09347_gb300 import cbs
+    cell = _cell(nx, ny, nz, fd, 0)
+    X = _random((systems, cell[0].n, L))
+    z, E = 1.8 * np.exp(1j * np.arange(systems)), np.linspace(-0.5, 0.5, systems)
+    H = _handle(cell)
+    before = cbs.kernel_launches()
+    Y = _apply(H, 0, z, E, X)
+    assert cbs.kernel_launches() - before == launches
+    _parts_within(cell, z, E, X, Y)
+
+
+def test_constant_field_on_a_long_march():
+    """On a constant column the neighbours' coefficients add up to the energy of the FP64 weights (on a
+    cell whose apply runs in fixed point): mean difference to the FP64 kernels below one rounding of
+    E minus the kinetic diagonal (about 30, half an ulp 1.8e-15) and the mean of the 3600 points' own."""
+    cell = _cell(12, 10, 30, 8, 0)
+    X = np.ones((1, cell[0].n, 1), complex)
+    X.imag = 1
+    H, z = _handle(cell), np.array([1.0])
+    a, b = (_apply(H, 0, z, ES[:1], X, k) for k in (False, True))
+    assert not np.array_equal(a, b)
+    assert abs((a - b).real.mean()) < 3e-15 and abs((a - b).imag.mean()) < 3e-15
