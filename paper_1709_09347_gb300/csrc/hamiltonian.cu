@@ -363,85 +363,112 @@ static cbs_status line_projectors(cbs_hamiltonian *h, const cbs_projectors *P, c
   v.fx_fp = h->fx_proj_ok ? std::min(56 - (ilogb(pmax) + 1), 61 - (ilogb(l1max) + 1)) : 0;
   v.fx_db = (float)(dmax * 1.001);
   v.fx_pb = (float)(cover * dmax * 1.001);
+  const double unit = ldexp(1.0, v.fx_fp);
   auto words = [&](int64_t t, int4 *out) {
     int w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int mu = 0; mu < (h->fx_proj_ok ? 4 : 0); ++mu) {
-      const long long f = mu < np ? llrint(ldexp(P->sup_val[t * np + mu], v.fx_fp)) : 0;
+    for (int mu = 0; mu < (h->fx_proj_ok ? np : 0); ++mu) {
+      const long long f = llrint(P->sup_val[t * np + mu] * unit);
       w[2 * mu] = balanced_hi(f);
       w[2 * mu + 1] = balanced_lo(f);
     }
     out[0] = make_int4(w[0], w[1], w[2], w[3]);
     out[1] = make_int4(w[4], w[5], w[6], w[7]);
   };
-  std::vector<int4> pp((size_t)nnz * 2 + 2, make_int4(0, 0, 0, 0)), gp((size_t)nnz * 2);   // one spare entry
-  std::vector<float4> p32((size_t)nnz + 1, make_float4(0, 0, 0, 0)), gp32(nnz);
-  std::vector<int2> gm(nnz, make_int2(0, 0));
-  std::vector<long long> gc((size_t)na * 12, 0);
-  std::vector<int> gi(nnz), gt(nnz), gptr((size_t)na * 4), img((size_t)nnz + 1, 0);
   auto single = [&](int64_t t) {
     float pv[4] = {0, 0, 0, 0};
     for (int mu = 0; mu < np; ++mu) pv[mu] = (float)P->sup_val[t * np + mu];
     return make_float4(pv[0], pv[1], pv[2], pv[3]);
   };
+  // one host buffer, one allocation and one copy for all tables: on small cells those are what they cost
   const int64_t nxy = (int64_t)v.nx * v.ny;
-  std::vector<int> ptr((size_t)nxy * (v.nz + 1));
+  size_t bytes = 0;
+  auto place = [&](size_t count, size_t size) {
+    const size_t at = bytes;
+    bytes += (count * size + 255) & ~(size_t)255;
+    return at;
+  };
+  const size_t n1 = (size_t)nnz + 1;   // a spare entry after the last of the line order
+  const size_t a_pp = place(2 * n1, sizeof(int4)), a_p32 = place(n1, sizeof(float4)), a_img = place(n1, sizeof(int)),
+               a_ptr = place((size_t)nxy * (v.nz + 1), sizeof(int)), a_gp = place(2 * (size_t)nnz, sizeof(int4)),
+               a_gp32 = place(nnz, sizeof(float4)), a_gi = place(nnz, sizeof(int)), a_gt = place(nnz, sizeof(int)),
+               a_gm = place(nnz, sizeof(int2)), a_gc = place((size_t)na * 12, sizeof(long long)),
+               a_gptr = place((size_t)na * 4, sizeof(int));
+  std::vector<unsigned char> host(bytes, 0);
+  unsigned char *hb = host.data();
+  int4 *pp = (int4 *)(hb + a_pp), *gp = (int4 *)(hb + a_gp);
+  float4 *p32 = (float4 *)(hb + a_p32), *gp32 = (float4 *)(hb + a_gp32);
+  int2 *gm = (int2 *)(hb + a_gm);
+  long long *gc = (long long *)(hb + a_gc);
+  int *img = (int *)(hb + a_img), *ptr = (int *)(hb + a_ptr), *gi = (int *)(hb + a_gi), *gt = (int *)(hb + a_gt),
+      *gptr = (int *)(hb + a_gptr);
+  std::vector<int> at(nnz);   // place of an entry in gather order
   int64_t o = 0;
-  for (int64_t line = 0; line < nxy; ++line) {
-    for (int iz = 0; iz < v.nz; ++iz) {
-      const int64_t i = (int64_t)iz * nxy + line;
-      ptr[(size_t)line * (v.nz + 1) + iz] = (int)o;
-      for (int64_t q = pt_ptr[i]; q < pt_ptr[i + 1]; ++q, ++o) {
-        words(pt_ent[q], &pp[2 * o]);
-        p32[o] = single(pt_ent[q]);
-        img[o] = ((int)P->sup_wrap[pt_ent[q]] + 1) * na + pt_atom[q];
-      }
-    }
-    ptr[(size_t)line * (v.nz + 1) + v.nz] = (int)o;
-  }
-  o = 0;
+  std::vector<double> size;
   for (int a = 0; a < na; ++a) {
     // the larger values of each projector: a quarter of the largest, at least six of them (a narrow
     // projector has one or two, and an ordinary column often something small there)
-    double large[4] = {0, 0, 0, 0};
+    double large[4] = {0, 0, 0, 0}, top[4] = {0, 0, 0, 0};
     const int64_t t0 = P->sup_ptr[a], entries = P->sup_ptr[a + 1] - t0;
-    std::vector<double> size(entries);
     for (int mu = 0; mu < np && entries > 0; ++mu) {
+      size.resize(entries);
       for (int64_t t = 0; t < entries; ++t) size[t] = fabs(P->sup_val[(t0 + t) * np + mu]);
       const int64_t sixth = std::min<int64_t>(6, entries) - 1;
       std::nth_element(size.begin(), size.begin() + sixth, size.end(), std::greater<double>());
-      large[mu] = std::min(size[sixth], *std::max_element(size.begin(), size.begin() + sixth + 1) / 4);
+      top[mu] = *std::max_element(size.begin(), size.begin() + sixth + 1);
+      large[mu] = std::min(size[sixth], top[mu] / 4);
     }
     for (int m = -1; m <= 2; ++m) {
       gptr[(size_t)a * 4 + m + 1] = (int)o;
       if (m == 2) break;
-      for (int64_t t = P->sup_ptr[a]; t < P->sup_ptr[a + 1]; ++t)
+      for (int64_t t = t0; t < t0 + entries; ++t)
         if (P->sup_wrap[t] == m) {
           gi[o] = P->sup_idx[t];
           gt[o] = (int)t;
+          at[t] = (int)o;
           words(t, &gp[2 * o]);
           const int4 w0 = gp[2 * o], w1 = gp[2 * o + 1];
           const int low[4] = {w0.y, w0.w, w1.y, w1.w};
           for (int mu = 0; mu < 4; ++mu) gc[((size_t)a * 3 + m + 1) * 4 + mu] += low[mu];
           gp32[o] = single(t);
-          for (int mu = 0; mu < np; ++mu)
-            if (fabs(P->sup_val[t * np + mu]) >= large[mu]) (mu < 2 ? gm[o].x : gm[o].y) |= mu % 2 ? (int)0xffff0000 : 0xffff;
+          for (int mu = 0; mu < np; ++mu) {
+            const double p = fabs(P->sup_val[t * np + mu]);
+            if (p >= large[mu] && (p > 0 || top[mu] == 0)) (mu < 2 ? gm[o].x : gm[o].y) |= mu % 2 ? (int)0xffff0000 : 0xffff;
+          }
           ++o;
         }
     }
   }
-  for (long long &c : gc) c /= 2;   // 2^28 of the 2^29 that a low word stands for
-  cbs_status s;
-  if ((s = upload(h, pp.data(), pp.size(), &v.fx_p)) != CBS_OK) return s;
-  if ((s = upload(h, p32.data(), p32.size(), &v.ln_p32)) != CBS_OK) return s;
-  if ((s = upload(h, img.data(), img.size(), &v.fx_img)) != CBS_OK) return s;
-  if ((s = upload(h, ptr.data(), ptr.size(), &v.fx_ptr)) != CBS_OK) return s;
-  if ((s = upload(h, gp.data(), gp.size(), &v.fx_gp)) != CBS_OK) return s;
-  if ((s = upload(h, gp32.data(), gp32.size(), &v.fx_gp32)) != CBS_OK) return s;
-  if ((s = upload(h, gi.data(), gi.size(), &v.fx_gi)) != CBS_OK) return s;
-  if ((s = upload(h, gc.data(), gc.size(), &v.fx_gc)) != CBS_OK) return s;
-  if ((s = upload(h, gm.data(), gm.size(), &v.fx_gm)) != CBS_OK) return s;
-  if ((s = upload(h, gt.data(), gt.size(), &v.fx_gt)) != CBS_OK) return s;
-  return upload(h, gptr.data(), gptr.size(), &v.fx_gptr);
+  for (int64_t k = 0; k < (int64_t)na * 12; ++k) gc[k] /= 2;   // 2^28 of the 2^29 that a low word stands for
+  o = 0;
+  for (int64_t line = 0; line < nxy; ++line) {
+    for (int iz = 0; iz < v.nz; ++iz) {
+      const int64_t i = (int64_t)iz * nxy + line;
+      ptr[line * (v.nz + 1) + iz] = (int)o;
+      for (int64_t q = pt_ptr[i]; q < pt_ptr[i + 1]; ++q, ++o) {
+        const int64_t g = at[pt_ent[q]];
+        pp[2 * o] = gp[2 * g];
+        pp[2 * o + 1] = gp[2 * g + 1];
+        p32[o] = gp32[g];
+        img[o] = ((int)P->sup_wrap[pt_ent[q]] + 1) * na + pt_atom[q];
+      }
+    }
+    ptr[line * (v.nz + 1) + v.nz] = (int)o;
+  }
+  const unsigned char *dev = nullptr;
+  const cbs_status s = upload(h, hb, bytes, &dev);
+  if (s != CBS_OK) return s;
+  v.fx_p = (const int4 *)(dev + a_pp);
+  v.ln_p32 = (const float4 *)(dev + a_p32);
+  v.fx_img = (const int *)(dev + a_img);
+  v.fx_ptr = (const int *)(dev + a_ptr);
+  v.fx_gp = (const int4 *)(dev + a_gp);
+  v.fx_gp32 = (const float4 *)(dev + a_gp32);
+  v.fx_gi = (const int *)(dev + a_gi);
+  v.fx_gt = (const int *)(dev + a_gt);
+  v.fx_gm = (const int2 *)(dev + a_gm);
+  v.fx_gc = (const long long *)(dev + a_gc);
+  v.fx_gptr = (const int *)(dev + a_gptr);
+  return CBS_OK;
 }
 
 static cbs_status create_impl(const cbs_grid *g, const double *v_loc, const cbs_projectors *P,
