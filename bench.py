@@ -52,10 +52,11 @@ STEP_ENERGIES = {"c3": (3, 11, 19, 27)}
 # kernel's source file hashes to `sha`.  The FP64 shifted-family update has none: its
 # captured launch does not record how many energies were still active.
 KERNEL_TRAFFIC = {
-    # 32x32x16 cell, 32 systems (16 points and their duals), 16.78 M outputs: 745.7 MB
-    ("c128_apply", "c2"): {"file": "apply.cu", "sha": "f77085a5a8f84789", "bytes_per_unit": 44.45},
-    # 64x64x24 cell, 128 systems, 402.7 M outputs: 8.681 GB
-    ("c64_apply", "c3"): {"file": "apply.cu", "sha": "f77085a5a8f84789", "bytes_per_unit": 21.56},
+    # 32x32x16 cell, 32 systems (16 points and their duals), 16.78 M outputs: 888.4 MB, the dual
+    # directions that the stencil reads for (p~, q) among them
+    ("c128_apply", "c2"): {"file": "apply_fixed.cu", "sha": "57b6e97d0f8919a0", "bytes_per_unit": 52.95},
+    # 64x64x24 cell, 32 systems, 100.7 M outputs: 2.145 GB
+    ("c64_apply", "c3"): {"file": "apply.cu", "sha": "8d471e55be2feda6", "bytes_per_unit": 21.31},
 }
 
 FORMS = {
@@ -477,13 +478,14 @@ def main():
                               peak_source=hbm_src, bytes_per_unit=bpu, unit_of_work="complex output",
                               traffic=_traffic("c64_apply", wl.name, p["outputs"] / launches))
                 elif key == "c128":
-                    # 64-bit integer sums, limited by integer issue; the rate against the FP64 peak
-                    # would exceed it, so the bytes are what is compared with a measured peak
+                    # 64-bit integer sums, limited by the latency of their instructions at 16 warps
+                    # per SM; the rate against the FP64 peak would exceed it, so the bytes are what is
+                    # compared with a measured peak
                     fpu, bpu = apply_flops_per_output(wl), apply_bytes_per_output(wl, 16)
                     ach = p["outputs"] * bpu / sec / 1e9
                     rl.update(bound="hbm", achieved=ach, peak=hbm, unit="GB/s", frac=ach / hbm,
                               peak_source=hbm_src, bytes_per_unit=bpu, unit_of_work="complex output",
-                              limiter="integer issue", real_TFLOP_s=p["outputs"] * fpu / sec / 1e12,
+                              limiter="integer instruction latency", real_TFLOP_s=p["outputs"] * fpu / sec / 1e12,
                               traffic=_traffic("c128_apply", wl.name, p["outputs"] / launches))
                 elif c64_family:
                     # per (energy, point, column) triple and grid point: scaled direction and

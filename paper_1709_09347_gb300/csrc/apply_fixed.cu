@@ -154,9 +154,10 @@ __device__ __noinline__ void gather_entries_fp64(const HamView *H, int t0, int t
   for (int mu = 0; mu < 4; ++mu) out[mu] = acc[mu];
 }
 
-// Bound by integer issue and the latency of the gathered rows: 32 systems of the 32x32x16 cell
-// (40 atoms, L = 32) take 194 us (175 without PARTS); the FP64 gather, at FP64 issue, 550 us.  About 90
-// instructions per entry and column, 24 of them products.
+// Bound by the latency of its integer products and of the gathered rows at 16 warps per SM (it issues
+// on 38 per cent of the cycles): 32 systems of the 32x32x16 cell (40 atoms, L = 32) take 194 us (175
+// without PARTS); the FP64 gather, at FP64 issue, 550 us.  About 90 instructions per entry and
+// column, 24 of them products.
 // One block per (atom, system, group of columns); threadIdx.x a column, threadIdx.y a lane over
 // the atom's support entries.  Per entry: one 16-byte load, two conversions and 3 word
 // products per projector and component.  The projector words are balanced (the low word is
@@ -542,9 +543,10 @@ struct Scatter {
 
 // Stencil and projector scatter: 677 us on 32 systems of the 32x32x16 cell (L = 32, 16.8 M
 // outputs), of which the stencil is 360; k_apply_zm<double>, at FP64 issue, 2400 us.  About 480
-// instructions per output for the stencil and 110 per covering entry; bound by their issue and,
-// in the scatter, by the latency of its loads (16 warps per SM at 128 registers, of which the
-// z queue takes 36; the widest stencils, of half-width 5 and 6, spill 30 to 270 bytes per thread).
+// instructions per output for the stencil and 110 per covering entry; they issue on 48 per cent of
+// the cycles, bound by the latency of dependent products, shared-memory reads and the scatter's loads
+// and by the barriers (16 warps per SM at 128 registers, of which the z queue takes 36; the widest
+// stencils, of half-width 5 and 6, spill 30 to 270 bytes per thread).
 // 8 x 8 x 4 tiles of 256 threads beat 16 x 8 x 4 of 512 (two blocks per SM
 // cover each other's barriers) and 8 x 4 x 8; the columns are cut in fours because the halo,
 // converted once per tile, shrinks with the tile's x-y extent.  A block covers TX x TY lines of CG
