@@ -170,7 +170,10 @@ cbs_status cbs_hamiltonian_norms(const cbs_hamiltonian *h, double E, double *n_p
 /* The QEP matrix applied to a batch (Eq. (4)):  Y[s] = P(z_s) X[s] = E_s X[s] - H(z_s) X[s].
  * z: host array of n_sys complex128 twists; E: host array of n_sys energies.
  * X, Y: DEVICE pointers to [n_sys][N][L] blocks of element type dtype (CBS_C128 or
- * CBS_C64).  1 <= L <= 256 (complex64 with even L: <= 512).  Runs on `stream`
+ * CBS_C64).  1 <= L <= 256 (complex64 with even L: <= 512).  Complex128 columns run in 64-bit
+ * fixed point at FP64 accuracy of the real and the imaginary parts; those that it cannot serve
+ * (zero, real, strongly localised or decaying columns, say) run in FP64, at a third of the speed.
+ * Runs on `stream`
  * (cudaStream_t, NULL = legacy default) and synchronises it.  Up to 16 MiB of scratch stay with
  * h, for one call at a time; larger scratch, and that of calls on h that overlap in several
  * threads, is allocated per call and freed. */
