@@ -54,9 +54,9 @@ STEP_ENERGIES = {"c3": (3, 11, 19, 27)}
 KERNEL_TRAFFIC = {
     # 32x32x16 cell, 32 systems (16 points and their duals), 16.78 M outputs: 888.4 MB, the dual
     # directions that the stencil reads for (p~, q) among them
-    ("c128_apply", "c2"): {"file": "apply_fixed.cu", "sha": "57b6e97d0f8919a0", "bytes_per_unit": 52.95},
+    ("c128_apply", "c2"): {"file": "apply_fixed.cu", "sha": "20434ae9b10f3c3f", "bytes_per_unit": 52.95},
     # 64x64x24 cell, 32 systems, 100.7 M outputs: 2.145 GB
-    ("c64_apply", "c3"): {"file": "apply.cu", "sha": "8d471e55be2feda6", "bytes_per_unit": 21.31},
+    ("c64_apply", "c3"): {"file": "apply.cu", "sha": "a1ed3252cc0330aa", "bytes_per_unit": 21.31},
 }
 
 FORMS = {

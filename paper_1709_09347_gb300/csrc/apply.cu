@@ -641,7 +641,7 @@ bool apply_supported(const HamView &H, int L, int dtype, const char *who) {
 template <typename R>
 cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *X,
                    typename CT<R>::T *Y, const double2 *twist, bool per_col, const double *E,
-                   void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st) {
+                   void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st, bool parts) {
   typename CT<R>::T *D = (typename CT<R>::T *)ws;
   if (per_col && !kPerCol<R>) {
     set_error("apply: twists per column need complex128");
@@ -649,7 +649,7 @@ cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *
   }
   if constexpr (sizeof(R) == sizeof(double)) {
     if (!fp64_quicker(H, n_sys, L) && fixed_serves(H, n_sys, L, ws_bytes))
-      return apply_fixed(H, n_sys, L, X, Y, twist, per_col, E, ws, sys_active, st);
+      return apply_fixed(H, n_sys, L, X, Y, twist, per_col, E, ws, sys_active, st, parts);
   }
   // 32-bit indices inside a system, in the gather too: refused before anything is queued
   if ((int64_t)H.n * L >= ((int64_t)1 << 31)) {
@@ -663,10 +663,10 @@ cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *
 
 template cbs_status apply_P<double>(const HamView &, int, int, const double2 *, double2 *,
                                     const double2 *, bool, const double *, void *, size_t,
-                                    const int *, cudaStream_t);
+                                    const int *, cudaStream_t, bool);
 template cbs_status apply_P<float>(const HamView &, int, int, const float2 *, float2 *,
                                    const double2 *, bool, const double *, void *, size_t,
-                                   const int *, cudaStream_t);
+                                   const int *, cudaStream_t, bool);
 template cbs_status launch_proj_gather<double>(const HamView &, int, int, const double2 *,
                                                const double2 *, bool, double2 *, const int *,
                                                cudaStream_t);

@@ -72,11 +72,12 @@ __device__ __forceinline__ uint2 words_around(const HamView &H, const double2 *X
 // One block of (L, lanes) per system: the FP64 work of the scales (a division, the conversions) is
 // done here once instead of by every thread of the kernels that use them.  The lanes share the
 // chunks and the samples of a column; bound by latency, so the samples are loaded beside the maxima.
+// Without `parts` no column is sent to the FP64 formula as a whole.
 __global__ void __launch_bounds__(1024) k_fix_scales(const __grid_constant__ HamView H, int L, int chunks,
                                                      const unsigned *__restrict__ maxhi, const double2 *__restrict__ X,
                                                      const double2 *__restrict__ twist, int per_col,
                                                      const double *__restrict__ E, ColumnScale *__restrict__ scales,
-                                                     const int *__restrict__ sys_active) {
+                                                     const int *__restrict__ sys_active, bool parts) {
   extern __shared__ unsigned smax[];   // [lanes][L], lim [L], poor [L]
   __shared__ int bad[256 / kFixRoute];
   const int s = blockIdx.x, c = threadIdx.x, ly = threadIdx.y, ry = blockDim.y;
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(1024) k_fix_scales(const __grid_constant__ Ham
 #pragma unroll
   for (int j = 0; j < U; ++j) {
     word[j] = ~0u;
-    if (ly + j * ry < kFixSamples) {
+    if (parts && ly + j * ry < kFixSamples) {
       const uint2 v = words_around(H, Xc, L, sample_point(ly + j * ry, H.n));
       word[j] = min(v.x, v.y);
     }
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(1024) k_fix_scales(const __grid_constant__ Ham
   for (int j = 0; j < U; ++j) p += word[j] < lm;
   if (p) atomicAdd(&poor[c], (unsigned)p);
   __syncthreads();
-  if (ly == 0 && (!o.f.ok || poor[c] >= kFixPoor)) bad[c / kFixRoute] = 1;
+  if (parts && ly == 0 && (!o.f.ok || poor[c] >= kFixPoor)) bad[c / kFixRoute] = 1;
   __syncthreads();
   if (ly) return;
   if (bad[c / kFixRoute]) o.skip = 2;
@@ -554,8 +555,10 @@ struct Scatter {
 // halo, as fixed-point pairs (two buffers, one barrier per plane), and each thread keeps the
 // 2 MH + 1 z neighbours of its point in registers.  The next plane's halo and the plane MH ahead
 // are loaded while the current one is computed.  Offsets inside a plane are 32-bit byte offsets
-// from a base that all threads share.  DOT: one of BiCG's iterations, with (p~, q).
-template <int MH, int CG, int TX, int TY, bool ISO, bool DOT>
+// from a base that all threads share.  PARTS: the real and the imaginary parts to the FP64 kernels'
+// accuracy; else the moduli, as BiCG's iterations and its residual check apply it (with (p~, q) over
+// the first dot.n systems).
+template <int MH, int CG, int TX, int TY, bool ISO, bool PARTS>
 __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
     k_stencil_fixed(const __grid_constant__ HamView H, int L, int groups, int tiles_x, int z_chunk,
                     const double2 *__restrict__ X, double2 *__restrict__ Y, const double *__restrict__ E,
@@ -571,7 +574,7 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
   if (sys_active && !sys_active[s]) return;
   const int nx = H.nx, ny = H.ny, nz = H.nz;
   const int g = blockIdx.x % groups, tb = blockIdx.x / groups;
-  if (!DOT && scales[(int64_t)s * L + g * CG].skip) {   // the same for the columns of the block
+  if (PARTS && scales[(int64_t)s * L + g * CG].skip) {   // the same for the columns of the block
     tile_fp64<MH, CG, TX, TY>(H, L, groups, tiles_x, z_chunk, X, Y, E, scales, D);
     return;
   }
@@ -593,8 +596,8 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
   const int base = sc->base;
   const bool own = g * CG + cl < L && bx + lx < nx && by + ly < ny && !sc->skip;
   // (p~, q): this thread's share, for primal systems
-  const bool dotted = DOT && s < dot.n;
-  const char *Xd = Xs + (DOT ? (int64_t)dot.n * H.n * L * (int64_t)sizeof(double2) : 0);
+  const bool dotted = !PARTS && s < dot.n;
+  const char *Xd = Xs + (!PARTS ? (int64_t)dot.n * H.n * L * (int64_t)sizeof(double2) : 0);
   double dx = 0, dy = 0;
   auto add_dot = [&](double2 pd, double2 q) {
     dx = fma(pd.x, q.x, fma(pd.y, q.y, dx));
@@ -696,7 +699,7 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
     }
     __syncthreads();
     const Fixed2 x0 = q[MH];
-    if (DOT && max(absword(x0.re), absword(x0.im)) < kFixSmallWord) {
+    if (!PARTS && max(absword(x0.re), absword(x0.im)) < kFixSmallWord) {
       // small at the point: its nearest neighbours decide (the moduli, since BiCG mixes the parts: its
       // updates round each against the larger one)
       const Fixed2 n[6] = {mid[CG], mid[-CG], mid[WX * CG], mid[-WX * CG], q[MH + 1], q[MH - 1]};
@@ -741,8 +744,8 @@ __global__ void __launch_bounds__(CG *TX *TY, 512 / (CG * TX * TY))
         yi.add(ti.shifted(H.fx_st), H.fx_c1[dir], H.fx_c0[dir]);
       }
     }
-    if (!DOT && ((within((int)(x0.re >> 32), kFixSmallWord) && within(near_re, 8 * kFixSmallWord)) ||
-                 (within((int)(x0.im >> 32), kFixSmallWord) && within(near_im, 8 * kFixSmallWord)))) {
+    if (PARTS && ((within((int)(x0.re >> 32), kFixSmallWord) && within(near_re, 8 * kFixSmallWord)) ||
+                  (within((int)(x0.im >> 32), kFixSmallWord) && within(near_im, 8 * kFixSmallWord)))) {
       // a part that is small at the point, and may be at its nearest neighbours: their sum, which
       // is at hand, is then below 6 times the limit (seldom otherwise)
       const Fixed2 *at = mid;
@@ -925,7 +928,7 @@ int fixed_dot_parts(const HamView &H, int n_sys, int L) {
 }
 
 cbs_status apply_fixed_scaled(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y, const double *E,
-                              void *ws, const int *sys_active, cudaStream_t st, const FixedDot *dot) {
+                              void *ws, const int *sys_active, cudaStream_t st, bool parts, const FixedDot *dot) {
   double2 *D = (double2 *)ws;
   int4 *Df = (int4 *)((char *)ws + (H.n_atoms ? apply_coef_bytes(H, n_sys, L, CBS_C128) : 0));
   const ColumnScale *scales = fixed_scales(H, n_sys, L, ws);
@@ -934,8 +937,8 @@ cbs_status apply_fixed_scaled(const HamView &H, int n_sys, int L, const double2 
     const int py = 256 / cg > 32 ? 32 : 256 / cg;
     const dim3 blk((unsigned)cg, (unsigned)py, 1), grd((unsigned)H.n_atoms, (unsigned)n_sys, (unsigned)groups);
     const size_t sm = (size_t)py * 16 * cg * sizeof(long long) + 4 * cg * sizeof(double2) + 2 * cg * sizeof(int);
-    if (dot) k_gather_fixed<false><<<grd, blk, sm, st>>>(H, L, X, scales, D, Df, sys_active);
-    else k_gather_fixed<true><<<grd, blk, sm, st>>>(H, L, X, scales, D, Df, sys_active);
+    if (parts) k_gather_fixed<true><<<grd, blk, sm, st>>>(H, L, X, scales, D, Df, sys_active);
+    else k_gather_fixed<false><<<grd, blk, sm, st>>>(H, L, X, scales, D, Df, sys_active);
     count_launches(1);
     CBS_CUDA(cudaGetLastError());
   }
@@ -943,21 +946,21 @@ cbs_status apply_fixed_scaled(const HamView &H, int n_sys, int L, const double2 
   const dim3 grd((unsigned)(g.groups * g.tiles), (unsigned)g.z_blocks, (unsigned)n_sys);
   const size_t sm = (size_t)2 * (kFixTX + 2 * H.m) * (kFixTY + 2 * H.m) * kFixCG * sizeof(Fixed2);
   const FixedDot d = dot ? *dot : FixedDot();
-#define FK(MH, ISO, DOT)                                                                                   \
+#define FK(MH, ISO, PARTS)                                                                                 \
   do {                                                                                                     \
     if (sm > 48 * 1024)                                                                                    \
-      CBS_CUDA(cudaFuncSetAttribute(k_stencil_fixed<MH, kFixCG, kFixTX, kFixTY, ISO, DOT>,                 \
+      CBS_CUDA(cudaFuncSetAttribute(k_stencil_fixed<MH, kFixCG, kFixTX, kFixTY, ISO, PARTS>,               \
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));                \
-    k_stencil_fixed<MH, kFixCG, kFixTX, kFixTY, ISO, DOT><<<grd, kFixCG * kFixTX * kFixTY, sm, st>>>(      \
+    k_stencil_fixed<MH, kFixCG, kFixTX, kFixTY, ISO, PARTS><<<grd, kFixCG * kFixTX * kFixTY, sm, st>>>(    \
         H, L, g.groups, g.tiles_x, g.z_chunk, X, Y, E, scales, D, Df, sys_active, d);                      \
   } while (0)
 #define FM(MH)                        \
   case MH:                            \
     if (H.fx_iso) {                   \
-      if (d.n) FK(MH, true, true);    \
+      if (parts) FK(MH, true, true);  \
       else FK(MH, true, false);       \
     } else {                          \
-      if (d.n) FK(MH, false, true);   \
+      if (parts) FK(MH, false, true); \
       else FK(MH, false, false);      \
     }                                 \
     break
@@ -974,7 +977,7 @@ cbs_status apply_fixed_scaled(const HamView &H, int n_sys, int L, const double2 
 
 cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y,
                        const double2 *twist, bool per_col, const double *E, void *ws,
-                       const int *sys_active, cudaStream_t st) {
+                       const int *sys_active, cudaStream_t st, bool parts) {
   ColumnScale *scales = fixed_scales(H, n_sys, L, ws);
   unsigned *maxhi = (unsigned *)(scales + (size_t)n_sys * L);
   int64_t pts;
@@ -984,10 +987,10 @@ cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, dou
       H.n, L, (int)pts, X, maxhi, sys_active);
   const dim3 sblk((unsigned)L, (unsigned)std::min(kFixSamples, 1024 / L), 1);
   k_fix_scales<<<n_sys, sblk, (size_t)(sblk.y + 2) * L * sizeof(unsigned), st>>>(H, L, chunks, maxhi, X, twist, per_col ? 1 : 0,
-                                                                               E, scales, sys_active);
+                                                                               E, scales, sys_active, parts);
   count_launches(2);
   CBS_CUDA(cudaGetLastError());
-  return apply_fixed_scaled(H, n_sys, L, X, Y, E, ws, sys_active, st, nullptr);
+  return apply_fixed_scaled(H, n_sys, L, X, Y, E, ws, sys_active, st, parts, nullptr);
 }
 
 }  // namespace cbs

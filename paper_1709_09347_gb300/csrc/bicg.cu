@@ -651,7 +651,7 @@ cbs_status Bicg<R>::advance(cudaStream_t st, int kk) {
       dot.part = dot_part;
       dot.tail = at;
       if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk], st, cudaEventRecordExternal));
-      CBS_TRY_B(apply_fixed_scaled(H, 2 * n, L, p, q, E, D, sys_active, st, &dot));
+      CBS_TRY_B(apply_fixed_scaled(H, 2 * n, L, p, q, E, D, sys_active, st, false, &dot));
       if (prof) CBS_CUDA(cudaEventRecordWithFlags(prof_ev[2 * kk + 1], st, cudaEventRecordExternal));
       return CBS_OK;
     }

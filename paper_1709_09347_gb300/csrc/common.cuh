@@ -220,17 +220,19 @@ bool apply_supported(const HamView &H, int L, int dtype, const char *who);
 // coefficients D; complex128 scratch of only that size is served by the FP64 kernels.
 size_t apply_coef_bytes(const HamView &H, int n_sys, int L, int dtype);
 size_t apply_ws_bytes(const HamView &H, int n_sys, int L, int dtype);
-// Y = P(w) X for n_sys systems; ws: scratch of ws_bytes
+// Y = P(w) X for n_sys systems; ws: scratch of ws_bytes.  parts: complex128 results are as accurate as
+// the FP64 kernels' in the real and the imaginary part, else in the modulus (as BiCG applies it: its
+// residual check sees the same operator)
 template <typename R>
 cbs_status apply_P(const HamView &H, int n_sys, int L, const typename CT<R>::T *X,
                    typename CT<R>::T *Y, const double2 *twist, bool per_col, const double *E,
-                   void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st);
+                   void *ws, size_t ws_bytes, const int *sys_active, cudaStream_t st, bool parts = true);
 // apply_fixed.cu: complex128 through fixed point
 bool fixed_serves(const HamView &H, int n_sys, int L, size_t ws_bytes);
 // whether the FP64 stencil takes about as long or less on a cell without projectors
 bool fp64_quicker(const HamView &H, int n_sys, int L);
 cbs_status apply_fixed(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y,
                        const double2 *twist, bool per_col, const double *E, void *ws,
-                       const int *sys_active, cudaStream_t st);
+                       const int *sys_active, cudaStream_t st, bool parts);
 
 }  // namespace cbs

@@ -14,8 +14,8 @@
 // units, and the imaginary parts too (k_gather_fixed has its own test, on the terms of its sums).
 // A point without them (one of a real field, say), a column whose largest component is zero, not
 // finite or extreme, and a system whose twist or energy is out of range take the FP64 formula
-// instead, point by point.  Inside BiCG the moduli are looked at: its updates with complex scalars
-// round a part against the larger of the two.
+// instead, point by point.  Inside BiCG and its residual check the moduli are looked at: its updates
+// with complex scalars round a part against the larger of the two.
 #pragma once
 
 #include "tails.cuh"
@@ -175,6 +175,6 @@ struct FixedDot {
 ColumnScale *fixed_scales(const HamView &H, int n_sys, int L, void *ws);
 int fixed_dot_parts(const HamView &H, int n_sys, int L);
 cbs_status apply_fixed_scaled(const HamView &H, int n_sys, int L, const double2 *X, double2 *Y, const double *E,
-                              void *ws, const int *sys_active, cudaStream_t st, const FixedDot *dot);
+                              void *ws, const int *sys_active, cudaStream_t st, bool parts, const FixedDot *dot);
 
 }  // namespace cbs

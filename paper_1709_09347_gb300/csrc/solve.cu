@@ -194,7 +194,7 @@ struct ResidualCheck {
       CBS_CUDA(cudaEventCreate(&e1));
       CBS_CUDA(cudaEventRecord(e0, st));
     }
-    CBS_TRY(apply_P<double>(H, 2 * n, L, Y, R, tw, false, E, D, d_bytes, nullptr, st));
+    CBS_TRY(apply_P<double>(H, 2 * n, L, Y, R, tw, false, E, D, d_bytes, nullptr, st, false));
     if (profile) {
       CBS_CUDA(cudaEventRecord(e1, st));
       CBS_CUDA(cudaEventSynchronize(e1));
