@@ -83,7 +83,9 @@ def test_time_does_not_follow_the_allocator():
         H = cbs.Hamiltonian(g, np.zeros(g.n))
         keep.append((H, cbs.Hamiltonian(synth.Grid(16, 16, 16, 0.4, 0.4, 0.4, 4), np.zeros(4096))))
         best = np.inf
-        for _ in range(3):
+        for k in range(8):
+            if k >= 3 and best < 1.5 * min(times, default=best):
+                break       # what the allocations cause stays however often it is timed
             t = []
             for _ in range(9):
                 torch.cuda.synchronize()
