@@ -158,6 +158,59 @@ __global__ void __launch_bounds__(32 * kFroWarps) k_frobenius(HamView H, double 
   }
 }
 
+// Cells without projectors: the off-diagonal entries are the merged stencil's, the same in every row
+// but for the cell faces, so their squares have a closed form (stencil_norms); what is left is the
+// sum of the diagonal and of its square.  part as above, with zeros in the other places.
+__global__ void k_diag_sums(int64_t n, double diag, const double *__restrict__ vloc, double *part) {
+  __shared__ double red[8][2];
+  double s = 0, s2 = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const double d = diag + vloc[i];
+    s += d;
+    s2 = fma(d, d, s2);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5][0] = s;
+    red[threadIdx.x >> 5][1] = s2;
+  }
+  __syncthreads();
+  if (threadIdx.x < 5) {
+    double t = 0;
+    for (int w = 0; w < 8 && threadIdx.x >= 3; ++w) t += red[w][threadIdx.x - 3];
+    part[(int64_t)blockIdx.x * 5 + threadIdx.x] = t;
+  }
+}
+
+// Squares of the merged stencil entries over all rows, by block (l = 0 off the diagonal, l = +1; l = -1
+// has the same), and what arms that wrap onto their own point add to the diagonal.
+static void stencil_norms(const HamView &v, double *off0, double *plus, double *diag) {
+  *diag = 0;
+  double row = 0;
+  auto wrapped = [&](int n, const double *w) {   // arms along x or y
+    std::vector<double> at(std::min(n, 2 * v.m + 1), 0.0);
+    for (int k = 1; k <= v.m; ++k)
+      for (int sg = -1; sg <= 1; sg += 2) {
+        const int o = n > 2 * v.m ? (sg > 0 ? k : v.m + k) : ((sg * k) % n + n) % n;   // apart where nothing coincides
+        at[o] += w[k];
+      }
+    *diag += at[0];
+    for (size_t o = 1; o < at.size(); ++o) row += at[o] * at[o];
+  };
+  wrapped(v.nx, v.wx);
+  wrapped(v.ny, v.wy);
+  const double nxy = (double)v.nx * v.ny;
+  *off0 = row * (double)v.n;
+  *plus = 0;
+  for (int k = 1; k <= v.m; ++k) {   // arms along z are apart: k <= nz
+    *off0 += nxy * 2.0 * (v.nz - k) * v.wz[k] * v.wz[k];
+    *plus += nxy * k * v.wz[k] * v.wz[k];
+  }
+}
+
 __global__ void k_sum_parts(const double *part, int nparts, double *out) {
   // one block, 128 lanes per sum, the lanes' sums added in order
   __shared__ double lanes[128][5];
@@ -302,14 +355,22 @@ extern "C" cbs_status cbs_hamiltonian_norms(const cbs_hamiltonian *h, double E, 
 static cbs_status compute_norms(cbs_hamiltonian *h) {
   HamView &v = h->v;
   // exact Frobenius norms on the device
-  const int nb = ceil_div(v.n, kFroWarps);
+  const bool bare = v.n_atoms == 0;
+  const int nb = bare ? std::min(304, ceil_div(v.n, 256)) : ceil_div(v.n, kFroWarps);
+  double off0 = 0, plus = 0, diag = 0;
   double *part = nullptr, *out = nullptr;
   int *err = nullptr;
   CBS_CUDA(cudaMalloc(&part, ((size_t)nb * 5 + 6) * sizeof(double)));
   out = part + (size_t)nb * 5;
   err = (int *)(out + 5);
   CBS_CUDA(cudaMemset(err, 0, sizeof(int)));
-  k_frobenius<<<nb, 32 * kFroWarps>>>(v, part, err); cbs::count_launches(1);
+  if (bare) {
+    stencil_norms(v, &off0, &plus, &diag);
+    k_diag_sums<<<nb, 256>>>(v.n, v.diag_kin + diag, v.vloc, part);
+  } else {
+    k_frobenius<<<nb, 32 * kFroWarps>>>(v, part, err);
+  }
+  cbs::count_launches(1);
   k_sum_parts<<<1, 128>>>(part, nb, out); cbs::count_launches(1);
   double res[5];
   int herr = 0;
@@ -320,7 +381,7 @@ static cbs_status compute_norms(cbs_hamiltonian *h) {
   if (e2 != cudaSuccess) return cuda_fail(e2, "Frobenius norm kernel");
   if (herr == 1) { set_error("more than 64 atoms cover one grid point"); return CBS_EINVAL; }
   if (herr == 2) { set_error("projector coupling beyond the neighbouring cells"); return CBS_EINVAL; }
-  h->fro_off0 = res[0]; h->fro_p2 = res[1]; h->fro_m2 = res[2];
+  h->fro_off0 = res[0] + off0; h->fro_p2 = res[1] + plus; h->fro_m2 = res[2] + plus;
   h->diag_sum = res[3]; h->diag_sum2 = res[4];
   return CBS_OK;
 }
